@@ -311,7 +311,8 @@ BF_API int bf_solve(const bf_abstraction *abs, const double *G, const uint8_t *t
 typedef struct {
     int32_t slice_target;
     int32_t fuse_mark;         /* 1: relax marks the next frontier                */
-    int32_t relax_blocks;
+    int32_t relax_blocks;      /* blocks of the relax launch (of the one-launch
+                                  form: its width in SMs)                        */
     int32_t candidates;        /* schedules timed (the default included)          */
     double best_ms;            /* mean solve time of the chosen schedule          */
     double default_ms;         /* the same for the default schedule               */

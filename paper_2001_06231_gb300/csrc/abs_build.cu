@@ -26,6 +26,7 @@
 #include "bf_internal.cuh"
 #include "dynamics.cuh"
 #include "solve_core.cuh"
+#include "word_engine.cuh"
 
 using namespace bfk;
 
@@ -829,6 +830,190 @@ static int build_templates(bf_abstraction* a, cudaStream_t st) {
     return BF_OK;
 }
 
+// Bitmaps of the pairs that have a box, a plane in whole words (warp per word;
+// the masks hold no other record: no mismatch).
+__global__ void k_valid_bits(GridDesc g, const unsigned long long* __restrict__ fmask, int plane_words,
+                             int plane_cells, int S, unsigned* vbits) {
+    const int lane = threadIdx.x & 31;
+    const int nw = gridDim.x * (blockDim.x >> 5);
+    for (int wd = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); wd < S; wd += nw) {
+        const int p = wd / plane_words;
+        const int i = (wd - p * plane_words) * 32 + lane;
+        const unsigned m = i < plane_cells ? (unsigned)fmask[(long long)p * plane_cells + i] : 0u;
+        for (int u = 0; u < g.U; ++u) {
+            const unsigned b = __ballot_sync(0xFFFFFFFFu, (m >> u) & 1u);
+            if (lane == 0) vbits[(long long)u * S + wd] = b;
+        }
+    }
+}
+
+// The word engine's list of record r on plane p (word_engine.cuh); a list that
+// does not fit has bit lookups 0xFF.
+template <int D>
+__device__ __forceinline__ void word_list(const GridDesc& g, unsigned long long r, int p, int plane_bits, int* out) {
+    out[0] = out[kWordHdr] = 0;
+    int w[4] = {1, 1, 1, 1}, rel[4] = {0, 0, 0, 0}, k[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        w[d] = rec_byte(r, 2 * d + 1) & 0x7F;
+        rel[d] = rec_sbyte(r, 2 * d);
+    }
+    if (w[0] == 0) return;                                    // no pair of the plane
+    if (D >= 3) { k[2] = p % g.n[2]; k[3] = p / g.n[2]; }
+#pragma unroll
+    for (int d = 2; d < D; ++d) {
+        int x = k[d] + rel[d];
+        if (g.periodic[d]) x = ((x % g.n[d]) + g.n[d]) % g.n[d];
+        lo[d] = x;
+    }
+    const bool use33 = w[0] >= 3 && w[1] >= 3;
+    const int tab = use33 ? 3 : (w[0] == 1 ? 0 : (w[0] == 2 ? 1 : 2));
+    const int np = w[0] < 3 ? 1 : (w[0] + 2) / 3;
+    const int n1 = use33 ? (w[1] + 2) / 3 : w[1];
+    for (int bits = 0; bits < 2; ++bits) {
+        // positions along dims 2 and 3: every plane, or (bits) two planes at a
+        // time, the last pair shifted back to end on the box's last plane
+        int n23[4] = {1, 1, 1, 1}, pair = 0;
+        for (int d = 2; d < D; ++d) {
+            const bool two = bits && w[d] >= 2;
+            n23[d] = two ? (w[d] + 1) / 2 : w[d];
+            if (two) pair |= d == 2 ? 4 : 8;
+        }
+        const long long L = (long long)np * n1 * n23[2] * n23[3];
+        if (L > (bits ? kWordBits : kWordVals)) { out[0] = 0xFF; return; }
+        int* o = out + (bits ? 1 : kWordVal);
+        int i = 0;
+        for (int j3 = 0; j3 < n23[3]; ++j3)
+            for (int j2 = 0; j2 < n23[2]; ++j2)
+                for (int j1 = 0; j1 < n1; ++j1)
+                    for (int q = 0; q < np; ++q) {
+                        int off = rel[0] + (w[0] < 3 ? 0 : min(3 * q, w[0] - 3));
+                        off += (rel[1] + (use33 ? min(3 * j1, w[1] - 3) : j1)) * (int)g.stride[1];
+                        int j[4] = {0, 0, j2, j3};
+#pragma unroll
+                        for (int d = 2; d < D; ++d) {
+                            if (pair & (d == 2 ? 4 : 8)) j[d] = min(2 * j[d], w[d] - 2);
+                            int x = lo[d] + j[d];
+                            if (g.periodic[d] && x >= g.n[d]) x -= g.n[d];
+                            // planes apart, in cells or in bits of the bitmaps
+                            const int planes = (x - k[d]) * (d == 2 ? 1 : g.n[2]);
+                            off += planes * (bits ? plane_bits : (int)g.stride[2]);
+                        }
+                        o[i++] = off;
+                    }
+        if (bits) {
+            out[0] = (int)L | ((tab + pair) << 8);
+        } else {
+            for (; i & 3; ++i) o[i] = o[0];
+            out[kWordHdr] = (int)L | (tab << 8);
+        }
+    }
+}
+
+template <int D>
+__global__ void k_word_lists(GridDesc g, const unsigned long long* __restrict__ shape, long long P, int plane_bits,
+                             int* out) {
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < P * g.U;
+         e += (long long)gridDim.x * blockDim.x)
+        word_list<D>(g, shape[e], (int)(e / g.U), plane_bits, out + e * kWordEnt);
+}
+
+// Static data of the word engine, where it applies (no mismatch, U <= 32, every
+// list fits).  A plane's bit lookups become one span of words per plane they
+// read, relative to the reader's word; a plane that reads more than kWordSpans
+// planes is always tested.
+static int build_word(bf_abstraction* a, cudaStream_t st) {
+    const GridDesc& g = a->g;
+    const long long pw = (g.stride[2] + 31) / 32;
+    if (!a->d_fmask || g.U > kWordMaxU || a->nplanes * pw * 32 > (1LL << 31) - 64 || a->nplanes >= (1LL << 24)) return BF_OK;
+    const size_t P = (size_t)a->nplanes, U = (size_t)g.U;
+    const int S = (int)(a->nplanes * pw), plane_bits = (int)pw * 32;
+    std::vector<int> lists(P * U * kWordEnt);
+    int* dl = nullptr;
+    unsigned* vb = nullptr;
+    int4* sp = nullptr;
+    cudaError_t e = cudaMalloc((void**)&dl, sizeof(int) * lists.size());
+    if (e == cudaSuccess) {
+        const int nb = grid_blocks((long long)(P * U), 128);
+        switch (g.D) {
+            case 2: k_word_lists<2><<<nb, 128, 0, st>>>(g, a->d_shape, (long long)P, plane_bits, dl); break;
+            case 3: k_word_lists<3><<<nb, 128, 0, st>>>(g, a->d_shape, (long long)P, plane_bits, dl); break;
+            default: k_word_lists<4><<<nb, 128, 0, st>>>(g, a->d_shape, (long long)P, plane_bits, dl); break;
+        }
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(lists.data(), dl, sizeof(int) * lists.size(), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    std::vector<unsigned long long> rec(P * U);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(rec.data(), a->d_shape, sizeof(rec[0]) * rec.size(), cudaMemcpyDeviceToHost);
+    std::vector<int4> spans(P * kWordSpans, make_int4(-1, 0, 0, 0));
+    int vtabs = 0, btabs = 0;
+    bool fits = true;
+    std::map<int, std::pair<int, int>> reach;                          // plane read -> offsets in cells
+    const int n0 = g.n[0], n2 = g.D >= 3 ? g.n[2] : 1, n3 = g.D >= 4 ? g.n[3] : 1;
+    for (size_t p = 0; e == cudaSuccess && p < P && fits; ++p) {
+        reach.clear();
+        const int k2 = (int)(p % n2), k3 = (int)(p / n2);
+        for (size_t u = 0; u < U; ++u) {
+            const int* l = &lists[(p * U + u) * kWordEnt];
+            const int L = l[0] & 0xFF;
+            if (L == 0xFF) { fits = false; break; }
+            if (L == 0) continue;
+            btabs |= 1 << (l[0] >> 8);
+            vtabs |= 1 << (l[kWordHdr] >> 8);
+            const unsigned long long r = rec[p * U + u];
+            int w[4] = {1, 1, 1, 1}, rel[4] = {0, 0, 0, 0};
+            for (int d = 0; d < g.D; ++d) {
+                w[d] = (int)((r >> (16 * d + 8)) & 0x7F);
+                rel[d] = (int)(signed char)((r >> (16 * d)) & 0xFF);
+            }
+            const int lo = rel[1] * n0 + rel[0], hi = (rel[1] + w[1] - 1) * n0 + rel[0] + w[0] - 1;
+            for (int j3 = 0; j3 < w[3]; ++j3)
+                for (int j2 = 0; j2 < w[2]; ++j2) {
+                    const int x2 = ((k2 + rel[2] + j2) % n2 + n2) % n2, x3 = ((k3 + rel[3] + j3) % n3 + n3) % n3;
+                    auto it = reach.find(x2 + n2 * x3);
+                    if (it == reach.end()) reach[x2 + n2 * x3] = {lo, hi};
+                    else it->second = {std::min(it->second.first, lo), std::max(it->second.second, hi)};
+                }
+        }
+        if (reach.size() > (size_t)kWordSpans) {
+            spans[p * kWordSpans].x = -2;
+            continue;
+        }
+        size_t i = 0;
+        for (const auto& q : reach)      // the lookup at bit off reads words off >> 5 and the next
+            spans[p * kWordSpans + i++] = make_int4(q.first, q.second.first >> 5, (q.second.second >> 5) + 1, 0);
+    }
+    if (e == cudaSuccess && (!fits || btabs == 0)) {                  // not for the word engine
+        cudaFree(dl);
+        return BF_OK;
+    }
+    if (e == cudaSuccess) e = cudaMalloc((void**)&vb, sizeof(unsigned) * S * U);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&sp, sizeof(int4) * spans.size());
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(sp, spans.data(), sizeof(int4) * spans.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+        k_valid_bits<<<grid_blocks((long long)S * 32, 256), 256, 0, st>>>(g, a->d_fmask, (int)pw, (int)g.stride[2], S,
+                                                                          vb);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        cudaFree(dl); cudaFree(vb); cudaFree(sp);
+        return bfh::cuda_fail(e, "word engine data");
+    }
+    a->d_vbits = vb;
+    a->d_wlists = dl;
+    a->d_spans = sp;
+    a->word_plane_words = (int)pw;
+    a->word_vtabs = vtabs;
+    a->word_btabs = btabs;
+    a->bytes += sizeof(unsigned) * S * U + sizeof(int4) * spans.size() + sizeof(int) * lists.size();
+    return BF_OK;
+}
+
 static int build_shapes(bf_abstraction* a, cudaStream_t st) {
     if (a->box_fmt != kBoxCompact || a->g.D < 2 || a->g.periodic[0] || a->g.periodic[1]) return BF_OK;
     int rc;
@@ -838,6 +1023,7 @@ static int build_shapes(bf_abstraction* a, cudaStream_t st) {
         default: rc = build_shapes_t<4>(a, st); break;
     }
     if (rc == BF_OK && a->d_shape && a->shape_mismatch == 0) rc = build_templates(a, st);
+    if (rc == BF_OK && a->d_tent) rc = build_word(a, st);
     return rc;
 }
 
@@ -863,6 +1049,9 @@ extern "C" void abs_free(bf_abstraction* a) {
     cudaFree(a->d_tent);
     cudaFree(a->d_uptr);
     cudaFree(a->d_uent);
+    cudaFree(a->d_vbits);
+    cudaFree(a->d_wlists);
+    cudaFree(a->d_spans);
     delete a;
 }
 

@@ -251,6 +251,16 @@ struct bf_abstraction {
     int* d_uptr;              // [2 nplanes + 1], as d_tptr
     int4* d_uent;             // [d_uptr[2 nplanes]]
     double utmpl_rows;        // mean per-input template entries per plane
+    // word engine (word_engine.cuh), where every box is its plane's entry, U <= 32
+    // and every list fits: bitmaps of the pairs that have a box [U][S] (S = P
+    // word_plane_words: a plane in whole words), the lists [P][U][kWordEnt], per
+    // plane the words its bit lookups read [P][kWordSpans], and the value and
+    // bit tables the lists read (bit t = table t); NULL / 0 otherwise
+    unsigned* d_vbits;
+    int* d_wlists;
+    int4* d_spans;
+    int word_plane_words;
+    int word_vtabs, word_btabs;
     // predecessor index [C][2*D] int16 offsets (x = y + off), empty: lo0 > hi0
     short* d_pred;
     double pred_rows;         // mean dim-0 rows of a predecessor box (cells with one)

@@ -21,6 +21,7 @@
 #include <math_constants.h>
 
 #include "solve_core.cuh"
+#include "word_engine.cuh"
 
 using namespace bfk;
 
@@ -29,6 +30,12 @@ struct TileState;
 int tile_setup(const bf_abstraction* a, long long* const tables[4], TileState** out);
 void tile_free(TileState* t);
 int launch_relax_tile(const InstView& v, TileState* t, bool mark, cudaStream_t st);
+
+// Word engine (solve_word.cu).
+int word_wave(int units);
+int word_solve(const WordInst& w, int blocks, cudaStream_t st);
+int word_solve_host(const WordInst& w, int blocks, cudaStream_t st, double* relax_ms, double* rest_ms,
+                    long long* launches);
 
 // Mean predecessor-box rows up to which relax marks the next frontier itself.
 constexpr double kFuseMarkRows = 64.0;
@@ -105,6 +112,12 @@ struct bf_solve_ws {
     long long* M2R = nullptr;
     long long* M3R = nullptr;
     double* stage_GR = nullptr;
+    // word engine (abstractions with d_vbits): used by plain Jacobi solves
+    bool use_word = true;           // bf_tune / bf_set_schedule may switch it off
+    int word_blocks = -1;           // widest launch, 0: not available, -1: not set up yet
+    int word_use = 0;               // launch width in use
+    void* word_mem = nullptr;       // bitmaps of the engine, one allocation
+    WordInst word;                  // views into it
     std::mutex mtx;
 };
 
@@ -122,6 +135,7 @@ void bf_solve_ws_free(bf_solve_ws* w) {
     cudaFree(w->f1bits);
     cudaFree(w->ubits);
     cudaFree(w->fc[0]); cudaFree(w->fc[1]); cudaFree(w->fc_tag);
+    cudaFree(w->word_mem);
     if (w->tile) tile_free(w->tile);
     delete w;
 }
@@ -270,7 +284,7 @@ size_t solve_ws_bytes(const bf_abstraction* a) {
     const size_t C = (size_t)a->g.C, U = (size_t)a->g.U, S = (C + 31) / 32;
     const size_t slice = 2ull * kSliceTargetMax * (size_t)sm_count() * 8 * 8 * 32;
     return C * (6 * 8 + 1 + 4 + 4) + 4 * S * (2 * U + 1) + 2 * 8 * C * U + 8 * C + 8 * C + 2 * C + slice * 12 + slice / 8 + 4 * S +
-           sizeof(Counters);
+           sizeof(Counters) + 8 * C + 160 * S + 8192;
 }
 
 static int ws_get(const bf_abstraction* a, bf_solve_ws** out) {
@@ -282,7 +296,7 @@ static int ws_get(const bf_abstraction* a, bf_solve_ws** out) {
     w->D = a->g.D;
     cudaGetDevice(&w->device);
     w->nwords = (a->g.C + 31) / 32;
-    const long long C = w->C, S = w->nwords;
+    const long long C = w->C;
     cudaError_t e = cudaSuccess;
     auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
     A((void**)&w->Vkey, 8 * C);
@@ -291,14 +305,84 @@ static int ws_get(const bf_abstraction* a, bf_solve_ws** out) {
     A((void**)&w->M3, 8 * C);
     if (w->D >= 2) A((void**)&w->M33, 8 * C);
     A((void**)&w->mu, C);
-    A((void**)&w->fbits, 4 * S);
-    A((void**)&w->cells, 4 * C);
-    A((void**)&w->chg, 4 * C);
-    A((void**)&w->Gint, 8 * C * w->U);
-    A((void**)&w->ctr, sizeof(Counters));
     if (e != cudaSuccess) { bf_solve_ws_free(w); return bfh::cuda_fail(e, "bf_solve workspace"); }
     am->ws = w;
     *out = w;
+    return BF_OK;
+}
+
+// The frontier list, the transposed costs and the counters (once per workspace;
+// the word engine needs none of them).
+static int ws_list(bf_solve_ws* w) {
+    if (w->ctr) return BF_OK;
+    cudaError_t e = cudaSuccess;
+    auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess && !*p) e = cudaMalloc(p, bytes); };
+    A((void**)&w->fbits, 4 * w->nwords);
+    A((void**)&w->cells, 4 * w->C);
+    A((void**)&w->chg, 4 * w->C);
+    A((void**)&w->Gint, 8 * w->C * w->U);
+    A((void**)&w->ctr, sizeof(Counters));
+    if (e != cudaSuccess) return bfh::cuda_fail(e, "bf_solve workspace");
+    return BF_OK;
+}
+
+// Word engine state (once per workspace): [counters][changed and infinite, by
+// parity][not avoid][windows][live words][changed units, by parity][smallest
+// costs], the
+// windows with room for a word before and after.  word_blocks = 0 where the
+// engine does not apply.
+static int ws_word(const bf_abstraction* a, bf_solve_ws* w, cudaStream_t st) {
+    if (w->word_blocks >= 0) return BF_OK;
+    if (!a->d_vbits) { w->word_blocks = 0; return BF_OK; }
+    WordInst& v = w->word;
+    memset(&v, 0, sizeof v);
+    v.g = a->g;
+    v.planes = (int)a->nplanes;
+    v.plane_cells = (int)a->g.stride[2];
+    v.plane_words = a->word_plane_words;
+    v.plane_units = (v.plane_words + 31) / 32;
+    v.unit_words = (v.plane_words + v.plane_units - 1) / v.plane_units;     // even units
+    v.units = v.planes * v.plane_units;
+    v.S = v.planes * v.plane_words;
+    const int blocks = word_wave(v.units);
+    if (blocks == 0) { w->word_blocks = 0; return BF_OK; }
+    auto up = [](size_t n) { return (n + 255) / 256 * 256; };
+    const size_t words = up(4 * (size_t)v.S), units = up((size_t)v.units), win = 2 * words + 512;
+    int nt = 0;
+    for (int t = 0; t < 16; ++t) nt += (a->word_btabs >> t) & 1;
+    const size_t bytes = up(sizeof(WordCtr)) + 5 * words + nt * win + up(4 * (size_t)v.units) + 2 * units +
+                         up(8 * (size_t)w->C);
+    cudaError_t e = cudaMalloc(&w->word_mem, bytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w->word_mem, 0, bytes, st);
+    if (e != cudaSuccess) {
+        cudaFree(w->word_mem);
+        w->word_mem = nullptr;
+        return bfh::cuda_fail(e, "word engine workspace");
+    }
+    unsigned char* p = (unsigned char*)w->word_mem;
+    auto take = [&](size_t n) { unsigned char* q = p; p += n; return q; };
+    v.ctr = (WordCtr*)take(up(sizeof(WordCtr)));
+    v.raw[0] = (uint2*)take(2 * words);
+    v.raw[1] = (uint2*)take(2 * words);
+    v.act = (unsigned*)take(words);
+    for (int t = 0; t < 16; ++t)
+        if ((a->word_btabs >> t) & 1) v.bt[t] = (uint2*)(take(win) + 256);
+    v.live = (unsigned*)take(up(4 * (size_t)v.units));
+    v.flags[0] = take(units);
+    v.flags[1] = take(units);
+    v.gmin = (double*)take(up(8 * (size_t)w->C));
+    v.vtabs = a->word_vtabs;
+    v.btabs = a->word_btabs;
+    v.lists = a->d_wlists;
+    v.vbits = a->d_vbits;
+    v.spans = a->d_spans;
+    v.Vnew = w->Vnew;
+    v.tab[0] = w->Vkey;
+    v.tab[1] = w->M2;
+    v.tab[2] = w->M3;
+    v.tab[3] = w->M33;
+    w->word_blocks = blocks;
+    if (w->word_use < 1 || w->word_use > blocks) w->word_use = blocks;
     return BF_OK;
 }
 
@@ -469,6 +553,8 @@ static void set_blocks(const bf_abstraction* a, bf_solve_ws* w) {
 // Launch shapes and slice buffers (once per workspace; caller holds w->mtx).
 static int ws_blocks(const bf_abstraction* a, bf_solve_ws* w, cudaStream_t st) {
     if (w->relax_blocks) return BF_OK;
+    const int lrc = ws_list(w);
+    if (lrc) return lrc;
     switch (a->g.D) {
         case 1: set_blocks<1>(a, w); break;
         case 2: set_blocks<2>(a, w); break;
@@ -555,6 +641,82 @@ static int stage_in(const void* src, size_t bytes, void** stage, cudaStream_t st
     return BF_OK;
 }
 
+// bf_solve by the word engine (arguments checked, w->mtx held).
+static int solve_by_words(const bf_abstraction* a, bf_solve_ws* w, const double* G, const uint8_t* target,
+                          const uint8_t* avoid, const bf_solve_opts* opts, double* V, uint8_t* mu, int64_t* iters,
+                          int32_t* status, cudaStream_t st) {
+    const long long C = w->C;
+    const double* terminal = opts ? opts->terminal : nullptr;
+    const int flags = opts ? opts->flags : 0;
+    const long long tcap = (opts && opts->trace && opts->trace_cap > 0) ? opts->trace_cap : 0;
+    if (tcap > w->trace_cap) {
+        cudaFree(w->trace);
+        w->trace = nullptr;
+        w->trace_cap = 0;
+        BF_CUDA(cudaMalloc((void**)&w->trace, sizeof(long long) * 4 * tcap));
+        w->trace_cap = tcap;
+        if (w->exec) { cudaGraphExecDestroy(w->exec); w->exec = nullptr; }     // it holds the old buffer
+        if (w->graph) { cudaGraphDestroy(w->graph); w->graph = nullptr; }
+    }
+    if (tcap > 0) BF_CUDA(cudaMemsetAsync(w->trace, 0xFF, sizeof(long long) * 4 * tcap, st));
+    const void *dG, *dT, *dTgt, *dAv;
+    int rc;
+    if ((rc = stage_in(G, sizeof(double) * C * w->U, (void**)&w->stage_G, st, &dG))) return rc;
+    if ((rc = stage_in(terminal, sizeof(double) * C, (void**)&w->stage_T, st, &dT))) return rc;
+    if ((rc = stage_in(terminal ? nullptr : target, C, (void**)&w->stage_tgt, st, &dTgt))) return rc;
+    if ((rc = stage_in(avoid, C, (void**)&w->stage_avoid, st, &dAv))) return rc;
+    const bool vdev = bfh::is_device_ptr(V), mdev = bfh::is_device_ptr(mu);
+    if (!vdev && !w->stage_V) BF_CUDA(cudaMalloc((void**)&w->stage_V, 8 * C));
+    WordInst v = w->word;
+    v.G = (const double*)dG;
+    v.terminal = (const double*)dT;
+    v.target = (const unsigned char*)dTgt;
+    v.avoid = (const unsigned char*)dAv;
+    v.mu = mdev ? mu : w->mu;
+    v.V = vdev ? V : w->stage_V;
+    v.trace = tcap > 0 ? w->trace : nullptr;
+    v.trace_cap = tcap;
+    v.cap = (opts && opts->max_iters > 0 && opts->max_iters < C) ? opts->max_iters : C;
+    BF_CUDA(cudaMemsetAsync(v.ctr, 0, sizeof(WordCtr), st));
+    const bool timed = (flags & BF_FLAG_TIME_KERNELS) != 0;
+    double relax_ms = 0.0, rest_ms = 0.0;
+    long long launches = 1;
+    if (timed || (flags & BF_FLAG_HOST_LOOP))
+        rc = word_solve_host(v, w->word_use, st, timed ? &relax_ms : nullptr, timed ? &rest_ms : nullptr, &launches);
+    else
+        rc = word_solve(v, w->word_use, st);
+    if (rc) return rc;
+    WordCtr hc;
+    if (!vdev) BF_CUDA(cudaMemcpyAsync(V, v.V, 8 * C, cudaMemcpyDeviceToHost, st));
+    if (!mdev) BF_CUDA(cudaMemcpyAsync(mu, v.mu, C, cudaMemcpyDeviceToHost, st));
+    BF_CUDA(cudaMemcpyAsync(&hc, v.ctr, sizeof hc, cudaMemcpyDeviceToHost, st));
+    if (tcap > 0)
+        BF_CUDA(cudaMemcpyAsync(opts->trace, w->trace, sizeof(long long) * 4 * tcap, cudaMemcpyDeviceToHost, st));
+    BF_CUDA(cudaStreamSynchronize(st));
+    if (hc.err) {
+        bfh::set_error("bf_solve: NaN, -inf or |value| > 2^64 in G or the terminal cost");
+        return BF_ERR_INVALID;
+    }
+    if (hc.fault) {
+        bfh::set_error("bf_solve: a block gave up waiting at the grid barrier");
+        return BF_ERR_TIMEOUT;
+    }
+    *iters = hc.round;
+    *status = hc.status;
+    if (opts && opts->stats) {
+        bf_solve_stats* o = opts->stats;
+        o->kernel_launches = launches;
+        o->relaxed_cells = (int64_t)hc.total_relaxed;
+        o->executed_pairs = (int64_t)hc.total_pairs;
+        o->exact_f1_cells = -1;
+        o->changed_cells = (int64_t)hc.total_changed;
+        o->relax_launches = hc.round;
+        o->relax_ms = relax_ms;
+        o->propagate_ms = rest_ms;
+    }
+    return BF_OK;
+}
+
 extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t* target,
                         const uint8_t* avoid, const bf_solve_opts* opts, double* V, uint8_t* mu,
                         int64_t* iters, int32_t* status, void* stream) {
@@ -574,6 +736,13 @@ extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t*
     std::lock_guard<std::mutex> lock(w->mtx);
     const long long C = w->C;
     const int U = w->U;
+    // plain Jacobi solves of abstractions that have its data take the word
+    // engine unless a schedule was set that names another form
+    if (w->use_word && a->d_vbits &&
+        (!opts || (opts->schedule == BF_SCHED_JACOBI && !opts->succ_class && !(opts->flags & BF_FLAG_COUNT_EXACT)))) {
+        if ((rc = ws_word(a, w, st))) return rc;
+        if (w->word_blocks > 0) return solve_by_words(a, w, G, target, avoid, opts, V, mu, iters, status, st);
+    }
     if ((rc = ws_blocks(a, w, st))) return rc;
     // schedule (the graph holds the view by value: rebuild it on a change)
     const int sched = opts ? opts->schedule : BF_SCHED_JACOBI;
@@ -806,12 +975,14 @@ struct Sched {
     int masked = 0;
     int pz = 0;
     bool pfront = false;
+    bool word = false;
+    int wblocks = 0;
 };
 
 static bool same_sched(const Sched& x, const Sched& y) {
     return x.slice == y.slice && x.fuse == y.fuse && x.blocks == y.blocks && x.use33 == y.use33 &&
            x.plane == y.plane && x.tmpl == y.tmpl && x.pair == y.pair && x.occ == y.occ && x.dense == y.dense &&
-           x.masked == y.masked && x.pz == y.pz && x.pfront == y.pfront;
+           x.masked == y.masked && x.pz == y.pz && x.pfront == y.pfront && x.word == y.word && x.wblocks == y.wblocks;
 }
 
 static bool base_plane_on(const Sched& s) { return s.plane; }
@@ -838,6 +1009,8 @@ static void set_schedule(const bf_abstraction* a, bf_solve_ws* w, const Sched& s
         }
     }
     w->pfront = pf;
+    w->use_word = s.word;
+    if (s.wblocks > 0) w->word_use = w->word_blocks > 0 && s.wblocks > w->word_blocks ? w->word_blocks : s.wblocks;
     w->slice_target = s.slice;
     w->fuse_mark = s.fuse;
     w->relax_blocks = s.blocks;
@@ -877,6 +1050,10 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     int rc = tune_time(a, G, target, avoid, &o, V, mu, st, &best);
     bf_solve_ws* w = a->ws;
     if (rc == BF_OK && !w) rc = BF_ERR_CUDA;
+    if (rc == BF_OK) {
+        std::lock_guard<std::mutex> lock(w->mtx);
+        rc = ws_blocks(a, w, st);
+    }
     if (rc) { cudaFree(V); cudaFree(mu); return rc; }
     const int full = w->relax_blocks_full;
     Sched b;
@@ -892,39 +1069,66 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     b.masked = w->masked;
     b.pz = w->pz;
     b.pfront = w->pfront;
+    b.word = w->use_word && w->word_blocks > 0 && o.schedule == BF_SCHED_JACOBI && !o.succ_class;
+    if (b.word) {
+        // the default was the word engine: as a schedule, the pair queue with
+        // the per-input frontier
+        b.use33 = b.plane = b.tmpl = b.pair = b.pfront = true;
+        b.masked = 2;
+        b.fuse = false;
+    }
     out->default_ms = best;
     int tried = 1;
     const bool cls = opts && opts->succ_class;
     const bool has33 = w->M33 && !cls, hasp = a->d_poffs[0] && !cls, hast = a->d_tent != nullptr;
     const bool hasd = !cls && ws_tile(a, w, st) == BF_OK;
-    // two whole schedules first (the pair-queue relax, with the per-input
-    // frontier and marking in its own launch, or without it and marking in
-    // relax): their settings help each other, which one dimension at a time
-    // would not find
-    if (hasp && has33 && a->d_fmask) {
-        for (int k = 0; k < 2 && rc == BF_OK; ++k) {
+    // time one schedule and keep it when it is the fastest so far
+    auto attempt = [&](const Sched& c) {
+        set_schedule(a, w, c);
+        double ms = 0.0;
+        rc = tune_time(a, G, target, avoid, &o, V, mu, st, &ms);
+        ++tried;
+        if (rc == BF_OK && ms < best) {
+            best = ms;
+            b = c;
+        }
+    };
+    // the word engine's width: fewer blocks make its barriers cheaper and leave
+    // each more work (4 widths)
+    if (b.word) {
+        b.wblocks = w->word_use;
+        const int wide = w->word_blocks;
+        for (int k = 0; k < 5 && rc == BF_OK; ++k) {
             Sched c = b;
+            c.wblocks = k == 0 ? wide : (wide * (5 - k) + 5) / 6;      // all, 2/3, 1/2, 1/3, 1/6
+            if (c.wblocks < 1 || same_sched(c, b)) continue;
+            attempt(c);
+        }
+    }
+    // whole schedules (the pair-queue relax, with the per-input frontier and
+    // marking in its own launch, or without it and marking in relax): their
+    // settings help each other, which one dimension at a time would not find.
+    // Against the word engine also the form every abstraction has (the lists in
+    // turn) and the cell masks in turn.
+    if (hasp && has33 && a->d_fmask) {
+        const Sched from = b;
+        for (int k = 0; k < (from.word ? 4 : 2) && rc == BF_OK; ++k) {
+            Sched c = from;
             c.use33 = true;
             c.plane = true;
             c.tmpl = hast;
-            c.masked = 2;
+            c.masked = k < 2 ? 2 : 3 - k;
             c.pair = true;
             c.pfront = k == 0 && a->d_uent != nullptr;
             c.fuse = k != 0;
-            if (same_sched(c, b)) continue;
-            set_schedule(a, w, c);
-            double ms = 0.0;
-            rc = tune_time(a, G, target, avoid, &o, V, mu, st, &ms);
-            ++tried;
-            if (rc == BF_OK && ms < best) {
-                best = ms;
-                b = c;
-            }
+            c.word = false;
+            if (same_sched(c, from)) continue;
+            attempt(c);
         }
     }
     // coordinate descent: each dimension's values with the others at the best
-    // so far, two rounds
-    for (int round = 0; round < 2 && rc == BF_OK; ++round) {
+    // so far, two rounds (all are dimensions of the list form)
+    for (int round = 0; round < 2 && rc == BF_OK && !b.word; ++round) {
         for (int dim = 0; dim < 12 && rc == BF_OK; ++dim) {
             const int nval = (dim == 0 || dim == 9) ? 4 : (dim == 7 ? 3 : (dim == 10 ? a->g.D - 1 : 2));
             if (dim == 7 && !hasd) continue;
@@ -956,14 +1160,7 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
                     default: c.pfront = k != 0; break;
                 }
                 if (same_sched(c, base)) continue;
-                set_schedule(a, w, c);
-                double ms = 0.0;
-                rc = tune_time(a, G, target, avoid, &o, V, mu, st, &ms);
-                ++tried;
-                if (rc == BF_OK && ms < best) {
-                    best = ms;
-                    b = c;
-                }
+                attempt(c);
             }
         }
     }
@@ -974,7 +1171,7 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     out->slice_target = b.slice;
     out->fuse_mark = b.fuse ? 1 : 0;
     out->window33 = b.use33 && w->M33 ? 1 : 0;
-    out->relax_blocks = b.blocks;
+    out->relax_blocks = b.word ? b.wblocks : b.blocks;
     out->plane_lists = (b.plane && hasp) ? 1 : 0;
     out->templates = (b.tmpl && hast) ? 1 : 0;
     out->pair_inputs = (b.pair && b.plane && hasp) ? 1 : 0;
@@ -1024,6 +1221,10 @@ extern "C" int bf_set_schedule(const bf_abstraction* a, const bf_tune_result* sc
     }
     c.pz = sched->pair_dim;
     c.pfront = sched->input_frontier != 0;
+    // the per-input frontier of the pair-queue form: the word engine, where the
+    // abstraction has its data
+    c.word = c.plane && c.tmpl && c.masked == 2 && c.pfront;
+    c.wblocks = sched->relax_blocks > 0 ? sched->relax_blocks : (w->word_blocks > 0 ? w->word_blocks : 1 << 20);
     if (c.pz != 0 && (c.pz < 2 || c.pz >= a->g.D)) {
         bfh::set_error("bf_set_schedule: pair_dim %d outside 0, 2 .. D - 1", c.pz);
         return BF_ERR_INVALID;

@@ -1,0 +1,910 @@
+// word_engine.cuh -- Algorithm 1 (Sec. IV-A) on bitmap words, for abstractions
+// whose every box is its plane's entry (plane shape table without mismatch):
+// all passes of a solve in one cooperative kernel.
+//
+// Of the pairs (x, u) whose box holds a cell changed in the previous pass (the
+// per-input frontier) most still have a cell of infinite value in their box,
+// so their candidate is +inf and they change nothing: on the fire model
+// 100 x 100 x 36 x 8 x 15 110 M such pairs are met over a solve, 34 M of them
+// with a finite box.  Both tests -- a changed cell in the box, no infinite
+// cell in the box -- are answered for 32 cells of one input at once, from
+// bitmaps over the cells whose entry says "the window of cells here holds a
+// changed (an infinite) cell".  The windows are those of the value tables (one
+// cell, 2 and 3 cells along dim 0, 3 x 3 cells on dims 0-1), each also over
+// two planes along dims 2 and 3, so a box takes a few unaligned 32-bit reads.
+// Only the pairs that pass both tests gather values.
+//
+// Bitmaps hold every plane (the cells with equal coordinates on dims >= 2) in
+// whole words, so a word's cells share their boxes' offsets, and a unit -- up
+// to 32 consecutive words of a plane, one per lane -- shares its lists.
+//
+// One pass, two phases with a grid barrier after each:
+//   relax   the units none of whose lookups can meet a changed entry are
+//           skipped (the planes' lookups as spans of words against one bit per
+//           word); of the others a warp takes one input at a time, lane per
+//           word, and the pairs of the masks go to a queue in shared memory; a
+//           thread takes a pair (its lookups and its cost in flight together),
+//           the smallest candidate of a cell wins, the lowest input among
+//           equals.
+//   tables  the windows of the units that hold a changed cell nearby; the
+//           value tables are recomputed at entries whose window holds a
+//           changed cell and no infinite one (entries with an infinite cell
+//           are never gathered), a thread per entry.
+// V, the tables and the bitmaps stay in the L2; the costs are read in the
+// caller's layout [C][U], only by the pairs that pass the tests.
+#pragma once
+#include "solve_core.cuh"
+
+namespace bfk {
+
+constexpr int kWordThreads = 1024;
+constexpr int kWordWarps = kWordThreads / 32;
+constexpr int kWordSpans = 32;        // spans of a plane's lookups
+constexpr int kWordUnits = 32;        // units a block relaxes at a time (a batch), at most
+constexpr int kWordRows = 320;        // ... and (unit, input) rows
+constexpr int kWordSlots = 192;       // words of a batch whose cells' candidates are kept at a time
+constexpr int kWordPer = 4;           // pairs of a thread at a time
+constexpr int kWordPairs = 6144;      // pair queue of a block
+constexpr int kWordHead = 8;          // value lookups of a list kept in shared memory
+constexpr int kWordEntries = 4096;    // table entries queued by a block
+constexpr int kWordMaxU = 32;
+constexpr int kWordTest = 256;        // units tested at a time
+constexpr unsigned kWordSpinMax = 1u << 22;
+constexpr long long kNoCand = 0x7FFFFFFFFFFFFFFFLL;
+
+// List of a (plane, input): int 0 = bit lookups | bit table << 8, ints 1 .. 31
+// their offsets in bits of the bitmaps; int 32 = value lookups | value table
+// << 8, ints 36 .. 95 their offsets in cells (padded to a multiple of 4 with
+// the first).  A count of 0: no pair of the plane has a box.  Bit table = value
+// table (0..3 = cell, 2 and 3 cells along dim 0, 3 x 3) + 4 when over two
+// planes along dim 2 + 8 when along dim 3.
+constexpr int kWordBits = 31;
+constexpr int kWordVals = 60;
+constexpr int kWordHdr = kWordBits + 1;          // the value lookups' header
+constexpr int kWordVal = kWordHdr + 4;           // their first offset
+constexpr int kWordEnt = kWordVal + kWordVals;
+
+struct WordCtr {
+    unsigned bar;                     // arrivals at the barrier after the set-up and the tables phases
+    int err;                          // invalid input seen during set-up
+    int fault;                        // a block gave up waiting at a barrier
+    int status;
+    int done;
+    long long round;                  // passes completed
+    unsigned long long gate[4];       // barrier after the relax phase of pass r: gate[r & 3] = blocks arrived |
+                                      // blocks with frontier cells << 16 | blocks with changed cells << 32
+    unsigned long long sums[4];       // pass r: frontier cells << 32 | changed cells in sums[r & 3]
+    unsigned long long total_relaxed, total_changed, total_pairs;
+};
+
+struct WordInst {
+    GridDesc g;
+    int planes, plane_cells;          // P, cells of a plane
+    int plane_words;                  // words of a plane: bit b of word p plane_words + k = cell 32 k + b of plane p
+    int unit_words, plane_units;      // words of a unit (the last of a plane may have fewer), units of a plane
+    int units;                        // P plane_units
+    int S;                            // P plane_words
+    int vtabs;                        // bit t: some list gathers from value table t
+    int btabs;                        // bit t: some list tests bit table t
+    const int* lists;                 // [P][U][kWordEnt]
+    const unsigned* vbits;            // [U][S] bit = the pair has a box
+    const int4* spans;                // [P][kWordSpans] {plane q, first, last word relative to the reader's, 0}: the
+                                      // words of q the plane's bit lookups read; q = -1: none, -2: anything
+    const double* G;                  // [C][U] the caller's costs
+    const double* terminal;           // [C] or NULL
+    const unsigned char* target;
+    const unsigned char* avoid;       // or NULL
+    long long* Vnew;                  // [C] keys
+    double* gmin;                     // [C] smallest cost of a cell's inputs
+    long long* tab[4];                // V at the start of the pass (kept when lists gather it), M2, M3, M33
+    uint2* raw[2];                    // [S] by pass parity: {cells changed in the pass, cells of infinite value}
+    unsigned char* flags[2];          // [units] by pass parity: some cell of the unit changed
+    unsigned* act;                    // [S] cells that are not avoid cells
+    uint2* bt[16];                    // [-1 .. S] {window holds a changed cell, ... an infinite cell}
+    unsigned* live;                   // [units] bit = some window of the word holds a changed cell
+    unsigned char* mu;                // [C]
+    double* V;                        // [C] output
+    WordCtr* ctr;
+    long long* trace;                 // [trace_cap][4] or NULL
+    long long trace_cap;
+    long long cap;                    // most passes
+};
+
+struct WordSmem {
+    long long best[kWordSlots * 32];          // smallest candidate of a slot's cells (kNoCand between windows)
+    unsigned bu[kWordSlots * 32];             // its lowest input
+    union {
+        struct {
+            unsigned pair[kWordPairs];        // slot of the window << 13 | bit << 8 | input, ~0: none
+            int4 list[kWordRows][1 + kWordHead / 4];    // (unit, input) rows: the value list's head
+            unsigned mask[kWordRows][32];     // ... the pairs to relax, by word
+            short over[kWordRows];            // rows whose pairs did not fit the queue, -1: queued since
+            unsigned f1[kWordUnits * 32];     // frontier cells of the batch's words
+            unsigned short slot[kWordUnits * 32];       // words with pairs: their slot in the batch, 0xFFFF: none
+            unsigned short word[kWordUnits * 32];       // slots: unit of the batch << 5 | word
+            int4 at[kWordSlots];              // slots of the window: {first cell, word, first row, plane}
+            int4 unit[kWordTest];             // units to relax {unit, plane | words << 24, first word, first cell}
+        } r;
+        struct {
+            int cell[kWordEntries];           // entries to recompute, -1: none
+        } t;
+    };
+    unsigned queued;                          // queue length
+    int nover;                                // rows that did not fit
+    int nslots;
+    int nlive;
+    int flag;
+    unsigned long long gate;
+    unsigned long long part[kWordWarps];
+};
+
+// ---------------------------------------------------------------------------
+// grid barrier (cooperative launch: every block is resident)
+// ---------------------------------------------------------------------------
+// Both barriers: every thread's writes before are visible to every thread
+// after (block barrier, fence and arrival of thread 0; acquire, fence, block
+// barrier).  A wait that gives up sets `fault` and the block leaves the kernel.
+
+// After the set-up and the tables phases; `target` counts arrivals over the
+// kernel's life.
+__device__ __forceinline__ bool word_barrier(WordCtr* k, unsigned& target, WordSmem& sm) {
+    __syncthreads();
+    target += gridDim.x;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&k->bar, 1u);
+        unsigned v, n = 0;
+        int ok = 1;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&k->bar) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if (++n > kWordSpinMax) { ok = 0; atomicExch(&k->fault, 1); break; }
+        }
+        __threadfence();
+        sm.flag = ok;
+    }
+    __syncthreads();
+    return sm.flag != 0;
+}
+
+// After the relax phase of pass r: the arrivals carry whether any block saw a
+// frontier cell and whether any cell changed, so the loop condition costs no
+// further read (a line that every warp reads takes microseconds).  count: the
+// warp's frontier cells << 32 | changed cells (lane 0).  Returns the gate's
+// value, 0 when the wait gave up.
+__device__ __forceinline__ unsigned long long word_gate(WordCtr* k, long long r, unsigned long long count,
+                                                        WordSmem& sm) {
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) sm.part[threadIdx.x >> 5] = count;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        unsigned long long s = lane < kWordWarps ? sm.part[lane] : 0ull;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+        if (lane == 0) {
+            if (s) atomicAdd(&k->sums[r & 3], s);
+            __threadfence();
+            unsigned long long* g = &k->gate[r & 3];
+            atomicAdd(g, 1ull + ((s >> 32) ? 1ull << 16 : 0ull) + ((s & 0xFFFFFFFFull) ? 1ull << 32 : 0ull));
+            unsigned long long v;
+            unsigned n = 0;
+            for (;;) {
+                asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(g) : "memory");
+                if ((v & 0xFFFFull) >= gridDim.x) break;
+                if (++n > kWordSpinMax) { v = 0ull; atomicExch(&k->fault, 1); break; }
+            }
+            __threadfence();
+            sm.gate = v;
+        }
+    }
+    __syncthreads();
+    return sm.gate;
+}
+
+// Exclusive prefix sum of n over the warp; *tot the total.
+__device__ __forceinline__ unsigned word_scan(unsigned n, unsigned& tot) {
+    const int lane = threadIdx.x & 31;
+    unsigned pre = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned x = __shfl_up_sync(0xFFFFFFFFu, pre, o);
+        if (lane >= o) pre += x;
+    }
+    tot = __shfl_sync(0xFFFFFFFFu, pre, 31);
+    return pre - n;
+}
+
+// ---------------------------------------------------------------------------
+// set-up: lines 1-9 of Algorithm 1
+// ---------------------------------------------------------------------------
+
+// Bit pattern test of clean_cost: NaN, -inf and |finite| > 2^64 are errors.
+__device__ __forceinline__ bool bad_cost(long long b) {
+    return (unsigned long long)(b & 0x7FFFFFFFFFFFFFFFLL) > 0x43F0000000000000ULL && b != kKeyInf;
+}
+
+// Costs staged by a warp at a time: its cells' rows, padded to an odd stride so
+// that a lane per cell reads its row without bank conflicts.
+constexpr int kWordSlab = 544;
+
+// W = terminal cost, mu = U (hand over), the bitmaps, and one pass over the
+// costs: checked, and the smallest of a cell kept (a bound that spares most
+// pairs their cost and their other lookups).  A stream at the HBM rate: 345 MB
+// on the fire model.
+__device__ __forceinline__ void word_init(const WordInst& w, double* slabs) {
+    const int lane = threadIdx.x & 31;
+    const int U = w.g.U;
+    const double inf = __longlong_as_double(kKeyInf);
+    double* slab = slabs + (threadIdx.x >> 5) * kWordSlab;
+    const unsigned per = (65536u + (unsigned)U - 1u) / (unsigned)U;      // i / U = i per >> 16 for i < 512
+    const unsigned pad = (U & 1) ? 0u : 1u;
+    const int nc = U <= 16 ? 32 : 16;                                    // cells staged at a time
+    bool bad = false;
+    for (int wd = blockIdx.x * kWordWarps + (int)(threadIdx.x >> 5); wd < w.S; wd += gridDim.x * kWordWarps) {
+        const int p = wd / w.plane_words;
+        const int i0 = (wd - p * w.plane_words) * 32;
+        const int nv = min(32, w.plane_cells - i0);
+        const long long c0 = (long long)p * w.plane_cells + i0;
+        bool fin = false, av = false;
+        if (lane < nv) {
+            const long long c = c0 + lane;
+            double x;
+            if (w.terminal) {
+                if (!clean_cost(w.terminal[c], x)) { bad = true; x = inf; }
+            } else {
+                x = w.target[c] ? 0.0 : inf;
+            }
+            av = w.avoid && w.avoid[c];
+            if (av) x = inf;
+            const long long k = key_of(x);
+            fin = k != kKeyInf;
+            w.Vnew[c] = k;
+            w.mu[c] = kHandover;
+        }
+        const unsigned im = __ballot_sync(0xFFFFFFFFu, lane < nv);
+        const unsigned f = __ballot_sync(0xFFFFFFFFu, fin);
+        const unsigned a = __ballot_sync(0xFFFFFFFFu, av);
+        if (lane == 0) {
+            w.raw[1][wd] = make_uint2(f, im & ~f);  // "changed" before pass 0
+            w.act[wd] = im & ~a;
+        }
+        for (int h = 0; h < nv; h += nc) {
+            const int n = min(nc, nv - h);
+            const long long* src = reinterpret_cast<const long long*>(w.G) + (c0 + h) * U;
+            long long v[16];
+#pragma unroll
+            for (int q = 0; q < 16; ++q) v[q] = q * 32 + lane < n * U ? __ldcs(src + q * 32 + lane) : 0ll;
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const unsigned i = (unsigned)(q * 32 + lane);
+                bad |= bad_cost(v[q]);
+                if ((int)i < n * U) slab[i + ((i * per) >> 16) * pad] = __longlong_as_double(v[q]);
+            }
+            __syncwarp();
+            if (lane < n) {
+                const double* row = slab + lane * (U + (int)pad);
+                double m = row[0];
+                for (int u = 1; u < U; ++u) m = row[u] < m ? row[u] : m;
+                w.gmin[c0 + h + lane] = m;
+            }
+            __syncwarp();
+        }
+    }
+    if (bad) atomicOr(&w.ctr->err, 1);
+}
+
+// No candidates yet (once per kernel; word_commit restores it).
+__device__ __forceinline__ void word_start(WordSmem& sm) {
+    for (int i = threadIdx.x; i < kWordSlots * 32; i += kWordThreads) {
+        sm.best[i] = kNoCand;
+        sm.bu[i] = 0xFFu;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// relax
+// ---------------------------------------------------------------------------
+
+// Words of unit un: its plane, its first word in the plane, its word count.
+__device__ __forceinline__ void word_unit(const WordInst& w, int un, int& p, int& k, int& n) {
+    p = un / w.plane_units;
+    k = (un - p * w.plane_units) * w.unit_words;
+    n = min(w.unit_words, w.plane_words - k);
+}
+
+// Can a lookup of the words k .. k + n - 1 of plane p meet a changed entry?
+// (whole warp; lanes take the plane's spans)
+__device__ __forceinline__ bool word_live(const WordInst& w, int p, int k, int n) {
+    const int lane = threadIdx.x & 31;
+    const int4 sp = __ldg(w.spans + (long long)p * kWordSpans + lane);
+    unsigned hit = sp.x == -2 ? 1u : 0u;
+    if (sp.x >= 0) {
+        const int a = max(k + sp.y, 0), b = min(k + n - 1 + sp.z, w.plane_words - 1);
+        if (a <= b) {
+            const int ua = a / w.unit_words, ub = b / w.unit_words;
+            const unsigned* l = w.live + (long long)sp.x * w.plane_units;
+#pragma unroll 4
+            for (int j = ua; j <= ub; ++j) {
+                const int lo = max(a - j * w.unit_words, 0), hi = min(b - j * w.unit_words, 31);
+                hit |= l[j] & bit_range(lo, hi);
+            }
+        }
+    }
+    return __any_sync(0xFFFFFFFFu, hit != 0u);
+}
+
+// One lookup of word wd: the 32 bits from its first on, moved by off.
+__device__ __forceinline__ void word_lookup(const uint2* at, int off, unsigned& chg, unsigned& inf) {
+    const uint2* q = at + (off >> 5);
+    const uint2 x = q[0], y = q[1];
+    chg |= __funnelshift_r(x.x, y.x, off);
+    inf |= __funnelshift_r(x.y, y.y, off);
+}
+
+// Masks of a word's cells for one input (vb: the pairs with a box): f1 those
+// whose box holds a changed cell, the result those whose box holds no infinite
+// cell either.
+__device__ __forceinline__ unsigned word_mask(const WordInst& w, const int* list, int wd, unsigned vb,
+                                              unsigned& f1) {
+    const int4 e0 = __ldg(reinterpret_cast<const int4*>(list)), e1 = __ldg(reinterpret_cast<const int4*>(list) + 1);
+    const int L = e0.x & 0xFF;
+    f1 = 0u;
+    if (vb == 0u) return 0u;
+    const uint2* at = w.bt[e0.x >> 8] + wd;
+    unsigned chg = 0u, inf = 0u;
+    word_lookup(at, e0.y, chg, inf);
+    if (L > 1) word_lookup(at, e0.z, chg, inf);
+    if (L > 2) word_lookup(at, e0.w, chg, inf);
+    if (L > 3) word_lookup(at, e1.x, chg, inf);
+    if (L > 4) {
+        word_lookup(at, e1.y, chg, inf);
+        if (L > 5) word_lookup(at, e1.z, chg, inf);
+        if (L > 6) word_lookup(at, e1.w, chg, inf);
+        for (int j = 7; j < L; ++j) word_lookup(at, __ldg(list + 1 + j), chg, inf);
+    }
+    f1 = vb & chg;
+    return f1 & ~inf;
+}
+
+// Queue the pairs of a row's masks m (whole warp; tag: the lane's word's slot and
+// the input).  False: they do not fit.
+__device__ __forceinline__ bool word_queue(WordSmem& sm, unsigned m, unsigned tag) {
+    if (!__any_sync(0xFFFFFFFFu, m != 0u)) return true;
+    const int lane = threadIdx.x & 31;
+    unsigned tot, at = 0u;
+    unsigned pos = word_scan((unsigned)__popc(m), tot);
+    if (lane == 0) at = atomicAdd(&sm.queued, tot);
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    if (at + tot > (unsigned)kWordPairs) {           // the queue's last places hold nothing
+        for (unsigned i = at + lane; i < (unsigned)kWordPairs; i += 32) sm.r.pair[i] = ~0u;
+        return false;
+    }
+    for (pos += at; m; m &= m - 1u) sm.r.pair[pos++] = tag + ((unsigned)(__ffs(m) - 1) << 8);
+    return true;
+}
+
+// Work the queued pairs off (whole block): a thread per pair, the smallest
+// candidate of a cell so far and its lowest input.  A pair whose cell's smallest
+// cost plus two of its lookups already reaches W cannot lower it: three of four
+// pairs go that way on the fire model (two of three on the unicycle), without
+// their own cost (from HBM) and their other lookups; the rest move together,
+// warp by warp.  A queue that gives a thread one pair at most skips the test:
+// it only adds a round of loads then.
+__device__ __forceinline__ void word_pairs(const WordInst& w, WordSmem& sm) {
+    const int np = (int)min(sm.queued, (unsigned)kWordPairs);
+    const int U = w.g.U;
+    const int lane = threadIdx.x & 31;
+    for (int k0 = 0; k0 < np; k0 += kWordPer * kWordThreads) {
+        // this thread's places: own[j kWordThreads]
+        unsigned* own = sm.r.pair + k0 + threadIdx.x;
+        int n = 0;                                         // the warp's pairs that are left
+        if (np <= kWordThreads) {
+            n = __popc(__ballot_sync(0xFFFFFFFFu, (int)threadIdx.x < np));
+        } else {
+#pragma unroll
+            for (int j0 = 0; j0 < kWordPer; j0 += 2) {
+                unsigned e[2];
+                long long v[2], a[2], b[2];
+                double gm[2];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    e[j] = k0 + (j0 + j) * kWordThreads + (int)threadIdx.x < np ? own[(j0 + j) * kWordThreads] : ~0u;
+                    v[j] = kKeyMin;                        // no pair: W below every candidate
+                    gm[j] = 0.0;
+                    a[j] = b[j] = kKeyInf;
+                    if (e[j] != ~0u) {
+                        const int4 at = sm.r.at[e[j] >> 13];
+                        const int c = at.x + (int)((e[j] >> 8) & 31u);
+                        const int* l = reinterpret_cast<const int*>(sm.r.list[at.z + (int)(e[j] & 0xFFu)]);
+                        const long long* tb = w.tab[l[0] >> 8] + c;
+                        v[j] = w.Vnew[c];
+                        gm[j] = w.gmin[c];
+                        a[j] = tb[l[4]];
+                        b[j] = tb[l[3 + min(l[0] & 0xFF, kWordHead)]];
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const bool left = key_of(gm[j] + val_of(max(a[j], b[j]))) < v[j];
+                    const unsigned m = __ballot_sync(0xFFFFFFFFu, left);
+                    if (left) {
+                        const int s = n + __popc(m & ((1u << lane) - 1u));
+                        // place s of the warp: every place up to it was read
+                        sm.r.pair[k0 + (s >> 5) * kWordThreads + ((int)threadIdx.x & ~31) + (s & 31)] = e[j];
+                    }
+                    n += __popc(m);
+                }
+            }
+            __syncwarp();
+        }
+        long long d[kWordPer];
+#pragma unroll
+        for (int j = 0; j < kWordPer; ++j) {
+            d[j] = kNoCand;
+            if (j * 32 + lane < n) {
+                const unsigned e = own[j * kWordThreads];
+                if (e != ~0u)
+                    d[j] = __double_as_longlong(
+                        __ldcs(w.G + (long long)(sm.r.at[e >> 13].x + (int)((e >> 8) & 31u)) * U + (e & 0xFFu)));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kWordPer; ++j) {
+            const unsigned e = j * 32 + lane < n ? own[j * kWordThreads] : ~0u;
+            if (e == ~0u) continue;
+            const int i = (int)(e >> 8), u = (int)(e & 0xFFu);
+            const int4 at = sm.r.at[i >> 5];
+            const int4* l = sm.r.list[at.z + u];
+            const int hdr = l[0].x;
+            const int L = hdr & 0xFF;
+            const long long* tb = w.tab[hdr >> 8] + (at.x + (i & 31));
+            const int4 o = l[1];
+            long long m = max(max(tb[o.x], tb[o.y]), max(tb[o.z], tb[o.w]));
+            if (L > 4) {
+                const int4 q = l[2];
+                m = max(m, max(max(tb[q.x], tb[q.y]), max(tb[q.z], tb[q.w])));
+                if (L > kWordHead) {
+                    const int4* rest = reinterpret_cast<const int4*>(
+                        w.lists + ((long long)at.w * U + u) * kWordEnt + kWordVal + kWordHead);
+                    for (int t = kWordHead; t < L; t += 4) {
+                        const int4 z = __ldg(rest++);
+                        m = max(m, max(max(tb[z.x], tb[z.y]), max(tb[z.z], tb[z.w])));
+                    }
+                }
+            }
+            d[j] = key_of(__longlong_as_double(d[j]) + val_of(m));        // the one FP64 add
+            // a smaller candidate: inputs found for the one before are stale
+            if (d[j] < *(volatile long long*)&sm.best[i] && d[j] < atomicMin(&sm.best[i], d[j])) sm.bu[i] = 0xFFu;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kWordPer; ++j)
+            if (d[j] < kKeyInf) {
+                const unsigned e = own[j * kWordThreads];
+                if (d[j] == sm.best[e >> 8]) atomicMin(&sm.bu[e >> 8], e & 0xFFu);
+            }
+        __syncthreads();
+    }
+}
+
+// The window's cells whose smallest candidate is below W (whole block).
+__device__ __forceinline__ void word_commit(const WordInst& w, uint2* raw, unsigned char* flags, const int4* unit,
+                                            int first, int ns, WordSmem& sm, unsigned long long& count) {
+    constexpr int K = 3;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int j0 = wid; j0 < ns; j0 += kWordWarps * K) {
+        long long b[K], old[K];
+        uint2 x[K];
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            const int j = j0 + q * kWordWarps;
+            b[q] = kNoCand;
+            if (j < ns) {
+                const int4 at = sm.r.at[j];
+                b[q] = sm.best[j * 32 + lane];
+                x[q] = raw[at.y];
+                if (b[q] != kNoCand) old[q] = w.Vnew[at.x + lane];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            const int j = j0 + q * kWordWarps;
+            if (j >= ns) continue;
+            const int4 at = sm.r.at[j];
+            bool changed = false;
+            if (b[q] != kNoCand) {
+                changed = b[q] < old[q];
+                if (changed) {
+                    w.Vnew[at.x + lane] = b[q];
+                    w.mu[at.x + lane] = (unsigned char)sm.bu[j * 32 + lane];
+                }
+                sm.best[j * 32 + lane] = kNoCand;
+                sm.bu[j * 32 + lane] = 0xFFu;
+            }
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, changed);
+            if (lane == 0 && m) {
+                raw[at.y] = make_uint2(m, x[q].y & ~m);
+                flags[unit[sm.r.word[first + j] >> 5].x] = 1;
+                count += (unsigned long long)__popc(m);
+            }
+        }
+    }
+}
+
+// The relax phase of one pass over this block's share of the units.  count_only:
+// the frontier is counted and nothing is relaxed (at the pass cap).  count (lane
+// 0 of every warp): frontier cells << 32 | changed cells; pairs (lane 0 of every
+// warp) counts the pairs relaxed.
+__device__ __forceinline__ void word_relax(const WordInst& w, long long round, bool count_only, WordSmem& sm,
+                                           unsigned long long& pairs, unsigned long long& count) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int U = w.g.U;
+    count = 0ull;
+    // consecutive units go to different blocks: the frontier is uneven
+    const int mine = (int)blockIdx.x < w.units ? (w.units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int batch = min(kWordUnits, kWordRows / U);
+    for (int t0 = 0; t0 < mine; t0 += kWordTest) {
+        if (threadIdx.x == 0) { sm.nlive = 0; sm.nslots = 0; }
+        if (threadIdx.x < kWordUnits * 32) sm.r.f1[threadIdx.x] = 0u;
+        __syncthreads();
+        for (int i = t0 + wid; i < min(mine, t0 + kWordTest); i += kWordWarps) {
+            const int un = i * gridDim.x + blockIdx.x;
+            int p, k, n;
+            word_unit(w, un, p, k, n);
+            if (word_live(w, p, k, n) && lane == 0)           // P < 2^24: checked at build
+                sm.r.unit[atomicAdd(&sm.nlive, 1)] =
+                    make_int4(un, p | n << 24, p * w.plane_words + k, p * w.plane_cells + k * 32);
+        }
+        __syncthreads();
+        const int nlive = sm.nlive;
+        for (int l0 = 0; l0 < nlive; l0 += batch) {
+            const int nu = min(batch, nlive - l0);
+            const int4* unit = sm.r.unit + l0;
+            // (unit, input) rows over the warps: the pairs to relax
+            const int rows = nu * U;
+            for (int it = wid; it < rows; it += kWordWarps) {
+                const int ui = it / U, u = it - ui * U;
+                const int4 un = unit[ui];
+                const int wd = un.z + lane;
+                const int* list = w.lists + ((long long)(un.y & 0xFFFFFF) * U + u) * kWordEnt;
+                unsigned vb = 0u, act = 0u;
+                if (lane < (un.y >> 24)) {
+                    vb = __ldg(w.vbits + (long long)u * w.S + wd);
+                    act = w.act[wd];
+                }
+                int4 head = make_int4(0, 0, 0, 0);
+                if (lane < 1 + kWordHead / 4) head = __ldg(reinterpret_cast<const int4*>(list + kWordHdr) + lane);
+                unsigned f1;
+                const unsigned m = word_mask(w, list, wd, vb, f1) & act;
+                if (f1) atomicOr(&sm.r.f1[ui * 32 + lane], f1);
+                if (lane < 1 + kWordHead / 4) sm.r.list[it][lane] = head;
+                sm.r.mask[it][lane] = m;
+            }
+            __syncthreads();
+            // slots of the words that have pairs
+            for (int ui = wid; ui < nu; ui += kWordWarps) {
+                unsigned any = 0u, n = 0u;
+                for (int u = 0; u < U; ++u) {
+                    const unsigned m = sm.r.mask[ui * U + u][lane];
+                    any |= m;
+                    n += (unsigned)__popc(m);
+                }
+                const unsigned f1 = sm.r.f1[ui * 32 + lane];
+                sm.r.f1[ui * 32 + lane] = 0u;
+                const unsigned nf = __reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(f1));
+                n = __reduce_add_sync(0xFFFFFFFFu, n);
+                const unsigned have = count_only ? 0u : __ballot_sync(0xFFFFFFFFu, any != 0u);
+                int s = 0;
+                if (lane == 0) {
+                    count += (unsigned long long)nf << 32;
+                    if (have) {
+                        pairs += n;
+                        s = atomicAdd(&sm.nslots, __popc(have));
+                    }
+                }
+                s = __shfl_sync(0xFFFFFFFFu, s, 0) + __popc(have & ((1u << lane) - 1u));
+                const bool mine_ = (have >> lane) & 1u;
+                sm.r.slot[ui * 32 + lane] = mine_ ? (unsigned short)s : (unsigned short)0xFFFFu;
+                if (mine_) sm.r.word[s] = (unsigned short)(ui << 5 | lane);
+            }
+            __syncthreads();
+            const int nslots = sm.nslots;
+            // the slots a window at a time
+            for (int s0 = 0; s0 < nslots; s0 += kWordSlots) {
+                const int ns = min(kWordSlots, nslots - s0);
+                if ((int)threadIdx.x < ns) {
+                    const int x = sm.r.word[s0 + threadIdx.x];
+                    const int4 un = unit[x >> 5];
+                    sm.r.at[threadIdx.x] =
+                        make_int4(un.w + (x & 31) * 32, un.z + (x & 31), (x >> 5) * U, un.y & 0xFFFFFF);
+                }
+                if (threadIdx.x == 0) { sm.queued = 0u; sm.nover = 0; }
+                __syncthreads();
+                for (int it = wid; it < rows; it += kWordWarps) {
+                    const int ui = it / U;
+                    const unsigned s = (unsigned)sm.r.slot[ui * 32 + lane] - (unsigned)s0;
+                    const unsigned m = s < (unsigned)ns ? sm.r.mask[it][lane] : 0u;
+                    if (!word_queue(sm, m, s << 13 | (unsigned)(it - ui * U)) && lane == 0)
+                        sm.r.over[atomicAdd(&sm.nover, 1)] = (short)it;
+                }
+                __syncthreads();
+                word_pairs(w, sm);
+                // rows that did not fit, until every one was queued
+                const int nover = sm.nover;
+                for (int more = nover; more;) {
+                    __syncthreads();
+                    if (threadIdx.x == 0) sm.queued = 0u;
+                    __syncthreads();
+                    bool again = false;
+                    for (int i = wid; i < nover; i += kWordWarps) {
+                        const int it = sm.r.over[i];
+                        if (it < 0) continue;
+                        const int ui = it / U;
+                        const unsigned s = (unsigned)sm.r.slot[ui * 32 + lane] - (unsigned)s0;
+                        const unsigned m = s < (unsigned)ns ? sm.r.mask[it][lane] : 0u;
+                        if (word_queue(sm, m, s << 13 | (unsigned)(it - ui * U))) {
+                            __syncwarp();
+                            if (lane == 0) sm.r.over[i] = -1;
+                        } else {
+                            again = true;
+                        }
+                    }
+                    more = __syncthreads_or(again ? 1 : 0);
+                    word_pairs(w, sm);
+                }
+                word_commit(w, w.raw[round & 1], w.flags[round & 1], unit, s0, ns, sm, count);
+                __syncthreads();
+            }
+            if (threadIdx.x == 0) sm.nslots = 0;
+            __syncthreads();
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// tables
+// ---------------------------------------------------------------------------
+
+__device__ __forceinline__ void word_or(uint2& a, const uint2& b) {
+    a.x |= b.x;
+    a.y |= b.y;
+}
+
+// The six words of a unit's word that its windows reach: row r (0..2) from word
+// k + (r n0 >> 5) of the plane, two words a row.  z: the third word of a row
+// whose first bit is bit 31 (34 bits are used), ORed in by the caller's shift.
+struct WordRows {
+    uint2 a[3], b[3], z[3];
+    __device__ __forceinline__ void load(const WordInst& w, const uint2* plane, int k, bool in, bool m33, bool add) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            if (r && !m33) break;
+            const int i = k + ((r * w.g.n[0]) >> 5);
+            const uint2 none = make_uint2(0u, 0u);
+            const uint2 x = in && i < w.plane_words ? plane[i] : none;
+            const uint2 y = in && i + 1 < w.plane_words ? plane[i + 1] : none;
+            const uint2 t = ((r * w.g.n[0]) & 31) == 31 && in && i + 2 < w.plane_words ? plane[i + 2] : none;
+            if (add) {
+                word_or(a[r], x);
+                word_or(b[r], y);
+                word_or(z[r], t);
+            } else {
+                a[r] = x;
+                b[r] = y;
+                z[r] = t;
+            }
+        }
+    }
+    // windows over 1, 2, 3 cells along dim 0 and 3 x 3 cells, of one component
+    __device__ __forceinline__ void windows(const WordInst& w, bool m33, uint2 out[4]) const {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            if (r && !m33) break;
+            const int s = (r * w.g.n[0]) & 31;
+            const unsigned lx = __funnelshift_r(a[r].x, b[r].x, s), hx = __funnelshift_r(b[r].x, z[r].x, s);
+            const unsigned ly = __funnelshift_r(a[r].y, b[r].y, s), hy = __funnelshift_r(b[r].y, z[r].y, s);
+            const uint2 w2 = make_uint2(lx | __funnelshift_r(lx, hx, 1), ly | __funnelshift_r(ly, hy, 1));
+            const uint2 w3 = make_uint2(w2.x | __funnelshift_r(lx, hx, 2), w2.y | __funnelshift_r(ly, hy, 2));
+            if (r == 0) {
+                out[0] = make_uint2(lx, ly);
+                out[1] = w2;
+                out[2] = w3;
+                out[3] = w3;
+            } else {
+                word_or(out[3], w3);
+            }
+        }
+    }
+};
+
+// The planes one step along dims 2 and 3 of plane p, relative in planes (0:
+// none).
+__device__ __forceinline__ void word_steps(const GridDesc& g, int p, int& s2, int& s3) {
+    const int k3 = (int)grid_div(g, 2, (unsigned)p), k2 = p - k3 * g.n[2];
+    s2 = g.D < 3 ? 0 : (k2 + 1 < g.n[2] ? 1 : (g.periodic[2] ? -k2 : 0));
+    s3 = g.D < 4 ? 0 : (k3 + 1 < g.n[3] ? g.n[2] : (g.periodic[3] ? -k3 * g.n[2] : 0));
+}
+
+// Did a cell change that a window of the unit holds (words k .. k + n - 1 of
+// plane p)?  One flag per unit; lanes take the planes the windows reach (own,
+// along dim 2, dim 3, both) and the units of their words.
+__device__ __forceinline__ bool word_touched(const WordInst& w, const unsigned char* flags, int p, int k, int n) {
+    const int lane = threadIdx.x & 31;
+    int s2, s3;
+    word_steps(w.g, p, s2, s3);
+    const int q = p + ((lane & 8) ? s2 : 0) + ((lane & 16) ? s3 : 0);
+    const int last = min(k + n - 1 + ((2 * w.g.n[0] + 33) >> 5), w.plane_words - 1);
+    bool hit = false;
+    for (int j = k / w.unit_words + (lane & 7); j * w.unit_words <= last; j += 8)
+        hit |= flags[q * w.plane_units + j] != 0;
+    return __any_sync(0xFFFFFFFFu, hit);
+}
+
+// Write the bit tables first .. first + 3 at word wd; changed bits of the tables
+// in use into any.
+__device__ __forceinline__ void word_put(const WordInst& w, int wd, int first, const uint2 x[4], unsigned& any) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+        if ((w.btabs >> (first + t)) & 1) {
+            any |= x[t].x;
+            w.bt[first + t][wd] = x[t];
+        }
+}
+
+// The windows of the unit's words (lane: word k + lane of plane p; in: the lane
+// has a word) into the bit tables; the result: the cells whose value-table
+// entries are to be recomputed.  The windows over two planes are the windows of
+// the planes' words ORed.
+__device__ __forceinline__ unsigned word_tables_at(const WordInst& w, const uint2* raw, int p, int k, bool in,
+                                                   unsigned& any) {
+    const bool m33 = ((w.btabs | w.vtabs) & 0x8888) != 0;
+    const int wd = p * w.plane_words + k;
+    const uint2* own = raw + (long long)p * w.plane_words;
+    int s2, s3;
+    word_steps(w.g, p, s2, s3);
+    const long long d2 = (long long)s2 * w.plane_words, d3 = (long long)s3 * w.plane_words;
+    WordRows r;
+    uint2 x[4];
+    unsigned need = 0u;
+    r.load(w, own, k, in, m33, false);
+    r.windows(w, m33, x);
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+        if ((w.vtabs >> t) & 1) {
+            need |= x[t].x & ~x[t].y;
+            any |= x[t].x;
+        }
+    if (in && (w.btabs & 0x000F)) word_put(w, wd, 0, x, any);
+    if (w.btabs & 0xF0F0) {
+        r.load(w, own + d2, k, in && s2 != 0, m33, true);
+        if (w.btabs & 0x00F0) {
+            r.windows(w, m33, x);
+            if (in) word_put(w, wd, 4, x, any);
+        }
+        if (w.btabs & 0xF000) {
+            r.load(w, own + d3, k, in && s3 != 0, m33, true);
+            r.load(w, own + d2 + d3, k, in && s2 != 0 && s3 != 0, m33, true);
+            r.windows(w, m33, x);
+            if (in) word_put(w, wd, 12, x, any);
+        }
+    }
+    if (w.btabs & 0x0F00) {
+        r.load(w, own, k, in, m33, false);
+        r.load(w, own + d3, k, in && s3 != 0, m33, true);
+        r.windows(w, m33, x);
+        if (in) word_put(w, wd, 8, x, any);
+    }
+    return need;
+}
+
+// Recompute the value tables at cell c.  Windows that reach past a row's or the
+// grid's end are never gathered; their cells are clamped to the array.
+__device__ __forceinline__ void word_entry(const WordInst& w, long long c) {
+    const long long n0 = w.g.n[0], last = w.g.C - 1;
+    const long long v0 = w.Vnew[c];
+    if (w.vtabs & 14) {
+        const long long v1 = w.Vnew[min(c + 1, last)], v2 = w.Vnew[min(c + 2, last)];
+        const long long m2 = max(v0, v1);
+        const long long m3 = max(m2, v2);
+        if (w.vtabs & 8) {
+            long long r[6];
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) r[b * 3 + a] = w.Vnew[min(c + (b + 1) * n0 + a, last)];
+            w.tab[3][c] = max(m3, max(max(r[0], max(r[1], r[2])), max(r[3], max(r[4], r[5]))));
+        }
+        if (w.vtabs & 4) w.tab[2][c] = m3;
+        if (w.vtabs & 2) w.tab[1][c] = m2;
+    }
+    if (w.vtabs & 1) w.tab[0][c] = v0;
+}
+
+// The tables phase after pass `round` (-1: after the set-up, every unit).
+__device__ __forceinline__ void word_tables(const WordInst& w, long long round, WordSmem& sm) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint2* raw = w.raw[round & 1];
+    uint2* next = w.raw[(round + 1) & 1];
+    const bool first = round < 0;
+    if (threadIdx.x == 0) sm.queued = 0u;
+    __syncthreads();
+    for (int un = wid * gridDim.x + blockIdx.x; un < w.units; un += kWordWarps * gridDim.x) {
+        int p, k, n;
+        word_unit(w, un, p, k, n);
+        const bool in = lane < n;
+        const int wd = p * w.plane_words + k + lane;
+        const bool before = w.live[un] != 0u;                    // windows to clear
+        const uint2 own = in ? raw[wd] : make_uint2(0u, 0u);
+        if (first || word_touched(w, w.flags[round & 1], p, k, n) || before) {
+            unsigned any = 0u, tot;
+            unsigned need = word_tables_at(w, raw, p, k + lane, in, any);
+            const unsigned live = __ballot_sync(0xFFFFFFFFu, any != 0u);
+            if (lane == 0) w.live[un] = live;
+            unsigned pos = word_scan((unsigned)__popc(need), tot);
+            if (tot) {
+                unsigned at = 0u;
+                if (lane == 0) at = atomicAdd(&sm.queued, tot);
+                at = __shfl_sync(0xFFFFFFFFu, at, 0);
+                const int c0 = p * w.plane_cells + (k + lane) * 32;
+                if (at + tot <= (unsigned)kWordEntries) {
+                    for (pos += at; need; need &= need - 1u) sm.t.cell[pos++] = c0 + __ffs(need) - 1;
+                } else {
+                    // the queue is full: its last places hold nothing, these
+                    // entries are recomputed here
+                    for (unsigned i = at + lane; i < (unsigned)kWordEntries; i += 32) sm.t.cell[i] = -1;
+                    for (; need; need &= need - 1u) word_entry(w, c0 + __ffs(need) - 1);
+                }
+            }
+        }
+        if (in) next[wd] = make_uint2(0u, own.y);
+        if (lane == 0) w.flags[(round + 1) & 1][un] = 0;
+    }
+    __syncthreads();
+    const int n = (int)min(sm.queued, (unsigned)kWordEntries);
+    for (int i = threadIdx.x; i < n; i += kWordThreads) {
+        const int c = sm.t.cell[i];
+        if (c >= 0) word_entry(w, c);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// pass end and output
+// ---------------------------------------------------------------------------
+
+// After the relax phase of pass r (one thread of the grid): trace, counters,
+// status.  `last`: the pass cap is reached and the frontier was only counted.
+__device__ __forceinline__ void word_close(const WordInst& w, long long r, bool last) {
+    WordCtr* k = w.ctr;
+    const unsigned long long s = *(volatile unsigned long long*)&k->sums[r & 3];
+    const unsigned long long f1 = s >> 32, nchg = s & 0xFFFFFFFFull;
+    if (f1 == 0 || last) {
+        k->done = 1;
+        k->status = f1 == 0 ? BF_CONVERGED : (r >= w.g.C ? BF_NEG_CYCLE : BF_ITER_CAP);
+        return;
+    }
+    if (w.trace && r < w.trace_cap) {
+        long long* t = w.trace + r * 4;
+        t[0] = (long long)f1;
+        t[1] = (long long)nchg;
+        t[2] = (long long)((f1 + 31) / 32);
+        t[3] = -1;
+    }
+    k->total_relaxed += f1;
+    k->total_changed += nchg;
+    k->round = r + 1;
+    k->sums[(r + 2) & 3] = 0ull;
+    k->gate[(r + 2) & 3] = 0ull;
+    if (nchg == 0) {
+        k->done = 1;
+        k->status = BF_CONVERGED;
+    }
+}
+
+__device__ __forceinline__ void word_output(const WordInst& w) {
+    for (long long c = blockIdx.x * (long long)kWordThreads + threadIdx.x; c < w.g.C;
+         c += (long long)gridDim.x * kWordThreads)
+        w.V[c] = val_of(w.Vnew[c]);
+}
+
+}  // namespace bfk

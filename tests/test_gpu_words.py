@@ -1,0 +1,103 @@
+"""The word engine (single solves on abstractions whose every box is its
+plane's entry) against the CPU oracle and against the list form on the same
+handle, at the sizes where its bitmaps can go wrong: planes of 31 to 33 and
+1023 to 1025 cells (word and unit edges), rows of 31, 63 and 95 cells (windows
+that need a third word), one plane, one cell wide planes, periodic and not on
+dims 2 and 3, 1 and 32 inputs.  Values are compared bit for bit: no tolerance.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2001_06231_gb300 as bf
+from test_gpu_solve import plane_instance, same
+
+pytestmark = pytest.mark.gpu
+INF = float("inf")
+
+
+def handle(n, periodic, boxes):
+    D = len(n)
+    return bf.abs_from_boxes(bf.make_grid(n, [0.0] * D, [float(k) for k in n], periodic), boxes)
+
+
+def list_form(A):
+    bf.bf_set_schedule(A, slice_target=2, fuse_mark=1, window33=0, plane_lists=1, cell_masks=0)
+
+
+@pytest.mark.parametrize("n,periodic,U,wmax,seed", [
+    ([31, 1, 5], [False, False, True], 3, (5, 1, 3, 1), 1),
+    ([8, 4, 6], [False, False, False], 4, (4, 3, 3, 1), 2),
+    ([11, 3, 7], [False, False, True], 5, (5, 2, 4, 1), 3),
+    ([33, 31, 4], [False, False, True], 4, (5, 5, 3, 1), 4),
+    ([32, 32, 3], [False, False, False], 4, (6, 6, 3, 1), 5),
+    ([41, 25, 5], [False, False, True], 1, (3, 3, 2, 1), 6),
+    ([63, 17, 6], [False, False, True], 6, (5, 5, 4, 1), 7),
+    ([95, 23, 3, 4], [False, False, True, True], 5, (4, 4, 3, 3), 8),
+    ([19, 18, 4, 3], [False, False, False, True], 32, (4, 4, 2, 2), 9),
+    ([70, 40], [False, False], 7, (6, 6, 1, 1), 10),
+    ([1, 50, 9], [False, False, True], 3, (1, 4, 3, 1), 11),
+    ([26, 90, 2, 2], [False, False, True, False], 6, (5, 4, 2, 2), 12),
+])
+def test_words_match_oracle_and_list_form(n, periodic, U, wmax, seed):
+    rng = np.random.default_rng(4000 + seed)
+    boxes, G, target, avoid = plane_instance(rng, n, periodic, U, wmax=wmax, p_differ=0.0)
+    A = handle(n, periodic, boxes)
+    assert A.shape_mismatch == 0
+    T = np.where(target.astype(bool), 0.0, INF)
+    ref = oracle.solve(n, periodic, boxes, G, T, avoid)
+    k = ref["iters"]
+    word = [bf.bf_solve(A, G, target=target, avoid=avoid, trace_cap=4096, host_loop=hl) for hl in (False, True, False)]
+    assert word[0]["stats"]["kernel_launches"] == 1            # the one-launch form ran
+    list_form(A)
+    word.append(bf.bf_solve(A, G, target=target, avoid=avoid, trace_cap=4096))
+    for r in word:
+        assert r["iters"] == k and r["status"] == ref["status"]
+        assert same(r["V"], ref["V"]) and same(r["mu"], ref["mu"])
+        assert same(r["trace"][:k, 1], ref["changed"][:k])
+    # the frontier of the word engine is Algorithm 1's exactly
+    assert same(word[0]["trace"][:k, 0], ref["f1"][:k])
+    assert word[0]["stats"]["relaxed_cells"] == int(ref["f1"][:k].sum())
+
+
+@pytest.mark.parametrize("cap", [1, 2, 5, 0])
+def test_words_cap_terminal_and_negative_cycle(cap):
+    """A pass cap, a terminal cost that is finite everywhere and costs below
+    zero (the loop then runs into the cap, or into |X| passes without one)."""
+    n, periodic, U = [9, 7, 4], [False, False, True], 3
+    rng = np.random.default_rng(77)
+    boxes, G, target, avoid = plane_instance(rng, n, periodic, U, wmax=(3, 3, 2, 1), p_differ=0.0)
+    G = G - 0.75
+    T = rng.integers(0, 40, size=boxes.shape[0]) * 0.25
+    A = handle(n, periodic, boxes)
+    for t in (T, np.where(target.astype(bool), 0.0, INF)):
+        ref = oracle.solve(n, periodic, boxes, G, t, avoid, max_iters=cap)
+        for hl in (False, True):
+            r = bf.bf_solve(A, G, terminal=t, avoid=avoid, max_iters=cap, host_loop=hl)
+            assert r["iters"] == ref["iters"] and r["status"] == ref["status"]
+            assert same(r["V"], ref["V"]) and same(r["mu"], ref["mu"])
+
+
+def test_words_check_every_cost():
+    """One bad cost anywhere (the first, the last, an unaligned array's ends)
+    is an error, and the handle solves again afterwards; device costs that
+    start 8 bytes past a 16-byte boundary give the same result."""
+    import torch
+    n, periodic, U = [13, 9, 5], [False, False, True], 3
+    rng = np.random.default_rng(5)
+    boxes, G, target, avoid = plane_instance(rng, n, periodic, U, wmax=(3, 3, 2, 1), p_differ=0.0)
+    A = handle(n, periodic, boxes)
+    good = bf.bf_solve(A, G, target=target, avoid=avoid)
+    N = G.size
+    for shift in (0, 1):
+        buf = torch.zeros(N + 2, dtype=torch.float64, device="cuda")
+        g = buf[shift:shift + N]
+        for at in (0, 1, N // 2, N - 2, N - 1):
+            for bad in (float("nan"), -INF, 1e300):
+                g.copy_(torch.from_numpy(G.reshape(-1)))
+                g[at] = bad
+                with pytest.raises(bf.BfError):
+                    bf.bf_solve(A, g, target=target, avoid=avoid)
+        g.copy_(torch.from_numpy(G.reshape(-1)))
+        r = bf.bf_solve(A, g, target=target, avoid=avoid)
+        assert same(r["V"], good["V"]) and same(r["mu"], good["mu"]) and r["iters"] == good["iters"]
