@@ -110,6 +110,133 @@ __global__ void k_rk_table(DynDesc dd, GridDesc g, const double* __restrict__ in
     }
 }
 
+// Range tables.  The right-hand sides of the 3- and 4-D built-in systems do not
+// read the coordinates of dims 0 and 1, so the box of (x, u) is a product of
+// ranges: on dim 0 one that depends on (x's coordinates on dims >= 2, u, x_0),
+// on dim 1 on (..., x_1), on dims >= 2 on (..., u) alone.  quantise_dim runs
+// once per table entry instead of once per (cell, input) -- 256,000 times
+// instead of 51 M on the unicycle 200 x 200 x 64 x 10 -- and boxes, records and
+// predecessor boxes are assembled from the tables: the build's box kernel went
+// from 96.7 ms (FP64 RK4 per pair) to a write of the records.  Entries hold the
+// values box_from_shared computes, operation by operation.  lo = kBlocked: the
+// range leaves the grid.
+struct RangeTabs {
+    short2* r0 = nullptr;      // [keys][U][n0] {lo, hi}
+    short2* r1 = nullptr;      // [keys][U][n1]
+    short4* r23 = nullptr;     // [keys][U] {lo2, hi2, lo3, hi3}, lo2 = kBlocked: blocked for every cell
+};
+
+template <int D>
+__global__ void k_range_tables(DynDesc dd, GridDesc g, const double* __restrict__ rk, long long nkeys, RangeTabs t) {
+    const int n0 = g.n[0], n1 = g.n[1];
+    const long long per = n0 + n1 + 1;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nkeys * g.U * per;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long e = i / per;
+        const int j = (int)(i - e * per);
+        const double* entry = rk + e * kRkEntry;
+        const double* cfinal = entry + 2 * kRkMaxSub;
+        const double* rfinal = cfinal + 2;
+        int lo, hi;
+        if (j < n0 + n1) {
+            const int d = j < n0 ? 0 : 1, k = d ? j - n0 : j;
+            double c = dd.glo[d] + ((double)k + 0.5) * dd.eta[d];
+            for (int s = 0; s < dd.substeps; ++s) c = c + entry[2 * s + d];
+            const double r = rfinal[d];
+            if (!quantise_dim(c - r, c + r, dd.glo[d], dd.eta[d], g.n[d], g.periodic[d], lo, hi)) lo = hi = kBlocked;
+            if (d) t.r1[e * n1 + k] = make_short2((short)lo, (short)hi);
+            else t.r0[e * n0 + k] = make_short2((short)lo, (short)hi);
+        } else {
+            short4 o = make_short4(0, 0, 0, 0);
+            bool ok = true;
+#pragma unroll
+            for (int d = 2; d < D; ++d) {
+                const double c = cfinal[d - 2], r = rfinal[d];
+                ok = ok && quantise_dim(c - r, c + r, dd.glo[d], dd.eta[d], g.n[d], g.periodic[d], lo, hi);
+                if (d == 2) { o.x = (short)lo; o.y = (short)hi; }
+                else { o.z = (short)lo; o.w = (short)hi; }
+            }
+            if (!ok) o = make_short4(kBlocked, 0, 0, 0);
+            t.r23[e] = o;
+        }
+    }
+}
+
+// Box of (cell k, input u) from the range tables.
+template <int D>
+__device__ __forceinline__ Box<D> box_from_ranges(const GridDesc& g, const RangeTabs& t, const int* k, int u) {
+    Box<D> b;
+    const long long e = (long long)rk_key<D>(g, k) * g.U + u;
+    const short2 a = t.r0[e * g.n[0] + k[0]], c = t.r1[e * g.n[1] + k[1]];
+    const short4 q = t.r23[e];
+    b.lo[0] = a.x; b.hi[0] = a.y;
+    b.lo[1] = c.x; b.hi[1] = c.y;
+    b.lo[2] = q.x; b.hi[2] = q.y;
+    if constexpr (D >= 4) { b.lo[3] = q.z; b.hi[3] = q.w; }
+    if (a.x == kBlocked || c.x == kBlocked || q.x == kBlocked) {
+        b.lo[0] = kBlocked;
+#pragma unroll
+        for (int d = 1; d < D; ++d) b.lo[d] = 0;
+#pragma unroll
+        for (int d = 0; d < D; ++d) b.hi[d] = 0;
+    }
+    return b;
+}
+
+// Predecessors along one dim: per (key, input) and coordinate y the offsets
+// x - y of the first and last x whose range holds y (first > last: none).
+__global__ void k_pred_ranges(long long entries, int n, const short2* __restrict__ r, short2* out) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < entries * n;
+         i += (long long)gridDim.x * blockDim.x) {
+        const long long e = i / n;
+        const int y = (int)(i - e * n);
+        int a = 32767, b = -32768;
+        for (int x = 0; x < n; ++x) {
+            const short2 q = __ldg(r + e * n + x);
+            if (q.x == kBlocked || y < q.x || y > q.y) continue;
+            a = min(a, x - y);
+            b = max(b, x - y);
+        }
+        out[i] = make_short2((short)a, (short)b);
+    }
+}
+
+// Predecessor boxes from the tables (thread per cell y): the bounding box over
+// the (source plane q, input) entries whose range on dims >= 2 holds y's plane;
+// ent {entry q U + u, offsets q - p on dims 2 and 3, 0}, those of plane p at
+// ptr[p] .. ptr[p + 1].
+template <int D>
+__global__ void k_pred_from_ranges(GridDesc g, const int* __restrict__ ptr, const int4* __restrict__ ent,
+                                   const short2* __restrict__ p0, const short2* __restrict__ p1, short* pred) {
+    for (long long y = blockIdx.x * (long long)blockDim.x + threadIdx.x; y < g.C;
+         y += (long long)gridDim.x * blockDim.x) {
+        const unsigned r = grid_div(g, 0, (unsigned)y);
+        const int k0 = (int)((unsigned)y - r * (unsigned)g.n[0]);
+        const int p = (int)grid_div(g, 1, r);
+        const int k1 = (int)(r - (unsigned)p * (unsigned)g.n[1]);
+        int lo[4], hi[4];
+#pragma unroll
+        for (int d = 0; d < 4; ++d) { lo[d] = 32767; hi[d] = -32768; }
+        const int e1 = __ldg(ptr + p + 1);
+        for (int e = __ldg(ptr + p); e < e1; ++e) {
+            const int4 t = __ldg(ent + e);
+            const short2 a = __ldg(p0 + (long long)t.x * g.n[0] + k0);
+            const short2 b = __ldg(p1 + (long long)t.x * g.n[1] + k1);
+            if (a.x > a.y || b.x > b.y) continue;
+            lo[0] = min(lo[0], (int)a.x); hi[0] = max(hi[0], (int)a.y);
+            lo[1] = min(lo[1], (int)b.x); hi[1] = max(hi[1], (int)b.y);
+            lo[2] = min(lo[2], t.y); hi[2] = max(hi[2], t.y);
+            lo[3] = min(lo[3], t.z); hi[3] = max(hi[3], t.z);
+        }
+        short* q = pred + y * (2 * D);
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            q[d] = (short)lo[d];
+            q[D + d] = (short)hi[d];
+        }
+    }
+}
+
 // external [C][U][2][D] -> internal [U][C] records, with validation
 template <int D>
 __global__ void k_import_boxes(GridDesc g, const short* __restrict__ ext, void* boxes,
@@ -258,6 +385,38 @@ __global__ void k_build_compact(DynDesc dd, GridDesc g, const double* __restrict
         const unsigned long long rec = encode_compact<D>(g, c, make_box<D>(dd, g, inputs, c, u), bad);
         if (bad) atomicExch(fail, 1);
         store_compact<D>(compact, p, rec);
+    }
+}
+
+// Compact records of the first U1 inputs from the range tables ([U1][C]); sets
+// *fail when some box does not fit.
+template <int D>
+__global__ void k_compact_ranges(GridDesc g, RangeTabs t, int U1, void* compact, int* fail) {
+    const long long total = g.C * U1;
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < total;
+         p += (long long)gridDim.x * blockDim.x) {
+        const int u = (int)(p / g.C);
+        const long long c = p - (long long)u * g.C;
+        int k[4];
+        cell_coords(g, c, k);
+        bool bad = false;
+        const unsigned long long rec = encode_compact<D>(g, c, box_from_ranges<D>(g, t, k, u), bad);
+        if (bad) atomicExch(fail, 1);
+        store_compact<D>(compact, p, rec);
+    }
+}
+
+// Wide records from the range tables (boxes too large for the compact form).
+template <int D>
+__global__ void k_wide_ranges(GridDesc g, RangeTabs t, void* boxes) {
+    const long long total = g.C * g.U;
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < total;
+         p += (long long)gridDim.x * blockDim.x) {
+        const int u = (int)(p / g.C);
+        int k[4];
+        cell_coords(g, p - (long long)u * g.C, k);
+        const Box<D> b = box_from_ranges<D>(g, t, k, u);
+        store_box<D>(boxes, p, b);
     }
 }
 
@@ -550,6 +709,23 @@ static DynDesc make_dyndesc(const bf_abstraction* a) {
 
 static size_t box_bytes(const GridDesc& g) { return (size_t)g.C * g.U * 4 * g.D; }
 
+// Mean predecessor-box rows: how much marking a changed cell costs.
+template <int D>
+static int pred_rows_t(bf_abstraction* a, cudaStream_t st) {
+    const GridDesc& g = a->g;
+    unsigned long long* sums = nullptr;
+    unsigned long long h[2] = {0, 0};
+    BF_CUDA(cudaMallocAsync((void**)&sums, 2 * sizeof(unsigned long long), st));
+    BF_CUDA(cudaMemsetAsync(sums, 0, 2 * sizeof(unsigned long long), st));
+    k_pred_rows<D><<<grid_blocks(g.C, 256), 256, 0, st>>>(g, a->d_pred, sums);
+    BF_CUDA(cudaGetLastError());
+    BF_CUDA(cudaMemcpyAsync(h, sums, sizeof h, cudaMemcpyDeviceToHost, st));
+    BF_CUDA(cudaFreeAsync(sums, st));
+    BF_CUDA(cudaStreamSynchronize(st));
+    a->pred_rows = h[1] ? (double)h[0] / (double)h[1] : 0.0;
+    return BF_OK;
+}
+
 template <int D>
 static int build_pred_t(bf_abstraction* a, cudaStream_t st) {
     const GridDesc& g = a->g;
@@ -564,18 +740,7 @@ static int build_pred_t(bf_abstraction* a, cudaStream_t st) {
     BF_CUDA(cudaGetLastError());
     BF_CUDA(cudaFreeAsync(plo, st));
     BF_CUDA(cudaFreeAsync(phi, st));
-    // mean predecessor-box rows: how much marking a changed cell costs
-    unsigned long long* sums = nullptr;
-    unsigned long long h[2] = {0, 0};
-    BF_CUDA(cudaMallocAsync((void**)&sums, 2 * sizeof(unsigned long long), st));
-    BF_CUDA(cudaMemsetAsync(sums, 0, 2 * sizeof(unsigned long long), st));
-    k_pred_rows<D><<<grid_blocks(g.C, 256), 256, 0, st>>>(g, a->d_pred, sums);
-    BF_CUDA(cudaGetLastError());
-    BF_CUDA(cudaMemcpyAsync(h, sums, sizeof h, cudaMemcpyDeviceToHost, st));
-    BF_CUDA(cudaFreeAsync(sums, st));
-    BF_CUDA(cudaStreamSynchronize(st));
-    a->pred_rows = h[1] ? (double)h[0] / (double)h[1] : 0.0;
-    return BF_OK;
+    return pred_rows_t<D>(a, st);
 }
 
 static int build_pred(bf_abstraction* a, cudaStream_t st) {
@@ -585,6 +750,119 @@ static int build_pred(bf_abstraction* a, cudaStream_t st) {
         case 3: return build_pred_t<3>(a, st);
         default: return build_pred_t<4>(a, st);
     }
+}
+
+// Scratch buffers of a build step, freed (on the stream) when it ends.
+struct BuildTemps {
+    cudaStream_t st;
+    std::vector<void*> p;
+    explicit BuildTemps(cudaStream_t s) : st(s) {}
+    ~BuildTemps() {
+        for (void* q : p) cudaFreeAsync(q, st);
+    }
+    template <typename T>
+    cudaError_t get(T** out, size_t n) {
+        void* q = nullptr;
+        const cudaError_t e = cudaMallocAsync(&q, sizeof(T) * (n ? n : 1), st);
+        if (e == cudaSuccess) p.push_back(q);
+        *out = (T*)q;
+        return e;
+    }
+};
+
+// Do the range tables apply?  (3- and 4-D built-in systems whose shared RK4
+// entries exist, dims 0 and 1 not periodic.)
+static bool has_ranges(const bf_abstraction* a) {
+    return a->g.D >= 3 && a->dyn.kind != 0 && a->dyn.rk4_substeps >= 1 && a->dyn.rk4_substeps <= kRkMaxSub &&
+           !a->g.periodic[0] && !a->g.periodic[1];
+}
+
+// The range tables, from the handle's shared RK4 entries or a scratch copy.
+template <int D>
+static int build_ranges_t(bf_abstraction* a, RangeTabs& t, BuildTemps& tmp, cudaStream_t st) {
+    const GridDesc& g = a->g;
+    const long long nkeys = g.C / g.stride[2], n = nkeys * g.U;
+    const DynDesc dd = make_dyndesc(a);
+    double* rk = a->d_rk;
+    if (!rk) {
+        BF_CUDA(tmp.get(&rk, (size_t)n * kRkEntry));
+        k_rk_table<D><<<grid_blocks(n, 64), 64, 0, st>>>(dd, g, a->d_inputs, nkeys, rk);
+    }
+    BF_CUDA(tmp.get(&t.r0, (size_t)n * g.n[0]));
+    BF_CUDA(tmp.get(&t.r1, (size_t)n * g.n[1]));
+    BF_CUDA(tmp.get(&t.r23, (size_t)n));
+    k_range_tables<D><<<grid_blocks(n * (g.n[0] + g.n[1] + 1), 128), 128, 0, st>>>(dd, g, rk, nkeys, t);
+    BF_CUDA(cudaGetLastError());
+    return BF_OK;
+}
+
+static int build_ranges(bf_abstraction* a, RangeTabs& t, BuildTemps& tmp, cudaStream_t st) {
+    return a->g.D == 3 ? build_ranges_t<3>(a, t, tmp, st) : build_ranges_t<4>(a, t, tmp, st);
+}
+
+// Offset of x - y along dim d, reduced to [-(n/2), n - n/2 - 1] on a periodic
+// dim (as k_pred_scatter does).
+static int pred_off(const GridDesc& g, int d, int x, int y) {
+    int o = x - y;
+    if (g.periodic[d]) {
+        const int n = g.n[d];
+        o %= n;
+        if (o < 0) o += n;
+        if (o >= n - n / 2) o -= n;
+    }
+    return o;
+}
+
+// The predecessor index from the range tables: what k_pred_scatter finds, without
+// walking every box (unicycle 200 x 200 x 64 x 10: 11.7 ms for 1.2 G cell visits).
+template <int D>
+static int build_pred_ranges_t(bf_abstraction* a, const RangeTabs& t, BuildTemps& tmp, cudaStream_t st) {
+    const GridDesc& g = a->g;
+    const long long P = g.C / g.stride[2], U = g.U, n = P * U;
+    short2 *p0 = nullptr, *p1 = nullptr;
+    int* ptr = nullptr;
+    int4* ent = nullptr;
+    BF_CUDA(tmp.get(&p0, (size_t)n * g.n[0]));
+    BF_CUDA(tmp.get(&p1, (size_t)n * g.n[1]));
+    k_pred_ranges<<<grid_blocks(n * g.n[0], 128), 128, 0, st>>>(n, g.n[0], t.r0, p0);
+    k_pred_ranges<<<grid_blocks(n * g.n[1], 128), 128, 0, st>>>(n, g.n[1], t.r1, p1);
+    std::vector<short4> r23((size_t)n);
+    BF_CUDA(cudaMemcpyAsync(r23.data(), t.r23, sizeof(short4) * n, cudaMemcpyDeviceToHost, st));
+    BF_CUDA(cudaStreamSynchronize(st));
+    const int n2 = g.n[2], n3 = D >= 4 ? g.n[3] : 1;
+    // two rounds over the entries: count per target plane, then fill
+    std::vector<int> hptr((size_t)P + 1, 0);
+    std::vector<int4> hent;
+    std::vector<int> at;
+    for (int fill = 0; fill < 2; ++fill) {
+        for (long long e = 0; e < n; ++e) {
+            const short4 r = r23[(size_t)e];
+            if (r.x == kBlocked) continue;
+            const int q = (int)(e / U), q2 = q % n2, q3 = q / n2;
+            const int lo3 = D >= 4 ? r.z : 0, hi3 = D >= 4 ? r.w : 0;
+            for (int x3 = lo3; x3 <= hi3; ++x3)
+                for (int x2 = r.x; x2 <= r.y; ++x2) {
+                    const int y2 = x2 >= n2 ? x2 - n2 : x2, y3 = x3 >= n3 ? x3 - n3 : x3;
+                    const size_t p = (size_t)(y2 + n2 * y3);
+                    if (!fill) ++hptr[p + 1];
+                    else hent[(size_t)at[p]++] =
+                             make_int4((int)e, pred_off(g, 2, q2, y2), D >= 4 ? pred_off(g, 3, q3, y3) : 0, 0);
+                }
+        }
+        if (!fill) {
+            for (size_t p = 0; p < (size_t)P; ++p) hptr[p + 1] += hptr[p];
+            hent.resize((size_t)hptr[(size_t)P]);
+            at.assign(hptr.begin(), hptr.end() - 1);
+        }
+    }
+    BF_CUDA(tmp.get(&ptr, hptr.size()));
+    BF_CUDA(tmp.get(&ent, hent.size()));
+    BF_CUDA(cudaMemcpyAsync(ptr, hptr.data(), sizeof(int) * hptr.size(), cudaMemcpyHostToDevice, st));
+    if (!hent.empty())
+        BF_CUDA(cudaMemcpyAsync(ent, hent.data(), sizeof(int4) * hent.size(), cudaMemcpyHostToDevice, st));
+    k_pred_from_ranges<D><<<grid_blocks(g.C, 256), 256, 0, st>>>(g, ptr, ent, p0, p1, a->d_pred);
+    BF_CUDA(cudaGetLastError());
+    return pred_rows_t<D>(a, st);                       // synchronizes: the host vectors are done
 }
 
 // Replace the wide records by compact ones when every box fits the format.
@@ -624,6 +902,37 @@ static int to_compact(bf_abstraction* a, cudaStream_t st) {
         case 3: return to_compact_t<3>(a, st);
         default: return to_compact_t<4>(a, st);
     }
+}
+
+// The stored records from the range tables: compact ones when every box fits
+// the format, else wide ones.
+static int boxes_from_ranges(bf_abstraction* a, const RangeTabs& t, cudaStream_t st) {
+    const GridDesc& g = a->g;
+    const size_t bytes = 8 * (size_t)g.C * g.U;
+    int* d_fail = nullptr;
+    int h_fail = 0;
+    BuildTemps tmp(st);
+    BF_CUDA(tmp.get(&d_fail, 1));
+    BF_CUDA(cudaMemsetAsync(d_fail, 0, sizeof(int), st));
+    BF_CUDA(cudaMalloc(&a->d_boxes, bytes));
+    const int nb = grid_blocks(g.C * g.U, 256);
+    if (g.D == 3) k_compact_ranges<3><<<nb, 256, 0, st>>>(g, t, g.U, a->d_boxes, d_fail);
+    else k_compact_ranges<4><<<nb, 256, 0, st>>>(g, t, g.U, a->d_boxes, d_fail);
+    BF_CUDA(cudaGetLastError());
+    BF_CUDA(cudaMemcpyAsync(&h_fail, d_fail, sizeof(int), cudaMemcpyDeviceToHost, st));
+    BF_CUDA(cudaStreamSynchronize(st));
+    if (!h_fail) {
+        a->box_fmt = kBoxCompact;
+        a->bytes = a->bytes - box_bytes(g) + bytes;
+        return BF_OK;
+    }
+    cudaFree(a->d_boxes);
+    a->d_boxes = nullptr;
+    BF_CUDA(cudaMalloc(&a->d_boxes, box_bytes(g)));
+    if (g.D == 3) k_wide_ranges<3><<<nb, 256, 0, st>>>(g, t, a->d_boxes);
+    else k_wide_ranges<4><<<nb, 256, 0, st>>>(g, t, a->d_boxes);
+    BF_CUDA(cudaGetLastError());
+    return BF_OK;
 }
 
 // The plane shape table of a compact-record abstraction (grids of 2+ dims,
@@ -1095,31 +1404,17 @@ extern "C" int abs_build(const bf_dynamics* dyn, const bf_grid* grid, const bf_i
     a->tau = tau;
     a->udim = inputs->udim;
     size_t in_bytes = sizeof(double) * inputs->ninputs * inputs->udim;
+    const bool ranges = has_ranges(a);
     cudaError_t e = cudaMalloc(&a->d_inputs, in_bytes);
     if (e == cudaSuccess) e = cudaMemcpyAsync(a->d_inputs, inputs->u, in_bytes, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMalloc((void**)&a->d_pred, sizeof(short) * 2 * g.D * g.C);
-    if (e == cudaSuccess && mode == BF_MODE_STORED) e = cudaMalloc(&a->d_boxes, box_bytes(a->g));
+    if (e == cudaSuccess && mode == BF_MODE_STORED && !ranges) e = cudaMalloc(&a->d_boxes, box_bytes(a->g));
     if (e != cudaSuccess) { abs_free(a); return bfh::cuda_fail(e, "abs_build allocation"); }
     a->bytes = in_bytes + sizeof(short) * 2 * g.D * g.C + (mode == BF_MODE_STORED ? box_bytes(a->g) : 0);
     DynDesc dd = make_dyndesc(a);
-    if (mode == BF_MODE_STORED) {
-        const int nb = grid_blocks(a->g.C * a->g.U, 128);
-        switch (g.D) {
-            case 2: k_build_boxes<2><<<nb, 128, 0, st>>>(dd, a->g, a->d_inputs, a->d_boxes); break;
-            case 3: k_build_boxes<3><<<nb, 128, 0, st>>>(dd, a->g, a->d_inputs, a->d_boxes); break;
-            default: k_build_boxes<4><<<nb, 128, 0, st>>>(dd, a->g, a->d_inputs, a->d_boxes); break;
-        }
-    }
     a->box_fmt = mode == BF_MODE_STORED ? kBoxWide : kBoxRecompute;
     a->nstored = mode == BF_MODE_STORED ? a->g.U : 0;
-    rc = build_pred(a, st);
-    if (rc == BF_OK) {
-        e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = bfh::cuda_fail(e, "abs_build kernels");
-    }
-    if (rc == BF_OK && mode == BF_MODE_STORED) rc = to_compact(a, st);
-    if (rc == BF_OK && mode == BF_MODE_STORED) rc = build_shapes(a, st);
-    if (rc == BF_OK && mode == BF_MODE_RECOMPUTE && g.D >= 3 && dyn->rk4_substeps <= kRkMaxSub) {
+    if (mode == BF_MODE_RECOMPUTE && g.D >= 3 && dyn->rk4_substeps <= kRkMaxSub) {
         // the RK4 work shared by cells with equal coordinates on dims >= 2
         const long long nkeys = g.C / g.stride[2];
         const size_t bytes = sizeof(double) * kRkEntry * nkeys * a->g.U;
@@ -1130,10 +1425,32 @@ extern "C" int abs_build(const bf_dynamics* dyn, const bf_grid* grid, const bf_i
             else k_rk_table<4><<<nb, 64, 0, st>>>(dd, a->g, a->d_inputs, nkeys, a->d_rk);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = bfh::cuda_fail(e, "recompute RK4 table");
-        else a->bytes += bytes;
+        if (e != cudaSuccess) { abs_free(a); return bfh::cuda_fail(e, "recompute RK4 table"); }
+        a->bytes += bytes;
     }
+    if (ranges) {
+        BuildTemps tmp(st);
+        RangeTabs t;
+        rc = build_ranges(a, t, tmp, st);
+        if (rc == BF_OK && mode == BF_MODE_STORED) rc = boxes_from_ranges(a, t, st);
+        if (rc == BF_OK) rc = g.D == 3 ? build_pred_ranges_t<3>(a, t, tmp, st) : build_pred_ranges_t<4>(a, t, tmp, st);
+    } else {
+        if (mode == BF_MODE_STORED) {
+            const int nb = grid_blocks(a->g.C * a->g.U, 128);
+            switch (g.D) {
+                case 2: k_build_boxes<2><<<nb, 128, 0, st>>>(dd, a->g, a->d_inputs, a->d_boxes); break;
+                case 3: k_build_boxes<3><<<nb, 128, 0, st>>>(dd, a->g, a->d_inputs, a->d_boxes); break;
+                default: k_build_boxes<4><<<nb, 128, 0, st>>>(dd, a->g, a->d_inputs, a->d_boxes); break;
+            }
+        }
+        rc = build_pred(a, st);
+        if (rc == BF_OK && mode == BF_MODE_STORED) rc = to_compact(a, st);
+    }
+    if (rc == BF_OK) {
+        e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) rc = bfh::cuda_fail(e, "abs_build kernels");
+    }
+    if (rc == BF_OK && mode == BF_MODE_STORED) rc = build_shapes(a, st);
     if (rc) { abs_free(a); return rc; }
     *out = a;
     return BF_OK;
@@ -1152,12 +1469,25 @@ static int add_stored_inputs(bf_abstraction* a, int K, cudaStream_t st) {
     void* comp = nullptr;
     int* d_fail = nullptr;
     int h_fail = 0;
+    BuildTemps tmp(st);
     BF_CUDA(cudaMalloc(&comp, bytes));
     cudaError_t e = cudaMalloc((void**)&d_fail, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(d_fail, 0, sizeof(int), st);
     if (e == cudaSuccess) {
-        DynDesc dd = make_dyndesc(a);
-        k_build_compact<D><<<grid_blocks(gk.C * K, 128), 128, 0, st>>>(dd, gk, a->d_inputs, comp, d_fail);
+        bool done = false;
+        if constexpr (D >= 3) {
+            if (has_ranges(a)) {
+                RangeTabs t;
+                const int rc = build_ranges_t<D>(a, t, tmp, st);
+                if (rc) { cudaFree(d_fail); cudaFree(comp); return rc; }
+                k_compact_ranges<D><<<grid_blocks(gk.C * K, 256), 256, 0, st>>>(a->g, t, K, comp, d_fail);
+                done = true;
+            }
+        }
+        if (!done) {
+            DynDesc dd = make_dyndesc(a);
+            k_build_compact<D><<<grid_blocks(gk.C * K, 128), 128, 0, st>>>(dd, gk, a->d_inputs, comp, d_fail);
+        }
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h_fail, d_fail, sizeof(int), cudaMemcpyDeviceToHost, st);

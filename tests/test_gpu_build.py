@@ -1,0 +1,58 @@
+"""The builder's range tables (one quantisation per plane, input and coordinate)
+against the general path: the recompute-mode export runs the RK4 scheme for
+every (cell, input) pair, and importing the exported boxes walks every box for
+the predecessor index.  Boxes, records and predecessor boxes are integers and
+must be identical.
+"""
+import math
+
+import numpy as np
+import pytest
+
+import paper_2001_06231_gb300 as bf
+from paper_2001_06231_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _with(w, **kw):
+    for k, v in kw.items():
+        setattr(w, k, v)
+    return w
+
+
+def _periodic(w, p):
+    w.grid = wl.Grid(w.grid.n, w.grid.lo, w.grid.hi, p)
+    return w
+
+
+CASES = {
+    "unicycle": lambda: wl.unicycle3d(n=(37, 41, 13), n_obstacles=2),
+    "unicycle one plane": lambda: wl.unicycle3d(n=(33, 20, 1), n_obstacles=2),
+    "unicycle theta open": lambda: _periodic(wl.unicycle3d(n=(30, 31, 9), n_obstacles=2), (False, False, False)),
+    "unicycle x periodic": lambda: _periodic(wl.unicycle3d(n=(24, 21, 8), n_obstacles=2), (True, False, True)),
+    "unicycle wide records": lambda: _with(wl.unicycle3d(n=(300, 6, 5), n_obstacles=2), tau=5.0),
+    "unicycle 11 substeps": lambda: _with(wl.unicycle3d(n=(21, 19, 8), n_obstacles=2), substeps=11),
+    "fire": lambda: wl.fire4d(n=(25, 23, 10, 3), n_blobs=1, n_nofly=1, tau=2.0),
+    "fire V periodic": lambda: _periodic(wl.fire4d(n=(21, 20, 9, 4), n_blobs=1, n_nofly=1, tau=1.0),
+                                         (False, False, True, True)),
+    "fire 2 substeps": lambda: _with(wl.fire4d(n=(26, 17, 12, 2), n_blobs=1, n_nofly=1, tau=1.5), substeps=2),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_range_tables_equal_the_general_path(name):
+    w = CASES[name]()
+    A = bf.abs_build_workload(w)
+    boxes = A.export_boxes()
+    R = bf.abs_build_workload(w, mode=bf.MODE_RECOMPUTE)
+    assert np.array_equal(boxes, R.export_boxes())
+    B = bf.abs_from_boxes(w.grid, boxes)
+    pred = B.export_pred()
+    assert np.array_equal(A.export_pred(), pred)
+    assert np.array_equal(R.export_pred(), pred)
+    assert A.box_record_bytes == B.box_record_bytes
+    assert (A.shape_planes, A.shape_mismatch) == (B.shape_planes, B.shape_mismatch)
+    K = max(1, w.ninputs // 3)
+    H = bf.abs_build_workload(w, box_budget=8 * w.ncells * K)
+    assert np.array_equal(H.export_boxes(), boxes) and np.array_equal(H.export_pred(), pred)
