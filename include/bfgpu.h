@@ -99,7 +99,11 @@ extern "C" {
 /* Storage mode of an abstraction (Sec. IV-B, memory control): STORED keeps the
  * image of F in device memory; RECOMPUTE keeps only the dynamics and
  * regenerates each box inside the relaxation kernel (bit-identical boxes,
- * 4*D*C*U fewer bytes, far more FP64 work). */
+ * 4*D*C*U fewer bytes, far more FP64 work).  Where every box of a plane (equal
+ * coordinates on dims >= 2) and input has the same shape relative to its cell
+ * -- the unicycle and the fire model -- the abstraction also keeps one bit per
+ * (cell, input) and the planes' lookup lists, and plain Jacobi solves use those
+ * instead of regenerating boxes. */
 #define BF_MODE_STORED 0
 #define BF_MODE_RECOMPUTE 1
 #define BF_MODE_HYBRID 2       /* records of the first K inputs stored, the
@@ -262,7 +266,8 @@ typedef struct {
      * pass's frontier are kept for the next pass, where the cells still in the
      * frontier read them instead of regenerating them; the others are dropped.
      * Device memory in the handle's workspace: 8 C + 16 (U - K) frontier_cache
-     * bytes.  0: no cache (stored-mode abstractions never use one). */
+     * bytes.  0: no cache (stored-mode abstractions never use one; nor do solves
+     * that need no box regenerated, see BF_MODE_RECOMPUTE). */
     int64_t frontier_cache;
 } bf_solve_opts;
 

@@ -420,6 +420,85 @@ __global__ void k_wide_ranges(GridDesc g, RangeTabs t, void* boxes) {
     }
 }
 
+// Shape table entries from the range tables (warp per (plane, input)): the
+// record every non-blocked pair shares, 0 when there is none; *mixed counts the
+// entries whose pairs have several records or one that the format cannot hold.
+template <int D>
+__global__ void k_shape_ranges(GridDesc g, RangeTabs t, long long n, unsigned long long* shape, unsigned* mixed) {
+    const int lane = threadIdx.x & 31;
+    const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
+    for (long long e = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); e < n; e += nw) {
+        int rel[D], wid[D];
+        bool none = false, bad = false, wrap = false;
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+            const short2* r = d ? t.r1 + e * g.n[1] : t.r0 + e * g.n[0];
+            int a = 0x7FFFFFFF, b = (int)0x80000000;       // smallest, largest of rel << 16 | width
+            for (int x = lane; x < g.n[d]; x += 32) {
+                const short2 q = r[x];
+                if (q.x == kBlocked) continue;
+                const int key = (int)((unsigned)(q.x - x) << 16 | (unsigned)(q.y - q.x + 1));
+                a = min(a, key);
+                b = max(b, key);
+            }
+            a = __reduce_min_sync(0xFFFFFFFFu, a);
+            b = __reduce_max_sync(0xFFFFFFFFu, b);
+            none |= a > b;
+            bad |= a < b;
+            rel[d] = a >> 16;
+            wid[d] = a & 0xFFFF;
+        }
+        const short4 q = t.r23[e];
+        none |= q.x == kBlocked;
+        const int k23[2] = {(int)((e / g.U) % g.n[2]), (int)((e / g.U) / g.n[2])};
+#pragma unroll
+        for (int d = 2; d < D; ++d) {
+            const int lo = d == 2 ? q.x : q.z, hi = d == 2 ? q.y : q.w, k = k23[d - 2], nn = g.n[d];
+            int o = lo - k;
+            wid[d] = hi - lo + 1;
+            if (g.periodic[d]) {                           // as encode_compact
+                o %= nn;
+                if (o < 0) o += nn;
+                if (o >= nn - nn / 2) o -= nn;
+                wrap |= k + o < 0 || k + o + wid[d] > nn;
+            }
+            rel[d] = o;
+        }
+        unsigned long long rec = 0;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            bad |= !none && (wid[d] > 127 || rel[d] < -128 || rel[d] > 127);
+            rec |= (unsigned long long)(unsigned char)(signed char)rel[d] << (16 * d);
+            rec |= (unsigned long long)(wid[d] & 0x7F) << (16 * d + 8);
+        }
+        if (wrap) rec |= 0x80ull << 8;
+        if (lane == 0) {
+            shape[e] = none ? 0ull : rec;
+            if (bad && !none) atomicAdd(mixed, 1u);
+        }
+    }
+}
+
+// Bitmaps of the pairs that have a box, from the range tables (warp per word).
+template <int D>
+__global__ void k_valid_ranges(GridDesc g, RangeTabs t, int plane_words, int plane_cells, int S, unsigned* vbits) {
+    const int lane = threadIdx.x & 31;
+    const int nw = gridDim.x * (blockDim.x >> 5);
+    for (int wd = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); wd < S; wd += nw) {
+        const int p = wd / plane_words;
+        const int i = (wd - p * plane_words) * 32 + lane;
+        const bool in = i < plane_cells;
+        const int k1 = in ? (int)grid_div(g, 0, (unsigned)i) : 0, k0 = in ? i - k1 * g.n[0] : 0;
+        for (int u = 0; u < g.U; ++u) {
+            const long long e = (long long)p * g.U + u;
+            const bool ok = in && t.r23[e].x != kBlocked && t.r0[e * g.n[0] + k0].x != kBlocked &&
+                            t.r1[e * g.n[1] + k1].x != kBlocked;
+            const unsigned b = __ballot_sync(0xFFFFFFFFu, ok);
+            if (lane == 0) vbits[(long long)u * S + wd] = b;
+        }
+    }
+}
+
 // Plane shape table.  A plane is the set of cells with equal coordinates on
 // dims >= 2 (the whole grid for D = 2); p = x / stride[2].  For dynamics
 // invariant under translation along dims 0 and 1 (the built-in unicycle and
@@ -938,64 +1017,71 @@ static int boxes_from_ranges(bf_abstraction* a, const RangeTabs& t, cudaStream_t
 // The plane shape table of a compact-record abstraction (grids of 2+ dims,
 // dims 0 and 1 not periodic); left NULL otherwise.  Best effort: the solver
 // works without it.
+// known: the table when it is known already (every pair has its entry's record).
 template <int D>
-static int build_shapes_t(bf_abstraction* a, cudaStream_t st) {
+static int build_shapes_t(bf_abstraction* a, const unsigned long long* known, cudaStream_t st) {
     const GridDesc& g = a->g;
     const long long P = g.C / g.stride[2];
     unsigned long long* shape = nullptr;
-    unsigned long long* d_bad = nullptr;
     unsigned long long h_bad = 0;
     const long long n = P * g.U;
-    unsigned long long *first = nullptr, *second = nullptr, *third = nullptr;
-    unsigned *hit1 = nullptr, *hit2 = nullptr, *nbk = nullptr, *idx = nullptr;
-    unsigned char* skip = nullptr;
     BF_CUDA(cudaMalloc((void**)&shape, sizeof(unsigned long long) * n));
-    cudaError_t e = cudaMalloc((void**)&d_bad, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&first, sizeof(unsigned long long) * 3 * n);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&hit1, sizeof(unsigned) * 4 * n);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&skip, n);
-    if (e == cudaSuccess) {
-        second = first + n;
-        third = first + 2 * n;
-        hit2 = hit1 + n;
-        nbk = hit1 + 2 * n;
-        idx = hit1 + 3 * n;
-        e = cudaMemsetAsync(hit1, 0, sizeof(unsigned) * 3 * n, st);
+    if (known) {
+        const cudaError_t e =
+            cudaMemcpyAsync(shape, known, sizeof(unsigned long long) * n, cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) { cudaFree(shape); return bfh::cuda_fail(e, "plane shape table"); }
+    } else {
+        unsigned long long *first = nullptr, *second = nullptr, *third = nullptr;
+        unsigned *hit1 = nullptr, *hit2 = nullptr, *nbk = nullptr, *idx = nullptr;
+        unsigned char* skip = nullptr;
+        unsigned long long* d_bad = nullptr;
+        cudaError_t e = cudaMalloc((void**)&d_bad, sizeof(unsigned long long));
+        if (e == cudaSuccess) e = cudaMalloc((void**)&first, sizeof(unsigned long long) * 3 * n);
+        if (e == cudaSuccess) e = cudaMalloc((void**)&hit1, sizeof(unsigned) * 4 * n);
+        if (e == cudaSuccess) e = cudaMalloc((void**)&skip, n);
+        if (e == cudaSuccess) {
+            second = first + n;
+            third = first + 2 * n;
+            hit2 = hit1 + n;
+            nbk = hit1 + 2 * n;
+            idx = hit1 + 3 * n;
+            e = cudaMemsetAsync(hit1, 0, sizeof(unsigned) * 3 * n, st);
+        }
+        if (e == cudaSuccess) e = cudaMemsetAsync(d_bad, 0, sizeof(unsigned long long), st);
+        if (e == cudaSuccess) {
+            const int nb = grid_blocks(g.C * g.U, 256);
+            const int ne = grid_blocks(n, 256);
+            auto pick = [&](unsigned long long* out, const unsigned long long* ex1, const unsigned long long* ex2,
+                            const unsigned char* sk) {
+                if (e == cudaSuccess) e = cudaMemsetAsync(idx, 0xFF, sizeof(unsigned) * n, st);
+                k_shape_first<D><<<nb, 256, 0, st>>>(g, a->d_boxes, idx, ex1, ex2, sk);
+                k_shape_take<D><<<ne, 256, 0, st>>>(g, a->d_boxes, idx, n, out);
+            };
+            pick(first, nullptr, nullptr, nullptr);
+            k_shape_count<D><<<nb, 256, 0, st>>>(g, a->d_boxes, first, hit1, nbk);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(shape, first, sizeof(unsigned long long) * n, cudaMemcpyDeviceToDevice, st);
+            // second round where the first pick is shared by less than half of the pairs
+            k_shape_retry<<<ne, 256, 0, st>>>(n, hit1, nbk, skip);
+            pick(second, first, nullptr, skip);
+            k_shape_count<D><<<nb, 256, 0, st>>>(g, a->d_boxes, second, hit2, nullptr);
+            k_shape_choose<<<ne, 256, 0, st>>>(n, shape, second, hit1, hit2);
+            // third round where neither is
+            if (e == cudaSuccess) e = cudaMemsetAsync(hit2, 0, sizeof(unsigned) * n, st);
+            k_shape_retry<<<ne, 256, 0, st>>>(n, hit1, nbk, skip);
+            pick(third, first, second, skip);
+            k_shape_count<D><<<nb, 256, 0, st>>>(g, a->d_boxes, third, hit2, nullptr);
+            k_shape_choose<<<ne, 256, 0, st>>>(n, shape, third, hit1, hit2);
+            k_shape_check<D><<<nb, 256, 0, st>>>(g, a->d_boxes, shape, d_bad);
+            if (e == cudaSuccess) e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&h_bad, d_bad, sizeof h_bad, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        cudaFree(d_bad);
+        cudaFree(first);
+        cudaFree(hit1);
+        cudaFree(skip);
+        if (e != cudaSuccess) { cudaFree(shape); return bfh::cuda_fail(e, "plane shape table"); }
     }
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_bad, 0, sizeof(unsigned long long), st);
-    if (e == cudaSuccess) {
-        const int nb = grid_blocks(g.C * g.U, 256);
-        const int ne = grid_blocks(n, 256);
-        auto pick = [&](unsigned long long* out, const unsigned long long* ex1, const unsigned long long* ex2,
-                        const unsigned char* sk) {
-            if (e == cudaSuccess) e = cudaMemsetAsync(idx, 0xFF, sizeof(unsigned) * n, st);
-            k_shape_first<D><<<nb, 256, 0, st>>>(g, a->d_boxes, idx, ex1, ex2, sk);
-            k_shape_take<D><<<ne, 256, 0, st>>>(g, a->d_boxes, idx, n, out);
-        };
-        pick(first, nullptr, nullptr, nullptr);
-        k_shape_count<D><<<nb, 256, 0, st>>>(g, a->d_boxes, first, hit1, nbk);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(shape, first, sizeof(unsigned long long) * n, cudaMemcpyDeviceToDevice, st);
-        // second round where the first pick is shared by less than half of the pairs
-        k_shape_retry<<<ne, 256, 0, st>>>(n, hit1, nbk, skip);
-        pick(second, first, nullptr, skip);
-        k_shape_count<D><<<nb, 256, 0, st>>>(g, a->d_boxes, second, hit2, nullptr);
-        k_shape_choose<<<ne, 256, 0, st>>>(n, shape, second, hit1, hit2);
-        // third round where neither is
-        if (e == cudaSuccess) e = cudaMemsetAsync(hit2, 0, sizeof(unsigned) * n, st);
-        k_shape_retry<<<ne, 256, 0, st>>>(n, hit1, nbk, skip);
-        pick(third, first, second, skip);
-        k_shape_count<D><<<nb, 256, 0, st>>>(g, a->d_boxes, third, hit2, nullptr);
-        k_shape_choose<<<ne, 256, 0, st>>>(n, shape, third, hit1, hit2);
-        k_shape_check<D><<<nb, 256, 0, st>>>(g, a->d_boxes, shape, d_bad);
-        if (e == cudaSuccess) e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_bad, d_bad, sizeof h_bad, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(d_bad);
-    cudaFree(first);
-    cudaFree(hit1);
-    cudaFree(skip);
-    if (e != cudaSuccess) { cudaFree(shape); return bfh::cuda_fail(e, "plane shape table"); }
     a->d_shape = shape;
     a->nplanes = P;
     a->shape_mismatch = (long long)h_bad;
@@ -1231,12 +1317,15 @@ __global__ void k_word_lists(GridDesc g, const unsigned long long* __restrict__ 
 // list fits).  A plane's bit lookups become one span of words per plane they
 // read, relative to the reader's word; a plane that reads more than kWordSpans
 // planes is always tested.
-static int build_word(bf_abstraction* a, cudaStream_t st) {
+// shape: the table; the pairs that have a box come from the range tables, or
+// (NULL) from the cell masks.
+static int build_word(bf_abstraction* a, const unsigned long long* shape, const RangeTabs* ranges, cudaStream_t st) {
     const GridDesc& g = a->g;
-    const long long pw = (g.stride[2] + 31) / 32;
-    if (!a->d_fmask || g.U > kWordMaxU || a->nplanes * pw * 32 > (1LL << 31) - 64 || a->nplanes >= (1LL << 24)) return BF_OK;
-    const size_t P = (size_t)a->nplanes, U = (size_t)g.U;
-    const int S = (int)(a->nplanes * pw), plane_bits = (int)pw * 32;
+    const long long planes = g.C / g.stride[2], pw = (g.stride[2] + 31) / 32;
+    if ((!ranges && !a->d_fmask) || g.U > kWordMaxU || planes * pw * 32 > (1LL << 31) - 64 || planes >= (1LL << 24))
+        return BF_OK;
+    const size_t P = (size_t)planes, U = (size_t)g.U;
+    const int S = (int)(planes * pw), plane_bits = (int)pw * 32;
     std::vector<int> lists(P * U * kWordEnt);
     int* dl = nullptr;
     unsigned* vb = nullptr;
@@ -1245,9 +1334,9 @@ static int build_word(bf_abstraction* a, cudaStream_t st) {
     if (e == cudaSuccess) {
         const int nb = grid_blocks((long long)(P * U), 128);
         switch (g.D) {
-            case 2: k_word_lists<2><<<nb, 128, 0, st>>>(g, a->d_shape, (long long)P, plane_bits, dl); break;
-            case 3: k_word_lists<3><<<nb, 128, 0, st>>>(g, a->d_shape, (long long)P, plane_bits, dl); break;
-            default: k_word_lists<4><<<nb, 128, 0, st>>>(g, a->d_shape, (long long)P, plane_bits, dl); break;
+            case 2: k_word_lists<2><<<nb, 128, 0, st>>>(g, shape, (long long)P, plane_bits, dl); break;
+            case 3: k_word_lists<3><<<nb, 128, 0, st>>>(g, shape, (long long)P, plane_bits, dl); break;
+            default: k_word_lists<4><<<nb, 128, 0, st>>>(g, shape, (long long)P, plane_bits, dl); break;
         }
         e = cudaGetLastError();
     }
@@ -1256,7 +1345,7 @@ static int build_word(bf_abstraction* a, cudaStream_t st) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     std::vector<unsigned long long> rec(P * U);
     if (e == cudaSuccess)
-        e = cudaMemcpy(rec.data(), a->d_shape, sizeof(rec[0]) * rec.size(), cudaMemcpyDeviceToHost);
+        e = cudaMemcpy(rec.data(), shape, sizeof(rec[0]) * rec.size(), cudaMemcpyDeviceToHost);
     std::vector<int4> spans(P * kWordSpans, make_int4(-1, 0, 0, 0));
     int vtabs = 0, btabs = 0;
     bool fits = true;
@@ -1304,8 +1393,10 @@ static int build_word(bf_abstraction* a, cudaStream_t st) {
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(sp, spans.data(), sizeof(int4) * spans.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
-        k_valid_bits<<<grid_blocks((long long)S * 32, 256), 256, 0, st>>>(g, a->d_fmask, (int)pw, (int)g.stride[2], S,
-                                                                          vb);
+        const int nb = grid_blocks((long long)S * 32, 256), cells = (int)g.stride[2];
+        if (!ranges) k_valid_bits<<<nb, 256, 0, st>>>(g, a->d_fmask, (int)pw, cells, S, vb);
+        else if (g.D == 3) k_valid_ranges<3><<<nb, 256, 0, st>>>(g, *ranges, (int)pw, cells, S, vb);
+        else k_valid_ranges<4><<<nb, 256, 0, st>>>(g, *ranges, (int)pw, cells, S, vb);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1323,16 +1414,43 @@ static int build_word(bf_abstraction* a, cudaStream_t st) {
     return BF_OK;
 }
 
-static int build_shapes(bf_abstraction* a, cudaStream_t st) {
-    if (a->box_fmt != kBoxCompact || a->g.D < 2 || a->g.periodic[0] || a->g.periodic[1]) return BF_OK;
+// The shape table, the lists and the templates of a stored abstraction, and the
+// word engine's data of any.  ranges: the builder's tables, or NULL (imported
+// boxes).  Where every entry of the range tables has one record, that is the
+// shape table, and an abstraction whose boxes are regenerated gets the word
+// engine's data too: a bit per pair and the lists stand for its boxes.
+static int build_shapes(bf_abstraction* a, const RangeTabs* ranges, cudaStream_t st) {
+    const GridDesc& g = a->g;
+    BuildTemps tmp(st);
+    unsigned long long* known = nullptr;
+    if (ranges) {
+        const long long n = g.C / g.stride[2] * g.U;
+        unsigned *d_mixed = nullptr, mixed = 0;
+        BF_CUDA(tmp.get(&known, (size_t)n));
+        BF_CUDA(tmp.get(&d_mixed, 1));
+        BF_CUDA(cudaMemsetAsync(d_mixed, 0, sizeof(unsigned), st));
+        const int nb = grid_blocks(n * 32, 256);
+        if (g.D == 3) k_shape_ranges<3><<<nb, 256, 0, st>>>(g, *ranges, n, known, d_mixed);
+        else k_shape_ranges<4><<<nb, 256, 0, st>>>(g, *ranges, n, known, d_mixed);
+        BF_CUDA(cudaGetLastError());
+        BF_CUDA(cudaMemcpyAsync(&mixed, d_mixed, sizeof mixed, cudaMemcpyDeviceToHost, st));
+        BF_CUDA(cudaStreamSynchronize(st));
+        if (mixed) known = nullptr;
+    }
+    if (a->box_fmt == kBoxRecompute) {
+        // best effort: without the memory the boxes are regenerated in relax
+        if (known && build_word(a, known, ranges, st) == BF_ERR_CUDA) return BF_ERR_CUDA;
+        return BF_OK;
+    }
+    if (a->box_fmt != kBoxCompact || g.D < 2 || g.periodic[0] || g.periodic[1]) return BF_OK;
     int rc;
-    switch (a->g.D) {
-        case 2: rc = build_shapes_t<2>(a, st); break;
-        case 3: rc = build_shapes_t<3>(a, st); break;
-        default: rc = build_shapes_t<4>(a, st); break;
+    switch (g.D) {
+        case 2: rc = build_shapes_t<2>(a, known, st); break;
+        case 3: rc = build_shapes_t<3>(a, known, st); break;
+        default: rc = build_shapes_t<4>(a, known, st); break;
     }
     if (rc == BF_OK && a->d_shape && a->shape_mismatch == 0) rc = build_templates(a, st);
-    if (rc == BF_OK && a->d_tent) rc = build_word(a, st);
+    if (rc == BF_OK && a->d_tent) rc = build_word(a, a->d_shape, known ? ranges : nullptr, st);
     return rc;
 }
 
@@ -1434,6 +1552,7 @@ extern "C" int abs_build(const bf_dynamics* dyn, const bf_grid* grid, const bf_i
         rc = build_ranges(a, t, tmp, st);
         if (rc == BF_OK && mode == BF_MODE_STORED) rc = boxes_from_ranges(a, t, st);
         if (rc == BF_OK) rc = g.D == 3 ? build_pred_ranges_t<3>(a, t, tmp, st) : build_pred_ranges_t<4>(a, t, tmp, st);
+        if (rc == BF_OK) rc = build_shapes(a, &t, st);
     } else {
         if (mode == BF_MODE_STORED) {
             const int nb = grid_blocks(a->g.C * a->g.U, 128);
@@ -1445,12 +1564,12 @@ extern "C" int abs_build(const bf_dynamics* dyn, const bf_grid* grid, const bf_i
         }
         rc = build_pred(a, st);
         if (rc == BF_OK && mode == BF_MODE_STORED) rc = to_compact(a, st);
+        if (rc == BF_OK && mode == BF_MODE_STORED) rc = build_shapes(a, nullptr, st);
     }
     if (rc == BF_OK) {
         e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = bfh::cuda_fail(e, "abs_build kernels");
     }
-    if (rc == BF_OK && mode == BF_MODE_STORED) rc = build_shapes(a, st);
     if (rc) { abs_free(a); return rc; }
     *out = a;
     return BF_OK;
@@ -1586,7 +1705,7 @@ extern "C" int abs_from_boxes(const bf_grid* grid, int32_t ninputs, const int16_
         if (e != cudaSuccess) rc = bfh::cuda_fail(e, "abs_from_boxes pred");
     }
     if (rc == BF_OK) rc = to_compact(a, st);
-    if (rc == BF_OK) rc = build_shapes(a, st);
+    if (rc == BF_OK) rc = build_shapes(a, nullptr, st);
     if (rc) { abs_free(a); return rc; }
     *out = a;
     return BF_OK;

@@ -337,7 +337,7 @@ static int ws_word(const bf_abstraction* a, bf_solve_ws* w, cudaStream_t st) {
     WordInst& v = w->word;
     memset(&v, 0, sizeof v);
     v.g = a->g;
-    v.planes = (int)a->nplanes;
+    v.planes = (int)(a->g.C / a->g.stride[2]);
     v.plane_cells = (int)a->g.stride[2];
     v.plane_words = a->word_plane_words;
     v.plane_units = (v.plane_words + 31) / 32;
