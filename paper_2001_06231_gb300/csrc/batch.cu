@@ -377,6 +377,8 @@ Engine::~Engine() {
     }
     insts_.clear();
     if (dev_mem_) cudaFreeAsync(dev_mem_, st_);
+    if (words_) cudaFreeAsync(words_, st_);
+    if (word_ctr_) cudaFreeAsync(word_ctr_, st_);
     cudaStreamSynchronize(st_);
     if (pool_) cudaMemPoolDestroy(pool_);
 }
@@ -394,6 +396,12 @@ size_t Engine::state_bytes_for(long long Cc, int Uc, bool stage_G, bool stage_T,
     if (stage_V) o += r256(8 * C);
     return o;
 }
+
+}  // namespace bfb
+// solve_word.cu
+int word_wave(int units);
+int word_solve_batch(const bfk::WordInst* insts, int n, int passes, bfk::WordCtr* k, cudaStream_t st);
+namespace bfb {
 
 static int group_of(const bf_abstraction* a) {
     return (a->g.D - 1) * 4 + a->box_fmt;
@@ -415,18 +423,29 @@ int Engine::add(const bf_abstraction* a, const double* G, const unsigned char* t
     const bool sAv = avoid && !bfh::is_device_ptr(avoid);
     const bool vdev = bfh::is_device_ptr(V);
     const bool mdev = bfh::is_device_ptr(mu);
+    // the word engine: its bitmaps instead of the lists and the transposed costs
+    // (where they take no more: tiny planes waste words)
+    const int bs = a->bsched >= 0 ? a->bsched : kBsDefault;
+    const size_t list_bytes = r256(4 * (size_t)S) + 2 * r256(4 * (size_t)C) + r256(8 * (size_t)C * U);
+    bfk::WordInst wi;
+    bool word = (bs & kBsWords) && a->d_vbits;
+    if (word) {
+        word_geometry(wi, a);
+        word = word_state_bytes(wi) <= list_bytes && word_wave(wi.units) > 0;
+    }
+    auto need = [&](int t) { return !word || ((a->word_vtabs >> t) & 1) ? r256(8 * (size_t)C) : 0; };
     size_t o = 0;
     const size_t o_ctr = o;  o += r256(sizeof(Counters));
-    const size_t o_vk = o;   o += r256(8 * (size_t)C);
+    const size_t o_vk = o;   o += need(0);
     const size_t o_vn = o;   o += r256(8 * (size_t)C);
-    const size_t o_m2 = o;   o += r256(8 * (size_t)C);
-    const size_t o_m3 = o;   o += r256(8 * (size_t)C);
-    const size_t o_m33 = o;  o += r256(8 * (size_t)C);
+    const size_t o_m2 = o;   o += need(1);
+    const size_t o_m3 = o;   o += need(2);
+    const size_t o_m33 = o;  o += need(3);
     const size_t o_mu = o;   o += r256((size_t)C);
-    const size_t o_fb = o;   o += r256(4 * (size_t)S);
-    const size_t o_cl = o;   o += r256(4 * (size_t)C);
-    const size_t o_chg = o;  o += r256(4 * (size_t)C);
-    const size_t o_gi = o;   o += r256(8 * (size_t)C * U);
+    const size_t o_fb = o;   o += word ? word_state_bytes(wi) : r256(4 * (size_t)S);
+    const size_t o_cl = o;   o += word ? 0 : r256(4 * (size_t)C);
+    const size_t o_chg = o;  o += word ? 0 : r256(4 * (size_t)C);
+    const size_t o_gi = o;   o += word ? 0 : r256(8 * (size_t)C * U);
     const size_t o_sg = o;   o += sG ? r256(8 * (size_t)C * U) : 0;
     const size_t o_st = o;   o += sT ? r256(8 * (size_t)C) : 0;
     const size_t o_stg = o;  o += sTg ? r256((size_t)C) : 0;
@@ -449,7 +468,6 @@ int Engine::add(const bf_abstraction* a, const double* G, const unsigned char* t
     v.M2 = reinterpret_cast<long long*>(m + o_m2);
     v.M3 = reinterpret_cast<long long*>(m + o_m3);
     // the batched schedule of the abstraction (bf_tune_batch) or the default
-    const int bs = a->bsched >= 0 ? a->bsched : kBsDefault;
     if ((bs & kBsWindow33) && a->g.D >= 2) v.M33 = reinterpret_cast<long long*>(m + o_m33);
     if ((bs & kBsPlane) && a->d_poffs[0]) v.poffs = a->d_poffs[v.M33 ? 1 : 0];
     if ((bs & kBsQueue) && a->d_fmask) v.fmask = a->d_fmask;
@@ -487,6 +505,27 @@ int Engine::add(const bf_abstraction* a, const double* G, const unsigned char* t
     s->V_host = vdev ? nullptr : V;
     s->mu_host = mdev ? nullptr : mu;
     s->mu_dev_out = mdev ? mu : nullptr;
+    if (word) {
+        // set up by the first launch
+        s->word = true;
+        BF_CUDA(cudaMemsetAsync(m + o_fb, 0, word_state_bytes(wi), st_));
+        word_state(wi, m + o_fb);
+        wi.G = dG;
+        wi.terminal = dT;
+        wi.target = dTg;
+        wi.avoid = dAv;
+        wi.Vnew = v.Vnew;
+        wi.tab[0] = v.Vkey;
+        wi.tab[1] = v.M2;
+        wi.tab[2] = v.M3;
+        wi.tab[3] = reinterpret_cast<long long*>(m + o_m33);
+        wi.mu = v.mu;
+        wi.cap = s->cap;
+        s->winst = wi;
+        insts_.push_back(s);
+        if (out) *out = s;
+        return BF_OK;
+    }
     // lines 1-10 of Algorithm 1
     k_b_counters<<<1, 1, 0, st_>>>(v.ctr, s->cap);
     BF_CUDA(cudaMemsetAsync(v.fbits, 0, 4 * (size_t)S, st_));
@@ -517,8 +556,34 @@ void Engine::remove(InstState* s) {
 
 int Engine::rebuild() {
     std::stable_sort(insts_.begin(), insts_.end(),
-                     [](const InstState* x, const InstState* y) { return x->group < y->group; });
-    const int n = (int)insts_.size();
+                     [](const InstState* x, const InstState* y) {
+                         return x->word != y->word ? !x->word : x->group < y->group;
+                     });
+    // the word engine's instances come last
+    int n = (int)insts_.size();
+    nwords_ = 0;
+    while (n > 0 && insts_[n - 1]->word) {
+        --n;
+        ++nwords_;
+    }
+    if (nwords_) {
+        host_words_.resize(nwords_);
+        for (int i = 0; i < nwords_; ++i) host_words_[i] = insts_[n + i]->winst;
+        const size_t bytes = r256(sizeof(bfk::WordInst) * (size_t)nwords_);
+        if (bytes > words_bytes_) {
+            if (words_) BF_CUDA(cudaFreeAsync(words_, st_));
+            words_ = nullptr;
+            words_bytes_ = 0;
+            if (int rc = alloc((void**)&words_, bytes)) return rc;
+            words_bytes_ = bytes;
+        }
+        if (!word_ctr_) {
+            if (int rc = alloc((void**)&word_ctr_, r256(sizeof(bfk::WordCtr)))) return rc;
+            BF_CUDA(cudaMemsetAsync(word_ctr_, 0, sizeof(bfk::WordCtr), st_));
+        }
+        BF_CUDA(cudaMemcpyAsync(words_, host_words_.data(), sizeof(bfk::WordInst) * nwords_, cudaMemcpyHostToDevice,
+                                st_));
+    }
     memset(&dev_, 0, sizeof dev_);
     dev_.n = n;
     // groups (same dimension and box format)
@@ -683,7 +748,25 @@ void Engine::launch_pass(cudaGraphConditionalHandle h, int use_graph) {
     k_b_plan<<<1, 1024, 0, st_>>>(dev_, 2, h, use_graph);
 }
 
+// The word engine's instances: at most `passes` passes (negative: all).
+int Engine::run_words(int passes) {
+    if (nwords_ == 0) return BF_OK;
+    return word_solve_batch(words_, nwords_, passes, word_ctr_, st_);
+}
+
+// Did a block give up waiting?  (synchronizes)
+int Engine::word_fault() {
+    if (!word_ctr_) return BF_OK;
+    int fault = 0;
+    BF_CUDA(cudaMemcpyAsync(&fault, &word_ctr_->fault, sizeof fault, cudaMemcpyDeviceToHost, st_));
+    BF_CUDA(cudaStreamSynchronize(st_));
+    if (!fault) return BF_OK;
+    bfh::set_error("batch: a block gave up waiting at the grid barrier");
+    return BF_ERR_TIMEOUT;
+}
+
 int Engine::run_to_completion() {
+    if (int rc = run_words(-1)) return rc;
     if (dev_.n == 0) return BF_OK;
     cudaGraph_t graph;
     BF_CUDA(cudaGraphCreate(&graph, 0));
@@ -790,7 +873,9 @@ int Engine::build_step_graph(int passes, cudaGraphExec_t* out) {
 }
 
 int Engine::step(int passes, bool graph) {
-    if (dev_.n == 0 || passes <= 0) return BF_OK;
+    if (passes <= 0) return BF_OK;
+    if (int rc = run_words(passes)) return rc;
+    if (dev_.n == 0) return BF_OK;
     if (!graph) {
         for (int p = 0; p < passes; ++p) launch_pass(0, 0);
         BF_CUDA(cudaGetLastError());
@@ -813,19 +898,41 @@ int Engine::step(int passes, bool graph) {
 
 int Engine::read_counters(std::vector<Counters>& out) {
     out.resize(insts_.size());
-    for (size_t i = 0; i < insts_.size(); ++i)
-        BF_CUDA(cudaMemcpyAsync(&out[i], insts_[i]->view.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, st_));
+    std::vector<bfk::WordCtr> wc(insts_.size());
+    for (size_t i = 0; i < insts_.size(); ++i) {
+        if (insts_[i]->word)
+            BF_CUDA(cudaMemcpyAsync(&wc[i], insts_[i]->winst.ctr, sizeof wc[i], cudaMemcpyDeviceToHost, st_));
+        else
+            BF_CUDA(cudaMemcpyAsync(&out[i], insts_[i]->view.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, st_));
+    }
     BF_CUDA(cudaStreamSynchronize(st_));
-    return BF_OK;
+    for (size_t i = 0; i < insts_.size(); ++i)
+        if (insts_[i]->word) {
+            memset(&out[i], 0, sizeof out[i]);
+            out[i].done = wc[i].done;
+            out[i].round = wc[i].round;
+            out[i].status = wc[i].status;
+            out[i].err = wc[i].err;
+        }
+    return word_fault();
 }
 
 int Engine::finish_instance(InstState* s, int64_t* iters, int32_t* status, int* err) {
     const long long C = s->a->g.C;
-    k_b_output<<<blocks_for(C), 256, 0, st_>>>(C, s->view.Vkey, s->Vdev);
+    k_b_output<<<blocks_for(C), 256, 0, st_>>>(C, s->word ? s->view.Vnew : s->view.Vkey, s->Vdev);
     BF_CUDA(cudaGetLastError());
     if (s->V_host) BF_CUDA(cudaMemcpyAsync(s->V_host, s->Vdev, 8 * (size_t)C, cudaMemcpyDeviceToHost, st_));
     if (s->mu_host) BF_CUDA(cudaMemcpyAsync(s->mu_host, s->view.mu, (size_t)C, cudaMemcpyDeviceToHost, st_));
     else BF_CUDA(cudaMemcpyAsync(s->mu_dev_out, s->view.mu, (size_t)C, cudaMemcpyDeviceToDevice, st_));
+    if (s->word) {
+        bfk::WordCtr wc;
+        BF_CUDA(cudaMemcpyAsync(&wc, s->winst.ctr, sizeof wc, cudaMemcpyDeviceToHost, st_));
+        BF_CUDA(cudaStreamSynchronize(st_));
+        *iters = wc.round;
+        *status = wc.status;
+        *err = wc.err;
+        return word_fault();
+    }
     Counters hc;
     BF_CUDA(cudaMemcpyAsync(&hc, s->view.ctr, sizeof hc, cudaMemcpyDeviceToHost, st_));
     BF_CUDA(cudaStreamSynchronize(st_));
@@ -930,10 +1037,33 @@ extern "C" int bf_tune_batch(int32_t n, const bf_abstraction* const* abs, const 
         ++tried;
     }
     const double default_ms = best;
+    // the word engine against two list schedules (marking by box size, and the
+    // pair queue with marking in relax); the descent below is over the list
+    // form's bits and is left out where the word engine stays ahead of them
+    bool words = false;
+    for (int i = 0; i < n; ++i) words |= abs[i]->d_vbits != nullptr;
+    if (words) {
+        const int lists = kBsDefault & ~kBsWords;
+        const int cands[5] = {lists, (lists & ~kBsMarkAuto) | kBsMark | kBsQueue, lists & ~kBsPair,
+                              (lists & ~kBsMarkAuto) | kBsMark, (lists & ~kBsMarkAuto) | kBsQueue};
+        for (int j = 0; j < 5 && rc == BF_OK; ++j) {
+            set_all(cands[j]);
+            double ms = 0.0;
+            rc = batch_time(n, abs, G, target, avoid, terminal, max_iters, V.data(), mu.data(), it.data(), stv.data(),
+                            st, &ms);
+            ++tried;
+            if (rc == BF_OK && ms < best) {
+                best = ms;
+                b = cands[j];
+            }
+        }
+    } else {
+        b &= ~kBsWords;
+    }
     // coordinate descent over the schedule bits, two rounds; the marking
     // dimension times both fixed choices against marking by box size
     const int bits[6] = {kBsMark, kBsWindow33, kBsPlane, kBsTemplates, kBsPair, kBsQueue};
-    for (int round = 0; round < 2 && rc == BF_OK; ++round)
+    for (int round = 0; round < 2 && rc == BF_OK && !(b & kBsWords); ++round)
         for (int k = 0; k < 6 && rc == BF_OK; ++k) {
             const int base = b;
             int cands[2];
@@ -969,6 +1099,15 @@ extern "C" int bf_tune_batch(int32_t n, const bf_abstraction* const* abs, const 
     set_all(b);
     const int bs = b;
     memset(out, 0, sizeof *out);
+    if (bs & kBsWords) {
+        // as a schedule: the pair queue with the per-input frontier
+        out->window33 = out->plane_lists = out->templates = out->pair_inputs = out->input_frontier = 1;
+        out->cell_masks = 2;
+        out->candidates = tried;
+        out->best_ms = best;
+        out->default_ms = default_ms;
+        return BF_OK;
+    }
     out->fuse_mark = (bs & kBsMarkAuto) ? -1 : ((bs & kBsMark) ? 1 : 0);
     out->window33 = (bs & kBsWindow33) ? 1 : 0;
     out->plane_lists = (bs & kBsPlane) ? 1 : 0;
@@ -993,6 +1132,7 @@ extern "C" int bf_set_batch_schedule(bf_abstraction* a, const bf_tune_result* sc
     int bs = (sched->window33 ? kBsWindow33 : 0) | (sched->plane_lists ? kBsPlane : 0) |
              (sched->templates ? kBsTemplates : 0) | (sched->pair_inputs ? kBsPair : 0) |
              (sched->cell_masks ? kBsQueue : 0);
+    if (sched->input_frontier && sched->cell_masks && sched->templates && sched->plane_lists) bs |= kBsWords;
     if (sched->fuse_mark == 1) bs |= kBsMark;
     if (sched->fuse_mark == -1) bs |= kBsMarkAuto;
     a->bsched = bs;

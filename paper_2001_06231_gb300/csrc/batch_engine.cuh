@@ -10,6 +10,10 @@
 // Instances keep their own pass counters, frontiers and termination, so each
 // result is identical to a solo bf_solve.
 //
+// Instances whose abstraction has the word engine's data (word_engine.cuh) and
+// whose batched schedule does not name another form run apart from the groups:
+// all of them in one cooperative launch, whole or a bounded number of passes.
+//
 // bf_solve_batch runs the pass loop inside a CUDA graph WHILE node; the
 // server (serve.cu) runs a bounded number of passes per engine step and lets
 // instances join and leave between steps.
@@ -19,6 +23,7 @@
 #include <vector>
 
 #include "solve_core.cuh"
+#include "word_engine.cuh"
 
 namespace bfb {
 
@@ -45,6 +50,8 @@ struct BatchDev {
 struct InstState {
     const bf_abstraction* a = nullptr;
     InstView view;
+    bool word = false;            // advanced by the word engine (winst), not by the groups
+    bfk::WordInst winst;
     void* mem = nullptr;          // owned allocation (state + staging)
     double* G = nullptr;          // device copies or caller device pointers
     const unsigned char* target = nullptr;
@@ -101,6 +108,14 @@ private:
     std::vector<InstState*> insts_;
     std::vector<InstView> host_views_;   // kept alive until the async copy is done
     BatchDev dev_{};
+    // instances of the word engine: device array, its barrier counters
+    bfk::WordInst* words_ = nullptr;
+    size_t words_bytes_ = 0;
+    bfk::WordCtr* word_ctr_ = nullptr;
+    int nwords_ = 0;
+    std::vector<bfk::WordInst> host_words_;
+    int run_words(int passes);
+    int word_fault();
     void* dev_mem_ = nullptr;
     size_t dev_mem_bytes_ = 0;
     int relax_blocks_ = 0, prop_blocks_ = 0, compact_blocks_ = 0;

@@ -326,32 +326,16 @@ static int ws_list(bf_solve_ws* w) {
     return BF_OK;
 }
 
-// Word engine state (once per workspace): [counters][changed and infinite, by
-// parity][not avoid][windows][live words][changed units, by parity][smallest
-// costs], the
-// windows with room for a word before and after.  word_blocks = 0 where the
-// engine does not apply.
+// Word engine state (once per workspace); word_blocks = 0 where the engine does
+// not apply.
 static int ws_word(const bf_abstraction* a, bf_solve_ws* w, cudaStream_t st) {
     if (w->word_blocks >= 0) return BF_OK;
     if (!a->d_vbits) { w->word_blocks = 0; return BF_OK; }
     WordInst& v = w->word;
-    memset(&v, 0, sizeof v);
-    v.g = a->g;
-    v.planes = (int)(a->g.C / a->g.stride[2]);
-    v.plane_cells = (int)a->g.stride[2];
-    v.plane_words = a->word_plane_words;
-    v.plane_units = (v.plane_words + 31) / 32;
-    v.unit_words = (v.plane_words + v.plane_units - 1) / v.plane_units;     // even units
-    v.units = v.planes * v.plane_units;
-    v.S = v.planes * v.plane_words;
+    word_geometry(v, a);
     const int blocks = word_wave(v.units);
     if (blocks == 0) { w->word_blocks = 0; return BF_OK; }
-    auto up = [](size_t n) { return (n + 255) / 256 * 256; };
-    const size_t words = up(4 * (size_t)v.S), units = up((size_t)v.units), win = 2 * words + 512;
-    int nt = 0;
-    for (int t = 0; t < 16; ++t) nt += (a->word_btabs >> t) & 1;
-    const size_t bytes = up(sizeof(WordCtr)) + 5 * words + nt * win + up(4 * (size_t)v.units) + 2 * units +
-                         up(8 * (size_t)w->C);
+    const size_t bytes = word_state_bytes(v);
     cudaError_t e = cudaMalloc(&w->word_mem, bytes);
     if (e == cudaSuccess) e = cudaMemsetAsync(w->word_mem, 0, bytes, st);
     if (e != cudaSuccess) {
@@ -359,23 +343,7 @@ static int ws_word(const bf_abstraction* a, bf_solve_ws* w, cudaStream_t st) {
         w->word_mem = nullptr;
         return bfh::cuda_fail(e, "word engine workspace");
     }
-    unsigned char* p = (unsigned char*)w->word_mem;
-    auto take = [&](size_t n) { unsigned char* q = p; p += n; return q; };
-    v.ctr = (WordCtr*)take(up(sizeof(WordCtr)));
-    v.raw[0] = (uint2*)take(2 * words);
-    v.raw[1] = (uint2*)take(2 * words);
-    v.act = (unsigned*)take(words);
-    for (int t = 0; t < 16; ++t)
-        if ((a->word_btabs >> t) & 1) v.bt[t] = (uint2*)(take(win) + 256);
-    v.live = (unsigned*)take(up(4 * (size_t)v.units));
-    v.flags[0] = take(units);
-    v.flags[1] = take(units);
-    v.gmin = (double*)take(up(8 * (size_t)w->C));
-    v.vtabs = a->word_vtabs;
-    v.btabs = a->word_btabs;
-    v.lists = a->d_wlists;
-    v.vbits = a->d_vbits;
-    v.spans = a->d_spans;
+    word_state(v, w->word_mem);
     v.Vnew = w->Vnew;
     v.tab[0] = w->Vkey;
     v.tab[1] = w->M2;

@@ -33,6 +33,8 @@
 // V, the tables and the bitmaps stay in the L2; the costs are read in the
 // caller's layout [C][U], only by the pairs that pass the tests.
 #pragma once
+#include <cstring>
+
 #include "solve_core.cuh"
 
 namespace bfk {
@@ -50,6 +52,7 @@ constexpr int kWordEntries = 4096;    // table entries queued by a block
 constexpr int kWordMaxU = 32;
 constexpr int kWordTest = 256;        // units tested at a time
 constexpr unsigned kWordSpinMax = 1u << 22;
+constexpr int kWordInsts = 256;       // instances of one batched launch
 constexpr long long kNoCand = 0x7FFFFFFFFFFFFFFFLL;
 
 // List of a (plane, input): int 0 = bit lookups | bit table << 8, ints 1 .. 31
@@ -70,6 +73,7 @@ struct WordCtr {
     int fault;                        // a block gave up waiting at a barrier
     int status;
     int done;
+    int ready;                        // batched form: the set-up was run
     long long round;                  // passes completed
     unsigned long long gate[4];       // barrier after the relax phase of pass r: gate[r & 3] = blocks arrived |
                                       // blocks with frontier cells << 16 | blocks with changed cells << 32
@@ -122,13 +126,24 @@ struct WordSmem {
             unsigned f1[kWordUnits * 32];     // frontier cells of the batch's words
             unsigned short slot[kWordUnits * 32];       // words with pairs: their slot in the batch, 0xFFFF: none
             unsigned short word[kWordUnits * 32];       // slots: unit of the batch << 5 | word
-            int4 at[kWordSlots];              // slots of the window: {first cell, word, first row, plane}
+            int4 at[kWordSlots];              // slots of the window: {first cell, word, first row, plane | instance << 24}
             int4 unit[kWordTest];             // units to relax {unit, plane | words << 24, first word, first cell}
+            // batched form: the units' instances; of the batch's units the first
+            // row and the counts, of its rows the unit
+            unsigned char inst[kWordTest], of_row[kWordRows];
+            int row0[kWordUnits + 1];
+            unsigned long long count[kWordUnits];
         } r;
         struct {
             int cell[kWordEntries];           // entries to recompute, -1: none
+            unsigned char inst[kWordEntries];
         } t;
     };
+    // batched form: units of this block before an instance's, its pass, active
+    int before[kWordInsts + 1];
+    long long round[kWordInsts];
+    unsigned char active[kWordInsts];
+    int nu;
     unsigned queued;                          // queue length
     int nover;                                // rows that did not fit
     int nslots;
@@ -137,6 +152,54 @@ struct WordSmem {
     unsigned long long gate;
     unsigned long long part[kWordWarps];
 };
+
+// Host: the geometry of an abstraction's bitmaps, and the bytes of an instance's
+// engine state: [counters][changed and infinite, by parity][not avoid][windows]
+// [live words][changed units, by parity][smallest costs], the windows with room
+// for a word before and after.
+inline size_t word_up(size_t n) { return (n + 255) / 256 * 256; }
+
+inline void word_geometry(WordInst& v, const bf_abstraction* a) {
+    memset(&v, 0, sizeof v);
+    v.g = a->g;
+    v.planes = (int)(a->g.C / a->g.stride[2]);
+    v.plane_cells = (int)a->g.stride[2];
+    v.plane_words = a->word_plane_words;
+    v.plane_units = (v.plane_words + 31) / 32;
+    v.unit_words = (v.plane_words + v.plane_units - 1) / v.plane_units;     // even units
+    v.units = v.planes * v.plane_units;
+    v.S = v.planes * v.plane_words;
+    v.vtabs = a->word_vtabs;
+    v.btabs = a->word_btabs;
+    v.lists = a->d_wlists;
+    v.vbits = a->d_vbits;
+    v.spans = a->d_spans;
+}
+
+inline size_t word_state_bytes(const WordInst& v) {
+    int nt = 0;
+    for (int t = 0; t < 16; ++t) nt += (v.btabs >> t) & 1;
+    const size_t words = word_up(4 * (size_t)v.S), units = word_up((size_t)v.units);
+    return word_up(sizeof(WordCtr)) + 5 * words + (size_t)nt * (2 * words + 512) + word_up(4 * (size_t)v.units) +
+           2 * units + word_up(8 * (size_t)v.g.C);
+}
+
+// Carve the state from p (word_state_bytes, zeroed).
+inline void word_state(WordInst& v, void* mem) {
+    unsigned char* p = (unsigned char*)mem;
+    auto take = [&](size_t n) { unsigned char* q = p; p += n; return q; };
+    const size_t words = word_up(4 * (size_t)v.S), units = word_up((size_t)v.units);
+    v.ctr = (WordCtr*)take(word_up(sizeof(WordCtr)));
+    v.raw[0] = (uint2*)take(2 * words);
+    v.raw[1] = (uint2*)take(2 * words);
+    v.act = (unsigned*)take(words);
+    for (int t = 0; t < 16; ++t)
+        if ((v.btabs >> t) & 1) v.bt[t] = (uint2*)(take(2 * words + 512) + 256);
+    v.live = (unsigned*)take(word_up(4 * (size_t)v.units));
+    v.flags[0] = take(units);
+    v.flags[1] = take(units);
+    v.gmin = (double*)take(word_up(8 * (size_t)v.g.C));
+}
 
 // ---------------------------------------------------------------------------
 // grid barrier (cooperative launch: every block is resident)
@@ -312,6 +375,44 @@ __device__ __forceinline__ void word_unit(const WordInst& w, int un, int& p, int
     n = min(w.unit_words, w.plane_words - k);
 }
 
+// Batched form: instance i's units of this block are first + j gridDim.x
+// (rotated from instance to instance: small instances spread over the blocks).
+__device__ __forceinline__ int word_first(int i) { return (int)((blockIdx.x + 53u * (unsigned)i) % gridDim.x); }
+
+__device__ __forceinline__ int word_share(int units, int first) {
+    return first < units ? (units - 1 - first) / (int)gridDim.x + 1 : 0;
+}
+
+// before[] of the active instances (whole block); the total.
+__device__ __forceinline__ int word_split(const WordInst* insts, int n, WordSmem& sm) {
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        unsigned sum = 0u;
+        for (int i = lane; i - lane < n; i += 32) {
+            unsigned tot;
+            const unsigned own = i < n && sm.active[i] ? (unsigned)word_share(insts[i].units, word_first(i)) : 0u;
+            const unsigned pre = word_scan(own, tot);
+            if (i < n) sm.before[i] = (int)(sum + pre);
+            sum += tot;
+        }
+        if (lane == 0) sm.before[n] = (int)sum;
+    }
+    __syncthreads();
+    return sm.before[n];
+}
+
+// The instance of the block's c-th unit: the last with before <= c that has units.
+__device__ __forceinline__ int word_find(const WordSmem& sm, int n, int c) {
+    int a = 0, b = n;
+    while (b - a > 1) {
+        const int h = (a + b) >> 1;
+        if (sm.before[h] <= c) a = h;
+        else b = h;
+    }
+    return a;
+}
+
 // Can a lookup of the words k .. k + n - 1 of plane p meet a changed entry?
 // (whole warp; lanes take the plane's spans)
 __device__ __forceinline__ bool word_live(const WordInst& w, int p, int k, int n) {
@@ -390,9 +491,9 @@ __device__ __forceinline__ bool word_queue(WordSmem& sm, unsigned m, unsigned ta
 // their own cost (from HBM) and their other lookups; the rest move together,
 // warp by warp.  A queue that gives a thread one pair at most skips the test:
 // it only adds a round of loads then.
-__device__ __forceinline__ void word_pairs(const WordInst& w, WordSmem& sm) {
+template <bool M>
+__device__ __forceinline__ void word_pairs(const WordInst& w0, const WordInst* insts, WordSmem& sm) {
     const int np = (int)min(sm.queued, (unsigned)kWordPairs);
-    const int U = w.g.U;
     const int lane = threadIdx.x & 31;
     for (int k0 = 0; k0 < np; k0 += kWordPer * kWordThreads) {
         // this thread's places: own[j kWordThreads]
@@ -414,6 +515,7 @@ __device__ __forceinline__ void word_pairs(const WordInst& w, WordSmem& sm) {
                     a[j] = b[j] = kKeyInf;
                     if (e[j] != ~0u) {
                         const int4 at = sm.r.at[e[j] >> 13];
+                        const WordInst& w = M ? insts[at.w >> 24] : w0;
                         const int c = at.x + (int)((e[j] >> 8) & 31u);
                         const int* l = reinterpret_cast<const int*>(sm.r.list[at.z + (int)(e[j] & 0xFFu)]);
                         const long long* tb = w.tab[l[0] >> 8] + c;
@@ -443,9 +545,12 @@ __device__ __forceinline__ void word_pairs(const WordInst& w, WordSmem& sm) {
             d[j] = kNoCand;
             if (j * 32 + lane < n) {
                 const unsigned e = own[j * kWordThreads];
-                if (e != ~0u)
+                if (e != ~0u) {
+                    const int4 at = sm.r.at[e >> 13];
+                    const WordInst& w = M ? insts[at.w >> 24] : w0;
                     d[j] = __double_as_longlong(
-                        __ldcs(w.G + (long long)(sm.r.at[e >> 13].x + (int)((e >> 8) & 31u)) * U + (e & 0xFFu)));
+                        __ldcs(w.G + (long long)(at.x + (int)((e >> 8) & 31u)) * w.g.U + (e & 0xFFu)));
+                }
             }
         }
 #pragma unroll
@@ -454,6 +559,7 @@ __device__ __forceinline__ void word_pairs(const WordInst& w, WordSmem& sm) {
             if (e == ~0u) continue;
             const int i = (int)(e >> 8), u = (int)(e & 0xFFu);
             const int4 at = sm.r.at[i >> 5];
+            const WordInst& w = M ? insts[at.w >> 24] : w0;
             const int4* l = sm.r.list[at.z + u];
             const int hdr = l[0].x;
             const int L = hdr & 0xFF;
@@ -465,7 +571,7 @@ __device__ __forceinline__ void word_pairs(const WordInst& w, WordSmem& sm) {
                 m = max(m, max(max(tb[q.x], tb[q.y]), max(tb[q.z], tb[q.w])));
                 if (L > kWordHead) {
                     const int4* rest = reinterpret_cast<const int4*>(
-                        w.lists + ((long long)at.w * U + u) * kWordEnt + kWordVal + kWordHead);
+                        w.lists + ((long long)(at.w & 0xFFFFFF) * w.g.U + u) * kWordEnt + kWordVal + kWordHead);
                     for (int t = kWordHead; t < L; t += 4) {
                         const int4 z = __ldg(rest++);
                         m = max(m, max(max(tb[z.x], tb[z.y]), max(tb[z.z], tb[z.w])));
@@ -488,8 +594,10 @@ __device__ __forceinline__ void word_pairs(const WordInst& w, WordSmem& sm) {
 }
 
 // The window's cells whose smallest candidate is below W (whole block).
-__device__ __forceinline__ void word_commit(const WordInst& w, uint2* raw, unsigned char* flags, const int4* unit,
-                                            int first, int ns, WordSmem& sm, unsigned long long& count) {
+template <bool M>
+__device__ __forceinline__ void word_commit(const WordInst& w0, const WordInst* insts, long long round0,
+                                            const int4* unit, int first, int ns, WordSmem& sm,
+                                            unsigned long long& count) {
     constexpr int K = 3;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int j0 = wid; j0 < ns; j0 += kWordWarps * K) {
@@ -501,8 +609,10 @@ __device__ __forceinline__ void word_commit(const WordInst& w, uint2* raw, unsig
             b[q] = kNoCand;
             if (j < ns) {
                 const int4 at = sm.r.at[j];
+                const WordInst& w = M ? insts[at.w >> 24] : w0;
+                const long long round = M ? sm.round[at.w >> 24] : round0;
                 b[q] = sm.best[j * 32 + lane];
-                x[q] = raw[at.y];
+                x[q] = w.raw[round & 1][at.y];
                 if (b[q] != kNoCand) old[q] = w.Vnew[at.x + lane];
             }
         }
@@ -511,6 +621,7 @@ __device__ __forceinline__ void word_commit(const WordInst& w, uint2* raw, unsig
             const int j = j0 + q * kWordWarps;
             if (j >= ns) continue;
             const int4 at = sm.r.at[j];
+            const WordInst& w = M ? insts[at.w >> 24] : w0;
             bool changed = false;
             if (b[q] != kNoCand) {
                 changed = b[q] < old[q];
@@ -523,9 +634,12 @@ __device__ __forceinline__ void word_commit(const WordInst& w, uint2* raw, unsig
             }
             const unsigned m = __ballot_sync(0xFFFFFFFFu, changed);
             if (lane == 0 && m) {
-                raw[at.y] = make_uint2(m, x[q].y & ~m);
-                flags[unit[sm.r.word[first + j] >> 5].x] = 1;
-                count += (unsigned long long)__popc(m);
+                const long long round = M ? sm.round[at.w >> 24] : round0;
+                const int ui = sm.r.word[first + j] >> 5;
+                w.raw[round & 1][at.y] = make_uint2(m, x[q].y & ~m);
+                w.flags[round & 1][unit[ui].x] = 1;
+                if (M) atomicAdd(&sm.r.count[ui], (unsigned long long)__popc(m));
+                else count += (unsigned long long)__popc(m);
             }
         }
     }
@@ -534,36 +648,70 @@ __device__ __forceinline__ void word_commit(const WordInst& w, uint2* raw, unsig
 // The relax phase of one pass over this block's share of the units.  count_only:
 // the frontier is counted and nothing is relaxed (at the pass cap).  count (lane
 // 0 of every warp): frontier cells << 32 | changed cells; pairs (lane 0 of every
-// warp) counts the pairs relaxed.
-__device__ __forceinline__ void word_relax(const WordInst& w, long long round, bool count_only, WordSmem& sm,
-                                           unsigned long long& pairs, unsigned long long& count) {
+// warp) counts the pairs relaxed.  M: the active ones of n instances, each at
+// its own pass (sm.round) and cap, its counts into its own sums.
+template <bool M>
+__device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* insts, int n_insts, long long round,
+                                           bool count_only0, WordSmem& sm, unsigned long long& pairs,
+                                           unsigned long long& count) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int U = w.g.U;
+    const int U0 = M ? 1 : w0.g.U;
     count = 0ull;
     // consecutive units go to different blocks: the frontier is uneven
-    const int mine = (int)blockIdx.x < w.units ? (w.units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    const int batch = min(kWordUnits, kWordRows / U);
+    const int mine = M ? sm.before[n_insts] : word_share(w0.units, (int)blockIdx.x);
     for (int t0 = 0; t0 < mine; t0 += kWordTest) {
         if (threadIdx.x == 0) { sm.nlive = 0; sm.nslots = 0; }
         if (threadIdx.x < kWordUnits * 32) sm.r.f1[threadIdx.x] = 0u;
         __syncthreads();
         for (int i = t0 + wid; i < min(mine, t0 + kWordTest); i += kWordWarps) {
-            const int un = i * gridDim.x + blockIdx.x;
+            const int inst = M ? word_find(sm, n_insts, i) : 0;
+            const WordInst& w = M ? insts[inst] : w0;
+            const int un = M ? word_first(inst) + (i - sm.before[inst]) * (int)gridDim.x : i * gridDim.x + blockIdx.x;
             int p, k, n;
             word_unit(w, un, p, k, n);
-            if (word_live(w, p, k, n) && lane == 0)           // P < 2^24: checked at build
-                sm.r.unit[atomicAdd(&sm.nlive, 1)] =
-                    make_int4(un, p | n << 24, p * w.plane_words + k, p * w.plane_cells + k * 32);
+            if (word_live(w, p, k, n) && lane == 0) {         // P < 2^24: checked at build
+                const int at = atomicAdd(&sm.nlive, 1);
+                sm.r.unit[at] = make_int4(un, p | n << 24, p * w.plane_words + k, p * w.plane_cells + k * 32);
+                if (M) sm.r.inst[at] = (unsigned char)inst;
+            }
         }
         __syncthreads();
         const int nlive = sm.nlive;
-        for (int l0 = 0; l0 < nlive; l0 += batch) {
-            const int nu = min(batch, nlive - l0);
+        for (int l0 = 0, nu; l0 < nlive; l0 += nu) {
             const int4* unit = sm.r.unit + l0;
+            int rows;
+            if (M) {
+                if (wid == 0) {
+                    // as many units as fit: their first rows
+                    const int U = l0 + lane < nlive ? insts[sm.r.inst[l0 + lane]].g.U : 0;
+                    unsigned tot;
+                    const int r0 = (int)word_scan((unsigned)U, tot);
+                    const bool fits = U > 0 && lane < kWordUnits && r0 + U <= kWordRows;
+                    const unsigned fm = __ballot_sync(0xFFFFFFFFu, fits);
+                    const int cnt = __popc(fm);                          // r0 grows: the first lanes
+                    if (fits) {
+                        sm.r.row0[lane] = r0;
+                        sm.r.count[lane] = 0ull;
+                        for (int q = 0; q < U; ++q) sm.r.of_row[r0 + q] = (unsigned char)lane;
+                        if (lane == cnt - 1) {
+                            sm.r.row0[cnt] = r0 + U;
+                            sm.nu = cnt;
+                        }
+                    }
+                }
+                __syncthreads();
+                nu = sm.nu;
+                rows = sm.r.row0[nu];
+            } else {
+                nu = min(min(kWordUnits, kWordRows / U0), nlive - l0);
+                rows = nu * U0;
+            }
             // (unit, input) rows over the warps: the pairs to relax
-            const int rows = nu * U;
             for (int it = wid; it < rows; it += kWordWarps) {
-                const int ui = it / U, u = it - ui * U;
+                const int ui = M ? sm.r.of_row[it] : it / U0;
+                const WordInst& w = M ? insts[sm.r.inst[l0 + ui]] : w0;
+                const int U = M ? w.g.U : U0;
+                const int u = it - (M ? sm.r.row0[ui] : ui * U);
                 const int4 un = unit[ui];
                 const int wd = un.z + lane;
                 const int* list = w.lists + ((long long)(un.y & 0xFFFFFF) * U + u) * kWordEnt;
@@ -584,8 +732,11 @@ __device__ __forceinline__ void word_relax(const WordInst& w, long long round, b
             // slots of the words that have pairs
             for (int ui = wid; ui < nu; ui += kWordWarps) {
                 unsigned any = 0u, n = 0u;
-                for (int u = 0; u < U; ++u) {
-                    const unsigned m = sm.r.mask[ui * U + u][lane];
+                const int r1 = M ? sm.r.row0[ui + 1] : (ui + 1) * U0;
+                bool count_only = count_only0;
+                if (M) count_only = sm.round[sm.r.inst[l0 + ui]] >= insts[sm.r.inst[l0 + ui]].cap;
+                for (int it = M ? sm.r.row0[ui] : ui * U0; it < r1; ++it) {
+                    const unsigned m = sm.r.mask[it][lane];
                     any |= m;
                     n += (unsigned)__popc(m);
                 }
@@ -596,7 +747,8 @@ __device__ __forceinline__ void word_relax(const WordInst& w, long long round, b
                 const unsigned have = count_only ? 0u : __ballot_sync(0xFFFFFFFFu, any != 0u);
                 int s = 0;
                 if (lane == 0) {
-                    count += (unsigned long long)nf << 32;
+                    if (M) atomicAdd(&sm.r.count[ui], (unsigned long long)nf << 32);
+                    else count += (unsigned long long)nf << 32;
                     if (have) {
                         pairs += n;
                         s = atomicAdd(&sm.nslots, __popc(have));
@@ -615,20 +767,23 @@ __device__ __forceinline__ void word_relax(const WordInst& w, long long round, b
                 if ((int)threadIdx.x < ns) {
                     const int x = sm.r.word[s0 + threadIdx.x];
                     const int4 un = unit[x >> 5];
+                    const int inst = M ? sm.r.inst[l0 + (x >> 5)] : 0;
                     sm.r.at[threadIdx.x] =
-                        make_int4(un.w + (x & 31) * 32, un.z + (x & 31), (x >> 5) * U, un.y & 0xFFFFFF);
+                        make_int4(un.w + (x & 31) * 32, un.z + (x & 31), M ? sm.r.row0[x >> 5] : (x >> 5) * U0,
+                                  (int)((unsigned)(un.y & 0xFFFFFF) | (unsigned)inst << 24));
                 }
                 if (threadIdx.x == 0) { sm.queued = 0u; sm.nover = 0; }
                 __syncthreads();
                 for (int it = wid; it < rows; it += kWordWarps) {
-                    const int ui = it / U;
+                    const int ui = M ? sm.r.of_row[it] : it / U0;
+                    const int u = it - (M ? sm.r.row0[ui] : ui * U0);
                     const unsigned s = (unsigned)sm.r.slot[ui * 32 + lane] - (unsigned)s0;
                     const unsigned m = s < (unsigned)ns ? sm.r.mask[it][lane] : 0u;
-                    if (!word_queue(sm, m, s << 13 | (unsigned)(it - ui * U)) && lane == 0)
+                    if (!word_queue(sm, m, s << 13 | (unsigned)u) && lane == 0)
                         sm.r.over[atomicAdd(&sm.nover, 1)] = (short)it;
                 }
                 __syncthreads();
-                word_pairs(w, sm);
+                word_pairs<M>(w0, insts, sm);
                 // rows that did not fit, until every one was queued
                 const int nover = sm.nover;
                 for (int more = nover; more;) {
@@ -639,10 +794,11 @@ __device__ __forceinline__ void word_relax(const WordInst& w, long long round, b
                     for (int i = wid; i < nover; i += kWordWarps) {
                         const int it = sm.r.over[i];
                         if (it < 0) continue;
-                        const int ui = it / U;
+                        const int ui = M ? sm.r.of_row[it] : it / U0;
+                        const int u = it - (M ? sm.r.row0[ui] : ui * U0);
                         const unsigned s = (unsigned)sm.r.slot[ui * 32 + lane] - (unsigned)s0;
                         const unsigned m = s < (unsigned)ns ? sm.r.mask[it][lane] : 0u;
-                        if (word_queue(sm, m, s << 13 | (unsigned)(it - ui * U))) {
+                        if (word_queue(sm, m, s << 13 | (unsigned)u)) {
                             __syncwarp();
                             if (lane == 0) sm.r.over[i] = -1;
                         } else {
@@ -650,10 +806,14 @@ __device__ __forceinline__ void word_relax(const WordInst& w, long long round, b
                         }
                     }
                     more = __syncthreads_or(again ? 1 : 0);
-                    word_pairs(w, sm);
+                    word_pairs<M>(w0, insts, sm);
                 }
-                word_commit(w, w.raw[round & 1], w.flags[round & 1], unit, s0, ns, sm, count);
+                word_commit<M>(w0, insts, round, unit, s0, ns, sm, count);
                 __syncthreads();
+            }
+            if (M && (int)threadIdx.x < nu && sm.r.count[threadIdx.x]) {
+                const int inst = sm.r.inst[l0 + threadIdx.x];
+                atomicAdd(&insts[inst].ctr->sums[sm.round[inst] & 3], sm.r.count[threadIdx.x]);
             }
             if (threadIdx.x == 0) sm.nslots = 0;
             __syncthreads();
@@ -821,22 +981,28 @@ __device__ __forceinline__ void word_entry(const WordInst& w, long long c) {
     if (w.vtabs & 1) w.tab[0][c] = v0;
 }
 
-// The tables phase after pass `round` (-1: after the set-up, every unit).
-__device__ __forceinline__ void word_tables(const WordInst& w, long long round, WordSmem& sm) {
+// The tables phase after pass `round` (-1: after the set-up, every unit).  M: of
+// the active instances, after the pass before sm.round.
+template <bool M>
+__device__ __forceinline__ void word_tables(const WordInst& w0, const WordInst* insts, int n_insts, long long round0,
+                                            WordSmem& sm) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint2* raw = w.raw[round & 1];
-    uint2* next = w.raw[(round + 1) & 1];
-    const bool first = round < 0;
     if (threadIdx.x == 0) sm.queued = 0u;
     __syncthreads();
-    for (int un = wid * gridDim.x + blockIdx.x; un < w.units; un += kWordWarps * gridDim.x) {
+    const int mine = M ? sm.before[n_insts] : word_share(w0.units, (int)blockIdx.x);
+    for (int i = wid; i < mine; i += kWordWarps) {
+        const int inst = M ? word_find(sm, n_insts, i) : 0;
+        const WordInst& w = M ? insts[inst] : w0;
+        const int un = M ? word_first(inst) + (i - sm.before[inst]) * (int)gridDim.x : i * gridDim.x + blockIdx.x;
+        const long long round = M ? sm.round[inst] - 1 : round0;
+        const uint2* raw = w.raw[round & 1];
         int p, k, n;
         word_unit(w, un, p, k, n);
         const bool in = lane < n;
         const int wd = p * w.plane_words + k + lane;
         const bool before = w.live[un] != 0u;                    // windows to clear
         const uint2 own = in ? raw[wd] : make_uint2(0u, 0u);
-        if (first || word_touched(w, w.flags[round & 1], p, k, n) || before) {
+        if (round < 0 || word_touched(w, w.flags[round & 1], p, k, n) || before) {
             unsigned any = 0u, tot;
             unsigned need = word_tables_at(w, raw, p, k + lane, in, any);
             const unsigned live = __ballot_sync(0xFFFFFFFFu, any != 0u);
@@ -848,23 +1014,26 @@ __device__ __forceinline__ void word_tables(const WordInst& w, long long round, 
                 at = __shfl_sync(0xFFFFFFFFu, at, 0);
                 const int c0 = p * w.plane_cells + (k + lane) * 32;
                 if (at + tot <= (unsigned)kWordEntries) {
-                    for (pos += at; need; need &= need - 1u) sm.t.cell[pos++] = c0 + __ffs(need) - 1;
+                    for (pos += at; need; need &= need - 1u, ++pos) {
+                        sm.t.cell[pos] = c0 + __ffs(need) - 1;
+                        if (M) sm.t.inst[pos] = (unsigned char)inst;
+                    }
                 } else {
                     // the queue is full: its last places hold nothing, these
                     // entries are recomputed here
-                    for (unsigned i = at + lane; i < (unsigned)kWordEntries; i += 32) sm.t.cell[i] = -1;
+                    for (unsigned q = at + lane; q < (unsigned)kWordEntries; q += 32) sm.t.cell[q] = -1;
                     for (; need; need &= need - 1u) word_entry(w, c0 + __ffs(need) - 1);
                 }
             }
         }
-        if (in) next[wd] = make_uint2(0u, own.y);
+        if (in) w.raw[(round + 1) & 1][wd] = make_uint2(0u, own.y);
         if (lane == 0) w.flags[(round + 1) & 1][un] = 0;
     }
     __syncthreads();
     const int n = (int)min(sm.queued, (unsigned)kWordEntries);
     for (int i = threadIdx.x; i < n; i += kWordThreads) {
         const int c = sm.t.cell[i];
-        if (c >= 0) word_entry(w, c);
+        if (c >= 0) word_entry(M ? insts[sm.t.inst[i]] : w0, c);
     }
 }
 
