@@ -111,6 +111,7 @@ struct bf_solve_ws {
     long long* VR = nullptr;
     long long* M2R = nullptr;
     long long* M3R = nullptr;
+    long long* M33R = nullptr;      // word engine
     double* stage_GR = nullptr;
     // word engine (abstractions with d_vbits): used by plain Jacobi solves
     bool use_word = true;           // bf_tune / bf_set_schedule may switch it off
@@ -131,7 +132,7 @@ void bf_solve_ws_free(bf_solve_ws* w) {
     cudaFree(w->stage_V); cudaFree(w->trace); cudaFree(w->stamp);
     cudaFree(w->cand_key); cudaFree(w->cand_u); cudaFree(w->slice_cnt);
     cudaFree(w->rmask); cudaFree(w->GRint); cudaFree(w->VN); cudaFree(w->VR); cudaFree(w->M2R);
-    cudaFree(w->M3R); cudaFree(w->stage_GR);
+    cudaFree(w->M3R); cudaFree(w->M33R); cudaFree(w->stage_GR);
     cudaFree(w->f1bits);
     cudaFree(w->ubits);
     cudaFree(w->fc[0]); cudaFree(w->fc[1]); cudaFree(w->fc_tag);
@@ -633,6 +634,18 @@ static int solve_by_words(const bf_abstraction* a, bf_solve_ws* w, const double*
     if ((rc = stage_in(terminal, sizeof(double) * C, (void**)&w->stage_T, st, &dT))) return rc;
     if ((rc = stage_in(terminal ? nullptr : target, C, (void**)&w->stage_tgt, st, &dTgt))) return rc;
     if ((rc = stage_in(avoid, C, (void**)&w->stage_avoid, st, &dAv))) return rc;
+    // successor class: its mask and costs, and the value tables over its cells
+    const uint8_t* cls = opts ? opts->succ_class : nullptr;
+    const void *dCls = nullptr, *dGc = nullptr;
+    if (cls) {
+        if ((rc = stage_in(cls, C, (void**)&w->rmask, st, &dCls))) return rc;
+        if ((rc = stage_in(opts->G_class, sizeof(double) * C * w->U, (void**)&w->stage_GR, st, &dGc))) return rc;
+        if (!w->VN) BF_CUDA(cudaMalloc((void**)&w->VN, 8 * C));
+        if (!w->VR) BF_CUDA(cudaMalloc((void**)&w->VR, 8 * C));
+        if (!w->M2R) BF_CUDA(cudaMalloc((void**)&w->M2R, 8 * C));
+        if (!w->M3R) BF_CUDA(cudaMalloc((void**)&w->M3R, 8 * C));
+        if (!w->M33R) BF_CUDA(cudaMalloc((void**)&w->M33R, 8 * C));
+    }
     const bool vdev = bfh::is_device_ptr(V), mdev = bfh::is_device_ptr(mu);
     if (!vdev && !w->stage_V) BF_CUDA(cudaMalloc((void**)&w->stage_V, 8 * C));
     WordInst v = w->word;
@@ -640,6 +653,15 @@ static int solve_by_words(const bf_abstraction* a, bf_solve_ws* w, const double*
     v.terminal = (const double*)dT;
     v.target = (const unsigned char*)dTgt;
     v.avoid = (const unsigned char*)dAv;
+    if (cls) {
+        v.cls = (const unsigned char*)dCls;
+        v.Gc = (const double*)dGc;
+        v.tab[0] = w->VN;
+        v.tabc[0] = w->VR;
+        v.tabc[1] = w->M2R;
+        v.tabc[2] = w->M3R;
+        v.tabc[3] = w->M33R;
+    }
     v.mu = mdev ? mu : w->mu;
     v.V = vdev ? V : w->stage_V;
     v.trace = tcap > 0 ? w->trace : nullptr;
@@ -648,7 +670,7 @@ static int solve_by_words(const bf_abstraction* a, bf_solve_ws* w, const double*
     BF_CUDA(cudaMemsetAsync(v.ctr, 0, sizeof(WordCtr), st));
     const bool timed = (flags & BF_FLAG_TIME_KERNELS) != 0;
     double relax_ms = 0.0, rest_ms = 0.0;
-    long long launches = 1;
+    long long launches = 2;
     if (timed || (flags & BF_FLAG_HOST_LOOP))
         rc = word_solve_host(v, w->word_use, st, timed ? &relax_ms : nullptr, timed ? &rest_ms : nullptr, &launches);
     else
@@ -707,7 +729,8 @@ extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t*
     // plain Jacobi solves of abstractions that have its data take the word
     // engine unless a schedule was set that names another form
     if (w->use_word && a->d_vbits &&
-        (!opts || (opts->schedule == BF_SCHED_JACOBI && !opts->succ_class && !(opts->flags & BF_FLAG_COUNT_EXACT)))) {
+        (!opts || (opts->schedule == BF_SCHED_JACOBI && !(opts->flags & BF_FLAG_COUNT_EXACT) &&
+                   (!opts->succ_class || opts->G_class)))) {
         if ((rc = ws_word(a, w, st))) return rc;
         if (w->word_blocks > 0) return solve_by_words(a, w, G, target, avoid, opts, V, mu, iters, status, st);
     }
@@ -731,13 +754,14 @@ extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t*
         w->inplace = sched;
         w->cls = cls;
     }
-    if (cls && !w->VN) {
-        BF_CUDA(cudaMalloc((void**)&w->rmask, C));
-        BF_CUDA(cudaMalloc((void**)&w->GRint, sizeof(double) * C * U));
-        BF_CUDA(cudaMalloc((void**)&w->VN, 8 * C));
-        BF_CUDA(cudaMalloc((void**)&w->VR, 8 * C));
-        BF_CUDA(cudaMalloc((void**)&w->M2R, 8 * C));
-        BF_CUDA(cudaMalloc((void**)&w->M3R, 8 * C));
+    if (cls) {
+        auto once = [&](void** p, size_t bytes) { return *p ? cudaSuccess : cudaMalloc(p, bytes); };
+        BF_CUDA(once((void**)&w->rmask, C));
+        BF_CUDA(once((void**)&w->GRint, sizeof(double) * C * U));
+        BF_CUDA(once((void**)&w->VN, 8 * C));
+        BF_CUDA(once((void**)&w->VR, 8 * C));
+        BF_CUDA(once((void**)&w->M2R, 8 * C));
+        BF_CUDA(once((void**)&w->M3R, 8 * C));
     }
     // frontier cache of the regenerated records (recompute / hybrid modes);
     // the graph holds the view by value: rebuild it when the size changes
@@ -1037,7 +1061,7 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     b.masked = w->masked;
     b.pz = w->pz;
     b.pfront = w->pfront;
-    b.word = w->use_word && w->word_blocks > 0 && o.schedule == BF_SCHED_JACOBI && !o.succ_class;
+    b.word = w->use_word && w->word_blocks > 0 && o.schedule == BF_SCHED_JACOBI;
     if (b.word) {
         // the default was the word engine: as a schedule, the pair queue with
         // the per-input frontier

@@ -1,5 +1,5 @@
-// solve_word.cu -- kernels of the word engine (word_engine.cuh): a whole solve
-// as one cooperative launch, and the same phases as separate launches for the
+// solve_word.cu -- kernels of the word engine (word_engine.cuh): all passes of a
+// solve as one cooperative launch, and the same phases as separate launches for the
 // host-driven and timed forms.
 #include "word_engine.cuh"
 
@@ -7,28 +7,28 @@ using namespace bfk;
 
 extern __shared__ __align__(16) unsigned char word_smem[];
 
-// One block per SM: 32 warps at 64 registers fill the register file.
+// One block per SM: 32 warps at 64 registers fill the register file.  The set-up
+// is a launch of its own before it (k_word_init): its registers would cost the
+// passes spills, and the launch costs no more than the grid barrier it saves.
+template <int K>
 __global__ void __launch_bounds__(kWordThreads, 1) k_word_solve(const __grid_constant__ WordInst w) {
     WordSmem& sm = *reinterpret_cast<WordSmem*>(word_smem);
     unsigned target = 0u;
-    unsigned long long pairs = 0ull, count;
-    word_init(w, reinterpret_cast<double*>(word_smem));
+    if (*(volatile int*)&w.ctr->err) return;                  // found by k_word_init
+    word_start(sm, w.units);
     __syncthreads();
-    word_start(sm);
-    if (!word_barrier(w.ctr, target, sm)) return;
-    if (*(volatile int*)&w.ctr->err) return;
-    long long r = 0;
-    for (;; ++r) {
-        word_tables<false>(w, nullptr, 0, r - 1, sm);
+    // the pass counter is an int: a solve of 2^31 passes would take hours
+    for (int r = 0;; ++r) {
+        word_tables<K>(w, nullptr, 0, (r + 1) & 1, r == 0, sm);
         if (!word_barrier(w.ctr, target, sm)) return;
         const bool last = r >= w.cap;
-        word_relax<false>(w, nullptr, 0, r, last, sm, pairs, count);
-        const unsigned long long v = word_gate(w.ctr, r, count, sm);
+        word_relax<K>(w, nullptr, 0, r & 1, last, sm);
+        const unsigned long long v = word_gate(w.ctr, r, sm);
         if (v == 0ull) return;
         if (blockIdx.x == 0 && threadIdx.x == 0) word_close(w, r, last);
         if (((v >> 16) & 0xFFFFull) == 0ull || last || (v >> 32) == 0ull) break;
     }
-    if (pairs) atomicAdd(&w.ctr->total_pairs, pairs);
+    if (threadIdx.x == 0 && sm.pairs) atomicAdd(&w.ctr->total_pairs, sm.pairs);
     word_output(w);
 }
 
@@ -40,16 +40,15 @@ __global__ void __launch_bounds__(kWordThreads, 1) k_word_batch(const WordInst* 
                                                                 WordCtr* k) {
     WordSmem& sm = *reinterpret_cast<WordSmem*>(word_smem);
     unsigned target = 0u;
-    unsigned long long pairs = 0ull, count;
     bool fresh = false;
     for (int i = 0; i < n; ++i)
         if (!insts[i].ctr->ready) {
             fresh = true;
-            word_init(insts[i], reinterpret_cast<double*>(word_smem));
+            word_init<kWordMany>(insts[i], reinterpret_cast<double*>(word_smem));
         }
     if (fresh && !word_barrier(k, target, sm)) return;
     __syncthreads();
-    word_start(sm);
+    word_start(sm, 0);
     for (int i = threadIdx.x; i < n; i += kWordThreads) {
         WordCtr* c = insts[i].ctr;
         const bool bad = *(volatile int*)&c->err != 0;
@@ -65,9 +64,9 @@ __global__ void __launch_bounds__(kWordThreads, 1) k_word_batch(const WordInst* 
         }
     for (int r = 0; passes < 0 || r < passes; ++r) {
         if (word_split(insts, n, sm) == 0 && !__syncthreads_or((int)threadIdx.x < n && sm.active[threadIdx.x])) break;
-        word_tables<true>(insts[0], insts, n, 0, sm);
+        word_tables<kWordMany>(insts[0], insts, n, 0, false, sm);
         if (!word_barrier(k, target, sm)) return;
-        word_relax<true>(insts[0], insts, n, 0, false, sm, pairs, count);
+        word_relax<kWordMany>(insts[0], insts, n, 0, false, sm);
         if (!word_barrier(k, target, sm)) return;
         for (int i = threadIdx.x; i < n; i += kWordThreads) {
             if (!sm.active[i]) continue;
@@ -81,21 +80,30 @@ __global__ void __launch_bounds__(kWordThreads, 1) k_word_batch(const WordInst* 
     }
 }
 
+template <int K>
 __global__ void __launch_bounds__(kWordThreads, 1) k_word_init(const __grid_constant__ WordInst w) {
-    word_init(w, reinterpret_cast<double*>(word_smem));
+    word_init<K>(w, reinterpret_cast<double*>(word_smem));
 }
 
+template <int K>
 __global__ void __launch_bounds__(kWordThreads, 1) k_word_relax(const __grid_constant__ WordInst w, long long r) {
     WordSmem& sm = *reinterpret_cast<WordSmem*>(word_smem);
-    unsigned long long pairs = 0ull, count;
-    word_start(sm);
-    word_relax<false>(w, nullptr, 0, r, r >= w.cap, sm, pairs, count);
-    if (pairs) atomicAdd(&w.ctr->total_pairs, pairs);
-    if ((threadIdx.x & 31) == 0 && count) atomicAdd(&w.ctr->sums[r & 3], count);
+    word_start(sm, w.units);
+    __syncthreads();
+    word_relax<K>(w, nullptr, 0, (int)(r & 1), r >= w.cap, sm);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (sm.npairs) atomicAdd(&w.ctr->total_pairs, (unsigned long long)sm.npairs);
+        if (sm.nf1) atomicAdd(&w.ctr->sums[r & 3], (unsigned long long)sm.nf1 << 32 | sm.nchg);
+    }
 }
 
+template <int K>
 __global__ void __launch_bounds__(kWordThreads, 1) k_word_tables(const __grid_constant__ WordInst w, long long r) {
-    word_tables<false>(w, nullptr, 0, r, *reinterpret_cast<WordSmem*>(word_smem));
+    WordSmem& sm = *reinterpret_cast<WordSmem*>(word_smem);
+    word_start(sm, w.units);
+    __syncthreads();
+    word_tables<K>(w, nullptr, 0, (int)(r & 1), r < 0, sm);
 }
 
 __global__ void k_word_close(const __grid_constant__ WordInst w, long long r) { word_close(w, r, r >= w.cap); }
@@ -104,13 +112,20 @@ __global__ void __launch_bounds__(kWordThreads, 1) k_word_output(const __grid_co
 
 static_assert(sizeof(WordSmem) >= kWordWarps * kWordSlab * sizeof(double), "the set-up stages costs there");
 
-static int word_attr() {
-    BF_CUDA(cudaFuncSetAttribute(k_word_init, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WordSmem)));
-    BF_CUDA(cudaFuncSetAttribute(k_word_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WordSmem)));
-    BF_CUDA(cudaFuncSetAttribute(k_word_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WordSmem)));
-    BF_CUDA(cudaFuncSetAttribute(k_word_relax, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WordSmem)));
-    BF_CUDA(cudaFuncSetAttribute(k_word_tables, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WordSmem)));
+template <int K>
+static int word_attr_k() {
+    const int b = (int)sizeof(WordSmem);
+    BF_CUDA(cudaFuncSetAttribute(k_word_init<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
+    BF_CUDA(cudaFuncSetAttribute(k_word_solve<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
+    BF_CUDA(cudaFuncSetAttribute(k_word_relax<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
+    BF_CUDA(cudaFuncSetAttribute(k_word_tables<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
     return BF_OK;
+}
+
+static int word_attr() {
+    BF_CUDA(cudaFuncSetAttribute(k_word_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WordSmem)));
+    const int rc = word_attr_k<kWordOne>();
+    return rc ? rc : word_attr_k<kWordClass>();
 }
 
 // Blocks of the engine's launches for a grid of `units` units: one per SM, and
@@ -121,7 +136,7 @@ int word_wave(int units) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (!coop || word_attr() != BF_OK) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_word_solve, kWordThreads, sizeof(WordSmem)) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_word_solve<kWordClass>, kWordThreads, sizeof(WordSmem)) !=
             cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         return 0;
@@ -129,11 +144,15 @@ int word_wave(int units) {
     return units < sms ? units : sms;
 }
 
-// A whole solve in one launch (counters zeroed by the caller on the stream).
+// A whole solve: set-up and passes, two launches (counters zeroed by the caller on the stream).
 int word_solve(const WordInst& w, int blocks, cudaStream_t st) {
+    if (w.cls) k_word_init<kWordClass><<<blocks, kWordThreads, sizeof(WordSmem), st>>>(w);
+    else k_word_init<kWordOne><<<blocks, kWordThreads, sizeof(WordSmem), st>>>(w);
+    BF_CUDA(cudaGetLastError());
     WordInst arg = w;
     void* args[] = {(void*)&arg};
-    BF_CUDA(cudaLaunchCooperativeKernel((const void*)k_word_solve, dim3(blocks), dim3(kWordThreads), args,
+    const void* k = w.cls ? (const void*)k_word_solve<kWordClass> : (const void*)k_word_solve<kWordOne>;
+    BF_CUDA(cudaLaunchCooperativeKernel(k, dim3(blocks), dim3(kWordThreads), args,
                                         sizeof(WordSmem), st));
     return BF_OK;
 }
@@ -157,15 +176,16 @@ int word_solve_batch(const WordInst* insts, int n, int passes, WordCtr* k, cudaS
 
 // The same phases launched one by one, the host reading the counters after
 // every pass; with relax_ms / rest_ms (or NULL) CUDA events around them.
-int word_solve_host(const WordInst& w, int blocks, cudaStream_t st, double* relax_ms, double* rest_ms,
+template <int K>
+static int word_solve_host_k(const WordInst& w, int blocks, cudaStream_t st, double* relax_ms, double* rest_ms,
                     long long* launches) {
     cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
     if (relax_ms)
         for (int i = 0; i < 3; ++i) BF_CUDA(cudaEventCreate(&e[i]));
     const size_t sb = sizeof(WordSmem);
     WordCtr hc;
-    k_word_init<<<blocks, kWordThreads, sb, st>>>(w);
-    k_word_tables<<<blocks, kWordThreads, sb, st>>>(w, -1);
+    k_word_init<K><<<blocks, kWordThreads, sb, st>>>(w);
+    k_word_tables<K><<<blocks, kWordThreads, sb, st>>>(w, -1);
     long long n = 2, r = 0;
     cudaError_t er = cudaGetLastError();
     for (; er == cudaSuccess; ++r) {
@@ -175,7 +195,7 @@ int word_solve_host(const WordInst& w, int blocks, cudaStream_t st, double* rela
             if (er != cudaSuccess || hc.err) break;
         }
         if (relax_ms) cudaEventRecord(e[0], st);
-        k_word_relax<<<blocks, kWordThreads, sb, st>>>(w, r);
+        k_word_relax<K><<<blocks, kWordThreads, sb, st>>>(w, r);
         if (relax_ms) cudaEventRecord(e[1], st);
         k_word_close<<<1, 1, 0, st>>>(w, r);
         n += 2;
@@ -189,7 +209,7 @@ int word_solve_host(const WordInst& w, int blocks, cudaStream_t st, double* rela
         }
         if (hc.done) break;
         if (relax_ms) cudaEventRecord(e[1], st);
-        k_word_tables<<<blocks, kWordThreads, sb, st>>>(w, r);
+        k_word_tables<K><<<blocks, kWordThreads, sb, st>>>(w, r);
         ++n;
         if (relax_ms) {
             cudaEventRecord(e[2], st);
@@ -209,4 +229,10 @@ int word_solve_host(const WordInst& w, int blocks, cudaStream_t st, double* rela
     *launches = n;
     if (er != cudaSuccess) return bfh::cuda_fail(er, "word engine passes");
     return BF_OK;
+}
+
+int word_solve_host(const WordInst& w, int blocks, cudaStream_t st, double* relax_ms, double* rest_ms,
+                    long long* launches) {
+    return w.cls ? word_solve_host_k<kWordClass>(w, blocks, st, relax_ms, rest_ms, launches)
+                 : word_solve_host_k<kWordOne>(w, blocks, st, relax_ms, rest_ms, launches);
 }

@@ -46,13 +46,17 @@ constexpr int kWordUnits = 32;        // units a block relaxes at a time (a batc
 constexpr int kWordRows = 320;        // ... and (unit, input) rows
 constexpr int kWordSlots = 192;       // words of a batch whose cells' candidates are kept at a time
 constexpr int kWordPer = 4;           // pairs of a thread at a time
-constexpr int kWordPairs = 6144;      // pair queue of a block
+constexpr int kWordPairs = 4096;      // pair queue of a block
 constexpr int kWordHead = 8;          // value lookups of a list kept in shared memory
 constexpr int kWordEntries = 4096;    // table entries queued by a block
 constexpr int kWordMaxU = 32;
-constexpr int kWordTest = 256;        // units tested at a time
+constexpr int kWordTest = 128;        // units tested at a time
 constexpr unsigned kWordSpinMax = 1u << 22;
-constexpr int kWordInsts = 256;       // instances of one batched launch
+// Forms of the engine's functions.
+constexpr int kWordOne = 0;           // one instance
+constexpr int kWordMany = 1;          // several instances, each at its own pass
+constexpr int kWordClass = 2;         // one instance with a successor class
+constexpr int kWordInsts = 128;       // instances of one batched launch
 constexpr long long kNoCand = 0x7FFFFFFFFFFFFFFFLL;
 
 // List of a (plane, input): int 0 = bit lookups | bit table << 8, ints 1 .. 31
@@ -88,6 +92,10 @@ struct WordInst {
     int unit_words, plane_units;      // words of a unit (the last of a plane may have fewer), units of a plane
     int units;                        // P plane_units
     int S;                            // P plane_words
+    // quotients without a divide: by plane_units and unit_words as grid_div, i / U
+    // of a row index (< 512) by a 16-bit product
+    unsigned pu_mul, uw_mul, u_mul;
+    int pu_shr, uw_shr;
     int vtabs;                        // bit t: some list gathers from value table t
     int btabs;                        // bit t: some list tests bit table t
     const int* lists;                 // [P][U][kWordEnt]
@@ -100,6 +108,12 @@ struct WordInst {
     const unsigned char* avoid;       // or NULL
     long long* Vnew;                  // [C] keys
     double* gmin;                     // [C] smallest cost of a cell's inputs
+    // successor class (K = kWordClass): the cells, their running cost, and the value
+    // tables over class cells; tab then holds those over the other cells (kKeyMin:
+    // a window without one)
+    const unsigned char* cls;         // [C]
+    const double* Gc;                 // [C][U]
+    long long* tabc[4];
     long long* tab[4];                // V at the start of the pass (kept when lists gather it), M2, M3, M33
     uint2* raw[2];                    // [S] by pass parity: {cells changed in the pass, cells of infinite value}
     unsigned char* flags[2];          // [units] by pass parity: some cell of the unit changed
@@ -132,7 +146,7 @@ struct WordSmem {
             // row and the counts, of its rows the unit
             unsigned char inst[kWordTest], of_row[kWordRows];
             int row0[kWordUnits + 1];
-            unsigned long long count[kWordUnits];
+            unsigned nf1[kWordUnits], nchg[kWordUnits];
         } r;
         struct {
             int cell[kWordEntries];           // entries to recompute, -1: none
@@ -140,6 +154,7 @@ struct WordSmem {
         } t;
     };
     // batched form: units of this block before an instance's, its pass, active
+    // (one instance: before[0] = the block's units)
     int before[kWordInsts + 1];
     long long round[kWordInsts];
     unsigned char active[kWordInsts];
@@ -150,7 +165,10 @@ struct WordSmem {
     int nlive;
     int flag;
     unsigned long long gate;
-    unsigned long long part[kWordWarps];
+    // of the relax phase (32-bit: the 64-bit shared-memory add is a compare-and-
+    // swap loop, which cost a microsecond a pass)
+    unsigned nf1, nchg, npairs;               // frontier cells, changed cells, pairs relaxed
+    unsigned long long pairs;                 // relaxed since the kernel began (thread 0)
 };
 
 // Host: the geometry of an abstraction's bitmaps, and the bytes of an instance's
@@ -169,6 +187,16 @@ inline void word_geometry(WordInst& v, const bf_abstraction* a) {
     v.unit_words = (v.plane_words + v.plane_units - 1) / v.plane_units;     // even units
     v.units = v.planes * v.plane_units;
     v.S = v.planes * v.plane_words;
+    GridDesc q;
+    memset(&q, 0, sizeof q);
+    q.n[0] = v.plane_units;
+    q.n[1] = v.unit_words;
+    grid_divisors(q);
+    v.pu_mul = q.dmul[0];
+    v.pu_shr = q.dshr[0];
+    v.uw_mul = q.dmul[1];
+    v.uw_shr = q.dshr[1];
+    v.u_mul = (65536u + (unsigned)v.g.U - 1u) / (unsigned)v.g.U;
     v.vtabs = a->word_vtabs;
     v.btabs = a->word_btabs;
     v.lists = a->d_wlists;
@@ -232,33 +260,26 @@ __device__ __forceinline__ bool word_barrier(WordCtr* k, unsigned& target, WordS
 
 // After the relax phase of pass r: the arrivals carry whether any block saw a
 // frontier cell and whether any cell changed, so the loop condition costs no
-// further read (a line that every warp reads takes microseconds).  count: the
-// warp's frontier cells << 32 | changed cells (lane 0).  Returns the gate's
-// value, 0 when the wait gave up.
-__device__ __forceinline__ unsigned long long word_gate(WordCtr* k, long long r, unsigned long long count,
-                                                        WordSmem& sm) {
-    const int lane = threadIdx.x & 31;
-    if (lane == 0) sm.part[threadIdx.x >> 5] = count;
+// further read (a line that every warp reads takes microseconds).  Returns the
+// gate's value, 0 when the wait gave up.
+__device__ __forceinline__ unsigned long long word_gate(WordCtr* k, int r, WordSmem& sm) {
     __syncthreads();
-    if (threadIdx.x < 32) {
-        unsigned long long s = lane < kWordWarps ? sm.part[lane] : 0ull;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-        if (lane == 0) {
-            if (s) atomicAdd(&k->sums[r & 3], s);
-            __threadfence();
-            unsigned long long* g = &k->gate[r & 3];
-            atomicAdd(g, 1ull + ((s >> 32) ? 1ull << 16 : 0ull) + ((s & 0xFFFFFFFFull) ? 1ull << 32 : 0ull));
-            unsigned long long v;
-            unsigned n = 0;
-            for (;;) {
-                asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(g) : "memory");
-                if ((v & 0xFFFFull) >= gridDim.x) break;
-                if (++n > kWordSpinMax) { v = 0ull; atomicExch(&k->fault, 1); break; }
-            }
-            __threadfence();
-            sm.gate = v;
+    if (threadIdx.x == 0) {
+        const unsigned long long s = (unsigned long long)sm.nf1 << 32 | sm.nchg;
+        sm.pairs += sm.npairs;
+        if (s) atomicAdd(&k->sums[r & 3], s);
+        __threadfence();
+        unsigned long long* g = &k->gate[r & 3];
+        atomicAdd(g, 1ull + ((s >> 32) ? 1ull << 16 : 0ull) + ((s & 0xFFFFFFFFull) ? 1ull << 32 : 0ull));
+        unsigned long long v;
+        unsigned n = 0;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(g) : "memory");
+            if ((v & 0xFFFFull) >= gridDim.x) break;
+            if (++n > kWordSpinMax) { v = 0ull; atomicExch(&k->fault, 1); break; }
         }
+        __threadfence();
+        sm.gate = v;
     }
     __syncthreads();
     return sm.gate;
@@ -294,12 +315,13 @@ constexpr int kWordSlab = 544;
 // costs: checked, and the smallest of a cell kept (a bound that spares most
 // pairs their cost and their other lookups).  A stream at the HBM rate: 345 MB
 // on the fire model.
+template <int K>
 __device__ __forceinline__ void word_init(const WordInst& w, double* slabs) {
     const int lane = threadIdx.x & 31;
     const int U = w.g.U;
     const double inf = __longlong_as_double(kKeyInf);
     double* slab = slabs + (threadIdx.x >> 5) * kWordSlab;
-    const unsigned per = (65536u + (unsigned)U - 1u) / (unsigned)U;      // i / U = i per >> 16 for i < 512
+    const unsigned per = w.u_mul;                                        // i / U = i per >> 16 for i < 512
     const unsigned pad = (U & 1) ? 0u : 1u;
     const int nc = U <= 16 ? 32 : 16;                                    // cells staged at a time
     bool bad = false;
@@ -333,46 +355,30 @@ __device__ __forceinline__ void word_init(const WordInst& w, double* slabs) {
         }
         for (int h = 0; h < nv; h += nc) {
             const int n = min(nc, nv - h);
-            const long long* src = reinterpret_cast<const long long*>(w.G) + (c0 + h) * U;
-            long long v[16];
+            double m = inf;
+#pragma unroll 1
+            for (int cost = 0; cost < (K == kWordClass ? 2 : 1); ++cost) {
+                const long long* src = reinterpret_cast<const long long*>(cost ? w.Gc : w.G) + (c0 + h) * U;
+                long long v[16];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) v[q] = q * 32 + lane < n * U ? __ldcs(src + q * 32 + lane) : 0ll;
+                for (int q = 0; q < 16; ++q) v[q] = q * 32 + lane < n * U ? __ldcs(src + q * 32 + lane) : 0ll;
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const unsigned i = (unsigned)(q * 32 + lane);
-                bad |= bad_cost(v[q]);
-                if ((int)i < n * U) slab[i + ((i * per) >> 16) * pad] = __longlong_as_double(v[q]);
+                for (int q = 0; q < 16; ++q) {
+                    const unsigned i = (unsigned)(q * 32 + lane);
+                    bad |= bad_cost(v[q]);
+                    if ((int)i < n * U) slab[i + ((i * per) >> 16) * pad] = __longlong_as_double(v[q]);
+                }
+                __syncwarp();
+                if (lane < n) {
+                    const double* row = slab + lane * (U + (int)pad);
+                    for (int u = 0; u < U; ++u) m = row[u] < m ? row[u] : m;
+                }
+                __syncwarp();
             }
-            __syncwarp();
-            if (lane < n) {
-                const double* row = slab + lane * (U + (int)pad);
-                double m = row[0];
-                for (int u = 1; u < U; ++u) m = row[u] < m ? row[u] : m;
-                w.gmin[c0 + h + lane] = m;
-            }
-            __syncwarp();
+            if (lane < n) w.gmin[c0 + h + lane] = m;
         }
     }
     if (bad) atomicOr(&w.ctr->err, 1);
-}
-
-// No candidates yet (once per kernel; word_commit restores it).
-__device__ __forceinline__ void word_start(WordSmem& sm) {
-    for (int i = threadIdx.x; i < kWordSlots * 32; i += kWordThreads) {
-        sm.best[i] = kNoCand;
-        sm.bu[i] = 0xFFu;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// relax
-// ---------------------------------------------------------------------------
-
-// Words of unit un: its plane, its first word in the plane, its word count.
-__device__ __forceinline__ void word_unit(const WordInst& w, int un, int& p, int& k, int& n) {
-    p = un / w.plane_units;
-    k = (un - p * w.plane_units) * w.unit_words;
-    n = min(w.unit_words, w.plane_words - k);
 }
 
 // Batched form: instance i's units of this block are first + j gridDim.x
@@ -381,6 +387,32 @@ __device__ __forceinline__ int word_first(int i) { return (int)((blockIdx.x + 53
 
 __device__ __forceinline__ int word_share(int units, int first) {
     return first < units ? (units - 1 - first) / (int)gridDim.x + 1 : 0;
+}
+
+// No candidates yet (once per kernel; word_commit restores it).
+// units: of the instance, where there is one.
+__device__ __forceinline__ void word_start(WordSmem& sm, int units) {
+    for (int i = threadIdx.x; i < kWordSlots * 32; i += kWordThreads) {
+        sm.best[i] = kNoCand;
+        sm.bu[i] = 0xFFu;
+    }
+    if (threadIdx.x == 0) {
+        sm.pairs = 0ull;
+        sm.before[0] = word_share(units, (int)blockIdx.x);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// relax
+// ---------------------------------------------------------------------------
+
+__device__ __forceinline__ int word_quot(unsigned x, unsigned mul, int shr) { return (int)((__umulhi(mul, x) + x) >> shr); }
+
+// Words of unit un: its plane, its first word in the plane, its word count.
+__device__ __forceinline__ void word_unit(const WordInst& w, int un, int& p, int& k, int& n) {
+    p = word_quot((unsigned)un, w.pu_mul, w.pu_shr);
+    k = (un - p * w.plane_units) * w.unit_words;
+    n = min(w.unit_words, w.plane_words - k);
 }
 
 // before[] of the active instances (whole block); the total.
@@ -422,7 +454,7 @@ __device__ __forceinline__ bool word_live(const WordInst& w, int p, int k, int n
     if (sp.x >= 0) {
         const int a = max(k + sp.y, 0), b = min(k + n - 1 + sp.z, w.plane_words - 1);
         if (a <= b) {
-            const int ua = a / w.unit_words, ub = b / w.unit_words;
+            const int ua = word_quot((unsigned)a, w.uw_mul, w.uw_shr), ub = word_quot((unsigned)b, w.uw_mul, w.uw_shr);
             const unsigned* l = w.live + (long long)sp.x * w.plane_units;
 #pragma unroll 4
             for (int j = ua; j <= ub; ++j) {
@@ -491,8 +523,9 @@ __device__ __forceinline__ bool word_queue(WordSmem& sm, unsigned m, unsigned ta
 // their own cost (from HBM) and their other lookups; the rest move together,
 // warp by warp.  A queue that gives a thread one pair at most skips the test:
 // it only adds a round of loads then.
-template <bool M>
+template <int K>
 __device__ __forceinline__ void word_pairs(const WordInst& w0, const WordInst* insts, WordSmem& sm) {
+    constexpr bool M = K == kWordMany;
     const int np = (int)min(sm.queued, (unsigned)kWordPairs);
     const int lane = threadIdx.x & 31;
     for (int k0 = 0; k0 < np; k0 += kWordPer * kWordThreads) {
@@ -519,10 +552,16 @@ __device__ __forceinline__ void word_pairs(const WordInst& w0, const WordInst* i
                         const int c = at.x + (int)((e[j] >> 8) & 31u);
                         const int* l = reinterpret_cast<const int*>(sm.r.list[at.z + (int)(e[j] & 0xFFu)]);
                         const long long* tb = w.tab[l[0] >> 8] + c;
+                        const int o0 = l[4], o1 = l[3 + min(l[0] & 0xFF, kWordHead)];
                         v[j] = w.Vnew[c];
                         gm[j] = w.gmin[c];
-                        a[j] = tb[l[4]];
-                        b[j] = tb[l[3 + min(l[0] & 0xFF, kWordHead)]];
+                        a[j] = tb[o0];
+                        b[j] = tb[o1];
+                        if (K == kWordClass) {
+                            const long long* tc = w.tabc[l[0] >> 8] + c;
+                            a[j] = max(a[j], tc[o0]);
+                            b[j] = max(b[j], tc[o1]);
+                        }
                     }
                 }
 #pragma unroll
@@ -564,21 +603,36 @@ __device__ __forceinline__ void word_pairs(const WordInst& w0, const WordInst* i
             const int hdr = l[0].x;
             const int L = hdr & 0xFF;
             const long long* tb = w.tab[hdr >> 8] + (at.x + (i & 31));
-            const int4 o = l[1];
-            long long m = max(max(tb[o.x], tb[o.y]), max(tb[o.z], tb[o.w]));
+            const long long* tc = nullptr;
+            double gc = 0.0;
+            if (K == kWordClass) {
+                tc = w.tabc[hdr >> 8] + (at.x + (i & 31));
+                gc = __ldcs(w.Gc + (long long)(at.x + (i & 31)) * w.g.U + u);
+            }
+            long long m = kKeyMin, mc = kKeyMin;
+            auto look = [&](const int4& o) {
+                m = max(m, max(max(tb[o.x], tb[o.y]), max(tb[o.z], tb[o.w])));
+                if (K == kWordClass) mc = max(mc, max(max(tc[o.x], tc[o.y]), max(tc[o.z], tc[o.w])));
+            };
+            look(l[1]);
             if (L > 4) {
-                const int4 q = l[2];
-                m = max(m, max(max(tb[q.x], tb[q.y]), max(tb[q.z], tb[q.w])));
+                look(l[2]);
                 if (L > kWordHead) {
                     const int4* rest = reinterpret_cast<const int4*>(
                         w.lists + ((long long)(at.w & 0xFFFFFF) * w.g.U + u) * kWordEnt + kWordVal + kWordHead);
-                    for (int t = kWordHead; t < L; t += 4) {
-                        const int4 z = __ldg(rest++);
-                        m = max(m, max(max(tb[z.x], tb[z.y]), max(tb[z.z], tb[z.w])));
-                    }
+                    for (int t = kWordHead; t < L; t += 4) look(__ldg(rest++));
                 }
             }
-            d[j] = key_of(__longlong_as_double(d[j]) + val_of(m));        // the one FP64 add
+            const double gv = __longlong_as_double(d[j]);
+            if (K == kWordClass) {
+                // the sup over the box of g(x,y,u) + V(y): each part that has cells
+                // is its cost + its max (fl(g + .) is monotone)
+                d[j] = kKeyMin;
+                if (m != kKeyMin) d[j] = key_of(gv + val_of(m));
+                if (mc != kKeyMin) d[j] = max(d[j], key_of(gc + val_of(mc)));
+            } else {
+                d[j] = key_of(gv + val_of(m));                            // the one FP64 add
+            }
             // a smaller candidate: inputs found for the one before are stale
             if (d[j] < *(volatile long long*)&sm.best[i] && d[j] < atomicMin(&sm.best[i], d[j])) sm.bu[i] = 0xFFu;
         }
@@ -594,30 +648,30 @@ __device__ __forceinline__ void word_pairs(const WordInst& w0, const WordInst* i
 }
 
 // The window's cells whose smallest candidate is below W (whole block).
-template <bool M>
-__device__ __forceinline__ void word_commit(const WordInst& w0, const WordInst* insts, long long round0,
-                                            const int4* unit, int first, int ns, WordSmem& sm,
-                                            unsigned long long& count) {
-    constexpr int K = 3;
+template <int K>
+__device__ __forceinline__ void word_commit(const WordInst& w0, const WordInst* insts, int par0, const int4* unit,
+                                            int first, int ns, WordSmem& sm) {
+    constexpr bool M = K == kWordMany;
+    constexpr int R = 3;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int j0 = wid; j0 < ns; j0 += kWordWarps * K) {
-        long long b[K], old[K];
-        uint2 x[K];
+    for (int j0 = wid; j0 < ns; j0 += kWordWarps * R) {
+        long long b[R], old[R];
+        uint2 x[R];
 #pragma unroll
-        for (int q = 0; q < K; ++q) {
+        for (int q = 0; q < R; ++q) {
             const int j = j0 + q * kWordWarps;
             b[q] = kNoCand;
             if (j < ns) {
                 const int4 at = sm.r.at[j];
                 const WordInst& w = M ? insts[at.w >> 24] : w0;
-                const long long round = M ? sm.round[at.w >> 24] : round0;
+                const int par = M ? (int)sm.round[at.w >> 24] & 1 : par0;
                 b[q] = sm.best[j * 32 + lane];
-                x[q] = w.raw[round & 1][at.y];
+                x[q] = w.raw[par][at.y];
                 if (b[q] != kNoCand) old[q] = w.Vnew[at.x + lane];
             }
         }
 #pragma unroll
-        for (int q = 0; q < K; ++q) {
+        for (int q = 0; q < R; ++q) {
             const int j = j0 + q * kWordWarps;
             if (j >= ns) continue;
             const int4 at = sm.r.at[j];
@@ -634,31 +688,30 @@ __device__ __forceinline__ void word_commit(const WordInst& w0, const WordInst* 
             }
             const unsigned m = __ballot_sync(0xFFFFFFFFu, changed);
             if (lane == 0 && m) {
-                const long long round = M ? sm.round[at.w >> 24] : round0;
+                const int par = M ? (int)sm.round[at.w >> 24] & 1 : par0;
                 const int ui = sm.r.word[first + j] >> 5;
-                w.raw[round & 1][at.y] = make_uint2(m, x[q].y & ~m);
-                w.flags[round & 1][unit[ui].x] = 1;
-                if (M) atomicAdd(&sm.r.count[ui], (unsigned long long)__popc(m));
-                else count += (unsigned long long)__popc(m);
+                w.raw[par][at.y] = make_uint2(m, x[q].y & ~m);
+                w.flags[par][unit[ui].x] = 1;
+                atomicAdd(M ? &sm.r.nchg[ui] : &sm.nchg, (unsigned)__popc(m));
             }
         }
     }
 }
 
 // The relax phase of one pass over this block's share of the units.  count_only:
-// the frontier is counted and nothing is relaxed (at the pass cap).  count (lane
-// 0 of every warp): frontier cells << 32 | changed cells; pairs (lane 0 of every
-// warp) counts the pairs relaxed.  M: the active ones of n instances, each at
+// the frontier is counted and nothing is relaxed (at the pass cap).  par: the
+// pass's parity.  The block's counts go to sm.nf1, sm.nchg and sm.npairs.
+// kWordMany: the active ones of n instances, each at
 // its own pass (sm.round) and cap, its counts into its own sums.
-template <bool M>
-__device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* insts, int n_insts, long long round,
-                                           bool count_only0, WordSmem& sm, unsigned long long& pairs,
-                                           unsigned long long& count) {
+template <int K>
+__device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* insts, int n_insts, int par,
+                                           bool count_only0, WordSmem& sm) {
+    constexpr bool M = K == kWordMany;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int U0 = M ? 1 : w0.g.U;
-    count = 0ull;
+    if (threadIdx.x == 0) sm.nf1 = sm.nchg = sm.npairs = 0u;
     // consecutive units go to different blocks: the frontier is uneven
-    const int mine = M ? sm.before[n_insts] : word_share(w0.units, (int)blockIdx.x);
+    const int mine = M ? sm.before[n_insts] : sm.before[0];
     for (int t0 = 0; t0 < mine; t0 += kWordTest) {
         if (threadIdx.x == 0) { sm.nlive = 0; sm.nslots = 0; }
         if (threadIdx.x < kWordUnits * 32) sm.r.f1[threadIdx.x] = 0u;
@@ -691,7 +744,7 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                     const int cnt = __popc(fm);                          // r0 grows: the first lanes
                     if (fits) {
                         sm.r.row0[lane] = r0;
-                        sm.r.count[lane] = 0ull;
+                        sm.r.nf1[lane] = sm.r.nchg[lane] = 0u;
                         for (int q = 0; q < U; ++q) sm.r.of_row[r0 + q] = (unsigned char)lane;
                         if (lane == cnt - 1) {
                             sm.r.row0[cnt] = r0 + U;
@@ -708,7 +761,7 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
             }
             // (unit, input) rows over the warps: the pairs to relax
             for (int it = wid; it < rows; it += kWordWarps) {
-                const int ui = M ? sm.r.of_row[it] : it / U0;
+                const int ui = M ? sm.r.of_row[it] : (int)((unsigned)it * w0.u_mul >> 16);
                 const WordInst& w = M ? insts[sm.r.inst[l0 + ui]] : w0;
                 const int U = M ? w.g.U : U0;
                 const int u = it - (M ? sm.r.row0[ui] : ui * U);
@@ -747,10 +800,9 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                 const unsigned have = count_only ? 0u : __ballot_sync(0xFFFFFFFFu, any != 0u);
                 int s = 0;
                 if (lane == 0) {
-                    if (M) atomicAdd(&sm.r.count[ui], (unsigned long long)nf << 32);
-                    else count += (unsigned long long)nf << 32;
+                    if (nf) atomicAdd(M ? &sm.r.nf1[ui] : &sm.nf1, nf);
                     if (have) {
-                        pairs += n;
+                        if (!M) atomicAdd(&sm.npairs, n);
                         s = atomicAdd(&sm.nslots, __popc(have));
                     }
                 }
@@ -775,7 +827,7 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                 if (threadIdx.x == 0) { sm.queued = 0u; sm.nover = 0; }
                 __syncthreads();
                 for (int it = wid; it < rows; it += kWordWarps) {
-                    const int ui = M ? sm.r.of_row[it] : it / U0;
+                    const int ui = M ? sm.r.of_row[it] : (int)((unsigned)it * w0.u_mul >> 16);
                     const int u = it - (M ? sm.r.row0[ui] : ui * U0);
                     const unsigned s = (unsigned)sm.r.slot[ui * 32 + lane] - (unsigned)s0;
                     const unsigned m = s < (unsigned)ns ? sm.r.mask[it][lane] : 0u;
@@ -783,7 +835,7 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                         sm.r.over[atomicAdd(&sm.nover, 1)] = (short)it;
                 }
                 __syncthreads();
-                word_pairs<M>(w0, insts, sm);
+                word_pairs<K>(w0, insts, sm);
                 // rows that did not fit, until every one was queued
                 const int nover = sm.nover;
                 for (int more = nover; more;) {
@@ -794,7 +846,7 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                     for (int i = wid; i < nover; i += kWordWarps) {
                         const int it = sm.r.over[i];
                         if (it < 0) continue;
-                        const int ui = M ? sm.r.of_row[it] : it / U0;
+                        const int ui = M ? sm.r.of_row[it] : (int)((unsigned)it * w0.u_mul >> 16);
                         const int u = it - (M ? sm.r.row0[ui] : ui * U0);
                         const unsigned s = (unsigned)sm.r.slot[ui * 32 + lane] - (unsigned)s0;
                         const unsigned m = s < (unsigned)ns ? sm.r.mask[it][lane] : 0u;
@@ -806,14 +858,15 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                         }
                     }
                     more = __syncthreads_or(again ? 1 : 0);
-                    word_pairs<M>(w0, insts, sm);
+                    word_pairs<K>(w0, insts, sm);
                 }
-                word_commit<M>(w0, insts, round, unit, s0, ns, sm, count);
+                word_commit<K>(w0, insts, par, unit, s0, ns, sm);
                 __syncthreads();
             }
-            if (M && (int)threadIdx.x < nu && sm.r.count[threadIdx.x]) {
+            if (M && (int)threadIdx.x < nu && sm.r.nf1[threadIdx.x]) {
                 const int inst = sm.r.inst[l0 + threadIdx.x];
-                atomicAdd(&insts[inst].ctr->sums[sm.round[inst] & 3], sm.r.count[threadIdx.x]);
+                atomicAdd(&insts[inst].ctr->sums[sm.round[inst] & 3],
+                          (unsigned long long)sm.r.nf1[threadIdx.x] << 32 | sm.r.nchg[threadIdx.x]);
             }
             if (threadIdx.x == 0) sm.nslots = 0;
             __syncthreads();
@@ -896,7 +949,7 @@ __device__ __forceinline__ bool word_touched(const WordInst& w, const unsigned c
     const int q = p + ((lane & 8) ? s2 : 0) + ((lane & 16) ? s3 : 0);
     const int last = min(k + n - 1 + ((2 * w.g.n[0] + 33) >> 5), w.plane_words - 1);
     bool hit = false;
-    for (int j = k / w.unit_words + (lane & 7); j * w.unit_words <= last; j += 8)
+    for (int j = word_quot((unsigned)k, w.uw_mul, w.uw_shr) + (lane & 7); j * w.unit_words <= last; j += 8)
         hit |= flags[q * w.plane_units + j] != 0;
     return __any_sync(0xFFFFFFFFu, hit);
 }
@@ -958,51 +1011,67 @@ __device__ __forceinline__ unsigned word_tables_at(const WordInst& w, const uint
     return need;
 }
 
-// Recompute the value tables at cell c.  Windows that reach past a row's or the
-// grid's end are never gathered; their cells are clamped to the array.
-__device__ __forceinline__ void word_entry(const WordInst& w, long long c) {
-    const long long n0 = w.g.n[0], last = w.g.C - 1;
-    const long long v0 = w.Vnew[c];
+// One value table family at cell c: windows of val(x) over 1, 2, 3 and 3 x 3
+// cells.  Windows that reach past a row's or the grid's end are never gathered;
+// their cells are clamped to the array.
+template <typename F>
+__device__ __forceinline__ void word_windows_at(const WordInst& w, long long* const* tab, int c, F val) {
+    const int n0 = w.g.n[0], last = (int)(w.g.C - 1);
+    const long long v0 = val(c);
     if (w.vtabs & 14) {
-        const long long v1 = w.Vnew[min(c + 1, last)], v2 = w.Vnew[min(c + 2, last)];
-        const long long m2 = max(v0, v1);
-        const long long m3 = max(m2, v2);
+        const long long m2 = max(v0, val(min(c + 1, last)));
+        const long long m3 = max(m2, val(min(c + 2, last)));
         if (w.vtabs & 8) {
             long long r[6];
 #pragma unroll
             for (int b = 0; b < 2; ++b)
 #pragma unroll
-                for (int a = 0; a < 3; ++a) r[b * 3 + a] = w.Vnew[min(c + (b + 1) * n0 + a, last)];
-            w.tab[3][c] = max(m3, max(max(r[0], max(r[1], r[2])), max(r[3], max(r[4], r[5]))));
+                for (int a = 0; a < 3; ++a)
+                    r[b * 3 + a] = val((int)min((unsigned)c + (unsigned)((b + 1) * n0 + a), (unsigned)last));
+            tab[3][c] = max(m3, max(max(r[0], max(r[1], r[2])), max(r[3], max(r[4], r[5]))));
         }
-        if (w.vtabs & 4) w.tab[2][c] = m3;
-        if (w.vtabs & 2) w.tab[1][c] = m2;
+        if (w.vtabs & 4) tab[2][c] = m3;
+        if (w.vtabs & 2) tab[1][c] = m2;
     }
-    if (w.vtabs & 1) w.tab[0][c] = v0;
+    if (w.vtabs & 1) tab[0][c] = v0;
 }
 
-// The tables phase after pass `round` (-1: after the set-up, every unit).  M: of
-// the active instances, after the pass before sm.round.
-template <bool M>
-__device__ __forceinline__ void word_tables(const WordInst& w0, const WordInst* insts, int n_insts, long long round0,
+// Recompute the value tables at cell c.
+template <int K>
+__device__ __forceinline__ void word_entry(const WordInst& w, int c) {
+    if (K == kWordClass) {
+        word_windows_at(w, w.tab, c, [&](int x) { return w.cls[x] ? kKeyMin : w.Vnew[x]; });
+        word_windows_at(w, w.tabc, c, [&](int x) { return w.cls[x] ? w.Vnew[x] : kKeyMin; });
+    } else {
+        word_windows_at(w, w.tab, c, [&](int x) { return w.Vnew[x]; });
+    }
+}
+
+// The tables phase after a pass of parity par (first: after the set-up, which
+// counts as parity 1, every unit).  kWordMany: of the active instances, after
+// the pass before sm.round.
+template <int K>
+__device__ __forceinline__ void word_tables(const WordInst& w0, const WordInst* insts, int n_insts, int par0, bool first0,
                                             WordSmem& sm) {
+    constexpr bool M = K == kWordMany;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x == 0) sm.queued = 0u;
     __syncthreads();
-    const int mine = M ? sm.before[n_insts] : word_share(w0.units, (int)blockIdx.x);
+    const int mine = M ? sm.before[n_insts] : sm.before[0];
     for (int i = wid; i < mine; i += kWordWarps) {
         const int inst = M ? word_find(sm, n_insts, i) : 0;
         const WordInst& w = M ? insts[inst] : w0;
         const int un = M ? word_first(inst) + (i - sm.before[inst]) * (int)gridDim.x : i * gridDim.x + blockIdx.x;
-        const long long round = M ? sm.round[inst] - 1 : round0;
-        const uint2* raw = w.raw[round & 1];
+        const int par = M ? (int)(sm.round[inst] + 1) & 1 : par0;
+        const bool first = M ? sm.round[inst] == 0 : first0;
+        const uint2* raw = w.raw[par];
         int p, k, n;
         word_unit(w, un, p, k, n);
         const bool in = lane < n;
         const int wd = p * w.plane_words + k + lane;
         const bool before = w.live[un] != 0u;                    // windows to clear
         const uint2 own = in ? raw[wd] : make_uint2(0u, 0u);
-        if (round < 0 || word_touched(w, w.flags[round & 1], p, k, n) || before) {
+        if (first || word_touched(w, w.flags[par], p, k, n) || before) {
             unsigned any = 0u, tot;
             unsigned need = word_tables_at(w, raw, p, k + lane, in, any);
             const unsigned live = __ballot_sync(0xFFFFFFFFu, any != 0u);
@@ -1022,18 +1091,18 @@ __device__ __forceinline__ void word_tables(const WordInst& w0, const WordInst* 
                     // the queue is full: its last places hold nothing, these
                     // entries are recomputed here
                     for (unsigned q = at + lane; q < (unsigned)kWordEntries; q += 32) sm.t.cell[q] = -1;
-                    for (; need; need &= need - 1u) word_entry(w, c0 + __ffs(need) - 1);
+                    for (; need; need &= need - 1u) word_entry<K>(w, c0 + __ffs(need) - 1);
                 }
             }
         }
-        if (in) w.raw[(round + 1) & 1][wd] = make_uint2(0u, own.y);
-        if (lane == 0) w.flags[(round + 1) & 1][un] = 0;
+        if (in) w.raw[par ^ 1][wd] = make_uint2(0u, own.y);
+        if (lane == 0) w.flags[par ^ 1][un] = 0;
     }
     __syncthreads();
     const int n = (int)min(sm.queued, (unsigned)kWordEntries);
     for (int i = threadIdx.x; i < n; i += kWordThreads) {
         const int c = sm.t.cell[i];
-        if (c >= 0) word_entry(M ? insts[sm.t.inst[i]] : w0, c);
+        if (c >= 0) word_entry<K>(M ? insts[sm.t.inst[i]] : w0, c);
     }
 }
 

@@ -48,7 +48,7 @@ def test_words_match_oracle_and_list_form(n, periodic, U, wmax, seed):
     ref = oracle.solve(n, periodic, boxes, G, T, avoid)
     k = ref["iters"]
     word = [bf.bf_solve(A, G, target=target, avoid=avoid, trace_cap=4096, host_loop=hl) for hl in (False, True, False)]
-    assert word[0]["stats"]["kernel_launches"] == 1            # the one-launch form ran
+    assert word[0]["stats"]["kernel_launches"] == 2            # set-up and one launch for all passes
     list_form(A)
     word.append(bf.bf_solve(A, G, target=target, avoid=avoid, trace_cap=4096))
     for r in word:
@@ -101,3 +101,35 @@ def test_words_check_every_cost():
         g.copy_(torch.from_numpy(G.reshape(-1)))
         r = bf.bf_solve(A, g, target=target, avoid=avoid)
         assert same(r["V"], good["V"]) and same(r["mu"], good["mu"]) and r["iters"] == good["iters"]
+
+
+@pytest.mark.parametrize("n,periodic,U,wmax,seed", [
+    ([33, 17, 5], [False, False, True], 4, (5, 4, 3, 1), 21),
+    ([12, 31, 4, 3], [False, False, True, False], 5, (4, 4, 3, 2), 22),
+    ([63, 9, 3], [False, False, False], 3, (2, 3, 2, 1), 23),
+    ([40, 30], [False, False], 6, (1, 4, 1, 1), 24),
+])
+@pytest.mark.parametrize("share", [0.0, 0.3, 1.0])
+def test_words_successor_class(n, periodic, U, wmax, seed, share):
+    """The class form (two value tables, the cost by the successor's class):
+    no cell, some cells, every cell in the class; finite terminal cost and
+    negative class costs included."""
+    rng = np.random.default_rng(4000 + seed)
+    boxes, G, target, avoid = plane_instance(rng, n, periodic, U, wmax=wmax, p_differ=0.0)
+    C = boxes.shape[0]
+    cls = (rng.random(C) < share).astype(np.uint8)
+    Gc = rng.integers(-2, 5, size=(C, U)) * 0.25
+    Gc[rng.random((C, U)) < 0.02] = INF
+    A = handle(n, periodic, boxes)
+    for T in (np.where(target.astype(bool), 0.0, INF), rng.integers(0, 30, size=C) * 0.5):
+        ref = oracle.solve(n, periodic, boxes, G, T, avoid, succ_class=cls, G_class=Gc, max_iters=200)
+        k = ref["iters"]
+        for hl in (False, True):
+            r = bf.bf_solve(A, G, terminal=T, avoid=avoid, succ_class=cls, G_class=Gc, max_iters=200, trace_cap=4096,
+                            host_loop=hl)
+            assert r["iters"] == k and r["status"] == ref["status"]
+            assert same(r["V"], ref["V"]) and same(r["mu"], ref["mu"])
+            assert same(r["trace"][:k, 1], ref["changed"][:k])
+    plain = bf.bf_solve(A, G, target=target, avoid=avoid)      # the same handle without a class again
+    ref = oracle.solve(n, periodic, boxes, G, np.where(target.astype(bool), 0.0, INF), avoid)
+    assert same(plain["V"], ref["V"]) and same(plain["mu"], ref["mu"])
