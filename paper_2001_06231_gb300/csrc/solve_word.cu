@@ -112,6 +112,79 @@ __global__ void __launch_bounds__(kWordThreads, 1) k_word_output(const __grid_co
 
 static_assert(sizeof(WordSmem) >= kWordWarps * kWordSlab * sizeof(double), "the set-up stages costs there");
 
+// kWordBox: the spans of every unit (block per unit): the words its cells' boxes
+// meet, as at most kWordSpans runs (runs up to 32 words apart are one), relative
+// to its first and last word; *used: the tables its lookups read.
+constexpr int kSpanWords = 4096;      // words of S bits of the block's bitmap
+
+__global__ void __launch_bounds__(256) k_word_spans(const __grid_constant__ WordInst w, int4* spans, int* used) {
+    __shared__ unsigned bits[kSpanWords];
+    __shared__ int tabs;
+    const int W = (w.S + 31) >> 5;
+    for (int un = blockIdx.x; un < w.units; un += gridDim.x) {
+        for (int i = threadIdx.x; i < W; i += blockDim.x) bits[i] = 0u;
+        if (threadIdx.x == 0) tabs = 0;
+        __syncthreads();
+        int p, k, n;
+        word_unit(w, un, p, k, n);
+        const long long last = min((long long)w.g.C, (long long)(k + n) * 32);
+        int mine = 0;
+        for (int u = 0; u < w.g.U; ++u)
+            for (long long c = (long long)k * 32 + threadIdx.x; c < last; c += blockDim.x) {
+                int lo[4], wd[4];
+                if (!word_box(w, (int)c, u, lo, wd)) continue;
+                word_cover(w.g, lo, wd, [&](int t, int e0, int e1, int e2, int e3) {
+                    mine |= 1 << t;
+                    const int e[4] = {e0, e1, e2, e3};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (!((bits[e[q] >> 10] >> ((e[q] >> 5) & 31)) & 1u))
+                            atomicOr(&bits[e[q] >> 10], 1u << ((e[q] >> 5) & 31));
+                });
+            }
+        if (mine) atomicOr(&tabs, mine);
+        __syncthreads();
+        // runs, found by one warp 1024 words at a time
+        if (threadIdx.x < 32) {
+            int4* out = spans + (long long)un * kWordSpans;
+            out[threadIdx.x] = make_int4(-1, 0, 0, 0);
+            __syncwarp();
+            if (threadIdx.x == 0) {
+                int first = -1, prev = -1, cnt = 0;
+                for (int i = 0; i <= W; ++i) {
+                    unsigned b = i < W ? bits[i] : 0u;
+                    if (i < W && !b) continue;
+                    for (; b || i == W; b &= b - 1u) {
+                        const int x = i == W ? 0x7FFFFFFF : i * 32 + __ffs(b) - 1;
+                        if (first >= 0 && (i == W || x - prev > 32)) {
+                            if (cnt < kWordSpans) out[cnt] = make_int4(0, first - k, prev - (k + n - 1), 0);
+                            ++cnt;
+                            first = -1;
+                        }
+                        if (i == W) break;
+                        if (first < 0) first = x;
+                        prev = x;
+                    }
+                }
+                if (cnt > kWordSpans) out[0] = make_int4(-2, 0, 0, 0);
+                atomicOr(used, tabs);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// The spans of an instance of the box form; *used on the device.  False: too
+// many words.
+bool word_spans(const WordInst& w, int4* spans, int* used, cudaStream_t st) {
+    if ((w.S + 31) / 32 > kSpanWords) return false;
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    k_word_spans<<<w.units < 4 * sms ? w.units : 4 * sms, 256, 0, st>>>(w, spans, used);
+    return cudaGetLastError() == cudaSuccess;
+}
+
 template <int K>
 static int word_attr_k() {
     const int b = (int)sizeof(WordSmem);
@@ -124,8 +197,9 @@ static int word_attr_k() {
 
 static int word_attr() {
     BF_CUDA(cudaFuncSetAttribute(k_word_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WordSmem)));
-    const int rc = word_attr_k<kWordOne>();
-    return rc ? rc : word_attr_k<kWordClass>();
+    int rc = word_attr_k<kWordOne>();
+    if (rc == BF_OK) rc = word_attr_k<kWordClass>();
+    return rc ? rc : word_attr_k<kWordBox>();
 }
 
 // Blocks of the engine's launches for a grid of `units` units: one per SM, and
@@ -146,12 +220,15 @@ int word_wave(int units) {
 
 // A whole solve: set-up and passes, two launches (counters zeroed by the caller on the stream).
 int word_solve(const WordInst& w, int blocks, cudaStream_t st) {
-    if (w.cls) k_word_init<kWordClass><<<blocks, kWordThreads, sizeof(WordSmem), st>>>(w);
-    else k_word_init<kWordOne><<<blocks, kWordThreads, sizeof(WordSmem), st>>>(w);
+    // (the set-up of the box form is the plain one)
+    const int words = (w.S + kWordWarps - 1) / kWordWarps, wide = word_wave(words);
+    if (w.cls) k_word_init<kWordClass><<<wide, kWordThreads, sizeof(WordSmem), st>>>(w);
+    else k_word_init<kWordOne><<<wide, kWordThreads, sizeof(WordSmem), st>>>(w);
     BF_CUDA(cudaGetLastError());
     WordInst arg = w;
     void* args[] = {(void*)&arg};
-    const void* k = w.cls ? (const void*)k_word_solve<kWordClass> : (const void*)k_word_solve<kWordOne>;
+    const void* k = w.cls ? (const void*)k_word_solve<kWordClass>
+                          : (w.lists ? (const void*)k_word_solve<kWordOne> : (const void*)k_word_solve<kWordBox>);
     BF_CUDA(cudaLaunchCooperativeKernel(k, dim3(blocks), dim3(kWordThreads), args,
                                         sizeof(WordSmem), st));
     return BF_OK;
@@ -234,5 +311,6 @@ static int word_solve_host_k(const WordInst& w, int blocks, cudaStream_t st, dou
 int word_solve_host(const WordInst& w, int blocks, cudaStream_t st, double* relax_ms, double* rest_ms,
                     long long* launches) {
     return w.cls ? word_solve_host_k<kWordClass>(w, blocks, st, relax_ms, rest_ms, launches)
-                 : word_solve_host_k<kWordOne>(w, blocks, st, relax_ms, rest_ms, launches);
+         : w.lists ? word_solve_host_k<kWordOne>(w, blocks, st, relax_ms, rest_ms, launches)
+                   : word_solve_host_k<kWordBox>(w, blocks, st, relax_ms, rest_ms, launches);
 }

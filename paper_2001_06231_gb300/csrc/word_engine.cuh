@@ -30,6 +30,10 @@
 //           value tables are recomputed at entries whose window holds a
 //           changed cell and no infinite one (entries with an infinite cell
 //           are never gathered), a thread per entry.
+// Boxes that differ from cell to cell (imported ones, the double integrator):
+// the whole grid is one plane, a lane takes a cell and reads its record, the
+// same tests go cell by cell, and a unit's spans are those of its own boxes.
+//
 // V, the tables and the bitmaps stay in the L2; the costs are read in the
 // caller's layout [C][U], only by the pairs that pass the tests.
 #pragma once
@@ -56,6 +60,7 @@ constexpr unsigned kWordSpinMax = 1u << 22;
 constexpr int kWordOne = 0;           // one instance
 constexpr int kWordMany = 1;          // several instances, each at its own pass
 constexpr int kWordClass = 2;         // one instance with a successor class
+constexpr int kWordBox = 3;           // one instance whose boxes differ from cell to cell
 constexpr int kWordInsts = 128;       // instances of one batched launch
 constexpr long long kNoCand = 0x7FFFFFFFFFFFFFFFLL;
 
@@ -100,8 +105,10 @@ struct WordInst {
     int btabs;                        // bit t: some list tests bit table t
     const int* lists;                 // [P][U][kWordEnt]
     const unsigned* vbits;            // [U][S] bit = the pair has a box
-    const int4* spans;                // [P][kWordSpans] {plane q, first, last word relative to the reader's, 0}: the
+    const int4* spans;                // [P] (kWordBox: [units]) [kWordSpans] {plane q, first, last word relative to the reader's, 0}: the
                                       // words of q the plane's bit lookups read; q = -1: none, -2: anything
+    const void* boxes;                // kWordBox: [U][C] records, compact or wide
+    int box_fmt;
     const double* G;                  // [C][U] the caller's costs
     const double* terminal;           // [C] or NULL
     const unsigned char* target;
@@ -177,14 +184,20 @@ struct WordSmem {
 // for a word before and after.
 inline size_t word_up(size_t n) { return (n + 255) / 256 * 256; }
 
-inline void word_geometry(WordInst& v, const bf_abstraction* a) {
+// box: the form for boxes that differ from cell to cell, about a unit per block
+// of `blocks` or more.
+inline void word_geometry(WordInst& v, const bf_abstraction* a, bool box = false, int blocks = 1) {
     memset(&v, 0, sizeof v);
     v.g = a->g;
-    v.planes = (int)(a->g.C / a->g.stride[2]);
-    v.plane_cells = (int)a->g.stride[2];
-    v.plane_words = a->word_plane_words;
+    v.planes = box ? 1 : (int)(a->g.C / a->g.stride[2]);
+    v.plane_cells = (int)(box ? a->g.C : a->g.stride[2]);
+    v.plane_words = box ? (int)((a->g.C + 31) / 32) : a->word_plane_words;
     v.plane_units = (v.plane_words + 31) / 32;
+    if (box && v.plane_units < blocks) v.plane_units = blocks < v.plane_words ? blocks : v.plane_words;
     v.unit_words = (v.plane_words + v.plane_units - 1) / v.plane_units;     // even units
+    if (box) v.plane_units = (v.plane_words + v.unit_words - 1) / v.unit_words;
+    v.boxes = a->d_boxes;
+    v.box_fmt = a->box_fmt;
     v.units = v.planes * v.plane_units;
     v.S = v.planes * v.plane_words;
     GridDesc q;
@@ -447,9 +460,10 @@ __device__ __forceinline__ int word_find(const WordSmem& sm, int n, int c) {
 
 // Can a lookup of the words k .. k + n - 1 of plane p meet a changed entry?
 // (whole warp; lanes take the plane's spans)
-__device__ __forceinline__ bool word_live(const WordInst& w, int p, int k, int n) {
+// at: the plane, or (kWordBox) the unit.
+__device__ __forceinline__ bool word_live(const WordInst& w, int at, int k, int n) {
     const int lane = threadIdx.x & 31;
-    const int4 sp = __ldg(w.spans + (long long)p * kWordSpans + lane);
+    const int4 sp = __ldg(w.spans + (long long)at * kWordSpans + lane);
     unsigned hit = sp.x == -2 ? 1u : 0u;
     if (sp.x >= 0) {
         const int a = max(k + sp.y, 0), b = min(k + n - 1 + sp.z, w.plane_words - 1);
@@ -499,6 +513,95 @@ __device__ __forceinline__ unsigned word_mask(const WordInst& w, const int* list
     return f1 & ~inf;
 }
 
+// kWordBox: the box of (c, u): first cell and width per dim; false: blocked.
+__device__ __forceinline__ bool word_box(const WordInst& w, int c, int u, int lo[4], int wd[4]) {
+    const GridDesc& g = w.g;
+    const long long at = (long long)u * g.C + c;
+#pragma unroll
+    for (int d = 0; d < 4; ++d) { lo[d] = 0; wd[d] = 1; }
+    if (w.box_fmt == kBoxCompact) {
+        const unsigned long long r = g.D <= 2 ? (unsigned long long)__ldg(reinterpret_cast<const unsigned*>(w.boxes) + at)
+                                              : __ldg(reinterpret_cast<const unsigned long long*>(w.boxes) + at);
+        if ((rec_byte(r, 1) & 0x7F) == 0) return false;
+        int k[4] = {0, 0, 0, 0};
+        cell_coords(g, c, k);
+#pragma unroll
+        for (int d = 0; d < 4; ++d)
+            if (d < g.D) {
+                wd[d] = rec_byte(r, 2 * d + 1) & 0x7F;
+                int l = k[d] + rec_sbyte(r, 2 * d);
+                if (g.periodic[d]) {
+                    if (l < 0) l += g.n[d];
+                    else if (l >= g.n[d]) l -= g.n[d];
+                }
+                lo[d] = l;
+            }
+        return true;
+    }
+    const short* q = reinterpret_cast<const short*>(w.boxes) + at * (2 * g.D);
+    if (__ldg(q) == kBlocked) return false;
+#pragma unroll
+    for (int d = 0; d < 4; ++d)
+        if (d < g.D) {
+            lo[d] = __ldg(q + d);
+            wd[d] = __ldg(q + g.D + d) - lo[d] + 1;
+        }
+    return true;
+}
+
+// The lookups that cover a box, four at a time: f(table, cells e0 .. e3), some of
+// them the same.  3 x 3 windows where the box is that large and wraps neither dim
+// 0 nor dim 1; else row by row, a row that wraps in two parts.
+template <typename F>
+__device__ __forceinline__ void word_cover(const GridDesc& g, const int lo[4], const int wd[4], F f) {
+    const int n0 = g.n[0], n1 = g.n[1];
+    const bool wrap0 = lo[0] + wd[0] > n0;
+    const bool big = wd[0] >= 3 && wd[1] >= 3 && !wrap0 && lo[1] + wd[1] <= n1;
+    const int step = big ? 6 : 2, top1 = big ? wd[1] - 3 : wd[1] - 1;
+    for (int part = 0; part < (wrap0 ? 2 : 1); ++part) {
+        const int a = part ? 0 : lo[0], len = part ? lo[0] + wd[0] - n0 : min(wd[0], n0 - lo[0]);
+        const int tab = big ? 3 : min(len, 3) - 1, top0 = max(len - 3, 0);
+        for (int j3 = 0; j3 < wd[3]; ++j3) {
+            int x3 = lo[3] + j3;
+            if (x3 >= g.n[3]) x3 -= g.n[3];
+            for (int j2 = 0; j2 < wd[2]; j2 += 2) {
+                int x2 = lo[2] + j2, y2 = lo[2] + min(j2 + 1, wd[2] - 1);
+                if (x2 >= g.n[2]) x2 -= g.n[2];
+                if (y2 >= g.n[2]) y2 -= g.n[2];
+                const int bx = (x3 * g.n[2] + x2) * n1, by = (x3 * g.n[2] + y2) * n1;
+                for (int j1 = 0;; j1 += step) {
+                    int x1 = lo[1] + min(j1, top1), y1 = lo[1] + min(j1 + (big ? 3 : 1), top1);
+                    if (x1 >= n1) x1 -= n1;
+                    if (y1 >= n1) y1 -= n1;
+                    for (int q = 0;; q += 3) {
+                        const int x0 = a + min(q, top0);
+                        f(tab, (bx + x1) * n0 + x0, (bx + y1) * n0 + x0, (by + x1) * n0 + x0, (by + y1) * n0 + x0);
+                        if (q >= top0) break;
+                    }
+                    if (j1 + (big ? 3 : 1) >= top1) break;
+                }
+            }
+        }
+    }
+}
+
+// kWordBox: a word's masks for input u, lane per cell: f1 the cells whose box
+// holds a changed cell, the result those whose box holds no infinite cell either.
+__device__ __forceinline__ unsigned word_box_mask(const WordInst& w, int wd, int u, unsigned& f1) {
+    const int c = wd * 32 + (threadIdx.x & 31);
+    unsigned chg = 0u, inf = 0u;
+    int lo[4], wid[4];
+    if (c < w.g.C && word_box(w, c, u, lo, wid))
+        word_cover(w.g, lo, wid, [&](int t, int e0, int e1, int e2, int e3) {
+            const uint2* bt = w.bt[t];
+            const uint2 x0 = bt[e0 >> 5], x1 = bt[e1 >> 5], x2 = bt[e2 >> 5], x3 = bt[e3 >> 5];
+            chg |= (x0.x >> (e0 & 31)) | (x1.x >> (e1 & 31)) | (x2.x >> (e2 & 31)) | (x3.x >> (e3 & 31));
+            inf |= (x0.y >> (e0 & 31)) | (x1.y >> (e1 & 31)) | (x2.y >> (e2 & 31)) | (x3.y >> (e3 & 31));
+        });
+    f1 = __ballot_sync(0xFFFFFFFFu, chg & 1u);
+    return __ballot_sync(0xFFFFFFFFu, (chg & ~inf) & 1u);
+}
+
 // Queue the pairs of a row's masks m (whole warp; tag: the lane's word's slot and
 // the input).  False: they do not fit.
 __device__ __forceinline__ bool word_queue(WordSmem& sm, unsigned m, unsigned tag) {
@@ -534,6 +637,11 @@ __device__ __forceinline__ void word_pairs(const WordInst& w0, const WordInst* i
         int n = 0;                                         // the warp's pairs that are left
         if (np <= kWordThreads) {
             n = __popc(__ballot_sync(0xFFFFFFFFu, (int)threadIdx.x < np));
+        } else if (K == kWordBox) {
+            // every pair: there is no list to take two lookups from
+#pragma unroll
+            for (int j = 0; j < kWordPer; ++j)
+                n += __popc(__ballot_sync(0xFFFFFFFFu, k0 + j * kWordThreads + (int)threadIdx.x < np));
         } else {
 #pragma unroll
             for (int j0 = 0; j0 < kWordPer; j0 += 2) {
@@ -599,6 +707,18 @@ __device__ __forceinline__ void word_pairs(const WordInst& w0, const WordInst* i
             const int i = (int)(e >> 8), u = (int)(e & 0xFFu);
             const int4 at = sm.r.at[i >> 5];
             const WordInst& w = M ? insts[at.w >> 24] : w0;
+            if (K == kWordBox) {
+                long long mb = kKeyMin;
+                int lo[4], wid[4];
+                word_box(w, at.x + (i & 31), u, lo, wid);
+                word_cover(w.g, lo, wid, [&](int t, int e0, int e1, int e2, int e3) {
+                    const long long* tb = w.tab[t];
+                    mb = max(mb, max(max(tb[e0], tb[e1]), max(tb[e2], tb[e3])));
+                });
+                d[j] = key_of(__longlong_as_double(d[j]) + val_of(mb));
+                if (d[j] < *(volatile long long*)&sm.best[i] && d[j] < atomicMin(&sm.best[i], d[j])) sm.bu[i] = 0xFFu;
+                continue;
+            }
             const int4* l = sm.r.list[at.z + u];
             const int hdr = l[0].x;
             const int L = hdr & 0xFF;
@@ -722,7 +842,7 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
             const int un = M ? word_first(inst) + (i - sm.before[inst]) * (int)gridDim.x : i * gridDim.x + blockIdx.x;
             int p, k, n;
             word_unit(w, un, p, k, n);
-            if (word_live(w, p, k, n) && lane == 0) {         // P < 2^24: checked at build
+            if (word_live(w, K == kWordBox ? un : p, k, n) && lane == 0) {         // P < 2^24: checked at build
                 const int at = atomicAdd(&sm.nlive, 1);
                 sm.r.unit[at] = make_int4(un, p | n << 24, p * w.plane_words + k, p * w.plane_cells + k * 32);
                 if (M) sm.r.inst[at] = (unsigned char)inst;
@@ -760,6 +880,22 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                 rows = nu * U0;
             }
             // (unit, input) rows over the warps: the pairs to relax
+            if (K == kWordBox) {
+                // word by word: lanes take its cells
+                for (int x = wid; x < rows * w0.unit_words; x += kWordWarps) {
+                    const int it = word_quot((unsigned)x, w0.uw_mul, w0.uw_shr), j = x - it * w0.unit_words;
+                    const int ui = (int)((unsigned)it * w0.u_mul >> 16);
+                    const int4 un = unit[ui];
+                    unsigned f1 = 0u, m = 0u;
+                    if (j < (un.y >> 24)) m = word_box_mask(w0, un.z + j, it - ui * U0, f1) & w0.act[un.z + j];
+                    if (lane == 0) {
+                        if (f1) atomicOr(&sm.r.f1[ui * 32 + j], f1);
+                        sm.r.mask[it][j] = m;
+                    }
+                }
+                for (int x = threadIdx.x; x < rows * 32; x += kWordThreads)
+                    if ((x & 31) >= w0.unit_words) sm.r.mask[x >> 5][x & 31] = 0u;
+            } else
             for (int it = wid; it < rows; it += kWordWarps) {
                 const int ui = M ? sm.r.of_row[it] : (int)((unsigned)it * w0.u_mul >> 16);
                 const WordInst& w = M ? insts[sm.r.inst[l0 + ui]] : w0;
@@ -944,8 +1080,8 @@ __device__ __forceinline__ void word_steps(const GridDesc& g, int p, int& s2, in
 // along dim 2, dim 3, both) and the units of their words.
 __device__ __forceinline__ bool word_touched(const WordInst& w, const unsigned char* flags, int p, int k, int n) {
     const int lane = threadIdx.x & 31;
-    int s2, s3;
-    word_steps(w.g, p, s2, s3);
+    int s2 = 0, s3 = 0;
+    if (w.btabs & 0xFFF0) word_steps(w.g, p, s2, s3);         // else no window reaches another plane
     const int q = p + ((lane & 8) ? s2 : 0) + ((lane & 16) ? s3 : 0);
     const int last = min(k + n - 1 + ((2 * w.g.n[0] + 33) >> 5), w.plane_words - 1);
     bool hit = false;
@@ -974,8 +1110,8 @@ __device__ __forceinline__ unsigned word_tables_at(const WordInst& w, const uint
     const bool m33 = ((w.btabs | w.vtabs) & 0x8888) != 0;
     const int wd = p * w.plane_words + k;
     const uint2* own = raw + (long long)p * w.plane_words;
-    int s2, s3;
-    word_steps(w.g, p, s2, s3);
+    int s2 = 0, s3 = 0;
+    if (w.btabs & 0xFFF0) word_steps(w.g, p, s2, s3);
     const long long d2 = (long long)s2 * w.plane_words, d3 = (long long)s3 * w.plane_words;
     WordRows r;
     uint2 x[4];

@@ -133,3 +133,32 @@ def test_words_successor_class(n, periodic, U, wmax, seed, share):
     plain = bf.bf_solve(A, G, target=target, avoid=avoid)      # the same handle without a class again
     ref = oracle.solve(n, periodic, boxes, G, np.where(target.astype(bool), 0.0, INF), avoid)
     assert same(plain["V"], ref["V"]) and same(plain["mu"], ref["mu"])
+
+
+@pytest.mark.parametrize("n,periodic,U,reach,width,seed", [
+    ([31], [False], 3, 3, 4, 31), ([33], [True], 2, 5, 33, 32), ([1], [False], 2, 0, 1, 33),
+    ([32, 33], [True, True], 4, 4, 9, 34), ([64, 16], [False, True], 32, 2, 5, 35),
+    ([41, 25], [False, False], 3, 40, 12, 36), ([7, 5, 31], [True, False, True], 5, 3, 6, 37),
+    ([95, 11, 3], [False, False, True], 4, 2, 7, 38), ([6, 7, 5, 9], [True, True, True, True], 3, 2, 5, 39),
+    ([300, 3, 2], [False, False, False], 6, 130, 2, 40),
+])
+def test_box_form_matches_oracle_and_list_form(n, periodic, U, reach, width, seed):
+    """Boxes that differ from cell to cell (the engine's box form): wrapping any
+    dim, whole circles, boxes that read 3 x 3 windows or rows of any length,
+    records too far for the compact form, one cell, 32 inputs."""
+    from test_gpu_solve import random_instance
+    rng = np.random.default_rng(4000 + seed)
+    boxes, G, target, avoid = random_instance(rng, n, periodic, U, reach=reach, width=width, neg=False)
+    target[rng.integers(0, boxes.shape[0])] = 1
+    A = handle(n, periodic, boxes)
+    T = np.where(target.astype(bool), 0.0, INF)
+    ref = oracle.solve(n, periodic, boxes, G, T, avoid)
+    k = ref["iters"]
+    res = [bf.bf_solve(A, G, target=target, avoid=avoid, trace_cap=4096, host_loop=hl) for hl in (False, True)]
+    list_form(A)
+    res.append(bf.bf_solve(A, G, target=target, avoid=avoid, trace_cap=4096))
+    for r in res:
+        assert r["iters"] == k and r["status"] == ref["status"]
+        assert same(r["V"], ref["V"]) and same(r["mu"], ref["mu"])
+        assert same(r["trace"][:k, 1], ref["changed"][:k])
+    assert same(res[0]["trace"][:k, 0], ref["f1"][:k])
