@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(kWordThreads, 1) k_word_solve(const __grid_con
     WordSmem& sm = *reinterpret_cast<WordSmem*>(word_smem);
     unsigned target = 0u;
     if (*(volatile int*)&w.ctr->err) return;                  // found by k_word_init
-    word_start(sm, w.units);
+    word_start(sm, &w);
     __syncthreads();
     // the pass counter is an int: a solve of 2^31 passes would take hours
     for (int r = 0;; ++r) {
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kWordThreads, 1) k_word_batch(const WordInst* 
         }
     if (fresh && !word_barrier(k, target, sm)) return;
     __syncthreads();
-    word_start(sm, 0);
+    word_start(sm, nullptr);
     for (int i = threadIdx.x; i < n; i += kWordThreads) {
         WordCtr* c = insts[i].ctr;
         const bool bad = *(volatile int*)&c->err != 0;
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kWordThreads, 1) k_word_init(const __grid_cons
 template <int K>
 __global__ void __launch_bounds__(kWordThreads, 1) k_word_relax(const __grid_constant__ WordInst w, long long r) {
     WordSmem& sm = *reinterpret_cast<WordSmem*>(word_smem);
-    word_start(sm, w.units);
+    word_start(sm, &w);
     __syncthreads();
     word_relax<K>(w, nullptr, 0, (int)(r & 1), r >= w.cap, sm);
     __syncthreads();
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kWordThreads, 1) k_word_relax(const __grid_con
 template <int K>
 __global__ void __launch_bounds__(kWordThreads, 1) k_word_tables(const __grid_constant__ WordInst w, long long r) {
     WordSmem& sm = *reinterpret_cast<WordSmem*>(word_smem);
-    word_start(sm, w.units);
+    word_start(sm, &w);
     __syncthreads();
     word_tables<K>(w, nullptr, 0, (int)(r & 1), r < 0, sm);
 }
@@ -218,15 +218,26 @@ int word_wave(int units) {
     return units < sms ? units : sms;
 }
 
+// The quotients by the launch's blocks.
+static void word_blocks(WordInst& w, int blocks) {
+    GridDesc q;
+    memset(&q, 0, sizeof q);
+    q.n[0] = blocks;
+    grid_divisors(q);
+    w.nb_mul = q.dmul[0];
+    w.nb_shr = q.dshr[0];
+}
+
 // A whole solve: set-up and passes, two launches (counters zeroed by the caller on the stream).
-int word_solve(const WordInst& w, int blocks, cudaStream_t st) {
+int word_solve(const WordInst& w0, int blocks, cudaStream_t st) {
+    WordInst w = w0;
+    word_blocks(w, blocks);
     // (the set-up of the box form is the plain one)
     const int words = (w.S + kWordWarps - 1) / kWordWarps, wide = word_wave(words);
     if (w.cls) k_word_init<kWordClass><<<wide, kWordThreads, sizeof(WordSmem), st>>>(w);
     else k_word_init<kWordOne><<<wide, kWordThreads, sizeof(WordSmem), st>>>(w);
     BF_CUDA(cudaGetLastError());
-    WordInst arg = w;
-    void* args[] = {(void*)&arg};
+    void* args[] = {(void*)&w};
     const void* k = w.cls ? (const void*)k_word_solve<kWordClass>
                           : (w.lists ? (const void*)k_word_solve<kWordOne> : (const void*)k_word_solve<kWordBox>);
     BF_CUDA(cudaLaunchCooperativeKernel(k, dim3(blocks), dim3(kWordThreads), args,
@@ -308,8 +319,10 @@ static int word_solve_host_k(const WordInst& w, int blocks, cudaStream_t st, dou
     return BF_OK;
 }
 
-int word_solve_host(const WordInst& w, int blocks, cudaStream_t st, double* relax_ms, double* rest_ms,
+int word_solve_host(const WordInst& w0, int blocks, cudaStream_t st, double* relax_ms, double* rest_ms,
                     long long* launches) {
+    WordInst w = w0;
+    word_blocks(w, blocks);
     return w.cls ? word_solve_host_k<kWordClass>(w, blocks, st, relax_ms, rest_ms, launches)
          : w.lists ? word_solve_host_k<kWordOne>(w, blocks, st, relax_ms, rest_ms, launches)
                    : word_solve_host_k<kWordBox>(w, blocks, st, relax_ms, rest_ms, launches);

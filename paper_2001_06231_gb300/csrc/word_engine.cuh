@@ -47,8 +47,8 @@ constexpr int kWordThreads = 1024;
 constexpr int kWordWarps = kWordThreads / 32;
 constexpr int kWordSpans = 32;        // spans of a plane's lookups
 constexpr int kWordUnits = 32;        // units a block relaxes at a time (a batch), at most
-constexpr int kWordRows = 320;        // ... and (unit, input) rows
-constexpr int kWordSlots = 192;       // words of a batch whose cells' candidates are kept at a time
+constexpr int kWordRows = 288;        // ... and (unit, input) rows
+constexpr int kWordSlots = 208;       // words of a batch whose cells' candidates are kept at a time
 constexpr int kWordPer = 4;           // pairs of a thread at a time
 constexpr int kWordPairs = 4096;      // pair queue of a block
 constexpr int kWordHead = 8;          // value lookups of a list kept in shared memory
@@ -99,8 +99,8 @@ struct WordInst {
     int S;                            // P plane_words
     // quotients without a divide: by plane_units and unit_words as grid_div, i / U
     // of a row index (< 512) by a 16-bit product
-    unsigned pu_mul, uw_mul, u_mul;
-    int pu_shr, uw_shr;
+    unsigned pu_mul, uw_mul, u_mul, nb_mul;
+    int pu_shr, uw_shr, nb_shr;       // (nb: by the blocks of the launch)
     int vtabs;                        // bit t: some list gathers from value table t
     int btabs;                        // bit t: some list tests bit table t
     const int* lists;                 // [P][U][kWordEnt]
@@ -246,8 +246,9 @@ inline void word_state(WordInst& v, void* mem) {
 // grid barrier (cooperative launch: every block is resident)
 // ---------------------------------------------------------------------------
 // Both barriers: every thread's writes before are visible to every thread
-// after (block barrier, fence and arrival of thread 0; acquire, fence, block
-// barrier).  A wait that gives up sets `fault` and the block leaves the kernel.
+// after (block barrier, releasing arrival of thread 0; acquiring polls, block
+// barrier).  2.4 us for 152 blocks of 1024 threads; a relaxed add and polls between
+// fences take 2.7.  A wait that gives up sets `fault` and the block leaves the kernel.
 
 // After the set-up and the tables phases; `target` counts arrivals over the
 // kernel's life.
@@ -255,8 +256,7 @@ __device__ __forceinline__ bool word_barrier(WordCtr* k, unsigned& target, WordS
     __syncthreads();
     target += gridDim.x;
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&k->bar, 1u);
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&k->bar) : "memory");
         unsigned v, n = 0;
         int ok = 1;
         for (;;) {
@@ -264,7 +264,6 @@ __device__ __forceinline__ bool word_barrier(WordCtr* k, unsigned& target, WordS
             if ((int)(v - target) >= 0) break;
             if (++n > kWordSpinMax) { ok = 0; atomicExch(&k->fault, 1); break; }
         }
-        __threadfence();
         sm.flag = ok;
     }
     __syncthreads();
@@ -281,9 +280,10 @@ __device__ __forceinline__ unsigned long long word_gate(WordCtr* k, int r, WordS
         const unsigned long long s = (unsigned long long)sm.nf1 << 32 | sm.nchg;
         sm.pairs += sm.npairs;
         if (s) atomicAdd(&k->sums[r & 3], s);
-        __threadfence();
         unsigned long long* g = &k->gate[r & 3];
-        atomicAdd(g, 1ull + ((s >> 32) ? 1ull << 16 : 0ull) + ((s & 0xFFFFFFFFull) ? 1ull << 32 : 0ull));
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(g),
+                     "l"(1ull + ((s >> 32) ? 1ull << 16 : 0ull) + ((s & 0xFFFFFFFFull) ? 1ull << 32 : 0ull))
+                     : "memory");
         unsigned long long v;
         unsigned n = 0;
         for (;;) {
@@ -291,7 +291,6 @@ __device__ __forceinline__ unsigned long long word_gate(WordCtr* k, int r, WordS
             if ((v & 0xFFFFull) >= gridDim.x) break;
             if (++n > kWordSpinMax) { v = 0ull; atomicExch(&k->fault, 1); break; }
         }
-        __threadfence();
         sm.gate = v;
     }
     __syncthreads();
@@ -394,32 +393,47 @@ __device__ __forceinline__ void word_init(const WordInst& w, double* slabs) {
     if (bad) atomicOr(&w.ctr->err, 1);
 }
 
+__device__ __forceinline__ int word_quot(unsigned x, unsigned mul, int shr) { return (int)((__umulhi(mul, x) + x) >> shr); }
+
 // Batched form: instance i's units of this block are first + j gridDim.x
 // (rotated from instance to instance: small instances spread over the blocks).
 __device__ __forceinline__ int word_first(int i) { return (int)((blockIdx.x + 53u * (unsigned)i) % gridDim.x); }
+
+// One instance: the block's j-th unit.  The blocks are rotated from one round of
+// units to the next: planes and bands of rows (a plane's units) of every kind
+// come to every block, and the frontier's work with them (without the rotation:
+// 1262 instead of 1202 us at 100x100x64 x 11, 1302 / 1240 at 61x61x25x7 x 9).
+__device__ __forceinline__ int word_mine(const WordInst& w, int j) {
+    const unsigned x = blockIdx.x + 61u * (unsigned)j;
+    return j * (int)gridDim.x + (int)(x - (unsigned)word_quot(x, w.nb_mul, w.nb_shr) * gridDim.x);
+}
 
 __device__ __forceinline__ int word_share(int units, int first) {
     return first < units ? (units - 1 - first) / (int)gridDim.x + 1 : 0;
 }
 
+// ... and how many it has: whole rounds, and one of the last round's.
+__device__ __forceinline__ int word_count(const WordInst& w) {
+    const int whole = w.units / (int)gridDim.x;
+    return whole + (word_mine(w, whole) < w.units ? 1 : 0);
+}
+
 // No candidates yet (once per kernel; word_commit restores it).
-// units: of the instance, where there is one.
-__device__ __forceinline__ void word_start(WordSmem& sm, int units) {
+// w: the instance, where there is one.
+__device__ __forceinline__ void word_start(WordSmem& sm, const WordInst* w) {
     for (int i = threadIdx.x; i < kWordSlots * 32; i += kWordThreads) {
         sm.best[i] = kNoCand;
         sm.bu[i] = 0xFFu;
     }
     if (threadIdx.x == 0) {
         sm.pairs = 0ull;
-        sm.before[0] = word_share(units, (int)blockIdx.x);
+        sm.before[0] = w ? word_count(*w) : 0;
     }
 }
 
 // ---------------------------------------------------------------------------
 // relax
 // ---------------------------------------------------------------------------
-
-__device__ __forceinline__ int word_quot(unsigned x, unsigned mul, int shr) { return (int)((__umulhi(mul, x) + x) >> shr); }
 
 // Words of unit un: its plane, its first word in the plane, its word count.
 __device__ __forceinline__ void word_unit(const WordInst& w, int un, int& p, int& k, int& n) {
@@ -786,8 +800,10 @@ __device__ __forceinline__ void word_commit(const WordInst& w0, const WordInst* 
                 const WordInst& w = M ? insts[at.w >> 24] : w0;
                 const int par = M ? (int)sm.round[at.w >> 24] & 1 : par0;
                 b[q] = sm.best[j * 32 + lane];
-                x[q] = w.raw[par][at.y];
-                if (b[q] != kNoCand) old[q] = w.Vnew[at.x + lane];
+                if (b[q] != kNoCand) {
+                    x[q] = w.raw[par][at.y];
+                    old[q] = w.Vnew[at.x + lane];
+                }
             }
         }
 #pragma unroll
@@ -807,7 +823,7 @@ __device__ __forceinline__ void word_commit(const WordInst& w0, const WordInst* 
                 sm.bu[j * 32 + lane] = 0xFFu;
             }
             const unsigned m = __ballot_sync(0xFFFFFFFFu, changed);
-            if (lane == 0 && m) {
+            if (changed && lane == __ffs(m) - 1) {                    // (a lane that has read the word)
                 const int par = M ? (int)sm.round[at.w >> 24] & 1 : par0;
                 const int ui = sm.r.word[first + j] >> 5;
                 w.raw[par][at.y] = make_uint2(m, x[q].y & ~m);
@@ -839,7 +855,7 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
         for (int i = t0 + wid; i < min(mine, t0 + kWordTest); i += kWordWarps) {
             const int inst = M ? word_find(sm, n_insts, i) : 0;
             const WordInst& w = M ? insts[inst] : w0;
-            const int un = M ? word_first(inst) + (i - sm.before[inst]) * (int)gridDim.x : i * gridDim.x + blockIdx.x;
+            const int un = M ? word_first(inst) + (i - sm.before[inst]) * (int)gridDim.x : word_mine(w0, i);
             int p, k, n;
             word_unit(w, un, p, k, n);
             if (word_live(w, K == kWordBox ? un : p, k, n) && lane == 0) {         // P < 2^24: checked at build
@@ -879,6 +895,22 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                 nu = min(min(kWordUnits, kWordRows / U0), nlive - l0);
                 rows = nu * U0;
             }
+            // few units: every word has its slot from the start and the rows' pairs are
+            // queued as they are found; else the words that have pairs get slots first
+            const bool direct = nu * 32 <= kWordSlots;
+            if (direct) {
+                if ((int)threadIdx.x < nu * 32) {
+                    const int4 un = unit[threadIdx.x >> 5];
+                    const int inst = M ? sm.r.inst[l0 + (threadIdx.x >> 5)] : 0, j = threadIdx.x & 31;
+                    sm.r.at[threadIdx.x] = make_int4(un.w + j * 32, un.z + j,
+                                                     M ? sm.r.row0[threadIdx.x >> 5] : (int)(threadIdx.x >> 5) * U0,
+                                                     (int)((unsigned)(un.y & 0xFFFFFF) | (unsigned)inst << 24));
+                    sm.r.slot[threadIdx.x] = (unsigned short)threadIdx.x;
+                    sm.r.word[threadIdx.x] = (unsigned short)threadIdx.x;
+                }
+                if (threadIdx.x == 0) { sm.queued = 0u; sm.nover = 0; sm.nslots = nu * 32; }
+                __syncthreads();
+            }
             // (unit, input) rows over the warps: the pairs to relax
             if (K == kWordBox) {
                 // word by word: lanes take its cells
@@ -895,31 +927,44 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                 }
                 for (int x = threadIdx.x; x < rows * 32; x += kWordThreads)
                     if ((x & 31) >= w0.unit_words) sm.r.mask[x >> 5][x & 31] = 0u;
-            } else
-            for (int it = wid; it < rows; it += kWordWarps) {
-                const int ui = M ? sm.r.of_row[it] : (int)((unsigned)it * w0.u_mul >> 16);
-                const WordInst& w = M ? insts[sm.r.inst[l0 + ui]] : w0;
-                const int U = M ? w.g.U : U0;
-                const int u = it - (M ? sm.r.row0[ui] : ui * U);
-                const int4 un = unit[ui];
-                const int wd = un.z + lane;
-                const int* list = w.lists + ((long long)(un.y & 0xFFFFFF) * U + u) * kWordEnt;
-                unsigned vb = 0u, act = 0u;
-                if (lane < (un.y >> 24)) {
-                    vb = __ldg(w.vbits + (long long)u * w.S + wd);
-                    act = w.act[wd];
+            } else {
+                for (int it = wid; it < rows; it += kWordWarps) {
+                    const int ui = M ? sm.r.of_row[it] : (int)((unsigned)it * w0.u_mul >> 16);
+                    const WordInst& w = M ? insts[sm.r.inst[l0 + ui]] : w0;
+                    const int U = M ? w.g.U : U0;
+                    const int u = it - (M ? sm.r.row0[ui] : ui * U);
+                    const int4 un = unit[ui];
+                    const int wd = un.z + lane;
+                    const int* list = w.lists + ((long long)(un.y & 0xFFFFFF) * U + u) * kWordEnt;
+                    unsigned vb = 0u, act = 0u;
+                    if (lane < (un.y >> 24)) {
+                        vb = __ldg(w.vbits + (long long)u * w.S + wd);
+                        act = w.act[wd];
+                    }
+                    int4 head = make_int4(0, 0, 0, 0);
+                    if (lane < 1 + kWordHead / 4) head = __ldg(reinterpret_cast<const int4*>(list + kWordHdr) + lane);
+                    unsigned f1;
+                    unsigned m = word_mask(w, list, wd, vb, f1) & act;
+                    if (f1) atomicOr(&sm.r.f1[ui * 32 + lane], f1);
+                    if (lane < 1 + kWordHead / 4) sm.r.list[it][lane] = head;
+                    sm.r.mask[it][lane] = m;
+                    if (direct) {
+                        if (M ? sm.round[sm.r.inst[l0 + ui]] >= w.cap : count_only0) m = 0u;
+                        const unsigned n = __reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(m));
+                        if (n && lane == 0) atomicAdd(&sm.npairs, n);
+                        if (n && !word_queue(sm, m, (unsigned)(ui * 32 + lane) << 13 | (unsigned)u) && lane == 0)
+                            sm.r.over[atomicAdd(&sm.nover, 1)] = (short)it;
+                    }
                 }
-                int4 head = make_int4(0, 0, 0, 0);
-                if (lane < 1 + kWordHead / 4) head = __ldg(reinterpret_cast<const int4*>(list + kWordHdr) + lane);
-                unsigned f1;
-                const unsigned m = word_mask(w, list, wd, vb, f1) & act;
-                if (f1) atomicOr(&sm.r.f1[ui * 32 + lane], f1);
-                if (lane < 1 + kWordHead / 4) sm.r.list[it][lane] = head;
-                sm.r.mask[it][lane] = m;
             }
             __syncthreads();
-            // slots of the words that have pairs
+            // frontier cells; slots of the words that have pairs
             for (int ui = wid; ui < nu; ui += kWordWarps) {
+                const unsigned f1 = sm.r.f1[ui * 32 + lane];
+                sm.r.f1[ui * 32 + lane] = 0u;
+                const unsigned nf = __reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(f1));
+                if (nf && lane == 0) atomicAdd(M ? &sm.r.nf1[ui] : &sm.nf1, nf);
+                if (direct) continue;
                 unsigned any = 0u, n = 0u;
                 const int r1 = M ? sm.r.row0[ui + 1] : (ui + 1) * U0;
                 bool count_only = count_only0;
@@ -929,48 +974,51 @@ __device__ __forceinline__ void word_relax(const WordInst& w0, const WordInst* i
                     any |= m;
                     n += (unsigned)__popc(m);
                 }
-                const unsigned f1 = sm.r.f1[ui * 32 + lane];
-                sm.r.f1[ui * 32 + lane] = 0u;
-                const unsigned nf = __reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(f1));
                 n = __reduce_add_sync(0xFFFFFFFFu, n);
                 const unsigned have = count_only ? 0u : __ballot_sync(0xFFFFFFFFu, any != 0u);
                 int s = 0;
-                if (lane == 0) {
-                    if (nf) atomicAdd(M ? &sm.r.nf1[ui] : &sm.nf1, nf);
-                    if (have) {
-                        if (!M) atomicAdd(&sm.npairs, n);
-                        s = atomicAdd(&sm.nslots, __popc(have));
-                    }
+                if (lane == 0 && have) {
+                    if (!M) atomicAdd(&sm.npairs, n);
+                    s = atomicAdd(&sm.nslots, __popc(have));
                 }
                 s = __shfl_sync(0xFFFFFFFFu, s, 0) + __popc(have & ((1u << lane) - 1u));
                 const bool mine_ = (have >> lane) & 1u;
                 sm.r.slot[ui * 32 + lane] = mine_ ? (unsigned short)s : (unsigned short)0xFFFFu;
                 if (mine_) sm.r.word[s] = (unsigned short)(ui << 5 | lane);
             }
-            __syncthreads();
+            if (!direct) __syncthreads();
             const int nslots = sm.nslots;
+            const bool found = direct && K != kWordBox;      // the pairs are queued already
             // the slots a window at a time
             for (int s0 = 0; s0 < nslots; s0 += kWordSlots) {
                 const int ns = min(kWordSlots, nslots - s0);
-                if ((int)threadIdx.x < ns) {
-                    const int x = sm.r.word[s0 + threadIdx.x];
-                    const int4 un = unit[x >> 5];
-                    const int inst = M ? sm.r.inst[l0 + (x >> 5)] : 0;
-                    sm.r.at[threadIdx.x] =
-                        make_int4(un.w + (x & 31) * 32, un.z + (x & 31), M ? sm.r.row0[x >> 5] : (x >> 5) * U0,
-                                  (int)((unsigned)(un.y & 0xFFFFFF) | (unsigned)inst << 24));
+                if (!direct) {
+                    if ((int)threadIdx.x < ns) {
+                        const int x = sm.r.word[s0 + threadIdx.x];
+                        const int4 un = unit[x >> 5];
+                        const int inst = M ? sm.r.inst[l0 + (x >> 5)] : 0;
+                        sm.r.at[threadIdx.x] =
+                            make_int4(un.w + (x & 31) * 32, un.z + (x & 31), M ? sm.r.row0[x >> 5] : (x >> 5) * U0,
+                                      (int)((unsigned)(un.y & 0xFFFFFF) | (unsigned)inst << 24));
+                    }
+                    if (threadIdx.x == 0) { sm.queued = 0u; sm.nover = 0; }
+                    __syncthreads();
                 }
-                if (threadIdx.x == 0) { sm.queued = 0u; sm.nover = 0; }
-                __syncthreads();
-                for (int it = wid; it < rows; it += kWordWarps) {
-                    const int ui = M ? sm.r.of_row[it] : (int)((unsigned)it * w0.u_mul >> 16);
-                    const int u = it - (M ? sm.r.row0[ui] : ui * U0);
-                    const unsigned s = (unsigned)sm.r.slot[ui * 32 + lane] - (unsigned)s0;
-                    const unsigned m = s < (unsigned)ns ? sm.r.mask[it][lane] : 0u;
-                    if (!word_queue(sm, m, s << 13 | (unsigned)u) && lane == 0)
-                        sm.r.over[atomicAdd(&sm.nover, 1)] = (short)it;
+                if (!found && !(K == kWordBox && direct && count_only0)) {
+                    for (int it = wid; it < rows; it += kWordWarps) {
+                        const int ui = M ? sm.r.of_row[it] : (int)((unsigned)it * w0.u_mul >> 16);
+                        const int u = it - (M ? sm.r.row0[ui] : ui * U0);
+                        const unsigned s = (unsigned)sm.r.slot[ui * 32 + lane] - (unsigned)s0;
+                        const unsigned m = s < (unsigned)ns ? sm.r.mask[it][lane] : 0u;
+                        if (K == kWordBox && direct) {
+                            const unsigned n = __reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(m));
+                            if (n && lane == 0) atomicAdd(&sm.npairs, n);
+                        }
+                        if (!word_queue(sm, m, s << 13 | (unsigned)u) && lane == 0)
+                            sm.r.over[atomicAdd(&sm.nover, 1)] = (short)it;
+                    }
+                    __syncthreads();
                 }
-                __syncthreads();
                 word_pairs<K>(w0, insts, sm);
                 // rows that did not fit, until every one was queued
                 const int nover = sm.nover;
@@ -1105,18 +1153,17 @@ __device__ __forceinline__ void word_put(const WordInst& w, int wd, int first, c
 // has a word) into the bit tables; the result: the cells whose value-table
 // entries are to be recomputed.  The windows over two planes are the windows of
 // the planes' words ORed.
+// r: the unit's own rows, loaded.
 __device__ __forceinline__ unsigned word_tables_at(const WordInst& w, const uint2* raw, int p, int k, bool in,
-                                                   unsigned& any) {
+                                                   WordRows& r, unsigned& any) {
     const bool m33 = ((w.btabs | w.vtabs) & 0x8888) != 0;
     const int wd = p * w.plane_words + k;
     const uint2* own = raw + (long long)p * w.plane_words;
     int s2 = 0, s3 = 0;
     if (w.btabs & 0xFFF0) word_steps(w.g, p, s2, s3);
     const long long d2 = (long long)s2 * w.plane_words, d3 = (long long)s3 * w.plane_words;
-    WordRows r;
     uint2 x[4];
     unsigned need = 0u;
-    r.load(w, own, k, in, m33, false);
     r.windows(w, m33, x);
 #pragma unroll
     for (int t = 0; t < 4; ++t)
@@ -1197,7 +1244,7 @@ __device__ __forceinline__ void word_tables(const WordInst& w0, const WordInst* 
     for (int i = wid; i < mine; i += kWordWarps) {
         const int inst = M ? word_find(sm, n_insts, i) : 0;
         const WordInst& w = M ? insts[inst] : w0;
-        const int un = M ? word_first(inst) + (i - sm.before[inst]) * (int)gridDim.x : i * gridDim.x + blockIdx.x;
+        const int un = M ? word_first(inst) + (i - sm.before[inst]) * (int)gridDim.x : word_mine(w0, i);
         const int par = M ? (int)(sm.round[inst] + 1) & 1 : par0;
         const bool first = M ? sm.round[inst] == 0 : first0;
         const uint2* raw = w.raw[par];
@@ -1206,10 +1253,14 @@ __device__ __forceinline__ void word_tables(const WordInst& w0, const WordInst* 
         const bool in = lane < n;
         const int wd = p * w.plane_words + k + lane;
         const bool before = w.live[un] != 0u;                    // windows to clear
-        const uint2 own = in ? raw[wd] : make_uint2(0u, 0u);
+        // the unit's rows are read with its flags: most units that are looked at
+        // late in a solve are touched, and the reads are in flight together
+        WordRows rows;
+        rows.load(w, raw + (long long)p * w.plane_words, k + lane, in, ((w.btabs | w.vtabs) & 0x8888) != 0, false);
+        const unsigned own = rows.a[0].y;                        // the word itself: row 0 starts at its first bit
         if (first || word_touched(w, w.flags[par], p, k, n) || before) {
             unsigned any = 0u, tot;
-            unsigned need = word_tables_at(w, raw, p, k + lane, in, any);
+            unsigned need = word_tables_at(w, raw, p, k + lane, in, rows, any);
             const unsigned live = __ballot_sync(0xFFFFFFFFu, any != 0u);
             if (lane == 0) w.live[un] = live;
             unsigned pos = word_scan((unsigned)__popc(need), tot);
@@ -1231,7 +1282,7 @@ __device__ __forceinline__ void word_tables(const WordInst& w0, const WordInst* 
                 }
             }
         }
-        if (in) w.raw[par ^ 1][wd] = make_uint2(0u, own.y);
+        if (in) w.raw[par ^ 1][wd] = make_uint2(0u, own);
         if (lane == 0) w.flags[par ^ 1][un] = 0;
     }
     __syncthreads();
