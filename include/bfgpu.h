@@ -227,10 +227,14 @@ BF_API void abs_free(bf_abstraction *abs);
 /* Statistics of one bf_solve call (all optional outputs). */
 typedef struct {
     int64_t kernel_launches;   /* kernels of this library the call launched      */
-    int64_t relaxed_cells;     /* sum over passes of cells relaxed (the frontier
-                                  flagged through predecessor bounding boxes:
-                                  a superset of the exact F1)                    */
-    int64_t executed_pairs;    /* relaxed_cells * U                              */
+    int64_t relaxed_cells;     /* sum over passes of cells relaxed: the exact F1
+                                  where all passes run in one launch, else the
+                                  frontier flagged through predecessor boxes or
+                                  templates (a superset)                         */
+    int64_t executed_pairs;    /* (cell, input) pairs evaluated: relaxed_cells * U,
+                                  with the per-input frontier the pairs with a
+                                  changed cell in their box, in the one-launch form
+                                  those of them without an infinite cell         */
     int64_t exact_f1_cells;    /* sum over passes of |F1| with exact pred (only
                                   with BF_FLAG_COUNT_EXACT, else -1)             */
     int64_t changed_cells;     /* sum over passes of cells whose V decreased    */

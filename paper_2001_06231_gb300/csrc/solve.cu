@@ -763,7 +763,9 @@ extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t*
     const long long C = w->C;
     const int U = w->U;
     // plain Jacobi solves of abstractions that have its data take the word
-    // engine unless a schedule was set that names another form
+    // engine unless a schedule was set that names another form: it was faster at
+    // every size measured, from 0.96 -> 0.50 ms (64 x 64 x 5) to 6.29 -> 2.93 ms
+    // (100 x 100 x 36 x 8 x 15, against the tuned list form)
     if (w->use_word && (a->d_vbits || (word_box_form(a) && !(opts && opts->succ_class))) &&
         (!opts || (opts->schedule == BF_SCHED_JACOBI && !(opts->flags & BF_FLAG_COUNT_EXACT) &&
                    (!opts->succ_class || opts->G_class)))) {

@@ -36,6 +36,19 @@
 //
 // V, the tables and the bitmaps stay in the L2; the costs are read in the
 // caller's layout [C][U], only by the pairs that pass the tests.
+//
+// What bounds it: latency.  A pass is two grid barriers (2.4 us each) and a chain
+// of about 17 dependent L2 trips; on the fire model's busiest pass the relax phase
+// issues in 40% of the cycles and DRAM is at 9%, tables 35% and 8%.  Solves, list
+// forms in a graph (tuned where noted) -> this, on one GB300:
+//   double integrator    64 x 64 x 5                    0.96 -> 0.50 ms
+//   unicycle             100 x 100 x 32 x 10            2.68 -> 1.28 ms
+//   unicycle             200 x 200 x 64 x 10 (tuned)    3.71 -> 1.89 ms
+//   fire                 61 x 57 x 24 x 6 x 15          1.54 -> 0.48 ms
+//   fire                 100 x 100 x 36 x 8 x 15 (tuned) 6.29 -> 2.93 ms
+//   fire, class cost     60 x 60 x 24 x 6 x 15          1.33 -> 0.40 ms
+//   fire, hybrid boxes   60 x 60 x 24 x 6 x 15          6.58 -> 0.48 ms
+//   16 unicycles in one batch                           11.3 -> 5.0 ms
 #pragma once
 #include <cstring>
 
@@ -402,7 +415,7 @@ __device__ __forceinline__ int word_first(int i) { return (int)((blockIdx.x + 53
 // One instance: the block's j-th unit.  The blocks are rotated from one round of
 // units to the next: planes and bands of rows (a plane's units) of every kind
 // come to every block, and the frontier's work with them (without the rotation:
-// 1262 instead of 1202 us at 100x100x64 x 11, 1302 / 1240 at 61x61x25x7 x 9).
+// 1262 instead of 1202 us at 100 x 100 x 32 x 10, 1302 / 1240 at 61 x 57 x 24 x 6 x 15).
 __device__ __forceinline__ int word_mine(const WordInst& w, int j) {
     const unsigned x = blockIdx.x + 61u * (unsigned)j;
     return j * (int)gridDim.x + (int)(x - (unsigned)word_quot(x, w.nb_mul, w.nb_shr) * gridDim.x);
