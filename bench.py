@@ -299,12 +299,13 @@ def ours(args, rank, world, local_rank):
         cm_ = vals[9] if len(vals) > 9 else 0
         pz_ = vals[10] if len(vals) > 10 else 0
         if_ = vals[11] if len(vals) > 11 else 0
+        ol_ = vals[12] if len(vals) > 12 else 0
         bf.bf_set_schedule(A, slice_target=st_, fuse_mark=fm_, relax_blocks=rb_, window33=w33_, plane_lists=pl_,
                            templates=tp_, pair_inputs=pr_, dense_pct=dn_, occupancy=oc_, cell_masks=cm_,
-                           pair_dim=pz_, input_frontier=if_, stream=stream)
+                           pair_dim=pz_, input_frontier=if_, one_launch=ol_, stream=stream)
         tuned = {"slice_target": st_, "fuse_mark": fm_, "relax_blocks": rb_, "window33": w33_, "plane_lists": pl_,
                  "templates": tp_, "pair_inputs": pr_, "dense_pct": dn_, "occupancy": oc_, "cell_masks": cm_,
-                 "pair_dim": pz_, "input_frontier": if_, "source": "--set-schedule"}
+                 "pair_dim": pz_, "input_frontier": if_, "one_launch": ol_, "source": "--set-schedule"}
     elif not args.no_tune:
         tuned = bf.bf_tune(A, G, target=tg, avoid=av, stream=stream)
     # canonical work (exact F1 of Algorithm 1 with Jacobi passes), counted once on the device
@@ -791,7 +792,7 @@ def main():
                     help="build the abstraction in recompute mode (boxes regenerated inside relax)")
     ap.add_argument("--no-cpu", action="store_true", help="skip the CPU oracle baseline")
     ap.add_argument("--no-tune", action="store_true", help="keep the default pass schedule (no bf_tune)")
-    ap.add_argument("--set-schedule", default=None, metavar="S,F,B,W[,P[,T[,I[,N[,O[,M[,Z[,R]]]]]]]]",
+    ap.add_argument("--set-schedule", default=None, metavar="S,F,B,W[,P[,T[,I[,N[,O[,M[,Z[,R[,L]]]]]]]]]",
                     help="put this pass schedule in force instead of bf_tune: slice target, marking in relax (0/1), "
                          "relax blocks (0: one wave), 3 x 3 window table (0/1), plane lookup lists (0/1, default 1), "
                          "predecessor templates (0/1, default 1), two inputs per relax iteration (0/1, default 0), "

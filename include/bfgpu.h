@@ -316,12 +316,15 @@ BF_API int bf_solve(const bf_abstraction *abs, const double *G, const uint8_t *t
  * candidate is solved five times (one warm, four timed) on the given inputs (G, target, avoid and the
  * optional terminal / succ_class / G_class / max_iters of opts; flags, trace
  * and stats are ignored); the fastest stays in force for later bf_solve calls
- * on the handle.  Results never depend on the schedule.  Errors: as bf_solve. */
+ * on the handle.  Where the one-launch form (one_launch) takes the given solve,
+ * its widths and a few whole list schedules are timed instead, and the descent
+ * only follows when a list schedule is the fastest.  Results never depend on
+ * the schedule.  Errors: as bf_solve. */
 typedef struct {
     int32_t slice_target;
     int32_t fuse_mark;         /* 1: relax marks the next frontier                */
-    int32_t relax_blocks;      /* blocks of the relax launch (of the one-launch
-                                  form: its width in SMs)                        */
+    int32_t relax_blocks;      /* blocks of the relax launch; with one_launch 1
+                                  the width of that launch in SMs                */
     int32_t candidates;        /* schedules timed (the default included)          */
     double best_ms;            /* mean solve time of the chosen schedule          */
     double default_ms;         /* the same for the default schedule               */
@@ -362,6 +365,13 @@ typedef struct {
                                   the previous pass: a pair whose box did not
                                   change cannot lower W(x), so results are the
                                   same                                          */
+    int32_t one_launch;        /* 1: plain Jacobi solves run all passes in one
+                                  cooperative launch (where the handle has that
+                                  form; the fields above are then those of its
+                                  other solves); 0: they take the list form the
+                                  fields above name; -1: not part of this
+                                  schedule (tuned for solves the one-launch form
+                                  does not take)                                */
 } bf_tune_result;
 
 BF_API int bf_tune(const bf_abstraction *abs, const double *G, const uint8_t *target,
@@ -372,7 +382,9 @@ BF_API int bf_tune(const bf_abstraction *abs, const double *G, const uint8_t *ta
  * relax_blocks (<= 0 or above one wave: one wave), window33, plane_lists,
  * templates, pair_inputs, occupancy, cell_masks, pair_dim (0 or 2 .. D - 1;
  * without effect unless window33 and plane_lists are on), input_frontier
- * (without effect unless templates are on and U <= 32) and dense_pct
+ * (without effect unless templates are on and U <= 32), one_launch (> 0: the
+ * one-launch form, relax_blocks is then its width and the list relax takes one
+ * wave; 0: the list form; < 0: stays as it is) and dense_pct
  * (0..100; ignored where the tile form does not apply) of *sched are read, the
  * rest ignored; window33 has no effect on
  * 1-D grids or solves with a successor class, plane_lists none on

@@ -115,7 +115,7 @@ struct bf_solve_ws {
     long long* M33R = nullptr;      // word engine
     double* stage_GR = nullptr;
     // word engine (abstractions with d_vbits): used by plain Jacobi solves
-    bool use_word = true;           // bf_tune / bf_set_schedule may switch it off
+    int form = -1;                  // 1: one launch, 0: list form, -1: no schedule named one (one launch)
     int word_blocks = -1;           // widest launch, 0: not available, -1: not set up yet
     int word_use = 0;               // launch width in use
     void* word_mem = nullptr;       // bitmaps of the engine, one allocation
@@ -766,7 +766,7 @@ extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t*
     // engine unless a schedule was set that names another form: it was faster at
     // every size measured, from 0.96 -> 0.50 ms (64 x 64 x 5) to 6.29 -> 2.93 ms
     // (100 x 100 x 36 x 8 x 15, against the tuned list form)
-    if (w->use_word && (a->d_vbits || (word_box_form(a) && !(opts && opts->succ_class))) &&
+    if (w->form != 0 && (a->d_vbits || (word_box_form(a) && !(opts && opts->succ_class))) &&
         (!opts || (opts->schedule == BF_SCHED_JACOBI && !(opts->flags & BF_FLAG_COUNT_EXACT) &&
                    (!opts->succ_class || opts->G_class)))) {
         if ((rc = ws_word(a, w, st))) return rc;
@@ -1005,8 +1005,8 @@ struct Sched {
     int masked = 0;
     int pz = 0;
     bool pfront = false;
-    bool word = false;
-    int wblocks = 0;
+    int word = -1;             // bf_solve_ws::form
+    int wblocks = 0;           // width of the one-launch form, 0: stays as it is
 };
 
 static bool same_sched(const Sched& x, const Sched& y) {
@@ -1039,7 +1039,7 @@ static void set_schedule(const bf_abstraction* a, bf_solve_ws* w, const Sched& s
         }
     }
     w->pfront = pf;
-    w->use_word = s.word;
+    w->form = s.word;
     if (s.wblocks > 0) w->word_use = w->word_blocks > 0 && s.wblocks > w->word_blocks ? w->word_blocks : s.wblocks;
     w->slice_target = s.slice;
     w->fuse_mark = s.fuse;
@@ -1099,10 +1099,11 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     b.masked = w->masked;
     b.pz = w->pz;
     b.pfront = w->pfront;
-    b.word = w->use_word && w->word_blocks > 0 && o.schedule == BF_SCHED_JACOBI;
+    b.word = w->form != 0 && w->word_blocks > 0 && o.schedule == BF_SCHED_JACOBI ? 1 : 0;
     if (b.word) {
-        // the default was the word engine: as a schedule, the pair queue with
-        // the per-input frontier
+        // the default was the word engine; the handle's other solves then take
+        // the pair queue with the per-input frontier
+        b.blocks = full;
         b.use33 = b.plane = b.tmpl = b.pair = b.pfront = true;
         b.masked = 2;
         b.fuse = false;
@@ -1151,7 +1152,7 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
             c.pair = true;
             c.pfront = k == 0 && a->d_uent != nullptr;
             c.fuse = k != 0;
-            c.word = false;
+            c.word = 0;
             if (same_sched(c, from)) continue;
             attempt(c);
         }
@@ -1210,6 +1211,7 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     out->cell_masks = (b.plane && hasp) ? w->masked : 0;
     out->pair_dim = (w->pz && b.use33 && b.plane && hasp) ? w->pz : 0;
     out->input_frontier = (w->pfront && b.tmpl && hast) ? 1 : 0;
+    out->one_launch = b.word;
     out->candidates = tried;
     out->best_ms = best;
     return BF_OK;
@@ -1232,9 +1234,11 @@ extern "C" int bf_set_schedule(const bf_abstraction* a, const bf_tune_result* sc
         std::lock_guard<std::mutex> lock(w->mtx);
         if ((rc = ws_blocks(a, w, (cudaStream_t)stream))) return rc;
     }
-    int blocks = sched->relax_blocks;
-    if (blocks <= 0 || blocks > w->relax_blocks_full) blocks = w->relax_blocks_full;
+    // relax_blocks is the width of the form that one_launch names
     Sched c;
+    c.word = sched->one_launch > 0 ? 1 : (sched->one_launch < 0 ? w->form : 0);
+    int blocks = sched->one_launch > 0 ? 0 : sched->relax_blocks;
+    if (blocks <= 0 || blocks > w->relax_blocks_full) blocks = w->relax_blocks_full;
     c.slice = st_;
     c.fuse = sched->fuse_mark != 0;
     c.blocks = blocks;
@@ -1251,10 +1255,8 @@ extern "C" int bf_set_schedule(const bf_abstraction* a, const bf_tune_result* sc
     }
     c.pz = sched->pair_dim;
     c.pfront = sched->input_frontier != 0;
-    // the per-input frontier of the pair-queue form: the word engine, where the
-    // abstraction has its data
-    c.word = c.plane && c.tmpl && c.masked == 2 && c.pfront;
-    c.wblocks = sched->relax_blocks > 0 ? sched->relax_blocks : (w->word_blocks > 0 ? w->word_blocks : 1 << 20);
+    if (sched->one_launch > 0)
+        c.wblocks = sched->relax_blocks > 0 ? sched->relax_blocks : (w->word_blocks > 0 ? w->word_blocks : 1 << 20);
     if (c.pz != 0 && (c.pz < 2 || c.pz >= a->g.D)) {
         bfh::set_error("bf_set_schedule: pair_dim %d outside 0, 2 .. D - 1", c.pz);
         return BF_ERR_INVALID;

@@ -162,3 +162,67 @@ def test_box_form_matches_oracle_and_list_form(n, periodic, U, reach, width, see
         assert same(r["V"], ref["V"]) and same(r["mu"], ref["mu"])
         assert same(r["trace"][:k, 1], ref["changed"][:k])
     assert same(res[0]["trace"][:k, 0], ref["f1"][:k])
+
+
+def one_launch(r):
+    """Did a solve run as its set-up and one launch for all passes?"""
+    return r["stats"]["kernel_launches"] == 2
+
+
+def schedule_of(t):
+    """The settings of a bf_tune result (what bf_set_schedule reads)."""
+    return {k: v for k, v in t.items() if k not in ("candidates", "best_ms", "default_ms")}
+
+
+def form_instance(kind):
+    """A grid with more than 128 units of work for a single block: 160 planes of
+    63 cells (every box its plane's entry), 141 words of boxes that differ."""
+    from test_gpu_solve import random_instance
+    rng = np.random.default_rng(4100)
+    if kind == "entries":
+        n, periodic, U = [9, 7, 40, 4], [False, False, True, False], 5
+        boxes, G, target, avoid = plane_instance(rng, n, periodic, U, wmax=(3, 3, 2, 2), p_differ=0.0)
+    else:
+        n, periodic, U = [75, 60], [True, False], 4
+        boxes, G, target, avoid = random_instance(rng, n, periodic, U, reach=3, width=4, neg=False)
+        target[rng.integers(0, boxes.shape[0])] = 1
+    ref = oracle.solve(n, periodic, boxes, G, np.where(target.astype(bool), 0.0, INF), avoid)
+    return n, periodic, boxes, G, target, avoid, ref
+
+
+@pytest.mark.parametrize("kind", ["entries", "boxes"])
+def test_schedule_names_its_form(kind):
+    """one_launch says which form a solve takes, whatever the list form's fields
+    say, at every width (one block then relaxes more units than it tests at a
+    time); the list form's own fields are in force when it is 0."""
+    n, periodic, boxes, G, target, avoid, ref = form_instance(kind)
+    A = handle(n, periodic, boxes)
+    pair_queue = dict(slice_target=0, fuse_mark=0, window33=1, plane_lists=1, templates=1, pair_inputs=1, cell_masks=2,
+                      input_frontier=1)
+    plain = dict(slice_target=2, fuse_mark=1, window33=0, plane_lists=0, templates=0)
+    for fields in (pair_queue, plain):
+        for form, width in ((1, 0), (1, 1), (0, 0), (1, 2), (1, 151), (0, 1), (1, 100000)):
+            bf.bf_set_schedule(A, one_launch=form, relax_blocks=width, **fields)
+            r = bf.bf_solve(A, G, target=target, avoid=avoid)
+            assert one_launch(r) == (form == 1), (fields, form, width)
+            assert r["iters"] == ref["iters"] and r["status"] == ref["status"]
+            assert same(r["V"], ref["V"]) and same(r["mu"], ref["mu"]), (fields, form, width)
+            bf.bf_set_schedule(A, one_launch=-1, **fields)           # leaves the form as it is
+            assert one_launch(bf.bf_solve(A, G, target=target, avoid=avoid)) == (form == 1)
+
+
+@pytest.mark.parametrize("kind", ["entries", "boxes"])
+def test_tuned_schedule_replays_on_another_handle(kind):
+    """What bf_tune reports, put in force on another handle of the same system,
+    takes the same form; so does what it reports when the handle starts from a
+    list schedule."""
+    n, periodic, boxes, G, target, avoid, ref = form_instance(kind)
+    for start in (None, dict(slice_target=2, fuse_mark=1)):
+        A, B = handle(n, periodic, boxes), handle(n, periodic, boxes)
+        if start:
+            bf.bf_set_schedule(A, **start)
+        t = bf.bf_tune(A, G, target=target, avoid=avoid)
+        bf.bf_set_schedule(B, **schedule_of(t))
+        a, b = (bf.bf_solve(H, G, target=target, avoid=avoid) for H in (A, B))
+        assert one_launch(a) == one_launch(b) == (t["one_launch"] == 1)
+        assert same(a["V"], ref["V"]) and same(b["V"], ref["V"]) and same(a["mu"], ref["mu"]) and same(b["mu"], ref["mu"])
