@@ -13,11 +13,10 @@
 //   3. reads the per-request counters, copies the results of finished
 //      requests to their host buffers and frees their state.
 // Requests that arrive while others are on the GPU thus join the next step.
-// While the engine is idle and at most kDirectMax requests wait, the oldest
-// runs at once as a plain bf_solve on the stream (one graph launch for all
-// its passes, on the abstraction's cached workspace, whose bytes count against
-// the budget from the first such request on); a longer queue goes to the
-// engine together.
+// While the engine is idle and one request waits, it runs at once as a plain
+// bf_solve on the stream (on the abstraction's cached workspace, whose bytes
+// count against the budget from the first such request on); two or more go to
+// the engine together.
 // The engine runs each request exactly as bf_solve would, so results do not
 // depend on what else is in the mix.
 #include <algorithm>
@@ -38,8 +37,11 @@ size_t solve_ws_bytes(const bf_abstraction* a);   // solve.cu
 namespace {
 
 // An idle engine takes up to this many waiting requests one at a time as plain
-// solves (one graph launch each); a longer queue goes to the batched engine.
-constexpr int kDirectMax = 4;
+// solves; a longer queue goes to the batched engine.  With more than one, plain
+// solves faster than the arrivals keep every queue that short and no request
+// ever shares the device with another: with 4, none of 21 requests submitted
+// at once overlapped.
+constexpr int kDirectMax = 1;
 
 double now_s() {
     using namespace std::chrono;
