@@ -340,6 +340,14 @@ static bool word_box_form(const bf_abstraction* a) {
            a->g.U <= kWordMaxU && a->g.C <= (1LL << 20);
 }
 
+// Does the one-launch form take a solve with these options?  (bf_solve and bf_tune
+// ask the same question; the launch itself may still not fit: ws_word.)
+static bool word_takes(const bf_abstraction* a, const bf_solve_opts* o) {
+    if (o && (o->schedule != BF_SCHED_JACOBI || (o->flags & BF_FLAG_COUNT_EXACT) || (o->succ_class && !o->G_class)))
+        return false;
+    return a->d_vbits || (word_box_form(a) && !(o && o->succ_class));
+}
+
 // Word engine state (once per workspace); word_blocks = 0 where the engine does
 // not apply.
 static int ws_word(const bf_abstraction* a, bf_solve_ws* w, cudaStream_t st) {
@@ -766,9 +774,7 @@ extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t*
     // engine unless a schedule was set that names another form: it was faster at
     // every size measured, from 0.96 -> 0.50 ms (64 x 64 x 5) to 6.29 -> 2.93 ms
     // (100 x 100 x 36 x 8 x 15, against the tuned list form)
-    if (w->form != 0 && (a->d_vbits || (word_box_form(a) && !(opts && opts->succ_class))) &&
-        (!opts || (opts->schedule == BF_SCHED_JACOBI && !(opts->flags & BF_FLAG_COUNT_EXACT) &&
-                   (!opts->succ_class || opts->G_class)))) {
+    if (w->form != 0 && word_takes(a, opts)) {
         if ((rc = ws_word(a, w, st))) return rc;
         if (w->word_blocks > 0) return solve_by_words(a, w, G, target, avoid, opts, V, mu, iters, status, st);
     }
@@ -1080,9 +1086,14 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     int rc = tune_time(a, G, target, avoid, &o, V, mu, st, &best);
     bf_solve_ws* w = a->ws;
     if (rc == BF_OK && !w) rc = BF_ERR_CUDA;
+    // does the one-launch form take these solves?  It is then timed against the
+    // list form whichever is in force; else the form is left as it is
+    bool can = word_takes(a, &o);
     if (rc == BF_OK) {
         std::lock_guard<std::mutex> lock(w->mtx);
         rc = ws_blocks(a, w, st);
+        if (rc == BF_OK && can) rc = ws_word(a, w, st);
+        can = can && w->word_blocks > 0;
     }
     if (rc) { cudaFree(V); cudaFree(mu); return rc; }
     const int full = w->relax_blocks_full;
@@ -1099,15 +1110,17 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     b.masked = w->masked;
     b.pz = w->pz;
     b.pfront = w->pfront;
-    b.word = w->form != 0 && w->word_blocks > 0 && o.schedule == BF_SCHED_JACOBI ? 1 : 0;
-    if (b.word) {
-        // the default was the word engine; the handle's other solves then take
-        // the pair queue with the per-input frontier
-        b.blocks = full;
-        b.use33 = b.plane = b.tmpl = b.pair = b.pfront = true;
-        b.masked = 2;
-        b.fuse = false;
-    }
+    const int form = w->form;
+    Sched list = b;                        // the list schedule in force
+    list.word = can ? 0 : form;
+    Sched word = b;                        // the one-launch form; the handle's other solves then
+    word.word = 1;                         // take the pair queue with the per-input frontier
+    word.wblocks = w->word_use;
+    word.blocks = full;
+    word.use33 = word.plane = word.tmpl = word.pair = word.pfront = true;
+    word.masked = 2;
+    word.fuse = false;
+    b = can && form != 0 ? word : list;
     out->default_ms = best;
     int tried = 1;
     const bool cls = opts && opts->succ_class;
@@ -1124,27 +1137,28 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
             b = c;
         }
     };
-    // the word engine's width: fewer blocks make its barriers cheaper and leave
-    // each more work (4 widths)
-    if (b.word) {
-        b.wblocks = w->word_use;
+    // the one-launch form, and its width: fewer blocks make its barriers cheaper
+    // and leave each more work (4 widths)
+    if (can) {
+        if (form == 0) attempt(word);
         const int wide = w->word_blocks;
         for (int k = 0; k < 5 && rc == BF_OK; ++k) {
-            Sched c = b;
+            Sched c = word;
             c.wblocks = k == 0 ? wide : (wide * (5 - k) + 5) / 6;      // all, 2/3, 1/2, 1/3, 1/6
-            if (c.wblocks < 1 || same_sched(c, b)) continue;
+            if (c.wblocks < 1 || same_sched(c, word)) continue;
             attempt(c);
         }
     }
-    // whole schedules (the pair-queue relax, with the per-input frontier and
+    // whole list schedules (the pair-queue relax, with the per-input frontier and
     // marking in its own launch, or without it and marking in relax): their
     // settings help each other, which one dimension at a time would not find.
-    // Against the word engine also the form every abstraction has (the lists in
-    // turn) and the cell masks in turn.
+    // Against the one-launch form also the form every abstraction has (the lists
+    // in turn) and the cell masks in turn; without lookup lists the schedule in
+    // force.
     if (hasp && has33 && a->d_fmask) {
-        const Sched from = b;
-        for (int k = 0; k < (from.word ? 4 : 2) && rc == BF_OK; ++k) {
-            Sched c = from;
+        const Sched first = b;
+        for (int k = 0; k < (can ? 4 : 2) && rc == BF_OK; ++k) {
+            Sched c = list;
             c.use33 = true;
             c.plane = true;
             c.tmpl = hast;
@@ -1152,14 +1166,15 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
             c.pair = true;
             c.pfront = k == 0 && a->d_uent != nullptr;
             c.fuse = k != 0;
-            c.word = 0;
-            if (same_sched(c, from)) continue;
+            if (same_sched(c, first)) continue;                // timed already
             attempt(c);
         }
+    } else if (can && form != 0 && rc == BF_OK) {
+        attempt(list);
     }
     // coordinate descent: each dimension's values with the others at the best
     // so far, two rounds (all are dimensions of the list form)
-    for (int round = 0; round < 2 && rc == BF_OK && !b.word; ++round) {
+    for (int round = 0; round < 2 && rc == BF_OK && !(can && b.word == 1); ++round) {
         for (int dim = 0; dim < 12 && rc == BF_OK; ++dim) {
             const int nval = (dim == 0 || dim == 9) ? 4 : (dim == 7 ? 3 : (dim == 10 ? a->g.D - 1 : 2));
             if (dim == 7 && !hasd) continue;
@@ -1202,7 +1217,7 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     out->slice_target = b.slice;
     out->fuse_mark = b.fuse ? 1 : 0;
     out->window33 = b.use33 && w->M33 ? 1 : 0;
-    out->relax_blocks = b.word ? b.wblocks : b.blocks;
+    out->relax_blocks = can && b.word == 1 ? b.wblocks : b.blocks;
     out->plane_lists = (b.plane && hasp) ? 1 : 0;
     out->templates = (b.tmpl && hast) ? 1 : 0;
     out->pair_inputs = (b.pair && b.plane && hasp) ? 1 : 0;
@@ -1211,7 +1226,7 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     out->cell_masks = (b.plane && hasp) ? w->masked : 0;
     out->pair_dim = (w->pz && b.use33 && b.plane && hasp) ? w->pz : 0;
     out->input_frontier = (w->pfront && b.tmpl && hast) ? 1 : 0;
-    out->one_launch = b.word;
+    out->one_launch = can ? b.word : -1;
     out->candidates = tried;
     out->best_ms = best;
     return BF_OK;

@@ -226,3 +226,47 @@ def test_tuned_schedule_replays_on_another_handle(kind):
         a, b = (bf.bf_solve(H, G, target=target, avoid=avoid) for H in (A, B))
         assert one_launch(a) == one_launch(b) == (t["one_launch"] == 1)
         assert same(a["V"], ref["V"]) and same(b["V"], ref["V"]) and same(a["mu"], ref["mu"]) and same(b["mu"], ref["mu"])
+
+
+def tune_inplace(A, G, target, avoid):
+    """bf_tune on solves with the in-place schedule, through the C interface."""
+    import ctypes
+    opts, res = bf.SolveOpts(), bf.TuneResult()
+    opts.schedule = bf.SCHED_INPLACE
+    rc = bf.lib().bf_tune(A.handle, G.ctypes.data, target.ctypes.data, avoid.ctypes.data, ctypes.byref(opts),
+                          ctypes.byref(res), None)
+    assert rc == 0
+    return {k: getattr(res, k) for k, _ in res._fields_}
+
+
+def test_tuner_leaves_the_form_to_the_solves_it_timed():
+    """Tuned for solves that the one-launch form does not take (in place; boxes
+    that differ with a successor class), a handle keeps its form, and the list
+    form's settings are searched, whether or not it was solved before."""
+    n, periodic, boxes, G, target, avoid, ref = form_instance("boxes")
+    cls = (np.random.default_rng(3).random(boxes.shape[0]) < 0.3).astype(np.uint8)
+    for solved in (False, True):
+        for tune in (lambda A: bf.bf_tune(A, G, target=target, avoid=avoid, succ_class=cls, G_class=G),
+                     lambda A: tune_inplace(A, G, target, avoid)):
+            A = handle(n, periodic, boxes)
+            if solved:
+                assert one_launch(bf.bf_solve(A, G, target=target, avoid=avoid))
+            t = tune(A)
+            assert t["one_launch"] == -1 and t["candidates"] > 5
+            r = bf.bf_solve(A, G, target=target, avoid=avoid)
+            assert one_launch(r) and same(r["V"], ref["V"]) and same(r["mu"], ref["mu"])
+
+
+def test_tuner_times_the_one_launch_form_from_a_list_schedule():
+    """A handle with a list schedule in force is tuned to the one-launch form
+    (on this unicycle 2.5 times as fast)."""
+    from paper_2001_06231_gb300 import workloads as wl
+    w = wl.unicycle3d(n=(40, 40, 100), n_obstacles=3)
+    A = bf.abs_build_workload(w)
+    bf.bf_set_schedule(A)
+    before = bf.bf_solve(A, w.G, target=w.target, avoid=w.avoid)
+    assert not one_launch(before)
+    t = bf.bf_tune(A, w.G, target=w.target, avoid=w.avoid)
+    after = bf.bf_solve(A, w.G, target=w.target, avoid=w.avoid)
+    assert t["one_launch"] == 1 and one_launch(after)
+    assert same(after["V"], before["V"]) and same(after["mu"], before["mu"])
