@@ -115,10 +115,11 @@ struct bf_solve_ws {
     long long* M33R = nullptr;      // word engine
     double* stage_GR = nullptr;
     // word engine (abstractions with d_vbits): used by plain Jacobi solves
-    int form = -1;                  // 1: one launch, 0: list form, -1: no schedule named one (one launch)
+    int form = -1;                  // 1: one launch, 0: list form, -1: no schedule named one (by the rules)
     int word_blocks = -1;           // widest launch, 0: not available, -1: not set up yet
     int word_use = 0;               // launch width in use
     void* word_mem = nullptr;       // bitmaps of the engine, one allocation
+    int* mixed = nullptr;           // word_box_pays' count
     int4* box_spans = nullptr;      // box form: the units' spans, then the tables read
     WordInst word;                  // views into it
     std::mutex mtx;
@@ -140,6 +141,7 @@ void bf_solve_ws_free(bf_solve_ws* w) {
     cudaFree(w->fc[0]); cudaFree(w->fc[1]); cudaFree(w->fc_tag);
     cudaFree(w->word_mem);
     cudaFree(w->box_spans);
+    cudaFree(w->mixed);
     if (w->tile) tile_free(w->tile);
     delete w;
 }
@@ -331,13 +333,50 @@ static int ws_list(bf_solve_ws* w) {
 }
 
 // Does the word engine's box form apply?  Stored records of any shape, at most
-// 32 inputs.  Up to a million cells: random boxes on a periodic grid take 99
-// against the list form's 154 us at 3,600 cells, 1.35 / 2.89 ms at 136,000, 3.35
-// / 4.32 ms at 480,000, 12.4 / 13.8 ms at 2.2 M, but 3.9 / 2.0 ms at 4.1 M with a
-// small frontier (every unit is tested every pass).
+// 32 inputs and a million cells.
 static bool word_box_form(const bf_abstraction* a) {
     return !a->d_vbits && a->d_boxes && a->nstored == a->g.U && (a->box_fmt == kBoxCompact || a->box_fmt == kBoxWide) &&
            a->g.U <= kWordMaxU && a->g.C <= (1LL << 20);
+}
+
+// Which form a solve takes on such boxes when no schedule names one.  The box
+// form reads the records of every unit of words that the frontier may have
+// reached, the list form those of the frontier's cells but with twice the fixed
+// cost of a pass.  So it goes by the (cell, input) pairs, and above a first line
+// by how broad the frontier is: the share of the bitmap's words that hold both
+// finite and infinite terminal values.  One launch / list form, GB300, boxes of 1
+// to 2 cells a dim unless noted:
+//   2-D  first line 0.85 M pairs: double integrator 300^2 477 / 562 us, 400^2
+//        (0.80 M) 585 / 609, 420^2 (0.88 M) 571 / 566, 500^2 (1.25 M) 684 / 569;
+//        imported 350^2 x 8 (0.98 M, boxes of 1 to 4 cells) from one target 5.5 /
+//        4.8 ms, 1000^2 x 8 46.4 / 25.8 ms.  0.4% targets: 350^2 x 8 633 / 1039
+//        us, 250^2 x 16 (1.0 M) 524 / 867, but 400^2 x 8 (1.28 M) 1.01 / 1.10 ms
+//        and with boxes of up to 4 cells 10.4 / 8.2 ms: up to 1.2 M.
+//   3-D  first line 2.2 M: from one target 64^3 x 8 (2.1 M) 2.76 / 3.06 ms, 90 x 90
+//        x 30 x 11 (2.7 M) 4.10 / 3.84, 80^3 x 8 (4.1 M) 5.5 / 4.6, 100^3 x 8 10.5 /
+//        7.0.  0.4% targets: 90 x 90 x 30 x 11 2.11 / 3.14 ms, 80^3 x 8 4.42 / 5.10,
+//        120 x 100 x 40 x 11 (5.3 M) 3.88 / 4.52, 80^3 x 16 (8.2 M) 2.09 / 1.64:
+//        up to 5.5 M.
+//   4-D  first line 6 M: from one target 24^4 x 16 (5.3 M) 3.03 / 3.60 ms, 32^4 x 8
+//        (8.4 M) 1.92 / 1.28.  0.4% targets: 32^4 x 16 (16.8 M) 3.92 / 3.94,
+//        19.6 / 31.4: every grid up to a million cells.
+constexpr double kBoxPairs[4] = {0.85e6, 0.85e6, 2.2e6, 6.0e6};
+constexpr double kBoxPairsBroad[4] = {1.2e6, 1.2e6, 5.5e6, 33.6e6};
+
+// Words of 32 cells with finite and infinite values in them.
+__global__ void k_mixed_words(long long C, const double* __restrict__ terminal, const unsigned char* __restrict__ target,
+                              const unsigned char* __restrict__ avoid, int* n) {
+    const int lane = threadIdx.x & 31;
+    int mixed = 0;
+    for (long long c0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) & ~31LL; c0 < C;
+         c0 += (long long)gridDim.x * blockDim.x) {
+        const long long c = c0 + lane;
+        bool fin = false;
+        if (c < C) fin = !(avoid && avoid[c]) && (terminal ? terminal[c] < CUDART_INF : target[c] != 0);
+        const unsigned f = __ballot_sync(0xFFFFFFFFu, fin), in = __ballot_sync(0xFFFFFFFFu, c < C);
+        mixed += f != 0u && f != in;
+    }
+    if (lane == 0 && mixed) atomicAdd(n, mixed);
 }
 
 // Does the one-launch form take a solve with these options?  (bf_solve and bf_tune
@@ -396,6 +435,30 @@ static int ws_word(const bf_abstraction* a, bf_solve_ws* w, cudaStream_t st) {
     v.tab[3] = w->M33;
     w->word_blocks = blocks;
     if (w->word_use < 1 || w->word_use > blocks) w->word_use = blocks;
+    return BF_OK;
+}
+
+static int stage_in(const void* src, size_t bytes, void** stage, cudaStream_t st, const void** dev);
+
+// Does the box form pay on these inputs (rule above)?
+static int word_box_pays(const bf_abstraction* a, bf_solve_ws* w, const uint8_t* target, const uint8_t* avoid,
+                         const double* terminal, cudaStream_t st, bool* pays) {
+    const double pairs = (double)a->g.C * a->g.U;
+    *pays = pairs <= kBoxPairs[a->g.D - 1];
+    if (*pays || pairs > kBoxPairsBroad[a->g.D - 1]) return BF_OK;
+    const void *dT, *dTgt, *dAv;
+    int rc, mixed = 0;
+    if ((rc = stage_in(terminal, sizeof(double) * w->C, (void**)&w->stage_T, st, &dT))) return rc;
+    if ((rc = stage_in(terminal ? nullptr : target, w->C, (void**)&w->stage_tgt, st, &dTgt))) return rc;
+    if ((rc = stage_in(avoid, w->C, (void**)&w->stage_avoid, st, &dAv))) return rc;
+    if (!w->mixed) BF_CUDA(cudaMalloc((void**)&w->mixed, sizeof(int)));
+    BF_CUDA(cudaMemsetAsync(w->mixed, 0, sizeof(int), st));
+    k_mixed_words<<<blocks_for(w->C, 256), 256, 0, st>>>(w->C, (const double*)dT, (const unsigned char*)dTgt,
+                                                         (const unsigned char*)dAv, w->mixed);
+    BF_CUDA(cudaGetLastError());
+    BF_CUDA(cudaMemcpyAsync(&mixed, w->mixed, sizeof mixed, cudaMemcpyDeviceToHost, st));
+    BF_CUDA(cudaStreamSynchronize(st));
+    *pays = 20LL * mixed >= w->nwords;         // 0.4% targets: 12% of the words, a block of cells: its rim
     return BF_OK;
 }
 
@@ -770,11 +833,13 @@ extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t*
     std::lock_guard<std::mutex> lock(w->mtx);
     const long long C = w->C;
     const int U = w->U;
-    // plain Jacobi solves of abstractions that have its data take the word
-    // engine unless a schedule was set that names another form: it was faster at
-    // every size measured, from 0.96 -> 0.50 ms (64 x 64 x 5) to 6.29 -> 2.93 ms
+    // plain Jacobi solves of abstractions that have its data take the word engine
+    // unless a schedule was set that names another form: with plane lists it was
+    // faster at every size measured, from 0.96 -> 0.50 ms (64 x 64 x 5) to 6.29 -> 2.93 ms
     // (100 x 100 x 36 x 8 x 15, against the tuned list form)
-    if (w->form != 0 && word_takes(a, opts)) {
+    bool one = w->form != 0 && word_takes(a, opts);
+    if (one && w->form < 0 && !a->d_vbits && (rc = word_box_pays(a, w, target, avoid, terminal, st, &one))) return rc;
+    if (one) {
         if ((rc = ws_word(a, w, st))) return rc;
         if (w->word_blocks > 0) return solve_by_words(a, w, G, target, avoid, opts, V, mu, iters, status, st);
     }
@@ -1088,12 +1153,14 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     if (rc == BF_OK && !w) rc = BF_ERR_CUDA;
     // does the one-launch form take these solves?  It is then timed against the
     // list form whichever is in force; else the form is left as it is
-    bool can = word_takes(a, &o);
+    bool can = word_takes(a, &o), one = w && w->form != 0;
     if (rc == BF_OK) {
         std::lock_guard<std::mutex> lock(w->mtx);
         rc = ws_blocks(a, w, st);
         if (rc == BF_OK && can) rc = ws_word(a, w, st);
         can = can && w->word_blocks > 0;
+        if (rc == BF_OK && can && w->form < 0 && !a->d_vbits)
+            rc = word_box_pays(a, w, target, avoid, o.terminal, st, &one);
     }
     if (rc) { cudaFree(V); cudaFree(mu); return rc; }
     const int full = w->relax_blocks_full;
@@ -1120,7 +1187,8 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     word.use33 = word.plane = word.tmpl = word.pair = word.pfront = true;
     word.masked = 2;
     word.fuse = false;
-    b = can && form != 0 ? word : list;
+    one = one && can;                      // the form that was timed
+    b = one ? word : list;
     out->default_ms = best;
     int tried = 1;
     const bool cls = opts && opts->succ_class;
@@ -1140,7 +1208,7 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
     // the one-launch form, and its width: fewer blocks make its barriers cheaper
     // and leave each more work (4 widths)
     if (can) {
-        if (form == 0) attempt(word);
+        if (!one) attempt(word);
         const int wide = w->word_blocks;
         for (int k = 0; k < 5 && rc == BF_OK; ++k) {
             Sched c = word;
@@ -1169,7 +1237,7 @@ extern "C" int bf_tune(const bf_abstraction* a, const double* G, const uint8_t* 
             if (same_sched(c, first)) continue;                // timed already
             attempt(c);
         }
-    } else if (can && form != 0 && rc == BF_OK) {
+    } else if (one && rc == BF_OK) {
         attempt(list);
     }
     // coordinate descent: each dimension's values with the others at the best

@@ -270,3 +270,41 @@ def test_tuner_times_the_one_launch_form_from_a_list_schedule():
     after = bf.bf_solve(A, w.G, target=w.target, avoid=w.avoid)
     assert t["one_launch"] == 1 and one_launch(after)
     assert same(after["V"], before["V"]) and same(after["mu"], before["mu"])
+
+
+@pytest.mark.parametrize("n,U,scattered,one", [
+    ([9000], 32, False, True), ([320, 320], 8, False, True),
+    ([340, 340], 8, False, False), ([340, 340], 8, True, True), ([500, 500], 5, True, False),
+    ([64, 64, 65], 8, False, True), ([70, 70, 70], 8, False, False), ([70, 70, 70], 8, True, True),
+    ([90, 90, 86], 8, True, False), ([24, 24, 24, 24], 16, False, True),
+    ([30, 30, 30, 30], 8, False, False), ([30, 30, 30, 30], 8, True, True),
+])
+def test_box_form_by_pairs_and_breadth_of_the_frontier(n, U, scattered, one):
+    """Boxes that differ from cell to cell, on both sides of the lines between
+    the one-launch form and the list form: the form a solve takes by itself, host
+    and device inputs, and the same V, mu and passes from either (40 passes)."""
+    import torch
+    rng = np.random.default_rng(4300)
+    C, D = int(np.prod(n)), len(n)
+    coords = np.stack(np.unravel_index(np.arange(C), tuple(reversed(n)))[::-1], axis=1)
+    boxes = np.empty((C, U, 2, D), dtype=np.int16)
+    for u in range(U):
+        lo = coords + rng.integers(-2, 3, size=(1, D)) * (np.arange(D) == u % D)
+        hi = lo + rng.integers(0, 2, size=(C, 1))
+        ok = np.all((lo >= 0) & (hi < np.array(n)), axis=1)
+        boxes[:, u, 0], boxes[:, u, 1] = np.where(ok[:, None], lo, 0), np.where(ok[:, None], hi, 0)
+        boxes[~ok, u, 0, 0] = bf.BLOCKED
+    G = rng.integers(1, 6, size=(C, U)) * 0.25
+    target = (rng.random(C) < 0.004 if scattered else np.all(np.abs(coords - np.array(n) // 2) <= 1, axis=1)).astype(np.uint8)
+    avoid = (rng.random(C) < 0.02).astype(np.uint8)
+    A = handle(n, [False] * D, boxes)
+    dev = [torch.from_numpy(x).cuda() for x in (G, target, avoid)]
+    r = bf.bf_solve(A, dev[0], target=dev[1], avoid=dev[2], max_iters=40)
+    assert one_launch(r) == one
+    T = np.where(target.astype(bool), 0.0, INF)
+    assert one_launch(bf.bf_solve(A, G, terminal=T, avoid=avoid, max_iters=40)) == one
+    for form in (0, 1):
+        bf.bf_set_schedule(A, one_launch=form)
+        q = bf.bf_solve(A, G, target=target, avoid=avoid, max_iters=40)
+        assert one_launch(q) == (form == 1)
+        assert same(q["V"], r["V"]) and same(q["mu"], r["mu"]) and (q["iters"], q["status"]) == (r["iters"], r["status"])
