@@ -400,7 +400,7 @@ size_t Engine::state_bytes_for(long long Cc, int Uc, bool stage_G, bool stage_T,
 }  // namespace bfb
 // solve_word.cu
 int word_wave(int units);
-int word_solve_batch(const bfk::WordInst* insts, int n, int passes, bfk::WordCtr* k, cudaStream_t st);
+int word_solve_batch(const bfk::WordInst* insts, int n, int passes, int blocks, bfk::WordCtr* k, cudaStream_t st);
 namespace bfb {
 
 static int group_of(const bf_abstraction* a) {
@@ -751,15 +751,17 @@ void Engine::launch_pass(cudaGraphConditionalHandle h, int use_graph) {
 // The word engine's instances: at most `passes` passes (negative: all).
 int Engine::run_words(int passes) {
     if (nwords_ == 0) return BF_OK;
-    return word_solve_batch(words_, nwords_, passes, word_ctr_, st_);
+    if (!turn_) turn_.reset(new bfk::WordTurn);
+    return word_solve_batch(words_, nwords_, passes, turn_->width(n_sms()), word_ctr_, st_);
 }
 
-// Did a block give up waiting?  (synchronizes)
+// Did a block give up waiting?  (synchronizes: no launch is on the device any more)
 int Engine::word_fault() {
     if (!word_ctr_) return BF_OK;
     int fault = 0;
     BF_CUDA(cudaMemcpyAsync(&fault, &word_ctr_->fault, sizeof fault, cudaMemcpyDeviceToHost, st_));
     BF_CUDA(cudaStreamSynchronize(st_));
+    turn_.reset();
     if (!fault) return BF_OK;
     bfh::set_error("batch: a block gave up waiting at the grid barrier");
     return BF_ERR_TIMEOUT;

@@ -20,6 +20,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <memory>
 #include <vector>
 
 #include "solve_core.cuh"
@@ -113,6 +114,7 @@ private:
     size_t words_bytes_ = 0;
     bfk::WordCtr* word_ctr_ = nullptr;
     int nwords_ = 0;
+    std::unique_ptr<bfk::WordTurn> turn_;     // while its launches are on the device
     std::vector<bfk::WordInst> host_words_;
     int run_words(int passes);
     int word_fault();

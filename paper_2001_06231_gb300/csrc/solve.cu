@@ -775,13 +775,15 @@ static int solve_by_words(const bf_abstraction* a, bf_solve_ws* w, const double*
     v.trace_cap = tcap;
     v.cap = (opts && opts->max_iters > 0 && opts->max_iters < C) ? opts->max_iters : C;
     BF_CUDA(cudaMemsetAsync(v.ctr, 0, sizeof(WordCtr), st));
+    const WordTurn turn;                        // to the end of the solve
+    const int width = turn.width(w->word_use);
     const bool timed = (flags & BF_FLAG_TIME_KERNELS) != 0;
     double relax_ms = 0.0, rest_ms = 0.0;
     long long launches = 2;
     if (timed || (flags & BF_FLAG_HOST_LOOP))
-        rc = word_solve_host(v, w->word_use, st, timed ? &relax_ms : nullptr, timed ? &rest_ms : nullptr, &launches);
+        rc = word_solve_host(v, width, st, timed ? &relax_ms : nullptr, timed ? &rest_ms : nullptr, &launches);
     else
-        rc = word_solve(v, w->word_use, st);
+        rc = word_solve(v, width, st);
     if (rc) return rc;
     WordCtr hc;
     if (!vdev) BF_CUDA(cudaMemcpyAsync(V, v.V, 8 * C, cudaMemcpyDeviceToHost, st));

@@ -1,6 +1,8 @@
 // solve_word.cu -- kernels of the word engine (word_engine.cuh): all passes of a
 // solve as one cooperative launch, and the same phases as separate launches for the
 // host-driven and timed forms.
+#include <atomic>
+
 #include "word_engine.cuh"
 
 using namespace bfk;
@@ -218,6 +220,30 @@ int word_wave(int units) {
     return units < sms ? units : sms;
 }
 
+// Callers with launches of the engine on a device now.
+static std::atomic<int> word_callers[64];
+
+WordTurn::WordTurn() {
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    callers = ++word_callers[dev & 63];
+}
+
+WordTurn::~WordTurn() { --word_callers[dev & 63]; }
+
+// An equal share of the SMs, an eighth at least.  Microseconds a solve of 1, 2, 4
+// and 8 threads with a handle and a stream each, at full width and by shares (GB300):
+//   double integrator 64 x 64      487 452 454 454    487 254 129  68
+//   double integrator 301 x 205    463 426 424 423    463 255 145  92
+//   unicycle 100 x 100 x 32       1121 1085 1082 1091 1121 651 384 261
+//   unicycle 200 x 200 x 64       1955 1914 1920 1922 1955 1498 1149 1104
+// Narrower than an eighth no more launches fit than threads were measured, and a
+// solve takes twice as long alone.
+int WordTurn::width(int blocks) const {
+    const int n = callers < 8 ? callers : 8, share = sms / n > 0 ? sms / n : 1;
+    return blocks < share ? blocks : share;
+}
+
 // The quotients by the launch's blocks.
 static void word_blocks(WordInst& w, int blocks) {
     GridDesc q;
@@ -245,18 +271,15 @@ int word_solve(const WordInst& w0, int blocks, cudaStream_t st) {
     return BF_OK;
 }
 
-// n instances (device array) together, at most `passes` passes (negative: all);
-// k: scratch counters (`fault` stays set when a block gave up waiting).
-int word_solve_batch(const WordInst* insts, int n, int passes, WordCtr* k, cudaStream_t st) {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+// n instances (device array) together, at most `passes` passes (negative: all) on
+// `blocks` SMs; k: scratch counters (`fault` stays set when a block gave up waiting).
+int word_solve_batch(const WordInst* insts, int n, int passes, int blocks, WordCtr* k, cudaStream_t st) {
     for (int i = 0; i < n; i += kWordInsts) {
         const WordInst* first = insts + i;
         int m = n - i < kWordInsts ? n - i : kWordInsts;
         BF_CUDA(cudaMemsetAsync(&k->bar, 0, sizeof k->bar, st));
         void* args[] = {(void*)&first, (void*)&m, (void*)&passes, (void*)&k};
-        BF_CUDA(cudaLaunchCooperativeKernel((const void*)k_word_batch, dim3(sms), dim3(kWordThreads), args,
+        BF_CUDA(cudaLaunchCooperativeKernel((const void*)k_word_batch, dim3(blocks), dim3(kWordThreads), args,
                                             sizeof(WordSmem), st));
     }
     return BF_OK;

@@ -255,6 +255,20 @@ inline void word_state(WordInst& v, void* mem) {
     v.gmin = (double*)take(word_up(8 * (size_t)v.g.C));
 }
 
+// Host: a caller whose launches by the engine are on the device, from before its
+// first until it has waited for its last (solve_word.cu).  A block of the engine
+// fills an SM and a launch starts when all its blocks fit, so launches at full
+// width run one after the other: callers at the same time share the SMs.
+struct WordTurn {
+    WordTurn();
+    ~WordTurn();
+    WordTurn(const WordTurn&) = delete;
+    WordTurn& operator=(const WordTurn&) = delete;
+    int width(int blocks) const;      // blocks of this caller's launches that take `blocks` alone
+private:
+    int dev = 0, callers = 1, sms = 0;
+};
+
 // ---------------------------------------------------------------------------
 // grid barrier (cooperative launch: every block is resident)
 // ---------------------------------------------------------------------------

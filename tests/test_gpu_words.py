@@ -308,3 +308,58 @@ def test_box_form_by_pairs_and_breadth_of_the_frontier(n, U, scattered, one):
         q = bf.bf_solve(A, G, target=target, avoid=avoid, max_iters=40)
         assert one_launch(q) == (form == 1)
         assert same(q["V"], r["V"]) and same(q["mu"], r["mu"]) and (q["iters"], q["status"]) == (r["iters"], r["status"])
+
+
+def test_solves_of_several_threads_share_the_device():
+    """Solves of four threads, a handle and a stream each, overlap (they took
+    four times a lone solve one after the other, 1.4 times when they share the
+    SMs) and give what a lone solve gives, beside a batched call too."""
+    import threading
+    import time
+
+    import torch
+    from paper_2001_06231_gb300 import workloads as wl
+    w = wl.unicycle3d(n=(100, 100, 32), n_obstacles=10)
+    ins = [torch.from_numpy(x).cuda() for x in (w.G, w.target, w.avoid)]
+
+    def job():
+        A, s = bf.abs_build_workload(w), torch.cuda.Stream()
+        V = torch.empty(w.ncells, dtype=torch.float64, device="cuda")
+        mu = torch.empty(w.ncells, dtype=torch.uint8, device="cuda")
+        return A, lambda: bf.bf_solve(A, ins[0], target=ins[1], avoid=ins[2], V=V, mu=mu, stream=s.cuda_stream)
+
+    jobs = [job() for _ in range(4)]
+    torch.cuda.synchronize()
+
+    def timed(fs, reps=12):
+        def go(f):
+            f()
+            gate.wait()
+            for _ in range(reps):
+                f()
+            gate.wait()
+        gate = threading.Barrier(len(fs) + 1)
+        th = [threading.Thread(target=go, args=(f,)) for f in fs]
+        for t in th:
+            t.start()
+        gate.wait()
+        t0 = time.perf_counter()
+        gate.wait()
+        dt = time.perf_counter() - t0
+        for t in th:
+            t.join()
+        return dt
+
+    lone = jobs[0][1]()
+    lone = (lone["V"].clone(), lone["mu"].clone(), lone["iters"])
+    one = min(timed([jobs[0][1]]) for _ in range(3))
+    four = min(timed([f for _, f in jobs]) for _ in range(3))
+    assert four < 2.5 * one, (one, four)
+    As, batch = [bf.abs_build_workload(w) for _ in range(3)], []
+    timed([f for _, f in jobs] + [lambda: batch.append(bf.bf_solve_batch(
+        As, [w.G] * 3, targets=[w.target] * 3, avoids=[w.avoid] * 3))], reps=3)
+    for r in [f() for _, f in jobs]:
+        assert torch.equal(r["V"], lone[0]) and torch.equal(r["mu"], lone[1]) and r["iters"] == lone[2]
+    for rs in batch:
+        for r in rs:
+            assert same(r["V"], lone[0].cpu().numpy()) and same(r["mu"], lone[1].cpu().numpy()) and r["iters"] == lone[2]
