@@ -579,7 +579,6 @@ int Engine::rebuild() {
         }
         if (!word_ctr_) {
             if (int rc = alloc((void**)&word_ctr_, r256(sizeof(bfk::WordCtr)))) return rc;
-            BF_CUDA(cudaMemsetAsync(word_ctr_, 0, sizeof(bfk::WordCtr), st_));
         }
         BF_CUDA(cudaMemcpyAsync(words_, host_words_.data(), sizeof(bfk::WordInst) * nwords_, cudaMemcpyHostToDevice,
                                 st_));
@@ -752,16 +751,18 @@ void Engine::launch_pass(cudaGraphConditionalHandle h, int use_graph) {
 int Engine::run_words(int passes) {
     if (nwords_ == 0) return BF_OK;
     if (!turn_) turn_.reset(new bfk::WordTurn);
+    // the fault flag is that of this run, which may be several launches
+    BF_CUDA(cudaMemsetAsync(word_ctr_, 0, sizeof(bfk::WordCtr), st_));
     return word_solve_batch(words_, nwords_, passes, turn_->width(n_sms()), word_ctr_, st_);
 }
 
-// Did a block give up waiting?  (synchronizes: no launch is on the device any more)
-int Engine::word_fault() {
-    if (!word_ctr_) return BF_OK;
+// Wait for the stream; did a block of the last run give up waiting at a barrier?
+int Engine::wait_words() {
     int fault = 0;
-    BF_CUDA(cudaMemcpyAsync(&fault, &word_ctr_->fault, sizeof fault, cudaMemcpyDeviceToHost, st_));
+    if (nwords_ && word_ctr_)
+        BF_CUDA(cudaMemcpyAsync(&fault, &word_ctr_->fault, sizeof fault, cudaMemcpyDeviceToHost, st_));
     BF_CUDA(cudaStreamSynchronize(st_));
-    turn_.reset();
+    turn_.reset();                           // no launch is on the device any more
     if (!fault) return BF_OK;
     bfh::set_error("batch: a block gave up waiting at the grid barrier");
     return BF_ERR_TIMEOUT;
@@ -907,7 +908,7 @@ int Engine::read_counters(std::vector<Counters>& out) {
         else
             BF_CUDA(cudaMemcpyAsync(&out[i], insts_[i]->view.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, st_));
     }
-    BF_CUDA(cudaStreamSynchronize(st_));
+    if (int rc = wait_words()) return rc;
     for (size_t i = 0; i < insts_.size(); ++i)
         if (insts_[i]->word) {
             memset(&out[i], 0, sizeof out[i]);
@@ -916,7 +917,7 @@ int Engine::read_counters(std::vector<Counters>& out) {
             out[i].status = wc[i].status;
             out[i].err = wc[i].err;
         }
-    return word_fault();
+    return BF_OK;
 }
 
 int Engine::finish_instance(InstState* s, int64_t* iters, int32_t* status, int* err) {
@@ -929,11 +930,11 @@ int Engine::finish_instance(InstState* s, int64_t* iters, int32_t* status, int* 
     if (s->word) {
         bfk::WordCtr wc;
         BF_CUDA(cudaMemcpyAsync(&wc, s->winst.ctr, sizeof wc, cudaMemcpyDeviceToHost, st_));
-        BF_CUDA(cudaStreamSynchronize(st_));
+        if (int rc = wait_words()) return rc;
         *iters = wc.round;
         *status = wc.status;
         *err = wc.err;
-        return word_fault();
+        return BF_OK;
     }
     Counters hc;
     BF_CUDA(cudaMemcpyAsync(&hc, s->view.ctr, sizeof hc, cudaMemcpyDeviceToHost, st_));

@@ -117,7 +117,7 @@ private:
     std::unique_ptr<bfk::WordTurn> turn_;     // while its launches are on the device
     std::vector<bfk::WordInst> host_words_;
     int run_words(int passes);
-    int word_fault();
+    int wait_words();
     void* dev_mem_ = nullptr;
     size_t dev_mem_bytes_ = 0;
     int relax_blocks_ = 0, prop_blocks_ = 0, compact_blocks_ = 0;

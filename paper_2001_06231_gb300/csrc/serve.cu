@@ -188,6 +188,25 @@ const bf_abstraction* resolve(bf_server* s, Req* r, std::unique_lock<std::mutex>
     return a;
 }
 
+// A step failed (a wait on the device ran out, a CUDA error): the requests on the
+// engine are completed with its code, their state is freed and their bytes are
+// given back.
+void fail_active(bf_server* s, std::unordered_map<bfb::InstState*, Req*>& owner, int rc) {
+    cudaStreamSynchronize(s->st);           // nothing reads the callers' buffers any more
+    for (auto& o : owner) s->eng->remove(o.first);
+    owner.clear();
+    s->eng->rebuild();
+    std::lock_guard<std::mutex> lk(s->m);
+    for (Req* r : s->active) {
+        r->res.error = rc;
+        r->res.done = 1;
+        r->res.finish_s = now_s();
+        s->used -= r->need;
+    }
+    s->active.clear();
+    s->cv_done.notify_all();
+}
+
 void engine_loop(bf_server* s) {
     cudaSetDevice(s->device);
     std::unordered_map<bfb::InstState*, Req*> owner;
@@ -296,22 +315,16 @@ void engine_loop(bf_server* s) {
             }
             s->cv_done.notify_all();
         }
-        if (changed) s->eng->rebuild();
+        int rc = changed ? s->eng->rebuild() : BF_OK;
         if (s->eng->list().empty()) continue;
         // with nobody waiting for a slot, longer steps cost no admission delay and
         // save host round trips; arrivals then wait at most one longer step
-        if (waiting) s->eng->step(s->passes);        // the set changes often: host-launched passes
-        else s->eng->step(4 * s->passes, true);    // light load: one graph launch per step
-        if (s->eng->read_counters(ctrs) != BF_OK) {
-            // a CUDA error: fail every active request
-            std::lock_guard<std::mutex> lk(s->m);
-            for (Req* r : s->active) {
-                r->res.error = BF_ERR_CUDA;
-                r->res.done = 1;
-                r->res.finish_s = now_s();
-            }
-            s->active.clear();
-            s->cv_done.notify_all();
+        if (rc == BF_OK)
+            rc = waiting ? s->eng->step(s->passes)             // the set changes often: host-launched passes
+                         : s->eng->step(4 * s->passes, true);  // light load: one graph launch per step
+        if (rc == BF_OK) rc = s->eng->read_counters(ctrs);
+        if (rc != BF_OK) {
+            fail_active(s, owner, rc);
             continue;
         }
         std::vector<bfb::InstState*> finished;
@@ -323,7 +336,7 @@ void engine_loop(bf_server* s) {
             int64_t it = 0;
             int32_t stt = 0;
             int err = 0;
-            const int rc = s->eng->finish_instance(inst, &it, &stt, &err);
+            rc = s->eng->finish_instance(inst, &it, &stt, &err);
             s->eng->remove(inst);
             owner.erase(inst);
             std::lock_guard<std::mutex> lk(s->m);
@@ -335,9 +348,12 @@ void engine_loop(bf_server* s) {
             s->used -= r->need;
             s->active.erase(std::find(s->active.begin(), s->active.end(), r));
         }
-        s->eng->rebuild();
-        std::lock_guard<std::mutex> lk(s->m);
-        s->cv_done.notify_all();
+        rc = s->eng->rebuild();
+        {
+            std::lock_guard<std::mutex> lk(s->m);
+            s->cv_done.notify_all();
+        }
+        if (rc != BF_OK) fail_active(s, owner, rc);
     }
 }
 

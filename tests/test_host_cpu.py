@@ -137,3 +137,78 @@ def test_bench_kernel_hash_ignores_comments_and_profiles_parse(tmp_path, monkeyp
         assert re.fullmatch(r"[0-9a-f]{16}", kv["kernel_hash"]), path
         form = dict(x.split("=") for x in kv["relax_form"].split())
         assert {"plane_lists", "cell_masks", "input_frontier"} <= set(form), path
+
+
+SERVE_CLIENT = r'''
+import ctypes, sys, time
+import numpy as np
+sys.path.insert(0, sys.argv[2])
+import paper_2001_06231_gb300 as bf
+L = ctypes.CDLL(sys.argv[1])
+P = ctypes.c_void_p
+L.fake_abstraction.restype = P
+L.fake_abstraction.argtypes = [ctypes.c_int64, ctypes.c_int32]
+L.bf_serve_open.argtypes = [ctypes.c_size_t, ctypes.c_int32, ctypes.c_int32, P]
+L.bf_serve_submit.argtypes = [P, P, P]
+L.bf_serve_poll.argtypes = [P, ctypes.c_uint64, ctypes.c_int32, P]
+L.bf_serve_close.argtypes = [P]
+A, C, U, N = L.fake_abstraction(64, 2), 64, 2, 6
+G, tg = np.ones((C, U)), np.ones(C, dtype=np.uint8)
+srv = P()
+assert L.bf_serve_open(100 * (N - 1) + 50, 64, 8, ctypes.byref(srv)) == 0    # room for N - 1 requests' state
+
+def wave(n=N):
+    """n requests: the first is a plain solve, the others wait for it and go to
+    the engine together."""
+    out, ids = [(np.zeros(C), np.zeros(C, dtype=np.uint8)) for _ in range(n)], []
+    for V, mu in out:
+        q, rid = bf.Request(), ctypes.c_uint64()
+        q.abs, q.G, q.target, q.V, q.mu = A, G.ctypes.data, tg.ctypes.data, V.ctypes.data, mu.ctypes.data
+        assert L.bf_serve_submit(srv, ctypes.byref(q), ctypes.byref(rid)) == 0
+        ids.append(rid.value)
+        if len(ids) == 1:
+            time.sleep(0.1)                    # it is running (0.3 s)
+    res = [bf.Result() for _ in ids]
+    for i, r in zip(ids, res):
+        assert L.bf_serve_poll(srv, i, 1, ctypes.byref(r)) == 0
+    return [(r.error, r.iters) for r in res], [V[0] for V, _ in out]
+
+TIMEOUT = -4
+for code in (TIMEOUT, -3, 0):
+    L.fake_fail(1 if code else 0, code)
+    before = L.fake_added()
+    res, V = wave()
+    want = [(0, 7)] + ([(code, 0)] if code else [(0, 7)]) * (N - 1)
+    assert res == want, (code, res)
+    assert V == [1.0] + [0.0 if code else 1.0] * (N - 1), V
+    # every one of them was on the engine, and none is left there
+    assert L.fake_added() - before == N - 1 and L.fake_removed() == L.fake_added()
+L.bf_serve_close(srv)
+print("served")
+'''
+
+
+def test_server_survives_a_step_that_times_out(tmp_path):
+    """A wait that runs out on the device fails the requests of that step, with its
+    code, and nothing else: their state leaves the engine, their bytes go back
+    to the budget, their buffers are not written later, and requests that
+    follow are served.  The server's own source over an engine that only
+    counts (serve_fake.cu), in a process of its own."""
+    import shutil
+    import subprocess
+    import sys
+    from paper_2001_06231_gb300 import _build
+    so = str(tmp_path / "libserve_fake.so")
+    flags = ["-std=c++17", "-Xcompiler", "-fPIC", "-I", _build.INCLUDE, "-I", _build.CSRC]
+    cuda = tmp_path / "cuda_calls.c"
+    cuda.write_text("int cudaSetDevice(int d) { return 0; }\n"
+                    "int cudaGetDevice(int *d) { *d = 0; return 0; }\n"
+                    "int cudaStreamCreateWithFlags(void **s, unsigned f) { *s = 0; return 0; }\n"
+                    "int cudaStreamSynchronize(void *s) { return 0; }\n"
+                    "int cudaStreamDestroy(void *s) { return 0; }\n")
+    src = [os.path.join(_build.CSRC, "serve.cu"), os.path.join(ROOT, "tests", "serve_fake.cu"), str(cuda)]
+    subprocess.run([shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"] + _build.ARCH + flags +
+                   ["-shared", "-cudart", "shared", "-o", so] + src + ["-lpthread"], check=True)
+    r = subprocess.run([sys.executable, "-c", SERVE_CLIENT, so, ROOT], capture_output=True, text=True, timeout=120,
+                       env=dict(os.environ, LD_LIBRARY_PATH="/usr/local/cuda/lib64"))
+    assert r.returncode == 0 and "served" in r.stdout, r.stdout + r.stderr
