@@ -68,7 +68,7 @@ constexpr int kWordHead = 8;          // value lookups of a list kept in shared 
 constexpr int kWordEntries = 4096;    // table entries queued by a block
 constexpr int kWordMaxU = 32;
 constexpr int kWordTest = 128;        // units tested at a time
-constexpr unsigned kWordSpinMax = 1u << 22;
+constexpr unsigned kWordSpinMax = 1u << 28;     // polls of a wait at a barrier
 // Forms of the engine's functions.
 constexpr int kWordOne = 0;           // one instance
 constexpr int kWordMany = 1;          // several instances, each at its own pass
@@ -275,10 +275,15 @@ private:
 // Both barriers: every thread's writes before are visible to every thread
 // after (block barrier, releasing arrival of thread 0; acquiring polls, block
 // barrier).  2.4 us for 152 blocks of 1024 threads; a relaxed add and polls between
-// fences take 2.7.  A wait that gives up sets `fault` and the block leaves the kernel.
+// fences take 2.7.  A wait that gives up (Spin polls) sets `fault` and the block
+// leaves the kernel.  kWordSpinMax polls are about 40 s (0.15 us each): a block may
+// work for long between two barriers while the others wait, up to 1e10 table lookups
+// (10 s) on boxes of a million cells.  (A limit read from memory costs 0.06 us a
+// barrier: 1103 -> 1116 us on a unicycle 100 x 100 x 32 x 10.)
 
 // After the set-up and the tables phases; `target` counts arrivals over the
 // kernel's life.
+template <unsigned Spin = kWordSpinMax>
 __device__ __forceinline__ bool word_barrier(WordCtr* k, unsigned& target, WordSmem& sm) {
     __syncthreads();
     target += gridDim.x;
@@ -289,7 +294,7 @@ __device__ __forceinline__ bool word_barrier(WordCtr* k, unsigned& target, WordS
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&k->bar) : "memory");
             if ((int)(v - target) >= 0) break;
-            if (++n > kWordSpinMax) { ok = 0; atomicExch(&k->fault, 1); break; }
+            if (++n > Spin) { ok = 0; atomicExch(&k->fault, 1); break; }
         }
         sm.flag = ok;
     }
@@ -301,6 +306,7 @@ __device__ __forceinline__ bool word_barrier(WordCtr* k, unsigned& target, WordS
 // frontier cell and whether any cell changed, so the loop condition costs no
 // further read (a line that every warp reads takes microseconds).  Returns the
 // gate's value, 0 when the wait gave up.
+template <unsigned Spin = kWordSpinMax>
 __device__ __forceinline__ unsigned long long word_gate(WordCtr* k, int r, WordSmem& sm) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -316,7 +322,7 @@ __device__ __forceinline__ unsigned long long word_gate(WordCtr* k, int r, WordS
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(g) : "memory");
             if ((v & 0xFFFFull) >= gridDim.x) break;
-            if (++n > kWordSpinMax) { v = 0ull; atomicExch(&k->fault, 1); break; }
+            if (++n > Spin) { v = 0ull; atomicExch(&k->fault, 1); break; }
         }
         sm.gate = v;
     }

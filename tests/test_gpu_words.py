@@ -363,3 +363,18 @@ def test_solves_of_several_threads_share_the_device():
     for rs in batch:
         for r in rs:
             assert same(r["V"], lone[0].cpu().numpy()) and same(r["mu"], lone[1].cpu().numpy()) and r["iters"] == lone[2]
+
+
+@pytest.mark.parametrize("gate", [0, 1])
+def test_a_wait_that_runs_out_sets_its_flag_and_leaves(tmp_path, gate):
+    """A block whose partner never arrives gives up after its polls, sets the fault
+    flag and returns; the device goes on (a solve afterwards)."""
+    import ctypes
+    from test_host_cpu import build_word_wait
+    lib = build_word_wait(tmp_path)
+    passed, fault = ctypes.c_int(-2), ctypes.c_int(-2)
+    assert lib.wait_runs_out(gate, ctypes.byref(passed), ctypes.byref(fault)) == 0
+    assert passed.value == 0 and fault.value == 1
+    n, periodic, boxes, G, target, avoid, ref = form_instance("entries")
+    r = bf.bf_solve(handle(n, periodic, boxes), G, target=target, avoid=avoid)
+    assert one_launch(r) and same(r["V"], ref["V"])

@@ -212,3 +212,32 @@ def test_server_survives_a_step_that_times_out(tmp_path):
     r = subprocess.run([sys.executable, "-c", SERVE_CLIENT, so, ROOT], capture_output=True, text=True, timeout=120,
                        env=dict(os.environ, LD_LIBRARY_PATH="/usr/local/cuda/lib64"))
     assert r.returncode == 0 and "served" in r.stdout, r.stdout + r.stderr
+
+
+def build_word_wait(tmp_path):
+    """tests/word_wait.cu as a library: the word engine's waits."""
+    import shutil
+    import subprocess
+    from paper_2001_06231_gb300 import _build
+    so = str(tmp_path / "libword_wait.so")
+    subprocess.run([shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"] + _build.ARCH +
+                   ["-std=c++17", "-Xcompiler", "-fPIC", "-I", _build.INCLUDE, "-I", _build.CSRC, "-shared", "-o", so,
+                    os.path.join(ROOT, "tests", "word_wait.cu")], check=True)
+    lib = ctypes.CDLL(so)
+    lib.spin_limit.restype = ctypes.c_double
+    return lib
+
+
+def test_barrier_waits_outlast_the_work_of_a_block(tmp_path):
+    """A block may work between two barriers while the others wait for it: the polls
+    of a wait (0.15 us at least) last longer than that at a rate no SM is below
+    (1e9 table lookups a second), on the most pairs that fit the memory with the
+    most lookups of a list, and on boxes that differ and hold the whole grid."""
+    polls = build_word_wait(tmp_path).spin_limit()
+    seconds = 0.15e-6 * polls
+    # 60 lookups a pair, costs of 8 bytes in 280 GB, all SMs
+    assert seconds > 60 * 280e9 / 8 / 152 / 1e9
+    # units of 1024 cells, windows of 3 cells (rows that wrap), most pairs of the box form
+    for cells, pairs in ((170e3, 0.85e6), (1 << 20, 5.5e6)):
+        units = -(-cells // 1024)
+        assert seconds > -(-units // 152) * (pairs / units) * (cells / 3) / 1e9
