@@ -102,8 +102,9 @@ extern "C" {
  * 4*D*C*U fewer bytes, far more FP64 work).  Where every box of a plane (equal
  * coordinates on dims >= 2) and input has the same shape relative to its cell
  * -- the unicycle and the fire model -- the abstraction also keeps one bit per
- * (cell, input) and the planes' lookup lists, and plain Jacobi solves use those
- * instead of regenerating boxes. */
+ * (cell, input) and the planes' lookup lists, where these take no more than a
+ * quarter of the compact records (planes of about 250 cells), and plain Jacobi
+ * solves use those instead of regenerating boxes. */
 #define BF_MODE_STORED 0
 #define BF_MODE_RECOMPUTE 1
 #define BF_MODE_HYBRID 2       /* records of the first K inputs stored, the

@@ -56,3 +56,20 @@ def test_range_tables_equal_the_general_path(name):
     K = max(1, w.ninputs // 3)
     H = bf.abs_build_workload(w, box_budget=8 * w.ncells * K)
     assert np.array_equal(H.export_boxes(), boxes) and np.array_equal(H.export_pred(), pred)
+
+
+@pytest.mark.parametrize("n,held", [((6, 6, 300), False), ((10, 10, 200), False), ((20, 20, 60), True),
+                                    ((40, 40, 20), True)])
+def test_recompute_handles_stay_small(n, held):
+    """What a recompute handle holds beside the inputs, the predecessor index and the
+    shared RK4 parts is at most a quarter of the compact records it avoids: on
+    planes of few cells nothing, and its solves regenerate the boxes."""
+    w = wl.unicycle3d(n=n, n_obstacles=1)
+    S, R = bf.abs_build_workload(w), bf.abs_build_workload(w, mode=bf.MODE_RECOMPUTE)
+    C, U, planes = w.ncells, w.ninputs, n[2]
+    base = 16 * U + 4 * 3 * C + 22 * 8 * planes * U
+    extra = R.device_bytes - base
+    assert 0 <= extra <= 8 * C * U // 4 and (extra > 0) == held
+    r, s = (bf.bf_solve(A, w.G, target=w.target, avoid=w.avoid) for A in (R, S))
+    assert (r["stats"]["kernel_launches"] == 2) == held
+    assert np.array_equal(r["V"], s["V"]) and np.array_equal(r["mu"], s["mu"]) and r["iters"] == s["iters"]
