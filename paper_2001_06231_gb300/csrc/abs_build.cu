@@ -44,6 +44,7 @@ void set_error(const char* fmt, ...) {
 }
 
 int cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();                    // reported here, not by the next call's launch check
     set_error("CUDA error %d (%s) in %s", (int)e, cudaGetErrorString(e), what);
     return e == cudaErrorMemoryAllocation ? BF_ERR_OOM : BF_ERR_CUDA;
 }

@@ -100,3 +100,16 @@ def test_large_grid_random_boxes():
     T[: n[0] * 4] = 0.0                                      # the first rows are the target
     res, _ = solve_both(n, [False, False], boxes, G, T, max_iters=40)
     assert res["status"] == bf.ITER_CAP
+
+
+def test_an_allocation_that_fails_is_reported_once():
+    """A system too large for the device is BF_ERR_OOM; the calls after it work."""
+    import ctypes
+    from paper_2001_06231_gb300 import workloads as wl
+    g, h, boxes = bf.make_grid([16383, 16383, 7]), ctypes.c_void_p(), np.zeros(16, dtype=np.int16)
+    w = wl.unicycle3d(n=(20, 18, 8), n_obstacles=2)
+    for _ in range(2):
+        rc = bf.lib().abs_from_boxes(ctypes.byref(g), 254, boxes.ctypes.data, None, ctypes.byref(h))   # 11 TB
+        assert rc == -2 and not h.value
+        r = bf.bf_solve(bf.abs_build_workload(w), w.G, target=w.target, avoid=w.avoid)
+        assert np.all(r["V"][w.target.astype(bool)] == 0.0)
