@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -830,6 +831,17 @@ static int build_pred(bf_abstraction* a, cudaStream_t st) {
     }
 }
 
+// A build step with lists on the host: no exception leaves the library.
+template <typename F>
+static int guarded(F f) {
+    try {
+        return f();
+    } catch (const std::bad_alloc&) {
+        bfh::set_error("abs_build: out of host memory");
+        return BF_ERR_OOM;
+    }
+}
+
 // Scratch buffers of a build step, freed (on the stream) when it ends.
 struct BuildTemps {
     cudaStream_t st;
@@ -848,11 +860,28 @@ struct BuildTemps {
     }
 };
 
+// Scratch of the range tables up to which they are always taken (bytes), and the
+// entries of the lists of target planes (16 bytes each, on the host and the
+// device).  The unicycle 200 x 200 x 64 x 10 takes 2.4 MB and some 2,000 entries,
+// the fire model 100 x 100 x 36 x 8 x 15 8 MB and 65,000; planes of few cells, or
+// ranges over thousands of planes, may take gigabytes.
+constexpr size_t kRangeScratch = 256u << 20;
+constexpr long long kPlaneHits = 1LL << 24;
+
 // Do the range tables apply?  (3- and 4-D built-in systems whose shared RK4
-// entries exist, dims 0 and 1 not periodic.)
+// entries exist, dims 0 and 1 not periodic, and tables no larger than what the
+// general path takes, kRangeScratch apart: the wide records of a stored build,
+// the bounds of the predecessor boxes of another.)
 static bool has_ranges(const bf_abstraction* a) {
-    return a->g.D >= 3 && a->dyn.kind != 0 && a->dyn.rk4_substeps >= 1 && a->dyn.rk4_substeps <= kRkMaxSub &&
-           !a->g.periodic[0] && !a->g.periodic[1];
+    const GridDesc& g = a->g;
+    if (g.D < 3 || a->dyn.kind == 0 || a->dyn.rk4_substeps < 1 || a->dyn.rk4_substeps > kRkMaxSub || g.periodic[0] ||
+        g.periodic[1])
+        return false;
+    const size_t entries = (size_t)(g.C / g.stride[2]) * g.U;
+    const size_t per = 2 * sizeof(short2) * (size_t)(g.n[0] + g.n[1]) + sizeof(short4) +
+                       (a->mode == BF_MODE_STORED ? sizeof(double) * kRkEntry : 0);
+    const size_t general = a->mode == BF_MODE_STORED ? box_bytes(g) : 2 * sizeof(int) * g.D * (size_t)g.C;
+    return entries * per <= std::max(general, kRangeScratch);
 }
 
 // The range tables, from the handle's shared RK4 entries or a scratch copy.
@@ -891,54 +920,85 @@ static int pred_off(const GridDesc& g, int d, int x, int y) {
     return o;
 }
 
-// The predecessor index from the range tables: what k_pred_scatter finds, without
-// walking every box (unicycle 200 x 200 x 64 x 10: 11.7 ms for 1.2 G cell visits).
-template <int D>
-static int build_pred_ranges_t(bf_abstraction* a, const RangeTabs& t, BuildTemps& tmp, cudaStream_t st) {
+// The source entries of every target plane, from the ranges on dims >= 2.
+struct PlaneHits {
+    std::vector<int> ptr;      // [P + 1]
+    std::vector<int4> ent;     // {entry q U + u, offsets q - p on dims 2 and 3, 0}
+};
+
+// BF_ERR_OOM where they are more than kPlaneHits.
+static int plane_hits(const bf_abstraction* a, const RangeTabs& t, PlaneHits& h, cudaStream_t st) {
     const GridDesc& g = a->g;
     const long long P = g.C / g.stride[2], U = g.U, n = P * U;
-    short2 *p0 = nullptr, *p1 = nullptr;
-    int* ptr = nullptr;
-    int4* ent = nullptr;
-    BF_CUDA(tmp.get(&p0, (size_t)n * g.n[0]));
-    BF_CUDA(tmp.get(&p1, (size_t)n * g.n[1]));
-    k_pred_ranges<<<grid_blocks(n * g.n[0], 128), 128, 0, st>>>(n, g.n[0], t.r0, p0);
-    k_pred_ranges<<<grid_blocks(n * g.n[1], 128), 128, 0, st>>>(n, g.n[1], t.r1, p1);
     std::vector<short4> r23((size_t)n);
     BF_CUDA(cudaMemcpyAsync(r23.data(), t.r23, sizeof(short4) * n, cudaMemcpyDeviceToHost, st));
     BF_CUDA(cudaStreamSynchronize(st));
-    const int n2 = g.n[2], n3 = D >= 4 ? g.n[3] : 1;
+    const int n2 = g.n[2], n3 = g.n[3];
+    auto hi3 = [&](const short4& r) { return g.D >= 4 ? (int)r.w : 0; };
+    auto lo3 = [&](const short4& r) { return g.D >= 4 ? (int)r.z : 0; };
+    long long hits = 0;
+    for (const short4& r : r23)
+        if (r.x != kBlocked) hits += (long long)(r.y - r.x + 1) * (hi3(r) - lo3(r) + 1);
+    if (hits > kPlaneHits) {
+        bfh::set_error("abs_build: %lld (plane, input) pairs per target plane", hits);
+        return BF_ERR_OOM;
+    }
     // two rounds over the entries: count per target plane, then fill
-    std::vector<int> hptr((size_t)P + 1, 0);
-    std::vector<int4> hent;
+    h.ptr.assign((size_t)P + 1, 0);
     std::vector<int> at;
     for (int fill = 0; fill < 2; ++fill) {
         for (long long e = 0; e < n; ++e) {
             const short4 r = r23[(size_t)e];
             if (r.x == kBlocked) continue;
             const int q = (int)(e / U), q2 = q % n2, q3 = q / n2;
-            const int lo3 = D >= 4 ? r.z : 0, hi3 = D >= 4 ? r.w : 0;
-            for (int x3 = lo3; x3 <= hi3; ++x3)
+            for (int x3 = lo3(r); x3 <= hi3(r); ++x3)
                 for (int x2 = r.x; x2 <= r.y; ++x2) {
                     const int y2 = x2 >= n2 ? x2 - n2 : x2, y3 = x3 >= n3 ? x3 - n3 : x3;
                     const size_t p = (size_t)(y2 + n2 * y3);
-                    if (!fill) ++hptr[p + 1];
-                    else hent[(size_t)at[p]++] =
-                             make_int4((int)e, pred_off(g, 2, q2, y2), D >= 4 ? pred_off(g, 3, q3, y3) : 0, 0);
+                    if (!fill) ++h.ptr[p + 1];
+                    else h.ent[(size_t)at[p]++] =
+                             make_int4((int)e, pred_off(g, 2, q2, y2), g.D >= 4 ? pred_off(g, 3, q3, y3) : 0, 0);
                 }
         }
         if (!fill) {
-            for (size_t p = 0; p < (size_t)P; ++p) hptr[p + 1] += hptr[p];
-            hent.resize((size_t)hptr[(size_t)P]);
-            at.assign(hptr.begin(), hptr.end() - 1);
+            for (size_t p = 0; p < (size_t)P; ++p) h.ptr[p + 1] += h.ptr[p];
+            h.ent.resize((size_t)h.ptr[(size_t)P]);
+            at.assign(h.ptr.begin(), h.ptr.end() - 1);
         }
     }
-    BF_CUDA(tmp.get(&ptr, hptr.size()));
-    BF_CUDA(tmp.get(&ent, hent.size()));
-    BF_CUDA(cudaMemcpyAsync(ptr, hptr.data(), sizeof(int) * hptr.size(), cudaMemcpyHostToDevice, st));
-    if (!hent.empty())
-        BF_CUDA(cudaMemcpyAsync(ent, hent.data(), sizeof(int4) * hent.size(), cudaMemcpyHostToDevice, st));
-    k_pred_from_ranges<D><<<grid_blocks(g.C, 256), 256, 0, st>>>(g, ptr, ent, p0, p1, a->d_pred);
+    return BF_OK;
+}
+
+// Predecessor ranges along dims 0 and 1.
+struct PredTabs {
+    short2* p0 = nullptr;      // [keys][U][n0]
+    short2* p1 = nullptr;      // [keys][U][n1]
+};
+
+static int build_pred_tabs(const bf_abstraction* a, const RangeTabs& t, PredTabs& p, BuildTemps& tmp, cudaStream_t st) {
+    const GridDesc& g = a->g;
+    const long long n = g.C / g.stride[2] * g.U;
+    BF_CUDA(tmp.get(&p.p0, (size_t)n * g.n[0]));
+    BF_CUDA(tmp.get(&p.p1, (size_t)n * g.n[1]));
+    k_pred_ranges<<<grid_blocks(n * g.n[0], 128), 128, 0, st>>>(n, g.n[0], t.r0, p.p0);
+    k_pred_ranges<<<grid_blocks(n * g.n[1], 128), 128, 0, st>>>(n, g.n[1], t.r1, p.p1);
+    BF_CUDA(cudaGetLastError());
+    return BF_OK;
+}
+
+// The predecessor index from the range tables: what k_pred_scatter finds, without
+// walking every box (unicycle 200 x 200 x 64 x 10: 11.7 ms for 1.2 G cell visits).
+template <int D>
+static int build_pred_ranges_t(bf_abstraction* a, const PredTabs& p, const PlaneHits& h, BuildTemps& tmp, cudaStream_t st) {
+    const GridDesc& g = a->g;
+    int* ptr = nullptr;
+    int4* ent = nullptr;
+    BF_CUDA(tmp.get(&ptr, h.ptr.size()));
+    BF_CUDA(tmp.get(&ent, h.ent.size()));
+    BF_CUDA(cudaMemcpyAsync(ptr, h.ptr.data(), sizeof(int) * h.ptr.size(), cudaMemcpyHostToDevice, st));
+    if (!h.ent.empty())
+        BF_CUDA(cudaMemcpyAsync(ent, h.ent.data(), sizeof(int4) * h.ent.size(), cudaMemcpyHostToDevice, st));
+    k_pred_from_ranges<D><<<grid_blocks(g.C, 256), 256, 0, st>>>(g, ptr, ent, p.p0, p.p1, a->d_pred);
     BF_CUDA(cudaGetLastError());
     return pred_rows_t<D>(a, st);                       // synchronizes: the host vectors are done
 }
@@ -1468,7 +1528,7 @@ static int build_word(bf_abstraction* a, const unsigned long long* shape, const 
 // boxes).  Where every entry of the range tables has one record, that is the
 // shape table, and an abstraction whose boxes are regenerated gets the word
 // engine's data too: a bit per pair and the lists stand for its boxes.
-static int build_shapes(bf_abstraction* a, const RangeTabs* ranges, cudaStream_t st) {
+static int build_shapes_of(bf_abstraction* a, const RangeTabs* ranges, cudaStream_t st) {
     const GridDesc& g = a->g;
     BuildTemps tmp(st);
     unsigned long long* known = nullptr;
@@ -1501,6 +1561,10 @@ static int build_shapes(bf_abstraction* a, const RangeTabs* ranges, cudaStream_t
     if (rc == BF_OK && a->d_shape && a->shape_mismatch == 0) rc = build_templates(a, st);
     if (rc == BF_OK && a->d_tent) rc = build_word(a, a->d_shape, known ? ranges : nullptr, st);
     return rc;
+}
+
+static int build_shapes(bf_abstraction* a, const RangeTabs* ranges, cudaStream_t st) {
+    return guarded([&] { return build_shapes_of(a, ranges, st); });
 }
 
 static bf_abstraction* new_abs() {
@@ -1571,11 +1635,10 @@ extern "C" int abs_build(const bf_dynamics* dyn, const bf_grid* grid, const bf_i
     a->tau = tau;
     a->udim = inputs->udim;
     size_t in_bytes = sizeof(double) * inputs->ninputs * inputs->udim;
-    const bool ranges = has_ranges(a);
+    bool ranges = has_ranges(a);
     cudaError_t e = cudaMalloc(&a->d_inputs, in_bytes);
     if (e == cudaSuccess) e = cudaMemcpyAsync(a->d_inputs, inputs->u, in_bytes, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMalloc((void**)&a->d_pred, sizeof(short) * 2 * g.D * g.C);
-    if (e == cudaSuccess && mode == BF_MODE_STORED && !ranges) e = cudaMalloc(&a->d_boxes, box_bytes(a->g));
     if (e != cudaSuccess) { abs_free(a); return bfh::cuda_fail(e, "abs_build allocation"); }
     a->bytes = in_bytes + sizeof(short) * 2 * g.D * g.C + (mode == BF_MODE_STORED ? box_bytes(a->g) : 0);
     DynDesc dd = make_dyndesc(a);
@@ -1598,12 +1661,33 @@ extern "C" int abs_build(const bf_dynamics* dyn, const bf_grid* grid, const bf_i
     if (ranges) {
         BuildTemps tmp(st);
         RangeTabs t;
-        rc = build_ranges(a, t, tmp, st);
-        if (rc == BF_OK && mode == BF_MODE_STORED) rc = boxes_from_ranges(a, t, st);
-        if (rc == BF_OK) rc = g.D == 3 ? build_pred_ranges_t<3>(a, t, tmp, st) : build_pred_ranges_t<4>(a, t, tmp, st);
-        if (rc == BF_OK) rc = build_shapes(a, &t, st);
-    } else {
+        PredTabs p;
+        PlaneHits h;
+        const size_t bytes = a->bytes;
+        rc = guarded([&] {
+            int r = build_ranges(a, t, tmp, st);
+            if (r == BF_OK && mode == BF_MODE_STORED) r = boxes_from_ranges(a, t, st);
+            if (r == BF_OK) r = build_pred_tabs(a, t, p, tmp, st);
+            return r ? r : plane_hits(a, t, h, st);
+        });
+        if (rc == BF_ERR_OOM) {
+            // the general path takes less
+            cudaFree(a->d_boxes);
+            a->d_boxes = nullptr;
+            a->box_fmt = mode == BF_MODE_STORED ? kBoxWide : kBoxRecompute;
+            a->bytes = bytes;
+            ranges = false;
+            rc = BF_OK;
+        } else {
+            if (rc == BF_OK)
+                rc = g.D == 3 ? build_pred_ranges_t<3>(a, p, h, tmp, st) : build_pred_ranges_t<4>(a, p, h, tmp, st);
+            if (rc == BF_OK) rc = build_shapes(a, &t, st);
+        }
+    }
+    if (!ranges) {
         if (mode == BF_MODE_STORED) {
+            e = cudaMalloc(&a->d_boxes, box_bytes(a->g));
+            if (e != cudaSuccess) { abs_free(a); return bfh::cuda_fail(e, "abs_build allocation"); }
             const int nb = grid_blocks(a->g.C * a->g.U, 128);
             switch (g.D) {
                 case 2: k_build_boxes<2><<<nb, 128, 0, st>>>(dd, a->g, a->d_inputs, a->d_boxes); break;
@@ -1647,9 +1731,10 @@ static int add_stored_inputs(bf_abstraction* a, int K, cudaStream_t st) {
             if (has_ranges(a)) {
                 RangeTabs t;
                 const int rc = build_ranges_t<D>(a, t, tmp, st);
-                if (rc) { cudaFree(d_fail); cudaFree(comp); return rc; }
-                k_compact_ranges<D><<<grid_blocks(gk.C * K, 256), 256, 0, st>>>(a->g, t, K, comp, d_fail);
-                done = true;
+                if (rc && rc != BF_ERR_OOM) { cudaFree(d_fail); cudaFree(comp); return rc; }
+                if (rc == BF_OK)
+                    k_compact_ranges<D><<<grid_blocks(gk.C * K, 256), 256, 0, st>>>(a->g, t, K, comp, d_fail);
+                done = rc == BF_OK;     // without the scratch: box by box
             }
         }
         if (!done) {

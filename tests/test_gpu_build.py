@@ -73,3 +73,40 @@ def test_recompute_handles_stay_small(n, held):
     r, s = (bf.bf_solve(A, w.G, target=w.target, avoid=w.avoid) for A in (R, S))
     assert (r["stats"]["kernel_launches"] == 2) == held
     assert np.array_equal(r["V"], s["V"]) and np.array_equal(r["mu"], s["mu"]) and r["iters"] == s["iters"]
+
+
+MANY_PLANES = r'''
+import sys
+import numpy as np
+sys.path.insert(0, sys.argv[1])
+import paper_2001_06231_gb300 as bf
+from paper_2001_06231_gb300 import workloads as wl
+def held():                                # most host memory the process held, MB
+    return int(next(l for l in open("/proc/self/status") if l.startswith("VmHWM")).split()[1]) / 1024
+w = wl.unicycle3d(n=(20, 18, 8), n_obstacles=2)
+bf.abs_build_workload(w)                   # the context is up
+g = bf.make_grid([3, 3, 16383], w.grid.lo, w.grid.hi, w.grid.periodic)
+before = held()
+A = [bf.abs_build(w.kind, [0.5] + list(w.params[1:]), w.substeps, g, w.inputs[:2], w.tau, m)
+     for m in (bf.MODE_STORED, bf.MODE_RECOMPUTE)]
+print("grew", held() - before)
+boxes = A[0].export_boxes()
+assert (boxes[:, :, 0, 0] != bf.BLOCKED).any() and np.array_equal(boxes, A[1].export_boxes())
+pred = bf.abs_from_boxes(g, boxes).export_pred()
+assert np.array_equal(A[0].export_pred(), pred) and np.array_equal(A[1].export_pred(), pred)
+assert A[0].box_record_bytes == 12
+'''
+
+
+def test_ranges_over_many_planes_take_the_general_path():
+    """A grid of 9 cells a plane whose boxes span 784 of 16,383 planes: the lists of
+    target planes would hold 26 M entries (411 MB on the host and on the device
+    each); the build takes the general path, with the same boxes and predecessor
+    boxes in either mode, and holds little host memory.  In a process of its own."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", MANY_PLANES, root], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+    assert float(r.stdout.split()[1]) < 150, r.stdout
