@@ -405,7 +405,14 @@ static int ws_word(const bf_abstraction* a, bf_solve_ws* w, cudaStream_t st) {
         blocks = word_wave(v.units);
         if (blocks == 0) return BF_OK;
         const size_t n = (size_t)v.units * kWordSpans;
-        if (!w->box_spans) BF_CUDA(cudaMalloc((void**)&w->box_spans, sizeof(int4) * n + 16));
+        if (!w->box_spans) {
+            const cudaError_t e = cudaMalloc((void**)&w->box_spans, sizeof(int4) * n + 16);
+            if (e != cudaSuccess) {
+                w->box_spans = nullptr;
+                w->word_blocks = -1;
+                return bfh::cuda_fail(e, "word engine workspace");
+            }
+        }
         int* used = (int*)(w->box_spans + n);
         int h_used = 0;
         BF_CUDA(cudaMemsetAsync(used, 0, sizeof(int), st));
@@ -842,8 +849,11 @@ extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t*
     bool one = w->form != 0 && word_takes(a, opts);
     if (one && w->form < 0 && !a->d_vbits && (rc = word_box_pays(a, w, target, avoid, terminal, st, &one))) return rc;
     if (one) {
-        if ((rc = ws_word(a, w, st))) return rc;
-        if (w->word_blocks > 0) return solve_by_words(a, w, G, target, avoid, opts, V, mu, iters, status, st);
+        // without the memory for it, the list form, whose workspace may be there
+        rc = ws_word(a, w, st);
+        if (rc == BF_OK && w->word_blocks > 0)
+            rc = solve_by_words(a, w, G, target, avoid, opts, V, mu, iters, status, st);
+        if (rc != BF_ERR_OOM && (rc || w->word_blocks > 0)) return rc;
     }
     if ((rc = ws_blocks(a, w, st))) return rc;
     // schedule (the graph holds the view by value: rebuild it on a change)

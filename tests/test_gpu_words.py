@@ -378,3 +378,44 @@ def test_a_wait_that_runs_out_sets_its_flag_and_leaves(tmp_path, gate):
     n, periodic, boxes, G, target, avoid, ref = form_instance("entries")
     r = bf.bf_solve(handle(n, periodic, boxes), G, target=target, avoid=avoid)
     assert one_launch(r) and same(r["V"], ref["V"])
+
+
+FULL_DEVICE = r'''
+import sys
+sys.path.insert(0, sys.argv[1])
+import torch
+import paper_2001_06231_gb300 as bf
+from paper_2001_06231_gb300 import workloads as wl
+w = wl.unicycle3d()
+A = bf.abs_build_workload(w)
+a = [torch.from_numpy(x).cuda() for x in (w.G, w.target, w.avoid)]
+V = torch.empty(w.ncells, dtype=torch.float64, device="cuda")
+mu = torch.empty(w.ncells, dtype=torch.uint8, device="cuda")
+solve = lambda **k: bf.bf_solve(A, a[0], target=a[1], avoid=a[2], V=V, mu=mu, **k)
+solve(schedule=bf.SCHED_INPLACE)           # the list form's workspace
+hog, step = [], 1 << 34
+while step >= 1 << 21:                     # the rest of the memory
+    try:
+        hog.append(torch.empty(step, dtype=torch.uint8, device="cuda"))
+    except torch.OutOfMemoryError:
+        step >>= 1
+full = solve()
+got = V.cpu()
+hog = None
+torch.cuda.empty_cache()
+again = solve()
+assert again["stats"]["kernel_launches"] == 2 and full["iters"] == again["iters"] and torch.equal(got, V.cpu())
+print("solved")
+'''
+
+
+def test_without_memory_for_the_one_launch_form_the_list_form_solves():
+    """A handle with the list form's workspace solves on a full device (the 40 MB of
+    the one-launch form cannot be had), and takes the one-launch form when there
+    is memory again.  In a process of its own."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FULL_DEVICE, root], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "solved" in r.stdout, r.stdout + r.stderr
