@@ -776,7 +776,15 @@ static int solve_by_words(const bf_abstraction* a, bf_solve_ws* w, const double*
         v.tabc[2] = w->M3R;
         v.tabc[3] = w->M33R;
     }
-    v.mu = mdev ? mu : w->mu;
+    // mu is written while the inputs are read: straight into the caller's buffer
+    // unless that holds one of them
+    auto held = [&](const void* p, size_t n) {
+        return p && (const uint8_t*)p < mu + C && mu < (const uint8_t*)p + n;
+    };
+    const size_t cost = sizeof(double) * C * w->U;
+    const bool direct = mdev && !held(dG, cost) && !held(dGc, cost) && !held(dT, sizeof(double) * C) && !held(dTgt, C) &&
+                        !held(dAv, C) && !held(dCls, C);
+    v.mu = direct ? mu : w->mu;
     v.V = vdev ? V : w->stage_V;
     v.trace = tcap > 0 ? w->trace : nullptr;
     v.trace_cap = tcap;
@@ -794,7 +802,7 @@ static int solve_by_words(const bf_abstraction* a, bf_solve_ws* w, const double*
     if (rc) return rc;
     WordCtr hc;
     if (!vdev) BF_CUDA(cudaMemcpyAsync(V, v.V, 8 * C, cudaMemcpyDeviceToHost, st));
-    if (!mdev) BF_CUDA(cudaMemcpyAsync(mu, v.mu, C, cudaMemcpyDeviceToHost, st));
+    if (!direct) BF_CUDA(cudaMemcpyAsync(mu, v.mu, C, cudaMemcpyDefault, st));
     BF_CUDA(cudaMemcpyAsync(&hc, v.ctr, sizeof hc, cudaMemcpyDeviceToHost, st));
     if (tcap > 0)
         BF_CUDA(cudaMemcpyAsync(opts->trace, w->trace, sizeof(long long) * 4 * tcap, cudaMemcpyDeviceToHost, st));

@@ -419,3 +419,29 @@ def test_without_memory_for_the_one_launch_form_the_list_form_solves():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", FULL_DEVICE, root], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "solved" in r.stdout, r.stdout + r.stderr
+
+
+def test_mu_may_be_written_over_an_input():
+    """A device buffer given as the class or the avoid mask and as mu too: read as
+    the input to the end, then written, as in the list form."""
+    import torch
+    n, periodic, U = [33, 17, 5], [False, False, True], 4
+    rng = np.random.default_rng(4400)
+    boxes, G, target, avoid = plane_instance(rng, n, periodic, U, wmax=(5, 4, 3, 1), p_differ=0.0)
+    C = boxes.shape[0]
+    cls = (rng.random(C) < 0.3).astype(np.uint8)
+    Gc = rng.integers(-2, 5, size=(C, U)) * 0.25
+    T = rng.integers(0, 30, size=C) * 0.5
+    A = handle(n, periodic, boxes)
+    ref = oracle.solve(n, periodic, boxes, G, T, avoid, succ_class=cls, G_class=Gc, max_iters=200)
+    assert ref["iters"] > 3
+    for over in ("cls", "avoid"):
+        for form in (1, 0):
+            bf.bf_set_schedule(A, one_launch=form)
+            d = {k: torch.from_numpy(x.copy()).cuda() for k, x in
+                 (("G", G), ("T", T), ("avoid", avoid), ("cls", cls), ("Gc", Gc))}
+            V = torch.empty(C, dtype=torch.float64, device="cuda")
+            r = bf.bf_solve(A, d["G"], terminal=d["T"], avoid=d["avoid"], succ_class=d["cls"], G_class=d["Gc"], V=V,
+                            mu=d[over], max_iters=200)
+            assert one_launch(r) == (form == 1) and r["iters"] == ref["iters"], (over, form)
+            assert same(V.cpu().numpy(), ref["V"]) and same(d[over].cpu().numpy(), ref["mu"]), (over, form)
