@@ -134,3 +134,21 @@ def test_batch_tuner_keeps_results():
     res = bf.bf_solve_batch(As, [w.G for w in ws], targets=[w.target for w in ws], avoids=[w.avoid for w in ws])
     for r, s in zip(res, solo):
         assert r["iters"] == s["iters"] and np.array_equal(r["V"], s["V"]) and np.array_equal(r["mu"], s["mu"])
+
+
+def test_batch_of_more_instances_than_one_launch_takes():
+    """131 instances of the one-launch form (a launch takes 128), each equal to its
+    solo solve."""
+    w = wl.unicycle3d(n=(24, 22, 12), n_obstacles=2)
+    A = bf.abs_build_workload(w)
+    rng = np.random.default_rng(8)
+    Gs, tgs = [], []
+    for i in range(131):
+        Gs.append(w.G * (1.0 + 0.25 * (i % 5)))
+        tgs.append((np.roll(w.target, int(rng.integers(0, w.ncells))) & (1 - w.avoid)).astype(np.uint8))
+    res = bf.bf_solve_batch([A] * 131, Gs, targets=tgs, avoids=[w.avoid] * 131)
+    for r, G, tg in zip(res, Gs, tgs):
+        s = bf.bf_solve(A, G, target=tg, avoid=w.avoid)
+        assert s["stats"]["kernel_launches"] == 2
+        assert r["iters"] == s["iters"] and r["status"] == s["status"]
+        assert np.array_equal(r["V"], s["V"]) and np.array_equal(r["mu"], s["mu"])
