@@ -39,10 +39,12 @@ import numpy as np  # noqa: E402
 
 METRIC = "(cell,input) relaxations/s"
 UNIT = "relaxations/s"
-PROFILES = {"unicycle3d": os.path.join(ROOT, "profiles", "k_relax_pq_unicycle3d_200x200x64.txt"),
-            "fire4d": os.path.join(ROOT, "profiles", "k_relax_pq_fire4d_100x100x36x8.txt")}
+# ncu summaries of the relax phase of the one-launch form (what bf_tune picks on
+# these workloads), and the sources they were taken on
+PROFILES = {"unicycle3d": os.path.join(ROOT, "profiles", "k_word_relax_unicycle3d_200x200x64.txt"),
+            "fire4d": os.path.join(ROOT, "profiles", "k_word_relax_fire4d_100x100x36x8.txt")}
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2001_06231_gb300", "csrc", f)
-                  for f in ("solve_core.cuh", "solve.cu", "solve_plane.cu", "bf_internal.cuh", "dynamics.cuh")]
+                  for f in ("word_engine.cuh", "solve_word.cu", "solve_core.cuh", "bf_internal.cuh")]
 FIRE_TARGET_WIDE = ((50.0, 250.0), (50.0, 150.0), (-0.5235987755982988, 0.5235987755982988), (10.0, 15.0))
 
 
@@ -82,10 +84,14 @@ def make_workload(name, rank=0):
     return w, desc
 
 
-def algorithmic_bytes_per_pair(A, masked=False):
+def algorithmic_bytes_per_pair(A, masked=False, one_launch=False):
     """HBM bytes one executed relaxation streams here: its box record + its cost
     (8 B); with the cell masks its cost and a U-th of the cell's 8-byte mask
-    (records only for the few boxes that are not their plane's entry)."""
+    (records only for the few boxes that are not their plane's entry); in the
+    one-launch form on plane lists its cost alone (values, bitmaps and lists
+    stay in the L2)."""
+    if one_launch:
+        return 8
     if masked:
         return 8 + 8.0 / A.ninputs
     return A.box_record_bytes + 8
@@ -326,6 +332,9 @@ def ours(args, rank, world, local_rank):
     for _ in range(args.warmup):
         r = solve()
     launches = r["stats"]["kernel_launches"]
+    # did the solves take the one-launch form?  (its set-up and one launch for all
+    # passes; under the host loop by the schedule)
+    one_launch = launches == 2 or bool(args.host_loop and tuned and tuned.get("one_launch") == 1)
     sampler = ClockSampler(local_rank)
     if dist:
         dist.barrier()
@@ -376,8 +385,8 @@ def ours(args, rank, world, local_rank):
     cbpp = canonical_bytes_per_pair(w.grid.ndim)
     bytes_per_launch = canonical * cbpp / max(1, passes)
     achieved = bytes_per_launch / (relax_ms_avg / 1e3) / 1e9
-    masked = bool(tuned and tuned.get("cell_masks") and tuned.get("plane_lists"))
-    bpp = algorithmic_bytes_per_pair(A, masked)
+    masked = bool(tuned and tuned.get("cell_masks") and tuned.get("plane_lists")) and not one_launch
+    bpp = algorithmic_bytes_per_pair(A, masked, one_launch and A.shape_planes > 0 and A.shape_mismatch == 0)
     exec_bytes_per_launch = executed * bpp / max(1, passes)
     # ncu DRAM bytes of the profiled relax launch, per relaxed (frontier) cell,
     # scaled to this run's mean launch -- only for the kernel sources and relax
@@ -448,15 +457,19 @@ def ours(args, rank, world, local_rank):
                    "schedule": tuned,
                    "builder_boxes_differing_from_oracle": builder_mismatch},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak, "traffic": traffic, "kernel": "k_relax",
+                     "frac": achieved / peak, "traffic": traffic,
+                     "kernel": "k_word_relax (relax phase of k_word_solve)" if one_launch else "k_relax",
                      "peak_source": peak_src, "relax_ms_per_launch": relax_ms_avg,
                      "rest_of_pass_ms_per_launch": prop_ms_avg,
                      "bytes_per_launch": bytes_per_launch,
-                     "bytes_note": "canonical (cell,input) pairs per launch x %d B (%d int16 box corners + FP64 G)" % (
-                         cbpp, 2 * w.grid.ndim),
+                     "bytes_note": "canonical (cell,input) pairs per launch x %d B (%d int16 box corners + FP64 G)%s" % (
+                         cbpp, 2 * w.grid.ndim, ": a rate of work, not of memory; the one-launch form reads no box "
+                         "and takes up few of these pairs" if one_launch else ""),
                      "executed_bytes_per_launch": exec_bytes_per_launch,
                      "executed_frac": exec_bytes_per_launch / (relax_ms_avg / 1e3) / 1e9 / peak,
-                     "executed_bytes_note": ("executed pairs per launch x %.2f B (G 8 B + a %d-th of the "
+                     "executed_bytes_note": "executed pairs per launch x %d B (G 8 B; the pairs whose box holds a "
+                                            "changed and no infinite cell)" % bpp if one_launch and bpp == 8 else
+                                            ("executed pairs per launch x %.2f B (G 8 B + a %d-th of the "
                                              "cell's 8-byte input mask)" % (bpp, U)) if masked else
                                             ("executed pairs per launch x %d B (box record %d B + G 8 B)" % (
                                                 bpp, bpp - 8))},
@@ -798,9 +811,11 @@ def main():
                          "predecessor templates (0/1, default 1), two inputs per relax iteration (0/1, default 0), "
                          "tile relax from this percentage of the cells in F1 (0: never, default), "
                          "one block per SM more for the plane relax (0/1, default 0), "
-                         "per-cell input masks (0/1, default 0: four inputs per iteration with I = 1, else two), "
+                         "per-cell input masks (0/1/2, default 0: four inputs per iteration with I = 1, else two; "
+                         "2: the pairs queued over the lanes), "
                          "plane-pair table dim (0: none, default; 2 .. D - 1), "
-                         "per-input frontier (0/1, default 0) "
+                         "per-input frontier (0/1, default 0), "
+                         "one launch for all passes (0/1, default 0; B is then its width in SMs) "
                          "-- reproduces a tuned schedule under a profiler, "
                          "whose timings would sway bf_tune")
     ap.add_argument("--cpu-budget", type=float, default=15.0)

@@ -852,7 +852,7 @@ extern "C" int bf_solve(const bf_abstraction* a, const double* G, const uint8_t*
     const int U = w->U;
     // plain Jacobi solves of abstractions that have its data take the word engine
     // unless a schedule was set that names another form: with plane lists it was
-    // faster at every size measured, from 0.96 -> 0.50 ms (64 x 64 x 5) to 6.29 -> 2.93 ms
+    // faster at every size measured (planes of 16 to 40,000 cells), from 0.96 -> 0.50 ms (64 x 64 x 5) to 6.29 -> 2.93 ms
     // (100 x 100 x 36 x 8 x 15, against the tuned list form)
     bool one = w->form != 0 && word_takes(a, opts);
     if (one && w->form < 0 && !a->d_vbits && (rc = word_box_pays(a, w, target, avoid, terminal, st, &one))) return rc;

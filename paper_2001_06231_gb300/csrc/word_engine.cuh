@@ -40,7 +40,9 @@
 // What bounds it: latency.  A pass is two grid barriers (2.4 us each) and a chain
 // of about 17 dependent L2 trips; on the fire model's busiest pass the relax phase
 // issues in 40% of the cycles and DRAM is at 9%, tables 35% and 8%.  Solves, list
-// forms in a graph (tuned where noted) -> this, on one GB300:
+// forms in a graph (tuned where noted) -> this, on one GB300 and the inputs of seed
+// 77 of perf/cases.py (another target, obstacles or fires move a case by 2 to 7
+// times, both forms alike):
 //   double integrator    64 x 64 x 5                    0.96 -> 0.50 ms
 //   unicycle             100 x 100 x 32 x 10            2.68 -> 1.28 ms
 //   unicycle             200 x 200 x 64 x 10 (tuned)    3.71 -> 1.89 ms
@@ -434,8 +436,11 @@ __device__ __forceinline__ int word_first(int i) { return (int)((blockIdx.x + 53
 
 // One instance: the block's j-th unit.  The blocks are rotated from one round of
 // units to the next: planes and bands of rows (a plane's units) of every kind
-// come to every block, and the frontier's work with them (without the rotation:
-// 1262 instead of 1202 us at 100 x 100 x 32 x 10, 1302 / 1240 at 61 x 57 x 24 x 6 x 15).
+// come to every block, and the frontier's work with them (without the rotation
+// 1262 instead of 1202 us on a unicycle 100 x 100 x 32 x 10, 1302 / 1240 on a fire
+// model 61 x 57 x 24 x 6 x 15; inputs of another seed than above).  61 and 53: primes
+// that divide neither the 152 SMs nor a share of them (a width they divide is not
+// rotated, nothing else).
 __device__ __forceinline__ int word_mine(const WordInst& w, int j) {
     const unsigned x = blockIdx.x + 61u * (unsigned)j;
     return j * (int)gridDim.x + (int)(x - (unsigned)word_quot(x, w.nb_mul, w.nb_shr) * gridDim.x);
