@@ -414,15 +414,15 @@ BF_API int bf_solve_batch(int32_t n, const bf_abstraction *const *abs, const dou
  * inputs per relax iteration and the relax by cell masks with the pairs queued
  * over the lanes (one at a time, keeping the others at the best so far, two
  * rounds; each candidate solved three times).  Where abstractions have the
- * one-launch form (bf_tune_result.input_frontier) it is timed against list
- * schedules first and the rest is left out when it is the fastest; it is reported
- * as cell_masks 2 with input_frontier 1.  The fastest schedule
+ * one-launch form it is timed against list schedules first and the rest is left
+ * out when it is the fastest (one_launch 1; the other fields are then those of
+ * the instances that lack the form).  The fastest schedule
  * is stored in every given abstraction and used by later bf_solve_batch calls
  * and by the server's engine (a group of instances that share a dimension and
  * storage form takes the schedule of its first instance).  In *out: fuse_mark
  * (-1: by predecessor-box size, the default), window33, plane_lists,
- * templates, pair_inputs, cell_masks (0 or 2), candidates, best_ms and
- * default_ms; the other fields are 0.  Results never depend on the schedule.  Errors: as bf_solve_batch. */
+ * templates, pair_inputs, cell_masks (0 or 2), one_launch, candidates, best_ms
+ * and default_ms; the other fields are 0.  Results never depend on the schedule.  Errors: as bf_solve_batch. */
 BF_API int bf_tune_batch(int32_t n, const bf_abstraction *const *abs, const double *const *G,
                   const uint8_t *const *target, const uint8_t *const *avoid,
                   const double *const *terminal, int64_t max_iters, bf_tune_result *out, void *stream);
@@ -431,8 +431,9 @@ BF_API int bf_tune_batch(int32_t n, const bf_abstraction *const *abs, const doub
  * abstraction without timing: fuse_mark (-1: relax marks when the
  * predecessor boxes are small, 0: a propagate launch, 1: relax marks),
  * window33, plane_lists, templates, pair_inputs, cell_masks (nonzero: the
- * pair-queue relax) and input_frontier (with the three before: the one-launch
- * form, where an abstraction has it) of *sched are read.  The
+ * pair-queue relax) and one_launch (> 0: the one-launch form, where an
+ * abstraction has it; so does input_frontier with plane_lists, templates and
+ * cell_masks) of *sched are read.  The
  * handle is modified; it must not be in use by a running batch or server.
  * Results never depend on the schedule.  Returns BF_OK or BF_ERR_INVALID. */
 BF_API int bf_set_batch_schedule(bf_abstraction *abs, const bf_tune_result *sched);

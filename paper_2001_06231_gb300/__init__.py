@@ -413,12 +413,12 @@ def bf_tune_batch(abstractions, Gs, targets=None, avoids=None, terminals=None, m
 
 
 def bf_set_batch_schedule(abstraction, fuse_mark=-1, window33=1, plane_lists=1, templates=1, pair_inputs=1,
-                          cell_masks=0, input_frontier=0):
+                          cell_masks=0, input_frontier=0, one_launch=0):
     """Put a batched-form schedule in force on this abstraction (no timing)."""
     s = TuneResult()
     s.fuse_mark, s.window33, s.plane_lists, s.templates, s.pair_inputs = (fuse_mark, window33, plane_lists,
                                                                          templates, pair_inputs)
-    s.cell_masks, s.input_frontier = cell_masks, input_frontier
+    s.cell_masks, s.input_frontier, s.one_launch = cell_masks, input_frontier, one_launch
     _check(lib().bf_set_batch_schedule(abstraction.handle, ctypes.byref(s)))
 
 

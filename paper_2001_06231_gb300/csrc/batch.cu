@@ -1102,15 +1102,7 @@ extern "C" int bf_tune_batch(int32_t n, const bf_abstraction* const* abs, const 
     set_all(b);
     const int bs = b;
     memset(out, 0, sizeof *out);
-    if (bs & kBsWords) {
-        // as a schedule: the pair queue with the per-input frontier
-        out->window33 = out->plane_lists = out->templates = out->pair_inputs = out->input_frontier = 1;
-        out->cell_masks = 2;
-        out->candidates = tried;
-        out->best_ms = best;
-        out->default_ms = default_ms;
-        return BF_OK;
-    }
+    out->one_launch = (bs & kBsWords) ? 1 : 0;
     out->fuse_mark = (bs & kBsMarkAuto) ? -1 : ((bs & kBsMark) ? 1 : 0);
     out->window33 = (bs & kBsWindow33) ? 1 : 0;
     out->plane_lists = (bs & kBsPlane) ? 1 : 0;
@@ -1135,7 +1127,9 @@ extern "C" int bf_set_batch_schedule(bf_abstraction* a, const bf_tune_result* sc
     int bs = (sched->window33 ? kBsWindow33 : 0) | (sched->plane_lists ? kBsPlane : 0) |
              (sched->templates ? kBsTemplates : 0) | (sched->pair_inputs ? kBsPair : 0) |
              (sched->cell_masks ? kBsQueue : 0);
-    if (sched->input_frontier && sched->cell_masks && sched->templates && sched->plane_lists) bs |= kBsWords;
+    if (sched->one_launch > 0 ||
+        (sched->input_frontier && sched->cell_masks && sched->templates && sched->plane_lists))
+        bs |= kBsWords;
     if (sched->fuse_mark == 1) bs |= kBsMark;
     if (sched->fuse_mark == -1) bs |= kBsMarkAuto;
     a->bsched = bs;

@@ -152,3 +152,22 @@ def test_batch_of_more_instances_than_one_launch_takes():
         assert s["stats"]["kernel_launches"] == 2
         assert r["iters"] == s["iters"] and r["status"] == s["status"]
         assert np.array_equal(r["V"], s["V"]) and np.array_equal(r["mu"], s["mu"])
+
+
+def test_batch_tuner_reports_what_it_put_in_force():
+    """A mix in which some instances lack the one-launch form: where that form is the
+    fastest, the others keep the default list schedule, the result says both, and
+    put in force on other handles it gives the same results."""
+    ws = [wl.unicycle3d(n=(60, 56, 24), n_obstacles=5, seed=3), wl.di2d(tau=0.3)]
+    args = dict(targets=[w.target for w in ws], avoids=[w.avoid for w in ws])
+    As, Bs = ([bf.abs_build_workload(w) for w in ws] for _ in range(2))
+    t = bf.bf_tune_batch(As, [w.G for w in ws], **args)
+    fields = {k: t[k] for k in ("fuse_mark", "window33", "plane_lists", "templates", "pair_inputs", "cell_masks",
+                                "input_frontier", "one_launch")}
+    if t["one_launch"]:
+        assert fields == dict(fuse_mark=-1, window33=1, plane_lists=1, templates=1, pair_inputs=1, cell_masks=0,
+                              input_frontier=0, one_launch=1)
+    for B in Bs:
+        bf.bf_set_batch_schedule(B, **fields)
+    for a, b in zip(*(bf.bf_solve_batch(H, [w.G for w in ws], **args) for H in (As, Bs))):
+        assert a["iters"] == b["iters"] and np.array_equal(a["V"], b["V"]) and np.array_equal(a["mu"], b["mu"])
